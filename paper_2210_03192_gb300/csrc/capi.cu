@@ -15,6 +15,7 @@
 
 #include "../../include/lx3c.h"
 #include "lx3c_internal.h"
+#include "primitives.h"
 
 namespace lx3c {
 cudaError_t init_constants();
@@ -246,21 +247,31 @@ void split_orientation(const lx3c_basis* orb, int a, int b, int la, int lb, std:
   double ab2 = 0;
   for (int x = 0; x < 3; ++x) ab2 += (A[x] - B[x]) * (A[x] - B[x]);
   const double dab = std::sqrt(ab2);
-  std::vector<double> wgt(Ka * Kb), ampA(Ka * Kb), ampB(Ka * Kb);
-  double wmax = 0;
+  // (small fixed-size arrays: this runs once per shell pair of a plan)
+  double wgt[LX3C_KMAX * LX3C_KMAX], ampA[LX3C_KMAX * LX3C_KMAX], ampB[LX3C_KMAX * LX3C_KMAX];
+  double K[LX3C_KMAX * LX3C_KMAX], q[LX3C_KMAX * LX3C_KMAX];
+  double wmax = 0, qmax = 0;
+  auto ipow = [](double x, int n) {
+    double r = 1.0;
+    for (int i = 0; i < n; ++i) r *= x;
+    return r;
+  };
   for (int ia = 0; ia < Ka; ++ia)
     for (int ib = 0; ib < Kb; ++ib) {
-      double za = orb->exps[orb->off[a] + ia], zb = orb->exps[orb->off[b] + ib], g = za + zb;
-      double w = std::fabs(orb->coefs[orb->off[a] + ia] * orb->coefs[orb->off[b] + ib]) *
-                 std::exp(-za * zb / g * ab2) / g;
-      double sg = 1.0 / std::sqrt(2.0 * g);
-      ampA[ia * Kb + ib] = std::pow((dab + sg) / (za / g * dab + sg), lb);
-      ampB[ia * Kb + ib] = std::pow((dab + sg) / (zb / g * dab + sg), la);
-      wgt[ia * Kb + ib] = w;
-      wmax = std::max(wmax, w);
+      const int r = ia * Kb + ib;
+      const double za = orb->exps[orb->off[a] + ia], zb = orb->exps[orb->off[b] + ib], g = za + zb;
+      q[r] = prim_bound(za, orb->coefs[orb->off[a] + ia], zb, orb->coefs[orb->off[b] + ib], ab2, la, lb, &K[r]);
+      qmax = std::max(qmax, q[r]);
+      if (lb == 0) continue;
+      const double sg = 1.0 / std::sqrt(2.0 * g);
+      ampA[r] = ipow((dab + sg) / (za / g * dab + sg), lb);
+      ampB[r] = ipow((dab + sg) / (zb / g * dab + sg), la);
+      wgt[r] = std::fabs(K[r]) / g;
+      wmax = std::max(wmax, wgt[r]);
     }
   double worstA = 0, worstB = 0;
   for (int r = 0; r < Ka * Kb; ++r) {
+    if (lb == 0 || !prim_kept(K[r], q[r], qmax)) continue;
     double f = wmax > 0 ? wgt[r] / wmax : 1.0;
     worstA = std::max(worstA, ampA[r] * f);
     worstB = std::max(worstB, ampB[r] * f);
@@ -272,6 +283,7 @@ void split_orientation(const lx3c_basis* orb, int a, int b, int la, int lb, std:
   else if (std::min(worstA, worstB) <= kAmpMax) whole = worstB < worstA ? 1 : 0;
   for (int ia = 0; ia < Ka; ++ia)
     for (int ib = 0; ib < Kb; ++ib) {
+      if (!prim_kept(K[ia * Kb + ib], q[ia * Kb + ib], qmax)) continue;
       const bool onB = whole >= 0 ? whole == 1 : orb->exps[orb->off[b] + ib] > orb->exps[orb->off[a] + ia];
       (onB ? primB : primA).push_back(ia * Kb + ib);
     }
@@ -414,6 +426,7 @@ namespace {
 // Fill one launch descriptor for class (l1, l2 | lc) over a sub-pair list.
 lx3c_status make_launch(DevState* ds, lx3c_plan* p, int orient, const std::vector<int4>& sub,
                         const std::vector<int>& prim, int kmax, cudaStream_t st) {
+  kmax = std::max(kmax, 1);
   Launch& L = p->L[orient];
   L.nsub = (long long)sub.size();
   if (L.nsub == 0) return LX3C_OK;
@@ -495,7 +508,8 @@ lx3c_status lx3c_eri3c_plan(lx3c_plan** out, const lx3c_basis* orb, const lx3c_b
     int oa = (int)primA.size(), ob = (int)primB.size();
     split_orientation(orb, pairs[2 * i], pairs[2 * i + 1], la, lb, primA, primB);
     int na = (int)primA.size() - oa, nb = (int)primB.size() - ob;
-    if (na) subA.push_back(int4{(int)i, oa, na, 0});
+    // a pair none of whose primitive pairs contributes: its blocks are zero
+    if (na || !nb) subA.push_back(int4{(int)i, oa, na, na ? 0 : 2});
     if (nb) subB.push_back(int4{(int)i, ob, nb, na > 0 ? 1 : 0});
     kA = std::max(kA, na);
     kB = std::max(kB, nb);
@@ -507,7 +521,8 @@ lx3c_status lx3c_eri3c_plan(lx3c_plan** out, const lx3c_basis* orb, const lx3c_b
     const ClassTables& ta = class_tables(la, lb, lc, p->bra_pure);
     const ClassTables& tb = class_tables(lb, la, lc, p->bra_pure);
     double f = 0;
-    for (auto& s4 : subA) f += ta.flops_prim * s4.z * Kc + ta.flops_contr;
+    for (auto& s4 : subA)
+      if (s4.z) f += ta.flops_prim * s4.z * Kc + ta.flops_contr;
     for (auto& s4 : subB) f += tb.flops_prim * s4.z * Kc + tb.flops_contr;
     p->flops = f * (double)naux;
   }

@@ -200,6 +200,7 @@ struct DfjLaunch {
 struct DfjGroup {
   int la, lb, lc, Ka, Kb, Kc;
   std::vector<int32_t> pairs, auxs, counts;
+  std::vector<int> at;  // position of each pair in its bra class
   long long ntasks = 0;
   double flops = 0, nint = 0;
   int32_t* d_pairs = nullptr;
@@ -392,6 +393,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
         g.pairs.push_back(pl[i].first);
         g.pairs.push_back(pl[i].second);
         g.counts.push_back(lo);
+        g.at.push_back((int)i);
         g.ntasks += lo;
       }
       if (g.counts.empty()) continue;
@@ -400,8 +402,16 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   }
   // contributions per atom to the gradient's fixed-point accumulators
   std::vector<double> fadds(std::max(p->natom, 1), 0.0);
-  // per group: orientation split, tiles, device lists
+  // per group: orientation split (once per bra class: its groups follow one
+  // another), tiles, device lists
+  struct { std::tuple<int, int, int, int> key{-1, 0, 0, 0}; std::vector<std::array<int, 4>> at; std::vector<int> prim[2]; } memo;
   for (auto& g : p->groups) {
+    if (memo.key != std::make_tuple(g.la, g.Ka, g.lb, g.Kb)) {
+      memo.key = std::make_tuple(g.la, g.Ka, g.lb, g.Kb);
+      memo.at.assign(bra[memo.key].size(), {-1, 0, 0, 0});  // first and count of each orientation
+      memo.prim[0].clear();
+      memo.prim[1].clear();
+    }
     const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
     const int nbra = (2 * g.la + 1) * (2 * g.lb + 1), nket = 2 * g.lc + 1;
     g.nint = (double)nbra * nket * (double)g.ntasks;
@@ -410,8 +420,17 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
     int kmax[2] = {0, 0}, cmax = 0;
     for (long long i = 0; i < np; ++i) {
       int oa = (int)prim[0].size(), ob = (int)prim[1].size();
-      split_orientation(orb, g.pairs[2 * i], g.pairs[2 * i + 1], g.la, g.lb, prim[0], prim[1]);
-      int na_ = (int)prim[0].size() - oa, nb_ = (int)prim[1].size() - ob;
+      auto& m = memo.at[g.at[i]];
+      if (m[0] < 0) {
+        m[0] = (int)memo.prim[0].size();
+        m[2] = (int)memo.prim[1].size();
+        split_orientation(orb, g.pairs[2 * i], g.pairs[2 * i + 1], g.la, g.lb, memo.prim[0], memo.prim[1]);
+        m[1] = (int)memo.prim[0].size() - m[0];
+        m[3] = (int)memo.prim[1].size() - m[2];
+      }
+      const int na_ = m[1], nb_ = m[3];
+      prim[0].insert(prim[0].end(), memo.prim[0].begin() + m[0], memo.prim[0].begin() + m[0] + na_);
+      prim[1].insert(prim[1].end(), memo.prim[1].begin() + m[2], memo.prim[1].begin() + m[2] + nb_);
       if (na_) sub[0].push_back(int4{(int)i, oa, na_, 0});
       if (nb_) sub[1].push_back(int4{(int)i, ob, nb_, 0});
       kmax[0] = std::max(kmax[0], na_);

@@ -422,7 +422,15 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
     const int4 sp = __ldg(d.subpairs + sub);
     const long long pair = sp.x;
     const int kab = sp.z, accum = sp.w;
-    if (kab == 0) return;  // a sub-pair without primitive pairs adds nothing (uniform across the CTA)
+    if (kab == 0) {  // (uniform across the CTA)
+      // a sub-pair without primitive pairs adds nothing; its blocks are zero
+      // when the pair has no other sub-pair
+      if (accum == 2 && d.digest == 0) {
+        double* o = d.out + ((pair - d.out_pair0) * d.naux + aux0) * (long long)d.nblk;
+        for (int w = tid; w < tv * d.nblk; w += kThreads) o[w] = 0.0;
+      }
+      return;
+    }
     const int K = kab * d.Kc;
     const int nchunk = (K + G - 1) / G;
     __syncthreads();  // previous tile done with shared memory
@@ -1084,7 +1092,7 @@ __global__ void __launch_bounds__(kSsThreads) eri3c_ss_kernel(const __grid_const
       const long long sub = w / d.naux;
       const long long q = w - sub * d.naux;
       const int4 sp = __ldg(d.subpairs + sub);
-      accum = sp.w;
+      accum = sp.w == 1;
       off = (((long long)sp.x - d.out_pair0) * d.naux + q) * (long long)d.nblk;
       ss_prims<LC>(d, sp.x, sp, q, acc);
     }
@@ -1329,7 +1337,7 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_kernel(const __grid_const
       const long long sub = w / d.naux;
       const long long q = w - sub * d.naux;
       const int4 sp = __ldg(d.subpairs + sub);
-      accum = sp.w;
+      accum = sp.w == 1;
       off = (((long long)sp.x - d.out_pair0) * d.naux + q) * (long long)d.nblk;
       ps_prims<LC>(d, sp.x, sp, q, A, Bm);
       double* row = sG + tid * 3 * (NC + 1);

@@ -51,7 +51,7 @@ struct ClassDesc {
   int orient;
   int onA, onB;            // output block dims of the caller's (la, lb) order
   long long nsub;          // sub-pairs in this launch
-  const int4* subpairs;    // {pair index, first entry in primidx, count, accumulate flag}
+  const int4* subpairs;    // {pair, first entry in primidx, count, 0 store / 1 add / 2 zero blocks}
   const int* primidx;      // primitive-pair indices (ia*Kb + ib) of each sub-pair
   // tiling: a tile is (one sub-pair, T consecutive ket shells of the list)
   int T, Tp, mode;         // mode 0: triple index fastest across lanes; 1: target index fastest
@@ -312,8 +312,9 @@ namespace lx3c {
 // Allocate and fill the device copy of a basis from its host vectors
 // (synchronises st).  No validation: callers check the shell table first.
 int basis_upload(lx3c_basis* b, cudaStream_t st);
-// Orientation of a pair: its primitive pairs go to primA or primB -- all to
-// the orientation with the smaller weighted HRR amplification when that is
+// Orientation of a pair: its contributing primitive pairs (primitives.h; none
+// when every Gaussian product underflows) go to primA or primB -- all to the
+// orientation with the smaller weighted HRR amplification when that is
 // at most the orientation threshold, else each to its more compact centre.
 void split_orientation(const lx3c_basis* orb, int a, int b, int la, int lb, std::vector<int>& primA,
                        std::vector<int>& primB);

@@ -17,6 +17,7 @@
 
 #include "../../include/lx3c.h"
 #include "lx3c_internal.h"
+#include "primitives.h"
 
 namespace lx3c {
 cudaError_t init_constants();
@@ -81,16 +82,19 @@ __global__ void noalloc_orient(const int32_t* __restrict__ pairs, long long npai
   double ab2 = 0;
   for (int x = 0; x < 3; ++x) ab2 += (xyz[3 * sa + x] - xyz[3 * sb + x]) * (xyz[3 * sa + x] - xyz[3 * sb + x]);
   const double dab = sqrt(ab2);
-  double wmax = 0;
+  double wmax = 0, qmax = 0, K;
   for (int ia = 0; ia < ka; ++ia)
     for (int ib = 0; ib < kb; ++ib) {
       const double za = exps[off[sa] + ia], zb = exps[off[sb] + ib], g = za + zb;
       wmax = fmax(wmax, fabs(coefs[off[sa] + ia] * coefs[off[sb] + ib]) * exp(-za * zb / g * ab2) / g);
+      qmax = fmax(qmax, prim_bound(za, coefs[off[sa] + ia], zb, coefs[off[sb] + ib], ab2, la, lb, &K));
     }
   double worstA = 0, worstB = 0;
   for (int ia = 0; ia < ka; ++ia)
     for (int ib = 0; ib < kb; ++ib) {
       const double za = exps[off[sa] + ia], zb = exps[off[sb] + ib], g = za + zb;
+      const double q = prim_bound(za, coefs[off[sa] + ia], zb, coefs[off[sb] + ib], ab2, la, lb, &K);
+      if (!prim_kept(K, q, qmax)) continue;
       const double w = fabs(coefs[off[sa] + ia] * coefs[off[sb] + ib]) * exp(-za * zb / g * ab2) / g;
       const double f = wmax > 0 ? w / wmax : 1.0, sg = 1.0 / sqrt(2.0 * g);
       worstA = fmax(worstA, pow((dab + sg) / (za / g * dab + sg), (double)lb) * f);
@@ -102,11 +106,14 @@ __global__ void noalloc_orient(const int32_t* __restrict__ pairs, long long npai
   int na = 0, nb = 0;
   for (int ia = 0; ia < ka; ++ia)
     for (int ib = 0; ib < kb; ++ib) {
+      const double q = prim_bound(exps[off[sa] + ia], coefs[off[sa] + ia], exps[off[sb] + ib], coefs[off[sb] + ib], ab2,
+                                  la, lb, &K);
+      if (!prim_kept(K, q, qmax)) continue;
       const bool onB = whole >= 0 ? whole == 1 : exps[off[sb] + ib] > exps[off[sa] + ia];
       if (onB) prim[(npair + p) * kab + nb++] = ia * kb + ib;
       else prim[p * kab + na++] = ia * kb + ib;
     }
-  sub[p] = int4{(int)p, (int)(p * kab), na, 0};
+  sub[p] = int4{(int)p, (int)(p * kab), na, na + nb ? 0 : 2};
   sub[npair + p] = int4{(int)p, (int)(p * kab), nb, na > 0 ? 1 : 0};
 }
 
