@@ -235,7 +235,8 @@ lx3c_status lx3c_hrr_tables_check(int la, int lb, int lc, int bra_pure, int vari
  *   and TwoSum) summation in the contracted stages -- bit 0 the n-quantum
  *   CVRR2 gather (Sec. 2.5.4), bit 1 the ket Cartesian-to-solid-harmonic
  *   transform; 0 (the default) for plain FMA chains.  bits outside 0..3 give
- *   LX3C_EINVAL.
+ *   LX3C_EINVAL.  (Both settings act on launches that form integrals; the
+ *   Hermite-basis DF-J and gradient have neither an HRR nor these stages.)
  */
 lx3c_status lx3c_set_orientation_threshold(double amp_max);
 lx3c_status lx3c_set_compensation(int bits);
@@ -277,17 +278,13 @@ lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap
  *   flags LX3C_DFJ_GRADIENT (bit 0): also prepare the nuclear gradient
  *   (lx3c_dfj_grad); needs an atom index on every shell and orbital shells
  *   with l < LX3C_LMAX_ORB.
- *   flags LX3C_DFJ_CONTRACT (bit 1): digest at the (e 0|c) level, the DF-J
- *   analogue of the J-engine the paper names as the follow-up (Sec. 4: the
- *   density is contracted with integral intermediates rather than with the
- *   integrals): per pair launch the bra map M (the HRR and bra transforms,
- *   (AB|C) = sum_e M[AB][e] (e 0|C)) is formed once per pair; per triple
- *   gamma_P = sum_c T_Cc sum_e (M^T D)_e (e 0|c) and y_e += sum_c (e 0|c)
- *   (T^T c_P)_c, then J_AB += M y per pair -- no ket transform, HRR or bra
- *   transform per triple.  A launch keeps the per-integral digestion when its
- *   bra map does not fit in shared memory, or when the contracted form would
- *   take more flops (few kets per pair: the per-pair bra maps cost more than
- *   the per-triple stages they replace).  Same results to rounding.
+ *   flags LX3C_DFJ_CONTRACT (bit 1): contract the density before the
+ *   integrals are formed, the J-engine the paper names as the follow-up
+ *   (Sec. 4).  Every plan does so where it is the faster form: in a Hermite
+ *   Gaussian basis, gamma_P = sum_a H_a (Lambda_a|P) with H the pair's
+ *   density in Hermite Gaussians and J_ab = sum_a E^ab_a sum_P (Lambda_a|P) c_P,
+ *   for all classes but (s s|C) and (p s|C), lc <= 4, whose integrals are
+ *   digested one by one.  The flag is accepted and changes nothing.
  *   Screening: a (pair, ket) triple is kept when Q_ab Q_P >= schwarz_tol, with
  *   Q_ab = 20 sum over primitive pairs of |c_a c_b| exp(-za zb/g AB^2)
  *   sqrt(2 pi^{5/2}/(g^2 sqrt(2g))) (|PA|^2+1/(2g))^{la/2} (|PB|^2+1/(2g))^{lb/2}
@@ -324,10 +321,11 @@ lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap
  *   tile slots of the integral launches (screened triples / slots is the
  *   tile fill).
  * lx3c_dfj_grad: dE/dR for E = c^T gamma with D and c held fixed (not in the
- *   paper): for every screened triple the derivative integrals
- *   d/dA (ab|P) = sum_prim [2 za (a+1 b|P) - a (a-1 b|P)] (same for B) are
- *   formed on the fly in Cartesian-bra classes and contracted with
- *   W = w D_ab c_P; dE/dC = -(dE/dA + dE/dB) (translational invariance).
+ *   paper), in the Hermite Gaussian basis: per screened triple the potential
+ *   y_a = sum_P (Lambda_a|P) c_P up to |a| = la + lb + 1 and the force on the
+ *   ket, -sum_a H_a (Lambda_{a+1}|P) c_P; per pair d/dA phi_a = 2 za phi_{a+1} -
+ *   a phi_{a-1} on the expansion coefficients, and dE/dB from dE/dA + dE/dB +
+ *   dE/dC = 0.
  *   grad (device, natom x 3) overwritten; summed in the same exact fixed
  *   point as gamma and J (bitwise reproducible).
  * lx3c_dfj_group: the screened task list of class group gi (for checks):

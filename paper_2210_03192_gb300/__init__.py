@@ -150,8 +150,8 @@ class DFJPlan:
     """Screened DF-J build (lx3c_dfj): gamma_P and J_mn from D and c, Sec. 3."""
 
     def __init__(self, orb, aux, schwarz_tol=1e-12, gradient=False, contract=False, stream=None):
-        """contract: digest at the (e 0|c) level (LX3C_DFJ_CONTRACT), the DF-J
-        analogue of a J-engine: no ket transform, HRR or bra transform per triple."""
+        """contract (LX3C_DFJ_CONTRACT): contract D and c before integrals are formed;
+        every plan does so where that is faster, so the flag changes nothing."""
         L = _lib.load()
         self.orb = orb if isinstance(orb, DeviceBasis) else DeviceBasis(orb, stream)
         self.aux = aux if isinstance(aux, DeviceBasis) else DeviceBasis(aux, stream)
@@ -430,8 +430,8 @@ class DFJEnergy:
 
     E = DFJEnergy.apply(R, orb, aux, D, c[, tol]) with R [natom, 3] float64
     atom positions (bohr); shells sit on R[atom].  Forward: lx3c_dfj_energy.
-    Backward: lx3c_dfj_grad (adjoint derivative integrals contracted with
-    D_ab c_P on the fly), dE/dR [natom, 3].  D and c are held fixed.
+    Backward: lx3c_dfj_grad (Hermite-basis potentials and forces, no derivative
+    integral is formed), dE/dR [natom, 3].  D and c are held fixed.
     """
 
     @staticmethod

@@ -7,12 +7,14 @@
 //
 // Setup (lx3c_dfj_plan): Schwarz-type screening estimates Q_ab, Q_P; every
 // (la lb | lc) class group keeps its ket shells sorted by Q_P so that the
-// ket shells surviving Q_ab Q_P >= tol for a pair form a prefix of the list;
-// tiles (sub-pair, ket range) are tabulated.  Execution runs the class kernel
-// in digest mode: gamma and J are accumulated from each tile's block in
-// shared memory into exact fixed-point accumulators (fixed128.cuh), so the
-// result does not depend on the order of the contributions; final kernels
-// convert them to FP64 and symmetrise J.
+// ket shells surviving Q_ab Q_P >= tol for a pair form a prefix of the list.
+// Execution: the (s s|C) and (p s|C) groups run the register-resident class
+// kernels in digest mode on tabulated tiles (sub-pair, ket range); all others,
+// and the gradient of every group, run in the Hermite basis (hermite.cu),
+// which forms no integral.  gamma, J and the gradient are accumulated into
+// exact fixed-point accumulators (fixed128.cuh), so the result does not
+// depend on the order of the contributions; final kernels convert them to
+// FP64 and symmetrise J.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,6 +32,7 @@
 
 #include "../../include/lx3c.h"
 #include "fixed128.cuh"
+#include "hermite.h"
 #include "lx3c_internal.h"
 
 namespace lx3c {
@@ -41,8 +44,6 @@ cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st);
 int eri3c_occupancy(int smem_bytes);
 cudaError_t launch_persistent(const ClassDesc* descs, const int2* work, long long nwork, unsigned long long* counter,
                               int grid, int smem_bytes, int three, cudaStream_t st);
-cudaError_t launch_jeng_matrix(const ClassDesc& d, int grid, cudaStream_t st);
-cudaError_t launch_jeng_pair(const ClassDesc& d, int finish, cudaStream_t st);
 int persistent_occupancy(int smem_bytes, int three);
 }  // namespace lx3c
 
@@ -180,15 +181,31 @@ double q_aux(const lx3c_basis* b, int s) { return q_aux_raw(b->l[s], b->k[s], &b
 // dropped triples stay below tol with that margin.
 constexpr double kSchwarzSafety = 20.0;
 
+// Ket shells a pair keeps: the prefix of the list (sorted by decreasing Q_P)
+// with kSchwarzSafety Q_ab Q_P >= tol.
+int kets_kept(double qpair, const std::vector<double>& qket, double tol) {
+  const double thr = qpair > 0 ? tol / (kSchwarzSafety * qpair) : 1e308;
+  int lo = 0, hi = (int)qket.size();
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (qket[mid] >= thr) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// Every group runs in the Hermite basis except those with a register-resident
+// class kernel, (s s|C) and (p s|C) with lc <= 4 (contracted when lc = 0):
+// there the digestion is a few FMAs per contracted triple, where the Hermite
+// form pays its two contractions per primitive triple.
+bool use_hermite(const HermBra& b, const HermKet& k) {
+  if (b.la + b.lb == 0) return false;
+  if (b.la + b.lb == 1) return k.lc > 4 || (k.lc == 0 && b.Ka * b.Kb * k.Kc == 1);
+  return true;
+}
+
 struct DfjLaunch {
   ClassDesc desc;
   int grid = 1;
-  // contraction at the (e 0|c) level (flag LX3C_DFJ_CONTRACT): the digest-5
-  // descriptor, the bra-map pass (one sub-pair per tile, nC = nkrow) and its grid
-  bool jeng = false;
-  ClassDesc jdesc, mdesc;
-  int mgrid = 1;
-  double jflops = 0, pflops = 0;
   long long ntiles = 0;
   int4* d_sub = nullptr;
   int* d_prim = nullptr;
@@ -212,58 +229,10 @@ struct DfjGroup {
   double* d_auxrec = nullptr;
   double* d_auxc = nullptr;
   DfjLaunch L[2];
-  // gradient: derivative classes (centre 0: (la+1,lb) scaled, (la-1,lb);
-  // centre 1: (la,lb+1) scaled, (la,lb-1)), each with two orientations
-  struct Deriv {
-    int centre, plus, l1, l2;
-    DfjLaunch L[2];
-    int4* d_gmap = nullptr;
-  };
-  std::vector<Deriv> deriv;
-  int2* d_pair_atoms = nullptr;
-  int* d_aux_atom = nullptr;
-  double gflops = 0;
+  // the group runs in the Hermite basis; its class launches L serve the
+  // several-density build alone
+  bool herm = false;
 };
-
-// Derivative map for one derivative class (see ClassDesc::gmap).
-std::vector<int4> derivative_map(int la, int lb, int centre, int plus, int gstart[4], int& nmax) {
-  std::vector<std::vector<int4>> byax(3);
-  const int l1 = la + (centre == 0 ? (plus ? 1 : -1) : 0), l2 = lb + (centre == 1 ? (plus ? 1 : -1) : 0);
-  const int ncB = ncart(lb);
-  auto carts = [](int l) {
-    std::vector<std::array<int, 3>> v;
-    for (int x = l; x >= 0; --x)
-      for (int y = l - x; y >= 0; --y) v.push_back({x, y, l - x - y});
-    return v;
-  };
-  auto c1 = carts(l1), c2 = carts(l2);
-  for (size_t i1 = 0; i1 < c1.size(); ++i1)
-    for (size_t i2 = 0; i2 < c2.size(); ++i2)
-      for (int ax = 0; ax < 3; ++ax) {
-        std::array<int, 3> a = c1[i1], b = c2[i2];
-        std::array<int, 3>& moved = centre == 0 ? a : b;
-        int factor;
-        if (plus) {  // (x + 1_ax) present in the block: original x = moved - 1_ax
-          if (moved[ax] < 1) continue;
-          moved[ax] -= 1;
-          factor = 1;
-        } else {     // (x - 1_ax) in the block: original x = moved + 1_ax, factor -x_ax
-          moved[ax] += 1;
-          factor = -moved[ax];
-        }
-        const int ia = cart_index(a[0], a[1], a[2]), ib = cart_index(b[0], b[1], b[2]);
-        byax[ax].push_back(int4{(int)i1, (int)i2, ia * ncB + ib, factor});
-      }
-  std::vector<int4> out;
-  nmax = 0;
-  for (int ax = 0; ax < 3; ++ax) {
-    gstart[ax] = (int)out.size();
-    out.insert(out.end(), byax[ax].begin(), byax[ax].end());
-    nmax = std::max(nmax, (int)byax[ax].size());
-  }
-  gstart[3] = (int)out.size();
-  return out;
-}
 
 }  // namespace
 
@@ -275,18 +244,12 @@ struct lx3c_dfj {
   int natom = 0;
   bool gradient = false;
   std::vector<DfjGroup> groups;
-  double* d_sph = nullptr;          // solid-harmonic matrices for l = 0..7
-  std::vector<int> sph_off;
-  // exact fixed-point accumulators (two words per element): gamma, J, gradient
+  HermPlan* hj = nullptr;           // gamma and J of the Hermite groups
+  HermPlan* hg = nullptr;           // gradient of every group
+  // exact fixed-point accumulators per element: gamma, J, gradient
   unsigned long long* d_gacc = nullptr;
   unsigned long long* d_Jacc = nullptr;
   unsigned long long* d_facc = nullptr;
-  // (e 0|c)-level contraction: bra maps, D through M^T and y, sized for the
-  // largest launch and reused launch after launch
-  bool contract = false;
-  double* d_jM = nullptr;
-  double* d_jD = nullptr;
-  unsigned long long* d_jY = nullptr;
 };
 
 namespace lx3c {
@@ -303,21 +266,12 @@ void lx3c_dfj_destroy(lx3c_dfj* p) {
     for (auto& L : g.L) {
       cudaFree(L.d_sub); cudaFree(L.d_prim); cudaFree(L.d_tiles);
     }
-    for (auto& dv : g.deriv) {
-      cudaFree(dv.d_gmap);
-      for (auto& L : dv.L) {
-        cudaFree(L.d_sub); cudaFree(L.d_prim); cudaFree(L.d_tiles);
-      }
-    }
-    cudaFree(g.d_pair_atoms); cudaFree(g.d_aux_atom);
   }
-  cudaFree(p->d_sph);
+  herm_destroy(p->hj);
+  herm_destroy(p->hg);
   cudaFree(p->d_gacc);
   cudaFree(p->d_Jacc);
   cudaFree(p->d_facc);
-  cudaFree(p->d_jM);
-  cudaFree(p->d_jD);
-  cudaFree(p->d_jY);
   delete p;
 }
 
@@ -329,7 +283,6 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   if (orb->nshell <= 0 || aux->nshell <= 0) return dfail(LX3C_EINVAL, "empty basis");
   if (!(schwarz_tol >= 0.0)) return dfail(LX3C_EINVAL, "negative or NaN tolerance");
   const bool want_grad = (flags & 1) != 0;
-  const bool contract = (flags & 2) != 0;
   for (int64_t s = 0; s < orb->nshell; ++s)
     if (orb->l[s] > LX3C_LMAX_ORB - (want_grad ? 1 : 0))
       return dfail(LX3C_ENOTSUP, "orbital shell beyond the supported l");
@@ -371,27 +324,38 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       bra[key].push_back({s1, s2});
       braq[key].push_back(q_pair(orb, s1, s2));
     }
+  std::vector<HermBra> hbra;
+  std::vector<HermKet> hket;
   for (auto& bk : bra) {
-    const auto& pl = bk.second;
-    const auto& ql = braq[bk.first];
-    for (auto& kk : kets) {
+    HermBra h{std::get<0>(bk.first), std::get<2>(bk.first), std::get<1>(bk.first), std::get<3>(bk.first), {}, {}};
+    for (auto& e : bk.second) {
+      h.pairs.push_back(e.first);
+      h.pairs.push_back(e.second);
+    }
+    h.q = braq[bk.first];
+    hbra.push_back(std::move(h));
+  }
+  for (auto& kk : kets) {
+    HermKet h{kk.first.first, kk.first.second, {}, {}};
+    for (auto& e : kk.second) {
+      h.shells.push_back(e.second);
+      h.q.push_back(e.first);
+    }
+    hket.push_back(std::move(h));
+  }
+  for (auto& hb : hbra) {
+    for (auto& hk : hket) {
       DfjGroup g;
-      g.la = std::get<0>(bk.first); g.Ka = std::get<1>(bk.first);
-      g.lb = std::get<2>(bk.first); g.Kb = std::get<3>(bk.first);
-      g.lc = kk.first.first; g.Kc = kk.first.second;
-      const auto& kl = kk.second;
-      for (auto& e : kl) g.auxs.push_back(e.second);
-      for (size_t i = 0; i < pl.size(); ++i) {
-        const double thr = ql[i] > 0 ? schwarz_tol / (kSchwarzSafety * ql[i]) : 1e308;
-        // number of ket shells with Q_P >= thr (prefix of the sorted list)
-        int lo = 0, hi = (int)kl.size();
-        while (lo < hi) {
-          int mid = (lo + hi) / 2;
-          if (kl[mid].first >= thr) lo = mid + 1; else hi = mid;
-        }
+      g.la = hb.la; g.Ka = hb.Ka;
+      g.lb = hb.lb; g.Kb = hb.Kb;
+      g.lc = hk.lc; g.Kc = hk.Kc;
+      g.herm = use_hermite(hb, hk);
+      g.auxs = hk.shells;
+      for (size_t i = 0; i < hb.q.size(); ++i) {
+        const int lo = kets_kept(hb.q[i], hk.q, schwarz_tol);
         if (lo == 0) continue;
-        g.pairs.push_back(pl[i].first);
-        g.pairs.push_back(pl[i].second);
+        g.pairs.push_back(hb.pairs[2 * i]);
+        g.pairs.push_back(hb.pairs[2 * i + 1]);
         g.counts.push_back(lo);
         g.at.push_back((int)i);
         g.ntasks += lo;
@@ -400,8 +364,14 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       p->groups.push_back(std::move(g));
     }
   }
-  // contributions per atom to the gradient's fixed-point accumulators
-  std::vector<double> fadds(std::max(p->natom, 1), 0.0);
+  rc = herm_build(&p->hj, orb, aux, hbra, hket, use_hermite, kets_kept, schwarz_tol, false, p->nao, st);
+  if (!rc && want_grad)
+    rc = herm_build(&p->hg, orb, aux, hbra, hket, [](const HermBra&, const HermKet&) { return true; }, kets_kept,
+                    schwarz_tol, true, p->nao, st);
+  if (rc) return rc;
+  // contributions to one element of the gradient's fixed-point accumulators
+  if (p->hg && herm_max_adds(p->hg) >= kFixMaxAdds)
+    return dfail(LX3C_ENOTSUP, "gradient: an atom's force accumulator would take 2^32 or more contributions");
   // per group: orientation split (once per bra class: its groups follow one
   // another), tiles, device lists
   struct { std::tuple<int, int, int, int> key{-1, 0, 0, 0}; std::vector<std::array<int, 4>> at; std::vector<int> prim[2]; } memo;
@@ -473,13 +443,15 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       {
         // executed flops: each sub-pair's primitive pairs through this
         // orientation's primitive stages, its contracted stages and the
-        // digestion (4 flops per integral) once per kept ket shell
+        // digestion (4 flops per integral) once per kept ket shell; in the
+        // Hermite basis a fixed count per primitive triple
         double tris = 0, primtris = 0;
         for (auto& sp : sub[o]) {
           tris += g.counts[sp.x];
           primtris += (double)g.counts[sp.x] * sp.z * g.Kc;
         }
-        g.flops += primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nbra * nket);
+        g.flops += g.herm ? primtris * herm_class_flops(g.la + g.lb, g.lc)
+                          : primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nbra * nket);
       }
       std::vector<int4> tiles;
       for (size_t s = 0; s < sub[o].size(); ++s) {
@@ -512,208 +484,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       d.aux_ao = g.d_aux_ao;
       const int occ = eri3c_occupancy(d.smem_doubles * 8);
       L.grid = (int)std::min<long long>(L.ntiles, (long long)dev_nsm(ds) * occ * 8);
-      if (contract) {
-        // the bra-map pass: the class stages with nC = nkrow, one sub-pair per tile
-        ClassTables ctm = *ct;
-        ctm.nC = ct->nkrow;
-        ctm.NV = ctm.NW = ctm.NF = ctm.NACC = 0;
-        ctm.ncc = 0;
-        LaunchShape shm{1, 1, 1, 0};
-        ClassDesc dm;
-        fill_desc_common(dm, ctm, *dc, dev_boys_tab(ds), dev_boys_mid(ds), o, kmax[o], Kab, g.Kc, shm);
-        ClassDesc dj = d;
-        dj.digest = 5;
-        {
-          // the gather output (X region) is live in this epilogue; the P
-          // accumulators before it (Y region) are dead after the gather
-          const long long need = ct->nkrow + 2LL * dj.T * ct->ncc;
-          if (need <= (long long)dj.V.base - dj.P.base) {
-            dj.dscr = dj.P.base;
-          } else {
-            dj.dscr = dj.smem_doubles;
-            dj.smem_doubles += (int)need;
-          }
-        }
-        // flops: per triple the primitive loop, the gather and the two
-        // contractions over (e, c) (plus gamma's ket transform); per sub-pair
-        // the bra map (the HRR and bra stages at nC = nkrow) and two GEMVs
-        const double gather = 2.0 * ct->gterm.size(), ket = 2.0 * ct->kent.size() * ct->nkrow;
-        const double hrrbra = (ct->flops_contr - gather - ket) / ct->nC * ct->nkrow;
-        const double nab = (double)d.onA * d.onB, nk = ct->nkrow;
-        double tris = 0, primtris = 0;
-        for (auto& sp : sub[o]) {
-          tris += g.counts[sp.x];
-          primtris += (double)g.counts[sp.x] * sp.z * g.Kc;
-        }
-        const double jflops = primtris * ct->flops_prim + tris * (gather + 4.0 * nk * ct->ncc + 2.0 * ct->kent.size()) +
-                              (double)d.nsub * (hrrbra + 4.0 * nab * nk);
-        // the same triples digested per integral (what the plain path counts)
-        const double pflops = primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nab * ct->nC);
-        // contract the launch only where that saves work: with few kets per
-        // pair the per-pair bra maps cost more than the per-triple stages
-        // they replace
-        if ((long long)dm.smem_doubles * 8 <= 232448 && (long long)dj.smem_doubles * 8 <= 232448 &&
-            jflops < pflops) {
-          dm.npair = np; dm.naux = na; dm.nsub = d.nsub; dm.subpairs = d.subpairs; dm.pairab = g.d_pairab;
-          L.jeng = true;
-          L.mdesc = dm;
-          L.jdesc = dj;
-          L.mgrid = (int)std::min<long long>(d.nsub, (long long)dev_nsm(ds) * 4);
-          L.jflops = jflops;
-          L.pflops = pflops;
-          p->contract = true;
-        }
-      }
     }
-    if (!want_grad) continue;
-    // ---- gradient launches
-    std::vector<int2> pat(np);
-    std::vector<int> aat(na);
-    for (long long i = 0; i < np; ++i) pat[i] = int2{orb->atom[g.pairs[2 * i]], orb->atom[g.pairs[2 * i + 1]]};
-    for (long long q = 0; q < na; ++q) aat[q] = aux->atom[g.auxs[q]];
-    DCUDA(cudaMalloc(&g.d_pair_atoms, np * sizeof(int2)));
-    DCUDA(cudaMalloc(&g.d_aux_atom, na * 4));
-    DCUDA(cudaMemcpyAsync(g.d_pair_atoms, pat.data(), np * sizeof(int2), cudaMemcpyHostToDevice, st));
-    DCUDA(cudaMemcpyAsync(g.d_aux_atom, aat.data(), na * 4, cudaMemcpyHostToDevice, st));
-    std::vector<double> gket_on_atom(p->natom, 0.0);
-    for (long long q = 0; q < na; ++q)
-      if (aat[q] >= 0) gket_on_atom[aat[q]] += 1.0;
-    for (int centre = 0; centre < 2; ++centre)
-      for (int plus = 1; plus >= 0; --plus) {
-        const int l1 = g.la + (centre == 0 ? (plus ? 1 : -1) : 0), l2 = g.lb + (centre == 1 ? (plus ? 1 : -1) : 0);
-        if (l1 < 0 || l2 < 0) continue;
-        DfjGroup::Deriv dv;
-        dv.centre = centre; dv.plus = plus; dv.l1 = l1; dv.l2 = l2;
-        int gst[4], nmax = 0;
-        std::vector<int4> gmap = derivative_map(g.la, g.lb, centre, plus, gst, nmax);
-        DCUDA(cudaMalloc(&dv.d_gmap, gmap.size() * sizeof(int4)));
-        DCUDA(cudaMemcpyAsync(dv.d_gmap, gmap.data(), gmap.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-        std::vector<int4> dsub[2];
-        std::vector<int> dprim[2];
-        int dk[2] = {0, 0};
-        for (long long i = 0; i < np; ++i) {
-          int oa = (int)dprim[0].size(), ob = (int)dprim[1].size();
-          split_orientation(orb, g.pairs[2 * i], g.pairs[2 * i + 1], l1, l2, dprim[0], dprim[1]);
-          int na_ = (int)dprim[0].size() - oa, nb_ = (int)dprim[1].size() - ob;
-          if (na_) dsub[0].push_back(int4{(int)i, oa, na_, 0});
-          if (nb_) dsub[1].push_back(int4{(int)i, ob, nb_, 0});
-          dk[0] = std::max(dk[0], na_);
-          dk[1] = std::max(dk[1], nb_);
-        }
-        for (int o = 0; o < 2; ++o) {
-          if (dsub[o].empty()) continue;
-          DfjLaunch& L = dv.L[o];
-          const ClassTables* ct;
-          try {
-            ct = &class_tables(o ? l2 : l1, o ? l1 : l2, g.lc, 0);
-          } catch (std::exception& e) {
-            return dfail(LX3C_ENOTSUP, e.what());
-          }
-          DevClass* dc;
-          rc = device_class_get(ds, *ct, &dc);
-          if (rc) return rc;
-          ClassDesc& d = L.desc;
-          if (fill_class_desc(d, *ct, *dc, ds, o, dk[o], Kab, g.Kc, fill_bound(dsub[o], g.counts, cmax)) < 0)
-            return dfail(LX3C_ENOTSUP, "derivative class does not fit in shared memory");
-          {
-            // executed flops of this derivative launch (as for the class
-            // launches) plus its contraction with D, c (2 flops per entry of
-            // the derivative map and ket function)
-            double tris = 0, primtris = 0;
-            for (auto& sp : dsub[o]) {
-              tris += g.counts[sp.x];
-              primtris += (double)g.counts[sp.x] * sp.z * g.Kc;
-            }
-            g.gflops += primtris * ct->flops_prim + tris * (ct->flops_contr + 2.0 * gmap.size() * (2 * g.lc + 1));
-          }
-          // entries per partial sum: balances the partial's FMA chain (E (nC+1))
-          // against the final sum over the nmax / E partials of an axis
-          const int E = std::max(1, std::min(32, (int)std::lround(std::sqrt((double)nmax / (d.nC + 1)))));
-          const int nch = std::max(1, (nmax + E - 1) / E);
-          const int nAp = 2 * g.la + 1, ncA = ncart(g.la), nBp = 2 * g.lb + 1, ncB = ncart(g.lb);
-          d.g_echunk = E;
-          d.g_base = place_epilogue_scratch(d, nAp * ncB + ncA * ncB + (long long)d.T * 3 * (nch + 1));
-          if (d.smem_doubles * 8 > 232448) return dfail(LX3C_ENOTSUP, "gradient epilogue does not fit");
-          d.g_centre = centre;
-          d.g_nAp = nAp; d.g_ncA = ncA; d.g_nBp = nBp; d.g_ncB = ncB; d.g_nch = nch;
-          for (int k = 0; k < 4; ++k) d.gstart[k] = gst[k];
-          d.gmap = dv.d_gmap;
-          std::vector<int4> tiles;
-          for (size_t s2 = 0; s2 < dsub[o].size(); ++s2) {
-            const int pi = dsub[o][s2].x, cnt = g.counts[pi];
-            const int tat = orb->atom[g.pairs[2 * pi + centre]];
-            for (int a0 = 0; a0 < cnt; a0 += d.T) {
-              tiles.push_back(int4{(int)s2, a0, std::min(d.T, cnt - a0), 0});
-              if (tat >= 0) fadds[tat] += 1.0;  // one add per axis per tile
-            }
-          }
-          // one add per triple to the ket shell's atom: at most this
-          // launch's sub-pairs times the group's kets on that atom
-          for (int a = 0; a < p->natom; ++a) fadds[a] += (double)dsub[o].size() * gket_on_atom[a];
-          L.ntiles = (long long)tiles.size();
-          DCUDA(cudaMalloc(&L.d_sub, dsub[o].size() * sizeof(int4)));
-          DCUDA(cudaMalloc(&L.d_prim, std::max<size_t>(dprim[o].size(), 1) * sizeof(int)));
-          DCUDA(cudaMalloc(&L.d_tiles, tiles.size() * sizeof(int4)));
-          DCUDA(cudaMemcpyAsync(L.d_sub, dsub[o].data(), dsub[o].size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-          DCUDA(cudaMemcpyAsync(L.d_prim, dprim[o].data(), dprim[o].size() * sizeof(int), cudaMemcpyHostToDevice, st));
-          DCUDA(cudaMemcpyAsync(L.d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-          d.npair = np; d.naux = na;
-          d.nsub = (long long)dsub[o].size();
-          d.ntiles = L.ntiles;
-          d.ntile_aux = 1;
-          d.tiles = L.d_tiles; d.subpairs = L.d_sub; d.primidx = L.d_prim;
-          d.pairrec = g.d_pairrec; d.pairab = g.d_pairab; d.auxrec = g.d_auxrec; d.auxc = g.d_auxc;
-          d.digest = 2;
-          d.ldD = p->nao;
-          d.pair_ao = g.d_pair_ao; d.aux_ao = g.d_aux_ao;
-          d.pair_atoms = g.d_pair_atoms; d.aux_atom = g.d_aux_atom;
-          const int occ = eri3c_occupancy(d.smem_doubles * 8);
-          L.grid = (int)std::min<long long>(L.ntiles, (long long)dev_nsm(ds) * occ * 8);
-        }
-        g.deriv.push_back(dv);
-      }
-  }
-  if (want_grad && *std::max_element(fadds.begin(), fadds.end()) >= kFixMaxAdds)
-    return dfail(LX3C_ENOTSUP, "gradient: an atom's force accumulator would take 2^32 or more contributions");
-  if (want_grad) {
-    std::vector<double> sph;
-    p->sph_off.assign(9, 0);
-    for (int l = 0; l <= 7; ++l) {
-      auto T = solid_matrix(l);
-      p->sph_off[l] = (int)sph.size();
-      sph.insert(sph.end(), T.begin(), T.end());
-    }
-    p->sph_off[8] = (int)sph.size();
-    DCUDA(cudaMalloc(&p->d_sph, sph.size() * 8));
-    DCUDA(cudaMemcpyAsync(p->d_sph, sph.data(), sph.size() * 8, cudaMemcpyHostToDevice, st));
-    DCUDA(cudaStreamSynchronize(st));
-    for (auto& g : p->groups)
-      for (auto& dv : g.deriv)
-        for (auto& L : dv.L) {
-          L.desc.Ta = p->d_sph + p->sph_off[g.la];
-          L.desc.Tb = p->d_sph + p->sph_off[g.lb];
-        }
-  }
-  if (p->contract) {
-    size_t nm = 1, nd = 1;
-    for (auto& g : p->groups)
-      for (auto& L : g.L)
-        if (L.jeng) {
-          nm = std::max(nm, (size_t)L.desc.nsub * L.desc.onA * L.desc.onB * L.mdesc.nkrow);
-          nd = std::max(nd, (size_t)L.desc.nsub * L.mdesc.nkrow);
-        }
-    DCUDA(cudaMalloc(&p->d_jM, nm * 8));
-    DCUDA(cudaMalloc(&p->d_jD, nd * 8));
-    DCUDA(cudaMalloc(&p->d_jY, nd * kFixBytes));
-    for (auto& g : p->groups)
-      for (auto& L : g.L)
-        if (L.jeng) {
-          for (ClassDesc* d : {&L.mdesc, &L.jdesc}) {
-            d->jM = p->d_jM;
-            d->jD = p->d_jD;
-            d->jY = p->d_jY;
-          }
-        }
   }
   DCUDA(cudaMalloc(&p->d_gacc, (size_t)p->naux_ao * kFixBytes));
   DCUDA(cudaMalloc(&p->d_Jacc, (size_t)p->nao * p->nao * kFixBytes));
@@ -729,33 +500,20 @@ lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, doub
   cudaStream_t st = (cudaStream_t)stream;
   if (gamma) DCUDA(cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, st));
   if (J) DCUDA(cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, st));
+  if (p->hj) DCUDA(herm_execute(p->hj, D, c, gamma ? p->d_gacc : nullptr, J ? p->d_Jacc : nullptr, st));
   for (auto& g : p->groups) {
+    if (g.herm) continue;
     const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
     DCUDA(launch_pair_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, st));
     DCUDA(launch_aux_precompute(p->aux->dev(), g.d_auxs, na, g.Kc, g.d_auxrec, g.d_auxc, st));
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
-      ClassDesc d = L.jeng ? L.jdesc : L.desc;
+      ClassDesc d = L.desc;
       d.D = D;
       d.cvec = c;
       d.gacc = gamma ? p->d_gacc : nullptr;
       d.Jacc = J ? p->d_Jacc : nullptr;
-      if (L.jeng) {
-        // bra maps, D through M^T, the tiles at the (e 0|c) level, then J = M y
-        ClassDesc dm = L.mdesc;
-        dm.D = D;
-        dm.gacc = d.gacc;
-        dm.Jacc = d.Jacc;
-        dm.ldD = d.ldD;
-        dm.pair_ao = d.pair_ao;
-        if (J) DCUDA(cudaMemsetAsync(p->d_jY, 0, (size_t)d.nsub * d.nkrow * kFixBytes, st));
-        DCUDA(launch_jeng_matrix(dm, L.mgrid, st));
-        if (gamma) DCUDA(launch_jeng_pair(dm, 0, st));
-        DCUDA(launch_eri3c(d, L.grid, st));
-        if (J) DCUDA(launch_jeng_pair(dm, 1, st));
-      } else {
-        DCUDA(launch_eri3c(d, L.grid, st));
-      }
+      DCUDA(launch_eri3c(d, L.grid, st));
     }
   }
   if (gamma) DCUDA(launch_fix_finish(p->d_gacc, p->naux_ao, gamma, st));
@@ -828,22 +586,7 @@ lx3c_status lx3c_dfj_grad(lx3c_dfj* p, const double* D, const double* c, double*
   if (!D || !c || !grad) return dfail(LX3C_EINVAL, "null pointer");
   cudaStream_t st = (cudaStream_t)stream;
   DCUDA(cudaMemsetAsync(p->d_facc, 0, (size_t)p->natom * 3 * kFixBytes, st));
-  for (auto& g : p->groups) {
-    const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
-    DCUDA(launch_aux_precompute(p->aux->dev(), g.d_auxs, na, g.Kc, g.d_auxrec, g.d_auxc, st));
-    for (auto& dv : g.deriv) {
-      DCUDA(launch_pair_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, st,
-                                   dv.centre == 0 && dv.plus, dv.centre == 1 && dv.plus));
-      for (auto& L : dv.L) {
-        if (!L.ntiles) continue;
-        ClassDesc d = L.desc;
-        d.D = D;
-        d.cvec = c;
-        d.facc = p->d_facc;
-        DCUDA(launch_eri3c(d, L.grid, st));
-      }
-    }
-  }
+  if (p->hg) DCUDA(herm_gradient(p->hg, D, c, p->d_facc, st));
   DCUDA(launch_fix_finish(p->d_facc, (long long)p->natom * 3, grad, st));
   return LX3C_OK;
 }
@@ -864,22 +607,15 @@ lx3c_status lx3c_schwarz_aux(int l, int k, const double* e, const double* c, dou
 
 lx3c_status lx3c_dfj_info(const lx3c_dfj* p, double* out, int n) {
   if (!p || (!out && n > 0)) return dfail(LX3C_EINVAL, "null pointer");
-  double tasks = 0, nint = 0, flops = 0, launches = 2, gflops = 0, glaunches = p->gradient ? 1 : 0, slots = 0;
+  double tasks = 0, nint = 0, flops = 0, launches = 2, slots = 0;
+  const double gflops = p->hg ? herm_flops(p->hg) : 0, glaunches = p->gradient ? 1 + (p->hg ? herm_launches(p->hg) : 0) : 0;
+  if (p->hj) launches += herm_launches(p->hj);
   for (auto& g : p->groups) {
-    for (auto& L : g.L) {
-      slots += (double)L.ntiles * L.desc.T;
-      if (L.jeng) {
-        flops += L.jflops - L.pflops;
-        launches += 3;  // bra maps, D through M^T, J = M y
-      }
-    }
+    for (auto& L : g.L) slots += (double)L.ntiles * L.desc.T;
     tasks += (double)g.ntasks;
     nint += g.nint;
     flops += g.flops;
-    gflops += g.gflops;
-    launches += 2 + (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
-    if (p->gradient) glaunches += 1;
-    for (auto& dv : g.deriv) glaunches += 1 + (dv.L[0].ntiles > 0) + (dv.L[1].ntiles > 0);
+    if (!g.herm) launches += 2 + (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
   }
   const double v[] = {(double)p->groups.size(), tasks, nint, flops, launches, (double)p->nao, (double)p->naux_ao,
                       (double)p->natom, gflops, glaunches, slots};
@@ -931,11 +667,7 @@ bool retile(DfjLaunch& L, const DfjGroup& g, const DevState* ds, int T) {
   sh.mode = mode;
   ClassDesc nd = d;
   fill_layout(nd, ct, sh);
-  if (d.digest == 2) {
-    nd.g_base = place_epilogue_scratch(nd, d.g_nAp * d.g_ncB + d.g_ncA * d.g_ncB + (long long)T * 3 * d.g_nch);
-  } else if (d.digest == 1) {
-    set_digest_scratch(nd);
-  }
+  set_digest_scratch(nd);
   if ((long long)nd.smem_doubles * 8 > 232448 - 64) return false;
   nd.nchunk = (nd.K + nd.G - 1) / nd.G;
   std::vector<int4> tiles;
@@ -1018,6 +750,7 @@ cudaError_t capture_branches(lx3c_batch* b, const std::vector<ClassDesc>& descs,
       cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
       cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
       for (auto& g : p->groups) {
+        if (g.herm) continue;
         launch_pair_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec,
                                g.d_pairab, cap);
         launch_aux_precompute(p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
@@ -1027,6 +760,22 @@ cudaError_t capture_branches(lx3c_batch* b, const std::vector<ClassDesc>& descs,
     cudaEventRecord(fork, cap);
     double load[kBranches] = {};
     for (int i = 0; i < kBranches; ++i) cudaStreamWaitEvent(br[i], fork, 0);
+    // each molecule's Hermite chain on one branch, the largest first
+    std::vector<int> by(nmol);
+    for (int m = 0; m < nmol; ++m) by[m] = m;
+    std::stable_sort(by.begin(), by.end(), [&](int x, int y) {
+      return (b->mols[x]->hj ? herm_flops(b->mols[x]->hj) : 0) > (b->mols[y]->hj ? herm_flops(b->mols[y]->hj) : 0);
+    });
+    for (int m : by) {
+      lx3c_dfj* p = b->mols[m];
+      if (!p->hj) continue;
+      int k = 0;
+      for (int i = 1; i < kBranches; ++i)
+        if (load[i] < load[k]) k = i;
+      load[k] += herm_flops(p->hj);
+      herm_execute(p->hj, b->D[m], b->c[m], p->d_gacc, p->d_Jacc, br[k]);
+      kernels += herm_launches(p->hj);
+    }
     for (auto& o : order) {
       int k = 0;
       for (int i = 1; i < kBranches; ++i)
@@ -1100,7 +849,7 @@ lx3c_status lx3c_batch_plan(lx3c_batch** out, int nmol, const lx3c_basis* const*
   for (auto* p : b->mols)
     for (auto& g : p->groups)
       for (auto& L : g.L) {
-        if (!L.ntiles) continue;
+        if (!L.ntiles || g.herm) continue;
         const std::string k = shape_key(L.desc);
         auto it = biggest.find(k);
         long long work = (long long)L.desc.T * L.ntiles;
@@ -1182,7 +931,7 @@ lx3c_status lx3c_batch_plan(lx3c_batch** out, int nmol, const lx3c_basis* const*
   for (auto* p : b->mols)
     for (auto& g : p->groups)
       for (auto& L : g.L) {
-        if (!L.ntiles) continue;
+        if (!L.ntiles || g.herm) continue;
         auto it = b->tuned.find(shape_key(L.desc));
         if (it != b->tuned.end() && it->second != L.desc.T) retile(L, g, b->ds, it->second);
       }
@@ -1210,8 +959,9 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
   b->plain_launches = 0;
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];
-    b->plain_launches += 2;
+    b->plain_launches += 2 + (p->hj ? herm_launches(p->hj) : 0);
     for (auto& g : p->groups) {
+      if (g.herm) continue;
       b->plain_launches += 2;
       for (auto& L : g.L) {
         if (!L.ntiles) continue;
@@ -1272,11 +1022,18 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
     cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
     for (auto& g : p->groups) {
+      if (g.herm) continue;
       launch_pair_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec,
                              g.d_pairab, cap);
       launch_aux_precompute(p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
       b->graph_kernels += 2;
     }
+  }
+  for (int m = 0; m < nmol; ++m) {
+    lx3c_dfj* p = b->mols[m];
+    if (!p->hj) continue;
+    herm_execute(p->hj, D[m], c[m], p->d_gacc, p->d_Jacc, cap);
+    b->graph_kernels += herm_launches(p->hj);
   }
   for (size_t t = 0; t < b->tiers.size(); ++t) {
     const auto& T = b->tiers[t];

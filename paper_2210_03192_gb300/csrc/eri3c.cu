@@ -24,6 +24,7 @@
 // memory and no atomics are needed.
 #include <cuda_runtime.h>
 
+#include "boys_device.cuh"
 #include "fixed128.cuh"
 #include "lx3c_internal.h"
 
@@ -40,31 +41,6 @@ struct FDiv {
   // exact for n * d < 2^32
   __device__ __forceinline__ unsigned div(unsigned n) const { return d <= 1u ? n : __umulhi(n, m); }
 };
-
-// 1/sqrt(x) for x > 0 in FP64: single-precision seed, then one Newton-Raphson
-// step carrying the second-order term (y1 = y0 (1 + e/2 + 3e^2/8),
-// e = 1 - x y0^2), which takes the ~1e-7 seed error to FP64 rounding level
-// with five FP64 operations.
-__device__ __forceinline__ double rsqrt_fp64(double x) {
-  float xf = __double2float_rn(x);
-  double y0 = (double)rsqrtf(xf);
-  double t = x * y0;
-  double e = fma(-t, y0, 1.0);
-  double p = fma(e, 0.375, 0.5);
-  double q = y0 * e;
-  return fma(q, p, y0);
-}
-
-// 1/x for x > 0 in FP64: single-precision seed, then two Newton-Raphson steps
-// r <- r (2 - x r) written as e = 1 - x r, r <- r + r e (quadratic
-// convergence: ~1e-7 -> ~1e-14 -> rounding level).
-__device__ __forceinline__ double rcp_fp64(double x) {
-  double r = (double)__frcp_rn(__double2float_rn(x));
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
-}
 
 // Compensated dot product (Ogita, Rump and Oishi's Dot2: TwoProduct by FMA,
 // TwoSum, errors summed separately): about twice the working precision for
@@ -103,38 +79,7 @@ __device__ __forceinline__ void boys_scaled(const double* __restrict__ tab, cons
                                             double cL, int hi, int lo, double T, double pref, double* v,
                                             int stride) {
   double FL, ex;
-  if (T < kBoysTMax) {
-    int i = __float2int_rz(__double2float_rz(T) * (float)kBoysPerUnit);
-    i = min(max(i, 0), kBoysNInt - 1);
-    double dx = T - __ldg(mid + i);
-    const double* c = tab + ((size_t)i * kBoysNF + hi) * 8;
-    const double* ce = tab + ((size_t)i * kBoysNF + (kBoysNF - 1)) * 8;
-    FL = __ldg(c + 7);
-    ex = 0.0;
-    if (hi > lo) {  // exp(-T) only feeds the downward relation
-      ex = __ldg(ce + 7);
-#pragma unroll
-      for (int j = 6; j >= 0; --j) {
-        FL = fma(FL, dx, __ldg(c + j));
-        ex = fma(ex, dx, __ldg(ce + j));
-      }
-    } else {
-#pragma unroll
-      for (int j = 6; j >= 0; --j) FL = fma(FL, dx, __ldg(c + j));
-    }
-  } else {
-    double rs = rsqrt_fp64(T);
-    double b = rcp_fp64(T);
-    double p = rs;
-    int e = hi;
-    while (e) {
-      if (e & 1) p *= b;
-      e >>= 1;
-      if (e) b *= b;
-    }
-    FL = cL * p;
-    ex = 0.0;
-  }
+  boys_top(tab, mid, cL, hi, hi > lo, T, FL, ex);  // exp(-T) only feeds the downward relation
   double G = pref * FL;
   v[(hi - lo) * stride] = G;
   if (hi > lo) {
@@ -244,21 +189,21 @@ __device__ __forceinline__ void dec3(unsigned w, int mode, const FDiv& fT, const
 
 // Segmented dot products out[o] += sum_{r < len} prod(o, r) for o < nout,
 // each partial result handed to emit(o, value), which adds it to global
-// memory with an atomic (whole: one lane per output, each emitted once).  The FP64 pipe charges a whole warp instruction
+// memory with an atomic.  The FP64 pipe charges a whole warp instruction
 // whatever the number of active lanes, and one lane's dependent FMAs are
 // serialised, so the mapping follows the estimated chain length: one lane per
 // output (two partial sums) when there are many outputs, else one warp per
 // (output, 128-term chunk) whose lanes each emit their own partial sum (a warp
 // shuffle reduction here costs the whole kernel registers).
 template <class Prod, class Emit>
-__device__ __forceinline__ void seg_dot(int nout, int len, const Prod& prod, const Emit& emit, bool whole = false) {
+__device__ __forceinline__ void seg_dot(int nout, int len, const Prod& prod, const Emit& emit) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kThreads / 32, kChunk = 128;
   if (nout <= 0 || len <= 0) return;
   const int nch = (len + kChunk - 1) / kChunk;
   const long long lane_steps = (long long)((nout + kThreads - 1) / kThreads) * ((len + 1) / 2);
   const long long warp_steps = (long long)((nout * nch + kWarps - 1) / kWarps) * ((min(len, kChunk) + 31) / 32 + 1);
-  if (whole || lane_steps <= warp_steps) {
+  if (lane_steps <= warp_steps) {
     for (int o = tid; o < nout; o += kThreads) {
       double s0 = 0.0, s1 = 0.0;
       int r = 0;
@@ -391,12 +336,10 @@ __device__ __forceinline__ Buf hrr_and_bra(const ClassDesc& d, double* sm, int T
 }
 
 // One tile: (sub-pair, up to T ket shells) through every stage, ending in the
-// store, the DF-J digestion or the gradient digestion.  kVar selects the
-// instantiation: 0 the plain kernel (store, per-integral DF-J and gradient
-// digestion), 1 adds the several-density digestion on FP64 tensor-core
-// tiles (digest == 4), 2 the contraction at the (e 0|c) level (digest ==
-// 5), each in a kernel of its own so that the plain launches keep their
-// register count.
+// store or the DF-J digestion.  kVar selects the instantiation: 0 the plain
+// kernel (store, per-integral DF-J digestion), 1 adds the several-density
+// digestion on FP64 tensor-core tiles (digest == 4), in a kernel of its own
+// so that the plain launches keep their register count.
 template <int kVar>
 __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, double* sm) {
   const unsigned tid = threadIdx.x;
@@ -667,65 +610,6 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       }
     }
     __syncthreads();
-    if (kVar == 2 && d.digest == 5) {
-      // ---- DF-J contracted at the (e 0|c) level (the analogue of a
-      // J-engine: D and c meet the intermediates, not the integrals).  With
-      // the pair's bra map M (HRR then bra transforms, (AB|C) = sum_e
-      // M[AB][e] (e 0|C)) and the ket transform T, (e 0|C) = sum_c T[C][c] (e 0|c):
-      //   gamma[t][C] = sum_c T[C][c] sum_e Dp[e] (e 0|c)_t,   Dp = w M^T D_pair
-      //   y[e]       += sum_{t,c} (e 0|c)_t cp[t][c],           cp = T^T c_t
-      // and J += wj M y per sub-pair once all its tiles are done
-      // (jeng_finish_kernel).  No ket transform, HRR or bra transform per triple.
-      const int nk = d.nkrow, ncc = d.ncc, nC = d.nC;
-      double* Dp = sm + d.dscr;       // [nk]
-      double* Cp = Dp + nk;           // [tv][ncc]
-      double* gq = Cp + T * ncc;      // [tv][ncc]
-      if (d.gacc)
-        for (int e = tid; e < nk; e += kThreads) Dp[e] = __ldg(d.jD + sub * nk + e);
-      if (d.Jacc)
-        for (int i = tid; i < tv * ncc; i += kThreads) {
-          const int t = i / ncc, c = i - t * ncc;
-          const double* cv = d.cvec + __ldg(d.aux_ao + aux0 + t);
-          double v = 0.0;
-          for (int q = __ldg(d.ktptr + c); q < __ldg(d.ktptr + c + 1); ++q) {
-            const int2 e = __ldg(d.ktent + q);
-            v = fma(__ldg(d.pal + e.y), __ldg(cv + e.x), v);
-          }
-          Cp[i] = v;
-        }
-      __syncthreads();
-      const Buf gb = d.Gb;
-      FDiv fc;
-      fc.init(ncc);
-      if (d.gacc) {
-        seg_dot(tv * ncc, nk,
-                [&](int o, int r, double acc) {
-                  const int t = (int)fc.div(o), c = o - t * ncc;
-                  return fma(sm[BUF_T(gb, r * ncc + c, t)], Dp[r], acc);
-                },
-                [&](int o, double v) { gq[o] = v; }, true);
-        __syncthreads();
-        FDiv fCC;
-        fCC.init(nC);
-        for (int i = tid; i < tv * nC; i += kThreads) {
-          const int t = (int)fCC.div(i), C = i - t * nC;
-          double v = 0.0;
-          for (int q = __ldg(d.kptr + C); q < __ldg(d.kptr + C + 1); ++q) {
-            const int2 e = __ldg(d.kent + q);
-            v = fma(__ldg(d.pal + e.y), gq[t * ncc + e.x], v);
-          }
-          fix_add(d.gacc + kFixWords * (__ldg(d.aux_ao + aux0 + t) + C), v);
-        }
-      }
-      if (d.Jacc)
-        seg_dot(nk, tv * ncc,
-                [&](int o, int r, double acc) {
-                  const int t = (int)fc.div(r), c = r - t * ncc;
-                  return fma(sm[BUF_T(gb, o * ncc + c, t)], Cp[r], acc);
-                },
-                [&](int o, double v) { fix_add(d.jY + kFixWords * (sub * nk + o), v); });
-      return;
-    }
     // ---- ket: Cartesian -> solid harmonic.  With targets across lanes
     // (mode 1) the items run C-major, so a warp's lanes share one C and with
     // it the loop trip count (a warp instruction costs the same whatever the
@@ -783,73 +667,6 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
         const int t = (int)fAC.div(w), r = (int)(w - (unsigned)t * nAC);
         const int A = (int)fC.div(r), C = r - A * nC;
         d.out[(long long)(pao.x + A) * d.ldD + __ldg(d.aux_ao + aux0 + t) + C] = sm[BUF_T(cur, A * nC + C, t)];
-      }
-      return;
-    }
-    if (d.digest == 2) {
-      // ---- gradient digestion: contract the derivative block with
-      // W = w D_ab c_P (Cartesian in the bra) without storing it.
-      const int4 pao = __ldg(d.pair_ao + pair);
-      const int2 pat = __ldg(d.pair_atoms + pair);
-      const double wp = pao.z ? 1.0 : 2.0;
-      const int nAp = d.g_nAp, ncA = d.g_ncA, nBp = d.g_nBp, ncB = d.g_ncB, nC = d.nC, nch = d.g_nch;
-      double* X = sm + d.g_base;     // [nAp][ncB]
-      double* Dc = X + nAp * ncB;    // [ncA][ncB]
-      double* part = Dc + ncA * ncB; // [tv][3][nch]
-      for (int w = tid; w < nAp * ncB; w += kThreads) {
-        const int A = w / ncB, b = w - A * ncB;
-        const double* Drow = d.D + (long long)(pao.x + A) * d.ldD + pao.y;
-        double s = 0.0;
-        for (int B = 0; B < nBp; ++B) s = fma(__ldg(Drow + B), __ldg(d.Tb + B * ncB + b), s);
-        X[w] = s;
-      }
-      __syncthreads();
-      for (int w = tid; w < ncA * ncB; w += kThreads) {
-        const int a = w / ncB, b = w - a * ncB;
-        double s = 0.0;
-        for (int A = 0; A < nAp; ++A) s = fma(__ldg(d.Ta + A * ncA + a), X[A * ncB + b], s);
-        Dc[w] = wp * s;
-      }
-      __syncthreads();
-      const int dnA = d.onA, dnB = d.onB;  // derivative class bra dims, caller order
-      for (int w = tid; w < tv * 3 * nch; w += kThreads) {
-        const int t = w / (3 * nch), rem = w - t * 3 * nch, ax = rem / nch, k = rem - ax * nch;
-        const int e0 = d.gstart[ax] + k * d.g_echunk, e1 = min(d.gstart[ax + 1], e0 + d.g_echunk);
-        const double* cv = d.cvec + __ldg(d.aux_ao + aux0 + t);
-        double s = 0.0;
-        for (int e = e0; e < e1; ++e) {
-          const int4 g = __ldg(d.gmap + e);
-          double tmp = 0.0;
-          for (int C = 0; C < nC; ++C) {
-            const int sidx = d.orient ? (g.y * dnA + g.x) * nC + C : (g.x * dnB + g.y) * nC + C;
-            tmp = fma(__ldg(cv + C), sm[BUF_T(cur, sidx, t)], tmp);
-          }
-          s = fma((double)g.w * Dc[g.z], tmp, s);
-        }
-        part[w] = s;
-      }
-      __syncthreads();
-      const int tatom = d.g_centre ? pat.y : pat.x;
-      double* tsum = part + T * 3 * nch;  // [tv][3]
-      for (int w = tid; w < tv * 3; w += kThreads) {
-        const int t = w / 3, ax = w - t * 3;
-        double s0 = 0.0, s1 = 0.0;
-        int k = 0;
-        for (; k + 1 < nch; k += 2) {
-          s0 += part[(t * 3 + ax) * nch + k];
-          s1 += part[(t * 3 + ax) * nch + k + 1];
-        }
-        if (k < nch) s0 += part[(t * 3 + ax) * nch + k];
-        const double s = s0 + s1;
-        tsum[w] = s;
-        fix_add(d.facc + kFixWords * (3 * __ldg(d.aux_atom + aux0 + t) + ax), -s);
-      }
-      __syncthreads();
-      // the pair's centre atom: the tile's kets summed first, one add per axis
-      if (tid < 3) {
-        double s = 0.0;
-        for (int t = 0; t < tv; ++t) s += tsum[t * 3 + tid];
-        fix_add(d.facc + kFixWords * (3 * tatom + tid), s);
       }
       return;
     }
@@ -1005,13 +822,6 @@ __global__ void __launch_bounds__(kThreads) eri3c_kernel(const __grid_constant__
 __global__ void __launch_bounds__(kThreads) eri3c_multi_kernel(const __grid_constant__ ClassDesc d) {
   extern __shared__ double sm[];
   for (long long tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) tile_body<1>(d, tile, sm);
-}
-
-// DF-J launches contracting at the (e 0|c) level (digest == 5), at the
-// plain kernel's three CTAs per SM.
-__global__ void __launch_bounds__(kThreads, 3) eri3c_contract_kernel(const __grid_constant__ ClassDesc d) {
-  extern __shared__ double sm[];
-  for (long long tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) tile_body<2>(d, tile, sm);
 }
 
 // (s s|C) classes (la = lb = 0) stored per integral, one thread per triple.
@@ -1427,81 +1237,6 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
   }
 }
 
-// The bra map M of every sub-pair of a launch (digest 5): HRR and bra
-// transforms applied to the unit vectors, i.e. the class stages with the nkrow
-// rows of the identity in place of (e 0|C) (the descriptor has nC = nkrow,
-// one "triple" per tile).  M[sub][s][e], s the block's storage index.
-__global__ void __launch_bounds__(kThreads) jeng_matrix_kernel(const __grid_constant__ ClassDesc d) {
-  extern __shared__ double sm[];
-  const unsigned tid = threadIdx.x;
-  const int nk = d.nkrow, nAB = d.onA * d.onB;
-  FDiv fT;
-  fT.init(1);
-  for (long long sub = blockIdx.x; sub < d.nsub; sub += gridDim.x) {
-    const long long pair = __ldg(d.subpairs + sub).x;
-    __syncthreads();
-    if (tid < 13) {
-      const double sg = d.orient ? -1.0 : 1.0;
-      const double x = sg * d.pairab[pair * 3], y = sg * d.pairab[pair * 3 + 1], z = sg * d.pairab[pair * 3 + 2];
-      const int ax = tid >= 1 && tid <= 9 ? (int)(tid - 1) % 3 : 0;
-      const double u = ax == 0 ? x : (ax == 1 ? y : z);
-      double v = 1.0;
-      if (tid >= 1 && tid <= 3) v = u;
-      else if (tid >= 4 && tid <= 6) v = 2.0 * u;
-      else if (tid >= 7 && tid <= 9) v = u * u;
-      else if (tid == 10) v = x * y;
-      else if (tid == 11) v = x * z;
-      else if (tid == 12) v = y * z;
-      sm[d.ab_base + tid] = v;
-    }
-    for (int w = tid; w < nk * nk; w += kThreads) sm[BUF_T(d.H[0], w, 0)] = (w / nk == w % nk) ? 1.0 : 0.0;
-    __syncthreads();
-    const Buf cur = hrr_and_bra(d, sm, 1, 1, 1, fT);
-    double* M = d.jM + sub * (long long)nAB * nk;
-    for (int w = tid; w < nAB * nk; w += kThreads) M[w] = sm[BUF_T(cur, w, 0)];
-  }
-}
-
-// Dp[sub][e] = w sum_s D_s M[sub][s][e] (the pair's D block through M^T),
-// one warp per sub-pair.
-__global__ void jeng_dprime_kernel(const __grid_constant__ ClassDesc d) {
-  const int lane = threadIdx.x & 31;
-  const long long sub = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (sub >= d.nsub) return;
-  const int nk = d.nkrow, nA = d.onA, nB = d.onB, nAB = nA * nB;
-  const long long pair = __ldg(d.subpairs + sub).x;
-  const int4 pao = __ldg(d.pair_ao + pair);
-  const double w = pao.z ? 1.0 : 2.0;
-  const double* M = d.jM + sub * (long long)nAB * nk;
-  for (int e = lane; e < nk; e += 32) {
-    double v = 0.0;
-    for (int s = 0; s < nAB; ++s) {
-      const int A = d.orient ? s % nA : s / nB, B = d.orient ? s / nA : s % nB;
-      v = fma(__ldg(d.D + (long long)(pao.x + A) * d.ldD + pao.y + B), M[s * nk + e], v);
-    }
-    d.jD[sub * nk + e] = w * v;
-  }
-}
-
-// J_pair += wj M y for every sub-pair (y from the fixed-point accumulators),
-// one warp per sub-pair.
-__global__ void jeng_finish_kernel(const __grid_constant__ ClassDesc d) {
-  const int lane = threadIdx.x & 31;
-  const long long sub = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (sub >= d.nsub) return;
-  const int nk = d.nkrow, nA = d.onA, nB = d.onB, nAB = nA * nB;
-  const long long pair = __ldg(d.subpairs + sub).x;
-  const int4 pao = __ldg(d.pair_ao + pair);
-  const double wj = pao.z ? 0.5 : 1.0;
-  const double* M = d.jM + sub * (long long)nAB * nk;
-  for (int s = lane; s < nAB; s += 32) {
-    double v = 0.0;
-    for (int e = 0; e < nk; ++e) v = fma(M[s * nk + e], fix_decode(d.jY + kFixWords * (sub * nk + e)), v);
-    const int A = d.orient ? s % nA : s / nB, B = d.orient ? s / nA : s % nB;
-    fix_add(d.Jacc + kFixWords * ((long long)(pao.x + A) * d.ldD + pao.y + B), wj * v);
-  }
-}
-
 // Persistent form for mixed workloads: every CTA pulls (descriptor, tile)
 // work items from one atomic counter until the list is exhausted (items are
 // ordered longest first on the host).  No CTA ever waits on another.  The
@@ -1592,8 +1327,6 @@ cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(eri3c_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(eri3c_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(eri3c_contract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1649,33 +1382,10 @@ cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
       case 5: eri3c_ss_dfj_kernel<5><<<g, kSsThreads, 0, st>>>(d); break;
       default: eri3c_ss_dfj_kernel<6><<<g, kSsThreads, 0, st>>>(d); break;
     }
-  } else if (d.digest == 5)
-    eri3c_contract_kernel<<<grid, kThreads, (size_t)d.smem_doubles * 8, st>>>(d);
-  else if (d.digest == 4)
+  } else if (d.digest == 4)
     eri3c_multi_kernel<<<grid, kThreads, (size_t)d.smem_doubles * 8, st>>>(d);
   else
     eri3c_kernel<<<grid, kThreads, (size_t)d.smem_doubles * 8, st>>>(d);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_jeng_matrix(const ClassDesc& d, int grid, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(jeng_matrix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  jeng_matrix_kernel<<<grid, kThreads, (size_t)d.smem_doubles * 8, st>>>(d);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_jeng_pair(const ClassDesc& d, int finish, cudaStream_t st) {
-  if (d.nsub == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((d.nsub + 7) / 8);
-  if (finish)
-    jeng_finish_kernel<<<grid, 256, 0, st>>>(d);
-  else
-    jeng_dprime_kernel<<<grid, 256, 0, st>>>(d);
   return cudaGetLastError();
 }
 

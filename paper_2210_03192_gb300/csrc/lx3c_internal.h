@@ -83,8 +83,6 @@ struct ClassDesc {
   const double* pal;       // coefficient palette
   const int* kptr;         // ket CSR by C
   const int2* kent;        // (c, coef_id)
-  const int* ktptr;        // the same transform transposed: CSR by c
-  const int2* ktent;       // (C, coef_id)
   // HRR rows {dst | nterm << 16, src0 | src1 << 16, src2 | src3 << 16, 4-bit
   // codes of the terms' AB-product coefficients}: dst = sum_t coef_t src_t
   const uint4* htab;
@@ -126,18 +124,10 @@ struct ClassDesc {
   // and the tile's c values [tv*nC padded to 4][8] (zero-padded to 8 columns)
   int nd;
   long long dstride, cstride;
-  // digest 1 and 2 add into exact fixed-point accumulators (fixed128.cuh),
-  // two words per element, instead of the FP64 outputs: gamma [naux_ao],
-  // J [nao][nao], gradient [natom][3]; NULL skips that output
+  // digest 1 adds into exact fixed-point accumulators (fixed128.cuh) instead
+  // of the FP64 outputs: gamma [naux_ao], J [nao][nao]; NULL skips that output
   unsigned long long* gacc;
   unsigned long long* Jacc;
-  unsigned long long* facc;
-  // contraction at the (e 0|c) level (digest == 5, the DF-J analogue of a
-  // J-engine): per sub-pair of the launch the bra map M [nAB][nkrow] (HRR and
-  // bra transforms), Dp = w M^T D [nkrow] and the fixed-point y [nkrow]
-  double* jM;
-  double* jD;
-  unsigned long long* jY;
   long long ldD;           // row stride of D and J
   const double* D;
   const double* cvec;
@@ -145,21 +135,6 @@ struct ClassDesc {
   double* J;
   const int4* pair_ao;     // per pair: {ao_a, ao_b, a == b, 0}
   const int* aux_ao;       // per ket-list entry: first AO
-  // Gradient digestion (digest == 2): the block is a Cartesian-bra derivative
-  // class ((la+-1, lb) or (la, lb+-1) in the caller's order); each entry of
-  // gmap = {a', b', index into the Cartesian weight block Dc[a][b], factor}
-  // adds factor * Dc[a][b] * sum_C c_C I[a'][b'][C] to dE/d(centre)_axis;
-  // entries are grouped by axis (gstart[0..3]).
-  int g_centre;            // 0: derivative on the pair's first shell, 1: second
-  int g_nAp, g_ncA, g_nBp, g_ncB, g_nch, g_base;
-  int g_echunk;            // map entries per partial sum (g_nch partials per axis)
-  int gstart[4];
-  const int4* gmap;
-  const double* Ta;        // [2la+1][ncart(la)] of the original la
-  const double* Tb;
-  double* grad;            // [natom][3]
-  const int2* pair_atoms;  // per pair: atoms of the two shells
-  const int* aux_atom;     // per ket-list entry
 };
 
 // Device view of a basis (shell tables in HBM).
@@ -187,8 +162,6 @@ struct ClassTables {
   std::vector<double> pal;
   std::vector<int> kptr;
   std::vector<int2> kent;
-  std::vector<int> ktptr;       // ket transform transposed (CSR by Cartesian c)
-  std::vector<int2> ktent;
   int nkrow;
   int nhrr = 0, hrr2 = 0;      // HRR rounds; 1 if rounds move two quanta (Sec. 2.5.5)
   std::vector<int4> erow_xyz;  // Cartesian exponents of the nkrow round-0 rows
@@ -219,8 +192,6 @@ struct DevClass {
   const double* pal;
   const int* kptr;
   const int2* kent;
-  const int* ktptr;
-  const int2* ktent;
   const uint4* htab;
   const int* baptr;
   const int2* baent;
@@ -248,8 +219,8 @@ void fill_desc_common(ClassDesc& d, const ClassTables& ct, const DevClass& dc, c
                       const double* boys_mid, int orient, int kmax, int Kab_rec, int Kc, const LaunchShape& sh);
 // Device pointers of every class table inside one uploaded blob laid out by
 // class_blob (same offsets on host and device).
-std::vector<char> class_blob(const ClassTables& ct, size_t offs[18]);
-void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t offs[18]);
+std::vector<char> class_blob(const ClassTables& ct, size_t offs[16]);
+void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t offs[16]);
 
 // planner entry points (plan.cu)
 const ClassTables& class_tables(int la, int lb, int lc, int bra_pure);  // HRR variant from the hints
