@@ -499,7 +499,7 @@ void lx3c_batch_destroy(lx3c_batch* batch);
  *                           doubles, same layout as lx3c_eri3c_execute.
  * Everything else the path needs (primitive records, sub-pair lists, Boys
  * and index tables) lives in one statically sized device array of about
- * 27 MB that every GPU loading the library holds until process exit.
+ * 34 MB that every GPU loading the library holds until process exit.
  * Limits: npair <= 65536, npair*ka*kb <= 65536, naux*kc <= 65536; larger
  * problems are rejected with LX3C_ENOTSUP and nothing is launched.
  * First call on a device (once per process and device): it looks up the

@@ -7,7 +7,11 @@
 // m = L-1 .. lc by the downward relation (2m+1) F_m = 2T F_{m+1} + exp(-T),
 // which is stable.  For T >= 117 exp(-T) is negligible next to every
 // F_m (m <= 24) in FP64 and F_L = Gamma(L+1/2)/2 * T^{-(L+1/2)} exactly to
-// FP64, so the same downward relation with exp(-T) = 0 applies.
+// FP64, so the same downward relation with exp(-T) = 0 applies.  That range
+// is tabulated too, on 256 intervals per octave up to 2^24: one FP64
+// instruction costs 64 issue slots, and a separate asymptotic branch (a root,
+// a reciprocal and powers, 16 instructions) was paid by nearly every warp,
+// whose kets lie on both sides of 117.
 //
 // Reference values for the fit: F_m(T) = exp(-T) sum_i (2T)^i /
 // ((2m+1)(2m+3)...(2m+2i+1)), a series of positive terms, summed in long double.
@@ -34,52 +38,87 @@ double boys_large_const(int L) {
   return (double)(g / 2.0L);
 }
 
+namespace {
+
+// Monomial coefficients, in powers of T - c, of the Chebyshev interpolant of a
+// function given by its values fk at the nodes c + h cos(pi (k + 1/2) / n).
+struct ChebFit {
+  static constexpr int n = kBoysDeg + 1;
+  long double x[n], cs[n][n], mono[n][n];  // nodes; T_j at the nodes; T_j in monomials
+  ChebFit() {
+    const long double pi = 3.14159265358979323846264338327950288L;
+    for (int k = 0; k < n; ++k) x[k] = std::cos(pi * (k + 0.5L) / n);
+    for (int j = 0; j < n; ++j)
+      for (int k = 0; k < n; ++k) {
+        cs[j][k] = std::cos(pi * j * (k + 0.5L) / n);
+        mono[j][k] = 0;
+      }
+    mono[0][0] = 1;
+    mono[1][1] = 1;
+    for (int j = 2; j < n; ++j)
+      for (int k = 0; k < n; ++k) mono[j][k] = -mono[j - 2][k] + (k > 0 ? 2 * mono[j - 1][k - 1] : 0);
+  }
+  void operator()(const long double* fk, long double h, double* out) const {
+    long double m[n] = {0};
+    for (int j = 0; j < n; ++j) {
+      long double s = 0;
+      for (int k = 0; k < n; ++k) s += fk[k] * cs[j][k];
+      s *= (j ? 2.0L : 1.0L) / n;
+      for (int k = 0; k <= j; ++k) m[k] += s * mono[j][k];
+    }
+    long double sc = 1;
+    for (int k = 0; k < n; ++k) {
+      out[k] = (double)(m[k] / sc);
+      sc *= h;
+    }
+  }
+};
+
+}  // namespace
+
 // tab[(i*kBoysNF + f)*8 + j]: coefficient of (T - mid_i)^j for function f
-// (f <= kBoysMmax: F_f, f = kBoysMmax+1: exp(-T)) on interval i.
+// (f <= kBoysMmax: F_f, f = kBoysMmax+1: exp(-T)) on interval i; intervals of
+// width 1/8 up to 117, then those of kBoysOct per octave.
 void boys_tables(std::vector<double>& tab, std::vector<double>& mid) {
-  const int n = kBoysDeg + 1;
+  const ChebFit fit;
+  const int n = ChebFit::n;
   tab.assign((size_t)kBoysNInt * kBoysNF * 8, 0.0);
   mid.assign(kBoysNInt, 0.0);
-  const long double pi = 3.14159265358979323846264338327950288L;
   const long double h = 0.5L / kBoysPerUnit;  // half width
-  for (int i = 0; i < kBoysNInt; ++i) {
-    long double c = (i + 0.5L) / kBoysPerUnit;
+  for (int i = 0; i < kBoysNLin; ++i) {
+    const long double c = (i + 0.5L) / kBoysPerUnit;
     mid[i] = (double)c;
-    long double xk[n], Tk[n];
-    for (int k = 0; k < n; ++k) {
-      xk[k] = std::cos(pi * (k + 0.5L) / n);
-      Tk[k] = c + h * xk[k];
-    }
     for (int f = 0; f < kBoysNF; ++f) {
       long double fk[n];
-      for (int k = 0; k < n; ++k) fk[k] = (f <= kBoysMmax) ? boys_ref(f, Tk[k]) : std::exp(-Tk[k]);
-      // Chebyshev coefficients of the interpolant
-      long double cc[n];
-      for (int j = 0; j < n; ++j) {
-        long double s = 0;
-        for (int k = 0; k < n; ++k) s += fk[k] * std::cos(pi * j * (k + 0.5L) / n);
-        cc[j] = s * 2.0L / n;
-      }
-      cc[0] *= 0.5L;
-      // monomial coefficients in x = (T - c)/h: sum_j cc_j T_j(x)
-      long double mono[n] = {0}, tm2[n] = {0}, tm1[n] = {0}, tcur[n];
-      tm2[0] = 1;  // T_0
-      tm1[1] = 1;  // T_1
-      for (int k = 0; k < n; ++k) mono[k] += cc[0] * tm2[k];
-      if (n > 1)
-        for (int k = 0; k < n; ++k) mono[k] += cc[1] * tm1[k];
-      for (int j = 2; j < n; ++j) {
-        for (int k = 0; k < n; ++k) tcur[k] = -tm2[k] + (k > 0 ? 2 * tm1[k - 1] : 0);
-        for (int k = 0; k < n; ++k) mono[k] += cc[j] * tcur[k];
-        for (int k = 0; k < n; ++k) { tm2[k] = tm1[k]; tm1[k] = tcur[k]; }
-      }
-      // rescale to powers of (T - c)
-      long double sc = 1;
-      for (int k = 0; k < n; ++k) {
-        tab[((size_t)i * kBoysNF + f) * 8 + k] = (double)(mono[k] / sc);
-        sc *= h;
+      for (int k = 0; k < n; ++k) fk[k] = (f <= kBoysMmax) ? boys_ref(f, c + h * fit.x[k]) : std::exp(-(c + h * fit.x[k]));
+      fit(fk, h, &tab[((size_t)i * kBoysNF + f) * 8]);
+    }
+  }
+  // T >= 117: F_f(4 T) = F_f(T) 2^{-(2f+1)}, so two octaves give all
+  const long double spi = std::sqrt(3.14159265358979323846264338327950288L);
+  std::vector<double> base((size_t)2 * kBoysOct * (kBoysMmax + 1) * 8);
+  for (int j = 0; j < 2 * kBoysOct; ++j) {
+    const long double w = j < kBoysOct ? 64.0L / kBoysOct : 128.0L / kBoysOct;
+    const long double c = (j < kBoysOct ? 64.0L : 128.0L) + (j % kBoysOct + 0.5L) * w;
+    long double F[kBoysMmax + 1][n];
+    for (int k = 0; k < n; ++k) {
+      const long double T = c + 0.5L * w * fit.x[k];
+      long double v = 0.5L * spi / std::sqrt(T);
+      for (int f = 0; f <= kBoysMmax; ++f) {
+        F[f][k] = v;
+        v *= (f + 0.5L) / T;
       }
     }
+    for (int f = 0; f <= kBoysMmax; ++f) fit(F[f], 0.5L * w, &base[((size_t)j * (kBoysMmax + 1) + f) * 8]);
+  }
+  for (int i = kBoysNLin; i < kBoysNInt; ++i) {
+    const int j = i - kBoysNLin + kBoysOctFirst, oct = j / kBoysOct, s = oct & ~1;  // T = 2^s x base T
+    const int bj = (oct & 1) * kBoysOct + j % kBoysOct;
+    mid[i] = std::ldexp((64.0 + (j % kBoysOct + 0.5) * (64.0 / kBoysOct)), oct);
+    for (int f = 0; f <= kBoysMmax; ++f)
+      for (int k = 0; k < n; ++k)
+        tab[((size_t)i * kBoysNF + f) * 8 + k] =
+            std::ldexp(base[((size_t)bj * (kBoysMmax + 1) + f) * 8 + k], -(s * (f + k) + s / 2));
   }
 }
 

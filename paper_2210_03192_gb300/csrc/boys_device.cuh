@@ -15,13 +15,24 @@ static __constant__ double c_inv[48] = {
     1.0 / 30, 1.0 / 31, 1.0 / 32, 1.0 / 33, 1.0 / 34, 1.0 / 35, 1.0 / 36, 1.0 / 37, 1.0 / 38, 1.0 / 39,
     1.0 / 40, 1.0 / 41, 1.0 / 42, 1.0 / 43, 1.0 / 44, 1.0 / 45, 1.0 / 46, 1.0 / 47};
 
+// FP64 <-> FP32 by shifting bits: the conversion instructions run at the FP64
+// rate (17 SM clocks per warp, measured), these in the integer pipe.  Values
+// outside the float range saturate to infinity and to zero.
+__device__ __forceinline__ float to_float_bits(double x) {  // x >= 0, truncated
+  const int hi = min(max(__double2hiint(x), 0x38000000), 0x47F00000);
+  return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)(hi - 0x38000000), 3));
+}
+__device__ __forceinline__ double to_double_bits(float y) {  // y > 0, or 0
+  const int b = __float_as_int(y);
+  return __hiloint2double(b ? (b >> 3) + 0x38000000 : 0, b << 29);
+}
+
 // 1/sqrt(x) for x > 0 in FP64: single-precision seed, then one Newton-Raphson
 // step carrying the second-order term (y1 = y0 (1 + e/2 + 3e^2/8),
 // e = 1 - x y0^2), which takes the ~1e-7 seed error to FP64 rounding level
 // with five FP64 operations.
 __device__ __forceinline__ double rsqrt_fp64(double x) {
-  float xf = __double2float_rn(x);
-  double y0 = (double)rsqrtf(xf);
+  double y0 = to_double_bits(rsqrtf(to_float_bits(x)));
   double t = x * y0;
   double e = fma(-t, y0, 1.0);
   double p = fma(e, 0.375, 0.5);
@@ -29,34 +40,29 @@ __device__ __forceinline__ double rsqrt_fp64(double x) {
   return fma(q, p, y0);
 }
 
-// F_hi(T) and, when want_ex, exp(-T) for the downward relation: interpolation
-// table for T < 117, else the asymptotic form with exp(-T) = 0.
+// F_hi(T) and, when want_ex, exp(-T) for the downward relation, by degree-7
+// interpolation: the interval from the bits of T (floor(8 T) below 117, the
+// top mantissa bits up to 2^24), the asymptotic form with exp(-T) = 0 beyond.
 __device__ __forceinline__ void boys_top(const double* __restrict__ tab, const double* __restrict__ mid, double cL,
                                          int hi, bool want_ex, double T, double& FL, double& ex) {
+  constexpr int kHi117 = 0x405D4000, kHi24 = 0x41700000;  // high words of 117 and 2^24
+  const int h = __double2hiint(T);
   ex = 0.0;
-  if (T < kBoysTMax) {
-    int i = __float2int_rz(__double2float_rz(T) * (float)kBoysPerUnit);
-    i = min(max(i, 0), kBoysNInt - 1);
+  if (h < kHi24) {
+    const int lin = ((h & 0xFFFFF) | 0x100000) >> min(1040 - (h >> 20), 31);
+    const int i = h < kHi117 ? lin : kBoysNLin + ((h >> 12) - (kHi117 >> 12));
     const double dx = T - __ldg(mid + i);
-    const double* c = tab + ((size_t)i * kBoysNF + hi) * 8;
-    const double* ce = tab + ((size_t)i * kBoysNF + (kBoysNF - 1)) * 8;
-    FL = __ldg(c + 7);
+    const double2* c = reinterpret_cast<const double2*>(tab + ((size_t)i * kBoysNF + hi) * 8);
+    const double2* ce = reinterpret_cast<const double2*>(tab + ((size_t)i * kBoysNF + (kBoysNF - 1)) * 8);
+    const double2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2), c3 = __ldg(c + 3);
+    FL = fma(fma(fma(fma(fma(fma(fma(c3.y, dx, c3.x), dx, c2.y), dx, c2.x), dx, c1.y), dx, c1.x), dx, c0.y), dx, c0.x);
     if (want_ex) {
-      ex = __ldg(ce + 7);
-#pragma unroll
-      for (int j = 6; j >= 0; --j) {
-        FL = fma(FL, dx, __ldg(c + j));
-        ex = fma(ex, dx, __ldg(ce + j));
-      }
-    } else {
-#pragma unroll
-      for (int j = 6; j >= 0; --j) FL = fma(FL, dx, __ldg(c + j));
+      const double2 e0 = __ldg(ce), e1 = __ldg(ce + 1), e2 = __ldg(ce + 2), e3 = __ldg(ce + 3);
+      ex = fma(fma(fma(fma(fma(fma(fma(e3.y, dx, e3.x), dx, e2.y), dx, e2.x), dx, e1.y), dx, e1.x), dx, e0.y), dx, e0.x);
     }
   } else {
     const double rs = rsqrt_fp64(T);
-    // 1/T from the root, one Newton step (a fresh reciprocal costs twice the
-    // instructions, and most warps hold lanes on both sides of 117)
-    double b = rs * rs;
+    double b = rs * rs;  // 1/T, one Newton step from the root
     b = fma(b, fma(-T, b, 1.0), b);
     double p = rs;
     int e = hi;

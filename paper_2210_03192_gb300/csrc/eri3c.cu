@@ -852,7 +852,7 @@ __device__ __forceinline__ void ss_prims(const ClassDesc& d, long long pair, con
       const double rs = rsqrt_fp64(sg);
       const double r = rs * rs;
       const double gr = gam * r;
-      const double Tb = gam * zc * r * pc2;
+      const double Tb = gr * zc * pc2;
       double V;
       boys_scaled(d.boys_tab, d.boys_mid, d.boys_cL, LC, LC, Tb, K * ccp * rs, &V, 0);
       if (LC == 0) {
@@ -1016,7 +1016,7 @@ __device__ __forceinline__ void ps_prims(const ClassDesc& d, long long pair, con
       const double rs = rsqrt_fp64(sg);
       const double r = rs * rs;
       const double gr = gam * r, rg = zc * r;
-      const double Tb = gam * zc * r * pc2;
+      const double Tb = gr * zc * pc2;
       double v2[2];
       boys_scaled(d.boys_tab, d.boys_mid, d.boys_cL, LC + 1, LC, Tb, K * ccp * rs, v2, 1);
       const double V0 = v2[0];

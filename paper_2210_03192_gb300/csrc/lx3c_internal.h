@@ -17,8 +17,10 @@ constexpr int kAuxRec = 2;               // doubles per ket primitive record: ze
 constexpr int kBoysMmax = 24;            // Boys table covers F_0..F_24
 constexpr int kBoysNF = kBoysMmax + 2;   // functions per interval: F_0..F_24, exp(-T)
 constexpr int kBoysPerUnit = 8;          // intervals per unit of T (width 1/8)
-constexpr int kBoysNInt = 117 * kBoysPerUnit;
-constexpr double kBoysTMax = 117.0;
+constexpr int kBoysNLin = 117 * kBoysPerUnit;  // intervals up to T = 117
+constexpr int kBoysOct = 256;            // intervals per octave beyond, up to T = 2^24
+constexpr int kBoysOctFirst = 212;       // 117 = (1 + 212/256) 64
+constexpr int kBoysNInt = kBoysNLin + 18 * kBoysOct - kBoysOctFirst;
 constexpr int kBoysDeg = 7;              // degree of the interpolating polynomial (Sec. 2.5.2)
 constexpr double kDefaultAmpMax = 300.0; // orientation: largest weighted HRR amplification kept unsplit
 

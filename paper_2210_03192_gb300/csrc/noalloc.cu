@@ -51,7 +51,7 @@ constexpr size_t kOffPrim = align256(kOffSub + sizeof(int4) * 2 * kMaxPairs);
 constexpr size_t kOffBoys = align256(kOffPrim + sizeof(int) * 2 * kMaxPrimPairs);
 constexpr size_t kOffBoysMid = align256(kOffBoys + sizeof(double) * kBoysNInt * kBoysNF * 8);
 constexpr size_t kOffTables = align256(kOffBoysMid + sizeof(double) * kBoysNInt);
-constexpr size_t kScratchBytes = align256(kOffTables + kTableBytes);  // about 27 MB
+constexpr size_t kScratchBytes = align256(kOffTables + kTableBytes);  // about 34 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
