@@ -11,12 +11,13 @@
 //   lx3c_dfj_coulomb          gamma -> c = V^{-1} gamma -> J in one call
 //
 // Cholesky kernels (row-major, lower triangle; the strictly upper triangle is
-// never written):
-//   chol_diag    one CTA factors the nb x nb diagonal block in shared memory
-//   chol_trsm    rows below it: L21 = A21 L11^{-T}, one thread per row
-//   chol_update  A22 -= L21 L21^T on 128 x 128 tiles of the lower triangle,
-//                8 x 8 FMA accumulators per thread (the FP64 pipe, not shared
-//                memory or HBM, bounds this GEMM on GB300)
+// never written), panels of 32 columns:
+//   factor_diag  one CTA factors the 32 x 32 diagonal block, a row per lane
+//   chol_trsm    rows below it: L21 = A21 L11^{-T}, a row per lane
+//   chol_update  A22 -= L21 L21^T on 64 x 64 (few left: 32 x 32) tiles of the
+//                lower triangle, the accumulators in registers (the FP64 pipe,
+//                not shared memory or HBM, bounds this GEMM on GB300); the CTA
+//                of the first tile goes on to factor the next diagonal block
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,6 +29,7 @@
 #include <vector>
 
 #include "../../include/lx3c.h"
+#include "boys_device.cuh"
 #include "lx3c_internal.h"
 
 namespace lx3c {
@@ -54,217 +56,332 @@ lx3c_status mfail(lx3c_status s, const std::string& m) {
     if (e_ != cudaSuccess) return mfail(LX3C_ECUDA, std::string(#expr) + ": " + cudaGetErrorString(e_));   \
   } while (0)
 
-constexpr int kNB = 64;        // panel width of the Cholesky and the solves
-constexpr int kTile = 128;     // trailing-update tile
-constexpr int kLd = kTile + 1; // padded shared-memory row of the update operands
-constexpr int kTrsmRows = 128; // rows per CTA of the panel solve
+// Each of an SM's four sub-partitions issues one FP64 warp instruction per 64
+// clocks, whether or not it depends on the last one (measured), so four warps
+// share each serial part and every FP64 instruction of a column's chain
+// counts: five for the reciprocal root, a product, an FMA.  32 columns take 12
+// us (a 64-wide panel by one CTA with a root, a division and two block
+// barriers per column took 110 us), and hide behind the update.  64 x 64 tiles
+// replace 128 x 128 ones, which kept an SM busy for 250 us and left half the
+// chip idle in matrices of a few thousand rows.
+constexpr int kNB = 32;        // panel width of the Cholesky
+constexpr int kSB = 64;        // block of the triangular solves
 
 // ---------------------------------------------------------------------------
 // Cholesky
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) chol_diag(double* __restrict__ A, long long lda, long long k, int nb,
-                                                 int* __restrict__ info, const double* __restrict__ diag0,
-                                                 double drop_tol) {
-  __shared__ double s[kNB][kNB + 1];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < nb * nb; idx += 256) {
-    const int i = idx / nb, j = idx - i * nb;
-    s[i][j] = j <= i ? A[(k + i) * lda + k + j] : 0.0;
-  }
-  __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    if (tid == 0) {
-      double dj = s[j][j];
-      if (diag0) {
-        // drop mode: a pivot at or below drop_tol of the original diagonal
-        // marks a function dependent on the earlier ones; an infinite pivot
-        // zeroes its column below and its coefficient in the solves
-        if (!(dj > drop_tol * diag0[k + j])) {
-          if (info) ++*info;
-          s[j][j] = __longlong_as_double(0x7FF0000000000000LL);
-        } else {
-          s[j][j] = sqrt(dj);
-        }
-      } else {
-        if (!(dj > 0.0)) {  // not positive definite: record the first such pivot, carry NaN on
-          if (info && *info == 0) *info = (int)(k + j + 1);
-          dj = nan("");
-        }
-        s[j][j] = sqrt(dj);
-      }
-    }
-    __syncthreads();
-    const double piv = s[j][j];
-    for (int i = j + 1 + tid; i < nb; i += 256) s[i][j] /= piv;
-    __syncthreads();
-    const int m = nb - j - 1;
-    for (int idx = tid; idx < m * m; idx += 256) {
-      const int r = idx / m, c = idx - r * m;
-      if (c <= r) s[j + 1 + r][j + 1 + c] = fma(-s[j + 1 + r][j], s[j + 1 + c][j], s[j + 1 + r][j + 1 + c]);
-    }
-    __syncthreads();
-  }
-  for (int idx = tid; idx < nb * nb; idx += 256) {
-    const int i = idx / nb, j = idx - i * nb;
-    if (j <= i) A[(k + i) * lda + k + j] = s[i][j];
-  }
+struct CholMode {
+  int* info;
+  const double* diag0;  // drop mode: the original diagonal
+  double drop_tol;
+};
+
+__device__ __forceinline__ bool is_zero(double x) {  // integer pipe: an FP64 compare costs 64 clocks
+  return (__double2hiint(x) << 1 | __double2loint(x)) == 0;
 }
 
-// Rows r0 .. r0+kTrsmRows-1 (r0 = k + nb + blockIdx.x * kTrsmRows) of the
-// panel: x L11^T = a, i.e. forward substitution with L11 per row.
-__global__ void __launch_bounds__(kTrsmRows) chol_trsm(double* __restrict__ A, long long lda, long long k, int nb,
-                                                       long long n) {
-  extern __shared__ double sm[];
-  double* L = sm;                     // [kNB][kNB + 1]
-  double* X = sm + kNB * (kNB + 1);   // [kTrsmRows][kNB + 1]
-  const int tid = threadIdx.x;
+// 1/sqrt of the pivot d of column g.  Dropped functions give 0 and a diagonal
+// that is not positive gives NaN; d becomes the square of the factor's diagonal
+// element in either case.
+__device__ __forceinline__ double pivot_rsqrt(const CholMode& m, long long g, double& d, bool lead) {
+  const int h = __double2hiint(d);
+  if (m.diag0) {
+    // drop mode: a pivot at or below drop_tol of the original diagonal marks
+    // a function dependent on the earlier ones; an infinite pivot zeroes its
+    // column below and its coefficient in the solves
+    if (!(d > m.drop_tol * m.diag0[g])) {
+      if (lead && m.info) ++*m.info;
+      d = __longlong_as_double(0x7FF0000000000000LL);
+      return 0.0;
+    }
+  }
+  if (h > 0x38800000 && h < 0x47800000) return rsqrt_fp64(d);  // the range of its FP32 seed
+  if (!(d > 0.0)) {  // not positive definite: record the first such pivot, carry NaN on
+    if (lead && m.info && *m.info == 0) *m.info = (int)(g + 1);
+    d = nan("");
+  }
+  return 1.0 / sqrt(d);
+}
+
+// Factor the nb x nb block at A[k][k] (nb <= 32) with 128 threads: lane i
+// holds row i, warp w its columns w, w + 4, ...  The warp of the next column
+// updates it first and publishes it before its other updates.
+__device__ __forceinline__ void factor_diag(double* A, long long lda, long long k, int nb, const CholMode& mode,
+                                            double (*s)[kNB + 1], double (*col)[kNB]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = warp; i < kNB; i += 4)
+    s[i][lane] = i < nb && lane <= i ? A[(k + i) * lda + k + lane] : (i == lane ? 1.0 : 0.0);
+  __syncthreads();
+  double a[kNB / 4];
+#pragma unroll
+  for (int m = 0; m < kNB / 4; ++m) a[m] = s[lane][4 * m + warp];
+  __syncthreads();
+  const auto publish = [&](int j, double x) {
+    double d = __shfl_sync(0xffffffffu, x, j);
+    const double r = pivot_rsqrt(mode, k + j, d, lane == 0);
+    const double v = lane > j && !is_zero(r) ? x * r : 0.0;
+    col[j & 1][lane] = v;
+    s[lane][j] = lane == j ? d : v;  // the diagonal's roots are taken together at the end
+  };
+  if (warp == 0 && nb > 0) publish(0, a[0]);
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j + 1 < kNB; ++j) {
+    if (j + 1 < nb) {
+      // (entries above the diagonal pick up values that nothing reads)
+      const double lj = -col[j & 1][lane];
+      if (warp == ((j + 1) & 3)) publish(j + 1, fma(lj, col[j & 1][j + 1], a[(j + 1) >> 2]));
+#pragma unroll
+      for (int m = 0; m < kNB / 4; ++m) {
+        const int c = 4 * m + warp;
+        if (4 * m + 3 > j + 1 && c > j + 1) a[m] = fma(lj, col[j & 1][c], a[m]);
+      }
+      __syncthreads();
+    }
+  }
+  if (warp == 0) s[lane][lane] = sqrt(s[lane][lane]);
+  __syncthreads();
+  for (int i = warp; i < nb; i += 4)
+    if (lane <= i) A[(k + i) * lda + k + lane] = s[i][lane];
+}
+
+__global__ void __launch_bounds__(128) chol_diag(double* __restrict__ A, long long lda, int nb, CholMode mode) {
+  __shared__ double s[kNB][kNB + 1];
+  __shared__ double col[2][kNB];
+  factor_diag(A, lda, 0, nb, mode, s, col);
+}
+
+// Rows k + nb + 16 blockIdx.x ... of the panel: x L11^T = a.  Warp w holds
+// columns 8 w ... 8 w + 7 of the 16 rows, four per lane: each warp solves its
+// columns in registers once the warps before it have published theirs.
+constexpr int kTrsmRows = 16;
+
+__global__ void __launch_bounds__(128) chol_trsm(double* __restrict__ A, long long lda, long long k, int nb,
+                                                 long long n) {
+  __shared__ double L[kNB][kNB + 1];
+  __shared__ double X[kTrsmRows][kNB + 1];
+  __shared__ double rd[kNB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row = lane & 15, half = lane >> 4;
   const long long r0 = k + nb + (long long)blockIdx.x * kTrsmRows;
-  for (int idx = tid; idx < nb * nb; idx += kTrsmRows) {
-    const int i = idx / nb, j = idx - i * nb;
-    L[i * (kNB + 1) + j] = j <= i ? A[(k + i) * lda + k + j] : 0.0;
-  }
-  for (int idx = tid; idx < kTrsmRows * nb; idx += kTrsmRows) {
-    const int r = idx / nb, j = idx - r * nb;
-    X[r * (kNB + 1) + j] = r0 + r < n ? A[(r0 + r) * lda + k + j] : 0.0;
-  }
+#pragma unroll
+  for (int i = warp; i < kNB; i += 4) L[i][lane] = i < nb && lane <= i ? A[(k + i) * lda + k + lane] : (i == lane ? 1.0 : 0.0);
+#pragma unroll
+  for (int r = warp; r < kTrsmRows; r += 4) X[r][lane] = r0 + r < n && lane < nb ? A[(r0 + r) * lda + k + lane] : 0.0;
   __syncthreads();
-  double* x = X + tid * (kNB + 1);
-  for (int j = 0; j < nb; ++j) {
-    double v = x[j];
-    for (int p = 0; p < j; ++p) v = fma(-x[p], L[j * (kNB + 1) + p], v);
-    x[j] = v / L[j * (kNB + 1) + j];
-  }
+  if (warp == 0) rd[lane] = 1.0 / L[lane][lane];  // 0 for the infinite pivot of a dropped function
+  double x[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) x[c] = X[row][8 * warp + 4 * half + c];
   __syncthreads();
-  for (int idx = tid; idx < kTrsmRows * nb; idx += kTrsmRows) {
-    const int r = idx / nb, j = idx - r * nb;
-    if (r0 + r < n) A[(r0 + r) * lda + k + j] = X[r * (kNB + 1) + j];
+  for (int w = 0; w < 4; ++w) {
+    if (warp == w) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const double r = rd[8 * w + j];
+        const double v = __shfl_sync(0xffffffffu, is_zero(r) ? 0.0 : x[j & 3] * r, row + 16 * (j >> 2));
+        if (half == (j >> 2)) x[j & 3] = v;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (4 + c > j && 4 * half + c > j) x[c] = fma(-v, L[8 * w + 4 * half + c][8 * w + j], x[c]);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) X[row][8 * w + 4 * half + c] = x[c];
+    }
+    __syncthreads();
+    if (warp > w) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const double v = X[row][8 * w + j];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[c] = fma(-v, L[8 * warp + 4 * half + c][8 * w + j], x[c]);
+      }
+    }
   }
+  for (int r = warp; r < kTrsmRows; r += 4)
+    if (r0 + r < n && lane < nb) A[(r0 + r) * lda + k + lane] = X[r][lane];
 }
 
 // Lower tile (bi, bj), bj <= bi, of the trailing matrix (rows/cols from
-// r0 = k + nb): A[i][j] -= sum_p L[i][k+p] L[j][k+p] for j <= i.
-__global__ void __launch_bounds__(256) chol_update(double* __restrict__ A, long long lda, long long k, int nb,
-                                                   long long n) {
-  extern __shared__ double sm[];
-  double* As = sm;              // [nb][kLd]: rows of tile bi, transposed
-  double* Bs = sm + nb * kLd;   // [nb][kLd]: rows of tile bj, transposed
+// r0 = k + nb): A[i][j] -= sum_p L[i][k+p] L[j][k+p] for j <= i.  128 threads,
+// (T/8) x (T/16) elements each.
+template <int T>
+__global__ void __launch_bounds__(128) chol_update(double* A, long long lda, long long k, int nb, long long n,
+                                                   CholMode mode) {
+  constexpr int RM = T / 8, CM = T / 16;
+  __shared__ double As[kNB][T + 1], Bs[kNB][T + 1];  // rows of tiles bi and bj, transposed
   const long long x = blockIdx.x;
   long long bi = (long long)((sqrt(8.0 * (double)x + 1.0) - 1.0) * 0.5);
   while (bi * (bi + 1) / 2 > x) --bi;
   while ((bi + 1) * (bi + 2) / 2 <= x) ++bi;
   const long long bj = x - bi * (bi + 1) / 2;
-  const long long r0 = k + nb, ri = r0 + bi * kTile, rj = r0 + bj * kTile;
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < kTile * nb; idx += 256) {
-    const int r = idx / nb, p = idx - r * nb;
-    As[p * kLd + r] = ri + r < n ? A[(ri + r) * lda + k + p] : 0.0;
-    Bs[p * kLd + r] = rj + r < n ? A[(rj + r) * lda + k + p] : 0.0;
+  const long long r0 = k + nb, ri = r0 + bi * T, rj = r0 + bj * T;
+  const int tid = threadIdx.x, p0 = tid & 31;
+#pragma unroll 4
+  for (int r = tid >> 5; r < T; r += 4) {
+    As[p0][r] = ri + r < n && p0 < nb ? A[(ri + r) * lda + k + p0] : 0.0;
+    Bs[p0][r] = rj + r < n && p0 < nb ? A[(rj + r) * lda + k + p0] : 0.0;
   }
   __syncthreads();
   const int ty = tid >> 4, tx = tid & 15;
-  double acc[8][8];
+  double acc[RM][CM];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int r = 0; r < RM; ++r)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[r][c] = 0.0;
+    for (int c = 0; c < CM; ++c) acc[r][c] = 0.0;
   for (int p = 0; p < nb; ++p) {
-    double a[8], b[8];
+    double a[RM], b[CM];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) a[r] = As[p * kLd + ty + 16 * r];
+    for (int r = 0; r < RM; ++r) a[r] = As[p][ty + 8 * r];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) b[c] = Bs[p * kLd + tx + 16 * c];
+    for (int c = 0; c < CM; ++c) b[c] = Bs[p][tx + 16 * c];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < RM; ++r)
 #pragma unroll
-      for (int c = 0; c < 8; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
+      for (int c = 0; c < CM; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
   }
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const long long i = ri + ty + 16 * r;
+  for (int r = 0; r < RM; ++r) {
+    const long long i = ri + ty + 8 * r;
     if (i >= n) continue;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
+    for (int c = 0; c < CM; ++c) {
       const long long j = rj + tx + 16 * c;
       if (j <= i) A[i * lda + j] -= acc[r][c];
     }
   }
+  if (x == 0) {
+    __syncthreads();
+    static_assert(T >= kNB, "the first tile holds the next diagonal block");
+    factor_diag(A, lda, r0, (int)min((long long)kNB, n - r0), mode, (double (*)[kNB + 1])&As[0][0],
+                (double (*)[kNB])&Bs[0][0]);
+  }
 }
 
 // ---------------------------------------------------------------------------
-// triangular solves, B row-major [n][nrhs]
+// triangular solves, B row-major [n][nrhs], blocks of 64 rows
 // ---------------------------------------------------------------------------
 
-// B[k..k+nb) <- L_kk^{-1} B[k..k+nb) (forward) or L_kk^{-T} (backward).
-__global__ void __launch_bounds__(256) solve_diag(const double* __restrict__ L, long long lda, long long k, int nb,
-                                                  double* __restrict__ B, long long nrhs, int backward) {
-  __shared__ double s[kNB][kNB + 1];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < nb * nb; idx += 256) {
-    const int i = idx / nb, j = idx - i * nb;
-    s[i][j] = j <= i ? L[(k + i) * lda + k + j] : 0.0;
-  }
-  __syncthreads();
-  for (long long q = tid; q < nrhs; q += 256) {
-    double* b = B + k * nrhs + q;
-    if (!backward) {
-      for (int j = 0; j < nb; ++j) {
-        double v = b[j * nrhs];
-        for (int p = 0; p < j; ++p) v = fma(-s[j][p], b[p * nrhs], v);
-        b[j * nrhs] = v / s[j][j];
+// Step of the solve for the block at k, with x the block solved before it (at
+// kp, nbp rows; nbp = 0 for the first): block 0 subtracts x's share from block
+// k and solves it, the others subtract it from the rows still to come, which
+// nothing else in the launch reads.  One launch per block: a separate
+// diagonal solve by one thread per right-hand side took 60 us a block.
+// Forward: L x = b, rows descending; backward: L^T x = b, rows ascending.
+template <bool kBack>
+__global__ void __launch_bounds__(256) solve_step(const double* __restrict__ L, long long lda, long long k, int nb,
+                                                  long long kp, int nbp, double* __restrict__ B, long long nrhs,
+                                                  long long n) {
+  __shared__ double s[kSB][kSB + 1];
+  __shared__ double rd[kSB];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x > 0) {
+    if (!kBack) {
+      // one warp per row, lanes over x's rows
+      const long long i = k + nb + (long long)(blockIdx.x - 1) * 8 + warp;
+      if (i >= n) return;
+      const double l0 = lane < nbp ? L[i * lda + kp + lane] : 0.0;
+      const double l1 = lane + 32 < nbp ? L[i * lda + kp + lane + 32] : 0.0;
+      for (long long q = 0; q < nrhs; ++q) {
+        double v = 0.0;
+        if (lane < nbp) v = l0 * B[(kp + lane) * nrhs + q];
+        if (lane + 32 < nbp) v = fma(l1, B[(kp + lane + 32) * nrhs + q], v);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) B[i * nrhs + q] -= v;
       }
     } else {
-      for (int j = nb - 1; j >= 0; --j) {
-        double v = b[j * nrhs];
-        for (int p = j + 1; p < nb; ++p) v = fma(-s[p][j], b[p * nrhs], v);
-        b[j * nrhs] = v / s[j][j];
+      // one thread per (row, right-hand side), reading a column of the block
+      // row (coalesced across rows)
+      const long long w = (long long)(blockIdx.x - 1) * 256 + tid;
+      if (w >= k * nrhs) return;
+      const long long j = w / nrhs, q = w - j * nrhs;
+      double v0 = 0.0, v1 = 0.0;
+      int i = 0;
+      for (; i + 1 < nbp; i += 2) {
+        v0 = fma(L[(kp + i) * lda + j], B[(kp + i) * nrhs + q], v0);
+        v1 = fma(L[(kp + i + 1) * lda + j], B[(kp + i + 1) * nrhs + q], v1);
+      }
+      if (i < nbp) v0 = fma(L[(kp + i) * lda + j], B[(kp + i) * nrhs + q], v0);
+      B[j * nrhs + q] -= v0 + v1;
+    }
+    return;
+  }
+  // the diagonal block, kept in registers until the share is subtracted
+  double dg[kSB * kSB / 256];
+#pragma unroll
+  for (int m = 0; m < kSB * kSB / 256; ++m) {
+    const int idx = tid + 256 * m, i = idx / kSB, j = idx - i * kSB;
+    dg[m] = i < nb && j <= i ? L[(k + i) * lda + k + j] : (i == j ? 1.0 : 0.0);
+  }
+  // x's share of block k (kBack: the transposed block below it)
+  if (nbp > 0) {
+    for (int idx = tid; idx < nb * nbp; idx += 256) {
+      if (!kBack) {
+        const int i = idx / nbp, p = idx - i * nbp;
+        s[i][p] = L[(k + i) * lda + kp + p];
+      } else {
+        const int p = idx / nb, i = idx - p * nb;
+        s[i][p] = L[(kp + p) * lda + k + i];
       }
     }
+    __syncthreads();
+    // four lanes per (row, right-hand side)
+    const int part = tid & 3;
+    for (long long w0 = 0; w0 < nb * nrhs; w0 += 64) {
+      const long long w = w0 + (tid >> 2);
+      const bool on = w < nb * nrhs;
+      const int i = on ? (int)(w / nrhs) : 0;
+      const long long q = on ? w - i * nrhs : 0;
+      double v0 = 0.0, v1 = 0.0;
+      if (on)
+#pragma unroll 4
+        for (int p = part; p < nbp; p += 8) {
+          v0 = fma(s[i][p], B[(kp + p) * nrhs + q], v0);
+          if (p + 4 < nbp) v1 = fma(s[i][p + 4], B[(kp + p + 4) * nrhs + q], v1);
+        }
+      double v = v0 + v1;
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (on && part == 0) B[(k + i) * nrhs + q] -= v;
+    }
+    __syncthreads();
   }
-}
-
-// Forward update: rows i >= k + nb, B[i] -= L[i][k..k+nb) B[k..k+nb); one
-// warp per row, lanes over the panel columns, shuffle reduction per rhs.
-__global__ void __launch_bounds__(256) solve_update_fwd(const double* __restrict__ L, long long lda, long long k,
-                                                        int nb, double* __restrict__ B, long long nrhs, long long n) {
-  const int lane = threadIdx.x & 31;
-  const long long i = k + nb + (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (i >= n) return;
-  const double l0 = lane < nb ? L[i * lda + k + lane] : 0.0;
-  const double l1 = lane + 32 < nb ? L[i * lda + k + lane + 32] : 0.0;
-  for (long long q = 0; q < nrhs; ++q) {
-    double v = 0.0;
-    if (lane < nb) v = l0 * B[(k + lane) * nrhs + q];
-    if (lane + 32 < nb) v = fma(l1, B[(k + lane + 32) * nrhs + q], v);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) B[i * nrhs + q] -= v;
+  for (int m = 0; m < kSB * kSB / 256; ++m) {
+    const int idx = tid + 256 * m, i = idx / kSB, j = idx - i * kSB;
+    if (kBack) s[j][i] = dg[m]; else s[i][j] = dg[m];
+    if (i == j) rd[i] = 1.0 / dg[m];  // 0 for the infinite pivot of a dropped function
   }
-}
-
-// Backward update: rows j < k, B[j] -= sum_i L[k+i][j] B[k+i]; one thread per
-// (row j, rhs q), reading a column of the block row (coalesced across j).
-__global__ void __launch_bounds__(256) solve_update_bwd(const double* __restrict__ L, long long lda, long long k,
-                                                        int nb, double* __restrict__ B, long long nrhs) {
-  const long long w = (long long)blockIdx.x * 256 + threadIdx.x;
-  if (w >= k * nrhs) return;
-  const long long j = w / nrhs, q = w - j * nrhs;
-  double v = 0.0;
-  for (int i = 0; i < nb; ++i) v = fma(L[(k + i) * lda + j], B[(k + i) * nrhs + q], v);
-  B[j * nrhs + q] -= v;
-}
-
-bool g_attr_done = false;
-
-cudaError_t chol_attributes() {
-  if (g_attr_done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(chol_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(2 * kNB * kLd * sizeof(double)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(chol_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((kNB + kTrsmRows) * (kNB + 1) * sizeof(double)));
-  if (e == cudaSuccess) g_attr_done = true;
-  return e;
+  __syncthreads();
+  // one warp per right-hand side, lane i holding rows i and i + 32
+  for (long long q = warp; q < nrhs; q += 8) {
+    double b0 = lane < nb ? B[(k + lane) * nrhs + q] : 0.0;
+    double b1 = lane + 32 < nb ? B[(k + lane + 32) * nrhs + q] : 0.0;
+    // first the half whose unknowns come first, updating both, then the other
+    double& f = kBack ? b1 : b0;
+    double& g = kBack ? b0 : b1;
+    const int of = kBack ? 32 : 0, og = 32 - of;
+#pragma unroll 4
+    for (int t = 0; t < 32; ++t) {
+      const int j = kBack ? 31 - t : t;
+      const double r = rd[of + j];
+      const double xj = is_zero(r) ? 0.0 : __shfl_sync(0xffffffffu, f, j) * r;
+      if (lane == j) f = xj;
+      if (kBack ? lane < j : lane > j) f = fma(-s[of + lane][of + j], xj, f);
+      g = fma(-s[og + lane][of + j], xj, g);
+    }
+#pragma unroll 4
+    for (int t = 0; t < 32; ++t) {
+      const int j = kBack ? 31 - t : t;
+      const double r = rd[og + j];
+      const double xj = is_zero(r) ? 0.0 : __shfl_sync(0xffffffffu, g, j) * r;
+      if (lane == j) g = xj;
+      if (kBack ? lane < j : lane > j) g = fma(-s[og + lane][og + j], xj, g);
+    }
+    if (lane < nb) B[(k + lane) * nrhs + q] = b0;
+    if (lane + 32 < nb) B[(k + lane + 32) * nrhs + q] = b1;
+  }
 }
 
 __global__ void copy_diag(const double* __restrict__ A, long long lda, long long n, double* __restrict__ d) {
@@ -274,19 +391,20 @@ __global__ void copy_diag(const double* __restrict__ A, long long lda, long long
 
 cudaError_t cholesky_launches(double* A, long long n, long long lda, int* info, const double* diag0,
                               double drop_tol, cudaStream_t st) {
-  cudaError_t e = chol_attributes();
-  for (long long k = 0; k < n && e == cudaSuccess; k += kNB) {
-    const int nb = (int)std::min<long long>(kNB, n - k);
-    chol_diag<<<1, 256, 0, st>>>(A, lda, k, nb, info, diag0, drop_tol);
-    e = cudaGetLastError();
-    const long long m = n - k - nb;
-    if (m <= 0 || e != cudaSuccess) continue;
-    chol_trsm<<<(unsigned)((m + kTrsmRows - 1) / kTrsmRows), kTrsmRows,
-                (kNB + kTrsmRows) * (kNB + 1) * sizeof(double), st>>>(A, lda, k, nb, n);
+  const CholMode mode{info, diag0, drop_tol};
+  chol_diag<<<1, 128, 0, st>>>(A, lda, (int)std::min<long long>(kNB, n), mode);
+  cudaError_t e = cudaGetLastError();
+  for (long long k = 0; k + kNB < n && e == cudaSuccess; k += kNB) {
+    const long long m = n - k - kNB;
+    chol_trsm<<<(unsigned)((m + kTrsmRows - 1) / kTrsmRows), 128, 0, st>>>(A, lda, k, kNB, n);
     e = cudaGetLastError();
     if (e != cudaSuccess) continue;
-    const long long T = (m + kTile - 1) / kTile;
-    chol_update<<<(unsigned)(T * (T + 1) / 2), 256, 2 * nb * kLd * sizeof(double), st>>>(A, lda, k, nb, n);
+    // 64 x 64 tiles while they fill the chip twice over, then 32 x 32 ones
+    const long long t64 = (m + 63) / 64, t32 = (m + 31) / 32;
+    if (t64 * (t64 + 1) / 2 >= 304)
+      chol_update<64><<<(unsigned)(t64 * (t64 + 1) / 2), 128, 0, st>>>(A, lda, k, kNB, n, mode);
+    else
+      chol_update<32><<<(unsigned)(t32 * (t32 + 1) / 2), 128, 0, st>>>(A, lda, k, kNB, n, mode);
     e = cudaGetLastError();
   }
   return e;
@@ -294,25 +412,19 @@ cudaError_t cholesky_launches(double* A, long long n, long long lda, int* info, 
 
 cudaError_t solve_launches(const double* L, long long n, long long lda, double* B, long long nrhs, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
-  for (long long k = 0; k < n && e == cudaSuccess; k += kNB) {
-    const int nb = (int)std::min<long long>(kNB, n - k);
-    solve_diag<<<1, 256, 0, st>>>(L, lda, k, nb, B, nrhs, 0);
+  for (long long k = 0; k < n && e == cudaSuccess; k += kSB) {
+    const int nb = (int)std::min<long long>(kSB, n - k);
+    const long long rest = k > 0 ? n - k - nb : 0;
+    solve_step<false><<<(unsigned)(1 + (rest + 7) / 8), 256, 0, st>>>(L, lda, k, nb, k - kSB, k > 0 ? kSB : 0, B, nrhs, n);
     e = cudaGetLastError();
-    const long long m = n - k - nb;
-    if (m > 0 && e == cudaSuccess) {
-      solve_update_fwd<<<(unsigned)((m + 7) / 8), 256, 0, st>>>(L, lda, k, nb, B, nrhs, n);
-      e = cudaGetLastError();
-    }
   }
-  const long long last = ((n - 1) / kNB) * kNB;
-  for (long long k = last; k >= 0 && e == cudaSuccess; k -= kNB) {
-    const int nb = (int)std::min<long long>(kNB, n - k);
-    solve_diag<<<1, 256, 0, st>>>(L, lda, k, nb, B, nrhs, 1);
+  const long long last = ((n - 1) / kSB) * kSB;
+  for (long long k = last; k >= 0 && e == cudaSuccess; k -= kSB) {
+    const int nb = (int)std::min<long long>(kSB, n - k);
+    const int nbp = k == last ? 0 : (int)std::min<long long>(kSB, n - k - kSB);
+    const long long rest = nbp > 0 ? k * nrhs : 0;
+    solve_step<true><<<(unsigned)(1 + (rest + 255) / 256), 256, 0, st>>>(L, lda, k, nb, k + kSB, nbp, B, nrhs, n);
     e = cudaGetLastError();
-    if (k > 0 && e == cudaSuccess) {
-      solve_update_bwd<<<(unsigned)((k * nrhs + 255) / 256), 256, 0, st>>>(L, lda, k, nb, B, nrhs);
-      e = cudaGetLastError();
-    }
   }
   return e;
 }
