@@ -19,11 +19,12 @@
 
 namespace lx3c {
 cudaError_t init_constants();
-cudaError_t launch_pair_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb,
-                                   double* rec, double* ab, cudaStream_t st, int scale_a = 0, int scale_b = 0);
-cudaError_t launch_aux_precompute(const DevBasis& aux, const int32_t* auxs, long long naux, int Kc, double* rec,
-                                  double* cxyz, cudaStream_t st);
+cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
+                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
+                              double* auxrec, double* auxc, cudaStream_t st);
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st);
+bool can_launch_both(const ClassDesc& a, const ClassDesc& b);
+cudaError_t launch_eri3c_both(const ClassDesc& a, int ga, const ClassDesc& b, int gb, cudaStream_t st);
 cudaError_t launch_boys(const double* T, long long n, int mmax, const double* tab, const double* mid, double cL,
                         double* out, cudaStream_t st);
 int eri3c_occupancy(int smem_bytes);
@@ -107,7 +108,7 @@ lx3c_status device_class(DevState* s, const ClassTables& ct, DevClass** out) {
     *out = &it->second;
     return LX3C_OK;
   }
-  size_t offs[16];
+  size_t offs[15];
   std::vector<char> blob = class_blob(ct, offs);
   DevClass dc;
   CUDA_TRY(cudaMalloc(&dc.blob, blob.size()));
@@ -139,21 +140,20 @@ size_t append(std::vector<char>& blob, const std::vector<T>& v) {
 }
 }  // namespace
 
-std::vector<char> class_blob(const ClassTables& ct, size_t f[16]) {
+std::vector<char> class_blob(const ClassTables& ct, size_t f[15]) {
   std::vector<char> blob;
-  f[0] = append(blob, ct.vtab); f[1] = append(blob, ct.wtab); f[2] = append(blob, ct.atab);
+  f[0] = append(blob, ct.vtab); f[1] = append(blob, ct.gslice); f[2] = append(blob, ct.atab);
   f[3] = append(blob, ct.gptr); f[4] = append(blob, ct.gterm); f[5] = append(blob, ct.gdst);
   f[6] = append(blob, ct.pal); f[7] = append(blob, ct.kptr); f[8] = append(blob, ct.kent);
   f[9] = append(blob, ct.htab); f[10] = append(blob, ct.baptr); f[11] = append(blob, ct.baent);
   f[12] = append(blob, ct.bbptr); f[13] = append(blob, ct.bbent); f[14] = append(blob, ct.gell);
-  f[15] = append(blob, ct.gslice);
   return blob;
 }
 
-void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t f[16]) {
+void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t f[15]) {
   const char* b = (const char*)dev_blob;
   dc.vtab = (const uint4*)(b + f[0]);
-  dc.wtab = (const int4*)(b + f[1]);
+  dc.gslice = (const int2*)(b + f[1]);
   dc.atab = (const unsigned*)(b + f[2]);
   dc.gptr = (const int*)(b + f[3]);
   dc.gterm = (const unsigned*)(b + f[4]);
@@ -167,7 +167,6 @@ void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t f[16])
   dc.bbptr = (const int*)(b + f[12]);
   dc.bbent = (const int2*)(b + f[13]);
   dc.gell = (const unsigned*)(b + f[14]);
-  dc.gslice = (const int2*)(b + f[15]);
 }
 
 void fill_desc_common(ClassDesc& d, const ClassTables& ct, const DevClass& dc, const double* boys_tab,
@@ -184,14 +183,14 @@ void fill_desc_common(ClassDesc& d, const ClassTables& ct, const DevClass& dc, c
   d.Kab_rec = Kab_rec;
   d.NV = ct.NV; d.NW = ct.NW; d.NF = ct.NF; d.NACC = ct.NACC;
   for (int e = 0; e <= d.Lab; ++e) d.vlev_start[e] = ct.vlev_start[e];
-  d.nW = ct.NW;
-  d.ngt = ct.nkrow * ct.ncc;
+  d.kmax = ct.kmax;
+  d.ngt = ct.nkrow * ct.nC;
   d.nkrow = ct.nkrow;
   d.nhrr = ct.nhrr;
   for (int j = 0; j <= ct.nhrr; ++j) d.hrows[j] = ct.hrows[j];
   for (int j = 0; j <= ct.nhrr + 1; ++j) d.hstart[j] = ct.hstart[j];
   d.nbA = ct.nbA; d.nbB = ct.nbB;
-  d.vtab = dc.vtab; d.wtab = dc.wtab; d.atab = dc.atab; d.gptr = dc.gptr; d.gterm = dc.gterm;
+  d.vtab = dc.vtab; d.atab = dc.atab; d.gptr = dc.gptr; d.gterm = dc.gterm;
   d.gdst = dc.gdst; d.pal = dc.pal; d.kptr = dc.kptr; d.kent = dc.kent; d.htab = dc.htab;
   d.gell = dc.gell; d.gslice = dc.gslice;
   d.baptr = dc.baptr; d.baent = dc.baent; d.bbptr = dc.bbptr; d.bbent = dc.bbent;
@@ -307,6 +306,7 @@ struct lx3c_plan {
   int64_t nblk = 0;
   double flops = 0;  // algorithmic flops of one execute, orientation by orientation
   Launch L[2];
+  bool both = false;  // the two orientations in one launch
   int32_t* d_pairs = nullptr;
   int32_t* d_auxs = nullptr;
   double* d_pairrec = nullptr;
@@ -527,6 +527,13 @@ lx3c_status lx3c_eri3c_plan(lx3c_plan** out, const lx3c_basis* orb, const lx3c_b
   rc = make_launch(ds, p.get(), 0, subA, primA, kA, st);
   if (!rc) rc = make_launch(ds, p.get(), 1, subB, primB, kB, st);
   if (rc) return rc;
+  // No pair has both orientations (its second one would add to the first
+  // one's blocks) and an SM gets one tile at most: one launch for both
+  // ((pp|d) 64 x 32: two launches of 31 and 33 tiles on 152 SMs).
+  p->both = p->L[0].nsub > 0 && p->L[1].nsub > 0 &&
+            std::none_of(subB.begin(), subB.end(), [](const int4& x) { return x.w == 1; }) &&
+            can_launch_both(p->L[0].desc, p->L[1].desc) &&
+            p->L[0].desc.ntiles + p->L[1].desc.ntiles <= ds->nsm;
   const int Kab = Ka * Kb;
   CUDA_TRY(cudaMalloc(&p->d_pairs, npair * 8));
   CUDA_TRY(cudaMalloc(&p->d_auxs, naux * 4));
@@ -549,8 +556,14 @@ lx3c_status lx3c_eri3c_execute(lx3c_plan* p, double* out, void* stream) {
   if (!p) return fail(LX3C_EINVAL, "eri3c_execute: null plan");
   if (!out) return fail(LX3C_EINVAL, "eri3c_execute: null output");
   cudaStream_t st = (cudaStream_t)stream;
-  CUDA_TRY(launch_pair_precompute(p->orb->dev(), p->d_pairs, p->npair, p->Ka, p->Kb, p->d_pairrec, p->d_pairab, st));
-  CUDA_TRY(launch_aux_precompute(p->aux->dev(), p->d_auxs, p->naux, p->Kc, p->d_auxrec, p->d_auxc, st));
+  CUDA_TRY(launch_precompute(p->orb->dev(), p->d_pairs, p->npair, p->Ka, p->Kb, p->d_pairrec, p->d_pairab, p->aux->dev(),
+                             p->d_auxs, p->naux, p->Kc, p->d_auxrec, p->d_auxc, st));
+  if (p->both) {
+    ClassDesc a = p->L[0].desc, b = p->L[1].desc;
+    a.out = b.out = out;
+    CUDA_TRY(launch_eri3c_both(a, p->L[0].grid, b, p->L[1].grid, st));
+    return LX3C_OK;
+  }
   for (auto& L : p->L) {
     if (!L.nsub) continue;
     ClassDesc d = L.desc;
@@ -563,7 +576,7 @@ lx3c_status lx3c_eri3c_execute(lx3c_plan* p, double* out, void* stream) {
 lx3c_status lx3c_plan_info(const lx3c_plan* p, int64_t* out, int n) {
   if (!p || (!out && n > 0)) return fail(LX3C_EINVAL, "plan_info: null pointer");
   std::vector<int64_t> v;
-  v.push_back(2 + (p->L[0].nsub > 0) + (p->L[1].nsub > 0));
+  v.push_back(1 + (p->both ? 1 : (p->L[0].nsub > 0) + (p->L[1].nsub > 0)));
   for (auto& l : p->L) {
     v.push_back(l.nsub);
     v.push_back(l.desc.T);
@@ -633,10 +646,9 @@ lx3c_status lx3c_eri3c_host(int64_t orb_nshell, const int32_t* orb_l, const int3
       if (e == cudaSuccess && !freed[b]) e = cudaEventCreateWithFlags(&freed[b], cudaEventDisableTiming);
     }
     cs = ds->host_cs;
-    if (e == cudaSuccess) e = launch_pair_precompute(plan->orb->dev(), plan->d_pairs, plan->npair, plan->Ka, plan->Kb,
-                                                     plan->d_pairrec, plan->d_pairab, st);
-    if (e == cudaSuccess) e = launch_aux_precompute(plan->aux->dev(), plan->d_auxs, plan->naux, plan->Kc, plan->d_auxrec,
-                                                    plan->d_auxc, st);
+    if (e == cudaSuccess) e = launch_precompute(plan->orb->dev(), plan->d_pairs, plan->npair, plan->Ka, plan->Kb,
+                                                plan->d_pairrec, plan->d_pairab, plan->aux->dev(), plan->d_auxs,
+                                                plan->naux, plan->Kc, plan->d_auxrec, plan->d_auxc, st);
     int c = 0;
     for (long long p0 = 0; p0 < npair && e == cudaSuccess; p0 += cp, ++c) {
       const long long p1 = std::min<long long>(npair, p0 + cp);
@@ -793,36 +805,23 @@ lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap
     if (a[i] < 0 || c[i] < 0) return fail(LX3C_EINVAL, "cvrr2_expansion: negative exponent");
   int la = a[0] + a[1] + a[2], lc = c[0] + c[1] + c[2];
   if (la > 2 * LX3C_LMAX_ORB || lc > LX3C_LMAX_AUX) return fail(LX3C_ENOTSUP, "cvrr2_expansion: too large");
-  // the class (la, 0 | lc) contains the target (a 0|c) at level 0
-  const ClassTables* ct;
-  try {
-    ct = &class_tables(la, 0, lc, 0);
-  } catch (std::exception& e) {
-    return fail(LX3C_ENOTSUP, e.what());
-  }
-  int row = cart_index(a[0], a[1], a[2]);
-  int id = row * ct->ncc + cart_index(c[0], c[1], c[2]);
-  int q0 = ct->gptr[id], q1 = ct->gptr[id + 1];
-  *nterms = q1 - q0;
-  for (int q = q0; q < q1 && q - q0 < cap; ++q) {
-    unsigned e = ct->gterm[q];
-    const int4 key = ct->acc_key[e & 0xFFFFF];
-    int el = key.x >> 16, ei = key.x & 0xFFFF, nl = key.z >> 16, ni = key.z & 0xFFFF;
-    // decode component indices back to exponents
-    auto decode = [](int l, int idx, double* o) {
-      int i = 0;
-      for (int x = l; x >= 0; --x)
-        for (int y = l - x; y >= 0; --y) {
-          if (i == idx) { o[0] = x; o[1] = y; o[2] = l - x - y; return; }
-          ++i;
+  // (a 0|c) = sum over u <= min(a, c) of prod_i C(a_i,u_i) C(c_i,u_i) u_i! (a-u 0)_{|u|, c-u}
+  int n = 0;
+  for (int ux = 0; ux <= std::min(a[0], c[0]); ++ux)
+    for (int uy = 0; uy <= std::min(a[1], c[1]); ++uy)
+      for (int uz = 0; uz <= std::min(a[2], c[2]); ++uz, ++n) {
+        if (n >= cap) continue;
+        const int u[3] = {ux, uy, uz};
+        double* t = terms + 8 * n;
+        t[3] = ux + uy + uz;
+        t[7] = 1.0;
+        for (int i = 0; i < 3; ++i) {
+          t[i] = a[i] - u[i];
+          t[4 + i] = c[i] - u[i];
+          for (int k = 0; k < u[i]; ++k) t[7] = t[7] * (a[i] - k) * (c[i] - k) / (k + 1);  // C(a,u) C(c,u) u!, exact
         }
-    };
-    double* t = terms + 8 * (q - q0);
-    decode(el, ei, t);
-    t[3] = key.y;
-    decode(nl, ni, t + 4);
-    t[7] = ct->pal[e >> 20];
-  }
+      }
+  *nterms = n;
   return LX3C_OK;
 }
 

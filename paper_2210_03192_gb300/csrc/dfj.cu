@@ -36,15 +36,14 @@
 #include "lx3c_internal.h"
 
 namespace lx3c {
-cudaError_t launch_pair_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb,
-                                   double* rec, double* ab, cudaStream_t st, int scale_a = 0, int scale_b = 0);
-cudaError_t launch_aux_precompute(const DevBasis& aux, const int32_t* auxs, long long naux, int Kc, double* rec,
-                                  double* cxyz, cudaStream_t st);
+cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
+                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
+                              double* auxrec, double* auxc, cudaStream_t st);
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st);
 int eri3c_occupancy(int smem_bytes);
 cudaError_t launch_persistent(const ClassDesc* descs, const int2* work, long long nwork, unsigned long long* counter,
-                              int grid, int smem_bytes, int three, cudaStream_t st);
-int persistent_occupancy(int smem_bytes, int three);
+                              int grid, int smem_bytes, int two, cudaStream_t st);
+int persistent_occupancy(int smem_bytes, int two);
 }  // namespace lx3c
 
 using namespace lx3c;
@@ -504,8 +503,8 @@ lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, doub
   for (auto& g : p->groups) {
     if (g.herm) continue;
     const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
-    DCUDA(launch_pair_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, st));
-    DCUDA(launch_aux_precompute(p->aux->dev(), g.d_auxs, na, g.Kc, g.d_auxrec, g.d_auxc, st));
+    DCUDA(launch_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, p->aux->dev(), g.d_auxs,
+                            na, g.Kc, g.d_auxrec, g.d_auxc, st));
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       ClassDesc d = L.desc;
@@ -554,8 +553,8 @@ lx3c_status lx3c_dfj_execute_multi(lx3c_dfj* p, int nd, const double* D, const d
   size_t li = 0;
   for (auto& g : p->groups) {
     const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
-    DCUDA(launch_pair_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, st));
-    DCUDA(launch_aux_precompute(p->aux->dev(), g.d_auxs, na, g.Kc, g.d_auxrec, g.d_auxc, st));
+    DCUDA(launch_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, p->aux->dev(), g.d_auxs,
+                            na, g.Kc, g.d_auxrec, g.d_auxc, st));
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       DCUDA(launch_eri3c(descs[li], grids[li], st));
@@ -615,7 +614,7 @@ lx3c_status lx3c_dfj_info(const lx3c_dfj* p, double* out, int n) {
     tasks += (double)g.ntasks;
     nint += g.nint;
     flops += g.flops;
-    if (!g.herm) launches += 2 + (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
+    if (!g.herm) launches += 1 + (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
   }
   const double v[] = {(double)p->groups.size(), tasks, nint, flops, launches, (double)p->nao, (double)p->naux_ao,
                       (double)p->natom, gflops, glaunches, slots};
@@ -705,11 +704,11 @@ struct lx3c_batch {
   int smem = 0;
   int grid = 0;
   // mode 1 splits the work items into occupancy tiers, each run by a
-  // persistent kernel sized for the tier's largest item: items that fit three
-  // CTAs per SM (the 40-register kernel), then two, then the rest
+  // persistent kernel sized for the tier's largest item: items that fit two
+  // CTAs per SM, then the rest
   struct Tier {
     long long off = 0, n = 0;
-    int smem = 0, grid = 0, three = 0;
+    int smem = 0, grid = 0, two = 0;
   };
   std::vector<Tier> tiers;
   cudaGraph_t graph = nullptr;        // mode 1: persistent kernels, one per tier
@@ -751,10 +750,9 @@ cudaError_t capture_branches(lx3c_batch* b, const std::vector<ClassDesc>& descs,
       cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
       for (auto& g : p->groups) {
         if (g.herm) continue;
-        launch_pair_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec,
-                               g.d_pairab, cap);
-        launch_aux_precompute(p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
-        kernels += 2;
+        launch_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
+                          p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
+        ++kernels;
       }
     }
     cudaEventRecord(fork, cap);
@@ -878,9 +876,8 @@ lx3c_status lx3c_batch_plan(lx3c_batch** out, int nmol, const lx3c_basis* const*
       DCUDA(cudaMemset(tg, 0, mxa * kFixBytes)); DCUDA(cudaMemset(tJ, 0, mx * mx * kFixBytes));
       DCUDA(cudaMemset(tc, 0, mxa * 8)); DCUDA(cudaMemset(tD, 0, mx * mx * 8));
     }
-    DCUDA(launch_pair_precompute(owner->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec,
-                                 g.d_pairab, st));
-    DCUDA(launch_aux_precompute(owner->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, st));
+    DCUDA(launch_precompute(owner->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
+                            owner->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, st));
     const int T0 = L.desc.T;
     std::vector<int> cands = {T0};
     if (T0 >= 2) cands.push_back(T0 / 2);
@@ -962,7 +959,7 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     b->plain_launches += 2 + (p->hj ? herm_launches(p->hj) : 0);
     for (auto& g : p->groups) {
       if (g.herm) continue;
-      b->plain_launches += 2;
+      b->plain_launches += 1;
       for (auto& L : g.L) {
         if (!L.ntiles) continue;
         ++b->plain_launches;
@@ -978,16 +975,15 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     }
   }
   std::stable_sort(order.begin(), order.end(), [](auto& x, auto& y) { return x.first > y.first; });
-  // tiers: the items whose shared memory lets the 40-register persistent
-  // kernel keep three CTAs per SM, then those that fit two CTAs of the
-  // unrestricted one, then the others; longest first within each tier
+  // tiers: the items whose shared memory lets two CTAs fit an SM, then the
+  // others; longest first within each tier
   std::vector<int2> work;
   b->tiers.clear();
-  auto tier_of = [&](int sm) { return persistent_occupancy(sm, 1) >= 3 ? 0 : (persistent_occupancy(sm, 0) >= 2 ? 1 : 2); };
-  for (int tier = 0; tier < 3; ++tier) {
+  auto tier_of = [&](int sm) { return persistent_occupancy(sm, 1) >= 2 ? 0 : 1; };
+  for (int tier = 0; tier < 2; ++tier) {
     lx3c_batch::Tier T;
     T.off = (long long)work.size();
-    T.three = tier == 0 ? 1 : 0;
+    T.two = tier == 0 ? 1 : 0;
     for (auto& o : order) {
       const int sm = descs[o.second].smem_doubles * 8;
       if (tier_of(sm) != tier) continue;
@@ -996,7 +992,7 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     }
     T.n = (long long)work.size() - T.off;
     if (!T.n) continue;
-    T.grid = dev_nsm(b->ds) * persistent_occupancy(T.smem, T.three);
+    T.grid = dev_nsm(b->ds) * persistent_occupancy(T.smem, T.two);
     b->tiers.push_back(T);
   }
   cudaFree(b->d_descs);
@@ -1023,10 +1019,9 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
     for (auto& g : p->groups) {
       if (g.herm) continue;
-      launch_pair_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec,
-                             g.d_pairab, cap);
-      launch_aux_precompute(p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
-      b->graph_kernels += 2;
+      launch_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
+                        p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
+      b->graph_kernels += 1;
     }
   }
   for (int m = 0; m < nmol; ++m) {
@@ -1038,7 +1033,7 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
   for (size_t t = 0; t < b->tiers.size(); ++t) {
     const auto& T = b->tiers[t];
     cudaMemsetAsync(b->d_counter + t, 0, sizeof(unsigned long long), cap);
-    launch_persistent(b->d_descs, b->d_work + T.off, T.n, b->d_counter + t, T.grid, T.smem, T.three, cap);
+    launch_persistent(b->d_descs, b->d_work + T.off, T.n, b->d_counter + t, T.grid, T.smem, T.two, cap);
     b->graph_kernels += 1;
   }
   for (int m = 0; m < nmol; ++m) {

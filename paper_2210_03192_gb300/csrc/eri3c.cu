@@ -6,8 +6,8 @@
 //                      [00|0]^(m) from the Boys function       Sec. 2.5.2
 //                      VRR1                                      Eq. vrr1
 //                      CVRR2 prerequisites, contracted early     Eq. a0cv2 / Sec. 2.5.4
-//                      CVRR2 targets (n-quantum form)            Sec. 2.5.4
-//                      Cartesian -> solid-harmonic ket           Sec. 2.5.1
+//                      CVRR2 targets (n-quantum form) on a solid-
+//                      harmonic ket                              Sec. 2.5.4, 2.5.1
 //                      HRR                                       Eq. hrr
 //                      optional solid-harmonic bra, store
 //
@@ -16,10 +16,13 @@
 // issue only the FP64 operations of the FLOP-minimal scheme with all 32 lanes
 // busy, while index decoding, shared-memory traffic and table reads (integer,
 // load/store pipes) hide under the FP64 pipe.  Each stage is a flat loop over
-// (triple, target) items driven by host-built tables; the triple index is the
-// fastest lane index when a tile holds >= 32 triples (warp-uniform table
+// (triple block, target) items driven by host-built tables; the triple index
+// is the fastest lane index when a tile holds >= 32 triples (warp-uniform table
 // entries, conflict-free strided shared memory) and the target index otherwise.
-// Primitive contraction happens in shared-memory accumulators (Eq. a0cv2
+// An item is one target of up to four triples: one decoded table entry and one
+// set of addresses serve them all (one triple per item took 47 instructions per
+// FP64 instruction at (ff|g), three quarters of the issue slots).
+// Primitive contraction happens in shared-memory accumulators (the CVRR2
 // prerequisites), so no intermediate CVRR2 value is ever stored to global
 // memory and no atomics are needed.
 #include <cuda_runtime.h>
@@ -31,6 +34,17 @@
 namespace lx3c {
 
 __constant__ double c_inv2m1[32];  // 1/(2m+1)
+
+// (l^2 - m^2) / (4 l^2 - 1): the solid-harmonic recursion
+// Q_{l+1,m} = z Q_{l,m} - c r^2 Q_{l-1,m}, l, m <= 5
+#define QC(l, m) ((double)((l) * (l) - (m) * (m)) / (4.0 * (l) * (l) - 1.0))
+#define QROW(l) QC(l, 0), QC(l, 1), QC(l, 2), QC(l, 3), QC(l, 4), QC(l, 5)
+__constant__ double c_q[36] = {0, 0, 0, 0, 0, 0, QROW(1), QROW(2), QROW(3), QROW(4), QROW(5)};
+
+template <int N>
+struct Int {
+  static constexpr int n = N;
+};
 
 struct FDiv {
   unsigned d, m;
@@ -97,11 +111,8 @@ __device__ __forceinline__ void boys_scaled(const double* __restrict__ tab, cons
 
 
 // One thread per primitive pair (pair p, a-primitive ia, b-primitive ib).
-__global__ void pair_precompute(DevBasis orb, const int32_t* __restrict__ pairs, long long npair, int Ka, int Kb,
-                                double* __restrict__ rec, double* __restrict__ ab, int scale_a, int scale_b) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long n = npair * Ka * Kb;
-  if (i >= n) return;
+__device__ __forceinline__ void pair_record(const DevBasis& orb, const int32_t* __restrict__ pairs, int Ka, int Kb,
+                                            double* __restrict__ rec, double* __restrict__ ab, long long i) {
   long long p = i / (Ka * Kb);
   int r = (int)(i - p * Ka * Kb);
   int ia = r / Kb, ib = r - ia * Kb;
@@ -117,10 +128,6 @@ __global__ void pair_precompute(DevBasis orb, const int32_t* __restrict__ pairs,
   double* o = rec + i * kPairRec;
   o[PR_G] = g;
   o[PR_K] = ca * cb * exp(-za * zb * ig * ab2) * two_pi52 * ig;
-  // derivative of a primitive: d/dA phi_a = 2 za phi_{a+1} - a phi_{a-1}; the
-  // 2 za factor of the first term rides on the coefficient
-  if (scale_a) o[PR_K] *= 2.0 * za;
-  if (scale_b) o[PR_K] *= 2.0 * zb;
   for (int x = 0; x < 3; ++x) {
     double P = (za * A[x] + zb * B[x]) * ig;
     o[PR_P + x] = P;
@@ -135,10 +142,8 @@ __global__ void pair_precompute(DevBasis orb, const int32_t* __restrict__ pairs,
 }
 
 // One thread per (ket list entry q, primitive ic): zeta_c and c_c / zeta_c.
-__global__ void aux_precompute(DevBasis aux, const int32_t* __restrict__ auxs, long long naux, int Kc,
-                               double* __restrict__ rec, double* __restrict__ cxyz) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= naux * Kc) return;
+__device__ __forceinline__ void aux_record(const DevBasis& aux, const int32_t* __restrict__ auxs, int Kc,
+                                           double* __restrict__ rec, double* __restrict__ cxyz, long long i) {
   long long q = i / Kc;
   int ic = (int)(i - q * Kc);
   int s = auxs[q];
@@ -147,6 +152,19 @@ __global__ void aux_precompute(DevBasis aux, const int32_t* __restrict__ auxs, l
   rec[i * kAuxRec + 1] = c / z;
   if (ic == 0)
     for (int x = 0; x < 3; ++x) cxyz[3 * q + x] = aux.xyz[3 * s + x];
+}
+
+// Pair records by the first threads, ket records by the others (one launch:
+// a small call is mostly launches).
+__global__ void precompute_kernel(DevBasis orb, const int32_t* __restrict__ pairs, long long npair, int Ka, int Kb,
+                                  double* __restrict__ rec, double* __restrict__ ab, DevBasis aux,
+                                  const int32_t* __restrict__ auxs, long long naux, int Kc,
+                                  double* __restrict__ auxrec, double* __restrict__ auxc) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x, n = npair * Ka * Kb;
+  if (i < n)
+    pair_record(orb, pairs, Ka, Kb, rec, ab, i);
+  else if (i - n < naux * Kc)
+    aux_record(aux, auxs, Kc, auxrec, auxc, i - n);
 }
 
 // ---------------------------------------------------------------------------
@@ -187,6 +205,38 @@ __device__ __forceinline__ void dec3(unsigned w, int mode, const FDiv& fT, const
   }
 }
 
+// A stage's loop over nx targets of T triples in blocks of TB: f(x, t0, ts)
+// for the triples t0, t0 + ts, ..., TB of them (those at or beyond the tile's
+// count are the caller's to skip).  Lanes run over triples first (mode 0) or
+// targets first (mode 1).
+template <int NT, int TB, class F>
+__device__ __forceinline__ void stage_items(int nx, int T, int tv, int mode, const F& f) {
+  FDiv fd;
+  const int nt = T / TB;
+  fd.init(mode == 0 ? nt : nx);
+  for (unsigned w = threadIdx.x; w < (unsigned)(nt * nx); w += NT) {
+    const unsigned q = fd.div(w), r = w - q * fd.d;
+    if (mode == 0) {
+      if ((int)r < tv) f((int)q, (int)r, nt);
+    } else {
+      if ((int)q * TB < tv) f((int)r, (int)q * TB, 1);
+    }
+  }
+}
+
+// Blocks of four, two or one triples, as T divides, as long as the items still
+// fill the block's threads and (mode 0) a warp keeps to one target.
+template <int NT, class F>
+__device__ __forceinline__ void stage(int nx, int T, int tv, int mode, const F& f) {
+  const int most = mode == 0 ? T >> 5 : 4;
+  if ((T & 3) == 0 && most >= 4 && nx * T >= 4 * NT)
+    stage_items<NT, 4>(nx, T, tv, mode, [&](int x, int t0, int ts) { f(x, t0, ts, Int<4>()); });
+  else if ((T & 1) == 0 && most >= 2 && nx * T >= 2 * NT)
+    stage_items<NT, 2>(nx, T, tv, mode, [&](int x, int t0, int ts) { f(x, t0, ts, Int<2>()); });
+  else
+    stage_items<NT, 1>(nx, T, tv, mode, [&](int x, int t0, int ts) { f(x, t0, ts, Int<1>()); });
+}
+
 // Segmented dot products out[o] += sum_{r < len} prod(o, r) for o < nout,
 // each partial result handed to emit(o, value), which adds it to global
 // memory with an atomic.  The FP64 pipe charges a whole warp instruction
@@ -195,16 +245,16 @@ __device__ __forceinline__ void dec3(unsigned w, int mode, const FDiv& fT, const
 // output (two partial sums) when there are many outputs, else one warp per
 // (output, 128-term chunk) whose lanes each emit their own partial sum (a warp
 // shuffle reduction here costs the whole kernel registers).
-template <class Prod, class Emit>
+template <int NT, class Prod, class Emit>
 __device__ __forceinline__ void seg_dot(int nout, int len, const Prod& prod, const Emit& emit) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kWarps = kThreads / 32, kChunk = 128;
+  constexpr int kWarps = NT / 32, kChunk = 128;
   if (nout <= 0 || len <= 0) return;
   const int nch = (len + kChunk - 1) / kChunk;
-  const long long lane_steps = (long long)((nout + kThreads - 1) / kThreads) * ((len + 1) / 2);
+  const long long lane_steps = (long long)((nout + NT - 1) / NT) * ((len + 1) / 2);
   const long long warp_steps = (long long)((nout * nch + kWarps - 1) / kWarps) * ((min(len, kChunk) + 31) / 32 + 1);
   if (lane_steps <= warp_steps) {
-    for (int o = tid; o < nout; o += kThreads) {
+    for (int o = tid; o < nout; o += NT) {
       double s0 = 0.0, s1 = 0.0;
       int r = 0;
       for (; r + 1 < len; r += 2) {
@@ -228,107 +278,110 @@ __device__ __forceinline__ void seg_dot(int nout, int len, const Prod& prod, con
 // HRR rounds (Eq. hrr; Sec. 2.5.5 for two-quantum rounds) and the optional
 // solid-harmonic bra transforms on tv triples of H[0]; returns the buffer
 // holding the final block.
-__device__ __forceinline__ Buf hrr_and_bra(const ClassDesc& d, double* sm, int T, int tv, int mode, const FDiv& fT) {
-  const unsigned tid = threadIdx.x;
+template <int NT>
+__device__ __forceinline__ Buf hrr_and_bra(const ClassDesc& d, double* sm, int T, int tv, int mode) {
   // ---- HRR (Eq. hrr) round by round: each row is dst = sum_t coef_t src_t
   // over 2 terms (one quantum moved, Eq. hrr) or 3-4 terms (two quanta,
   // Sec. 2.5.5), the coefficients products of AB components
+  FDiv fC;
+  fC.init(d.nC);
   for (int j = 1; j <= d.nhrr; ++j) {
-    FDiv fX, fC;
-    const int nx = d.hrows[j] * d.nC;
-    fX.init(nx);
-    fC.init(d.nC);
-    const unsigned n = (unsigned)(T * nx);
     const Buf hi = d.H[j - 1], ho = d.H[j];
     const double* abp = sm + d.ab_base;
-    for (unsigned w = tid; w < n; w += kThreads) {
-      int t, x;
-      dec2(w, mode, fT, fX, t, x);
-      if (t >= tv) continue;
-      const int r = (int)fC.div(x), C = x - r * d.nC;
-      const uint4 e = __ldg(d.htab + d.hstart[j] + r);
+    const uint4* tab = d.htab + d.hstart[j];
+    const int nC = d.nC;
+    stage<NT>(d.hrows[j] * nC, T, tv, mode, [&](int x, int t0, int ts, auto tb) {
+      constexpr int TB = decltype(tb)::n;
+      const int r = (int)fC.div(x), C = x - r * nC;
+      const uint4 e = __ldg(tab + r);
       const unsigned nt = e.x >> 16;
-      double v = fma(abp[(e.w >> 4) & 0xF], sm[BUF_T(hi, (int)(e.y >> 16) * d.nC + C, t)],
-                     sm[BUF_T(hi, (int)(e.y & 0xFFFF) * d.nC + C, t)]);
-      if (nt > 2) v = fma(abp[(e.w >> 8) & 0xF], sm[BUF_T(hi, (int)(e.z & 0xFFFF) * d.nC + C, t)], v);
-      if (nt > 3) v = fma(abp[(e.w >> 12) & 0xF], sm[BUF_T(hi, (int)(e.z >> 16) * d.nC + C, t)], v);
-      sm[BUF_T(ho, (int)(e.x & 0xFFFF) * d.nC + C, t)] = v;
-    }
+      const int st = hi.st * ts, base = hi.base + t0 * hi.st + C * hi.si, row = nC * hi.si;
+      const double* s0 = sm + base + (int)(e.y & 0xFFFF) * row;
+      const double* s1 = sm + base + (int)(e.y >> 16) * row;
+      double* o = sm + BUF_T(ho, (int)(e.x & 0xFFFF) * nC + C, t0);
+      const int so = ho.st * ts;
+      const double c1 = abp[(e.w >> 4) & 0xF];
+      double v[TB];
+#pragma unroll
+      for (int k = 0; k < TB; ++k)
+        if (t0 + k * ts < tv) v[k] = fma(c1, s1[k * st], s0[k * st]);
+      if (nt > 2) {
+        const double* s2 = sm + base + (int)(e.z & 0xFFFF) * row;
+        const double c2 = abp[(e.w >> 8) & 0xF];
+#pragma unroll
+        for (int k = 0; k < TB; ++k)
+          if (t0 + k * ts < tv) v[k] = fma(c2, s2[k * st], v[k]);
+        if (nt > 3) {
+          const double* s3 = sm + base + (int)(e.z >> 16) * row;
+          const double c3 = abp[(e.w >> 12) & 0xF];
+#pragma unroll
+          for (int k = 0; k < TB; ++k)
+            if (t0 + k * ts < tv) v[k] = fma(c3, s3[k * st], v[k]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < TB; ++k)
+        if (t0 + k * ts < tv) o[k * so] = v[k];
+    });
     __syncthreads();
   }
   // ---- optional solid-harmonic bra
   Buf cur = d.H[d.nhrr];
-  if (d.nbA) {
-    FDiv fX, fC, fB;
-    const int nx = d.nbA * d.nC;
-    fX.init(nx);
-    fC.init(d.nC);
-    fB.init(d.ncB);
-    const unsigned n = (unsigned)(T * nx);
-    for (unsigned w = tid; w < n; w += kThreads) {
-      int t, x;
-      dec2(w, mode, fT, fX, t, x);
-      if (t >= tv) continue;
-      const int row = (int)fC.div(x), C = x - row * d.nC;
-      const int A = (int)fB.div(row), ib = row - A * d.ncB;
-      const int q0 = __ldg(d.baptr + A), q1 = __ldg(d.baptr + A + 1);
-      double s;
-      const int2 e0 = __ldg(d.baent + q0);
-      if (q1 - q0 == 1 && e0.y == 0) {
-        s = sm[BUF_T(cur, (e0.x * d.ncB + ib) * d.nC + C, t)];
-      } else {
-        s = 0.0;
-        for (int q = q0; q < q1; ++q) {
-          const int2 e = __ldg(d.baent + q);
-          s = fma(__ldg(d.pal + e.y), sm[BUF_T(cur, (e.x * d.ncB + ib) * d.nC + C, t)], s);
-        }
-      }
-      sm[BUF_T(d.BA, x, t)] = s;
+  // out[dst] = sum of coef[q] src[entry q] over the CSR row [q0, q1); a single
+  // unit coefficient is a copy
+  const auto row_sum = [&](const int2* ent, int q0, int q1, const Buf& in, int in0, int stride, const Buf& out, int dst,
+                           int t0, int ts, auto tb) {
+    constexpr int TB = decltype(tb)::n;
+    const int st = in.st * ts, so = out.st * ts;
+    const double* src = sm + in.base + t0 * in.st + in0 * in.si;
+    double* o = sm + BUF_T(out, dst, t0);
+    double v[TB];
+    const int2 e0 = __ldg(ent + q0);
+    const double* p0 = src + e0.x * stride * in.si;
+    if (e0.y == 0) {
+#pragma unroll
+      for (int k = 0; k < TB; ++k) v[k] = t0 + k * ts < tv ? p0[k * st] : 0.0;
+    } else {
+      const double c = __ldg(d.pal + e0.y);
+#pragma unroll
+      for (int k = 0; k < TB; ++k)
+        if (t0 + k * ts < tv) v[k] = c * p0[k * st];
     }
+    for (int q = q0 + 1; q < q1; ++q) {
+      const int2 e = __ldg(ent + q);
+      const double* p = src + e.x * stride * in.si;
+      const double c = __ldg(d.pal + e.y);
+#pragma unroll
+      for (int k = 0; k < TB; ++k)
+        if (t0 + k * ts < tv) v[k] = fma(c, p[k * st], v[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < TB; ++k)
+      if (t0 + k * ts < tv) o[k * so] = v[k];
+  };
+  if (d.nbA) {
+    // items A-slowest: with targets across lanes they share A's trip count
+    const int nB = d.ncB * d.nC;
+    FDiv fB;
+    fB.init(nB);
+    stage<NT>(d.nbA * d.nC, T, tv, mode, [&](int x, int t0, int ts, auto tb) {
+      const int A = (int)fB.div(x), bC = x - A * nB;
+      row_sum(d.baent, __ldg(d.baptr + A), __ldg(d.baptr + A + 1), cur, bC, nB, d.BA, x, t0, ts, tb);
+    });
     __syncthreads();
     cur = d.BA;
   }
   if (d.nbB) {
-    // items B-slowest in mode 1: a warp's lanes share B's trip count
-    FDiv fX, fC, fB, fAC;
-    const int nx = d.nbB * d.nC;
-    const int nBs = d.nB, nAC = (d.nbB / d.nB) * d.nC;
-    fX.init(nx);
-    fC.init(d.nC);
-    fB.init(nBs);
+    // items B-slowest: with targets across lanes they share B's trip count
+    const int nBs = d.nB, nAC = (d.nbB / d.nB) * d.nC, nC = d.nC;
+    FDiv fAC;
     fAC.init(nAC);
-    const unsigned n = (unsigned)(T * nx);
-    for (unsigned w = tid; w < n; w += kThreads) {
-      int t, x;
-      dec2(w, mode, fT, fX, t, x);
-      if (t >= tv) continue;
-      int A, B, C;
-      if (mode == 0) {
-        const int row = (int)fC.div(x);
-        C = x - row * d.nC;
-        A = (int)fB.div(row);
-        B = row - A * nBs;
-      } else {
-        B = (int)fAC.div(x);
-        const int rem = x - B * nAC;
-        A = (int)fC.div(rem);
-        C = rem - A * d.nC;
-      }
-      x = (A * nBs + B) * d.nC + C;
-      const int q0 = __ldg(d.bbptr + B), q1 = __ldg(d.bbptr + B + 1);
-      double s;
-      const int2 e0 = __ldg(d.bbent + q0);
-      if (q1 - q0 == 1 && e0.y == 0) {
-        s = sm[BUF_T(cur, (A * d.ncB + e0.x) * d.nC + C, t)];
-      } else {
-        s = 0.0;
-        for (int q = q0; q < q1; ++q) {
-          const int2 e = __ldg(d.bbent + q);
-          s = fma(__ldg(d.pal + e.y), sm[BUF_T(cur, (A * d.ncB + e.x) * d.nC + C, t)], s);
-        }
-      }
-      sm[BUF_T(d.BB, x, t)] = s;
-    }
+    stage<NT>(d.nbB * nC, T, tv, mode, [&](int x, int t0, int ts, auto tb) {
+      const int B = (int)fAC.div(x), rem = x - B * nAC;
+      const int A = (int)fC.div(rem), C = rem - A * nC;
+      row_sum(d.bbent, __ldg(d.bbptr + B), __ldg(d.bbptr + B + 1), cur, A * d.ncB * nC + C, nC, d.BB,
+              (A * nBs + B) * nC + C, t0, ts, tb);
+    });
     __syncthreads();
     cur = d.BB;
   }
@@ -340,7 +393,7 @@ __device__ __forceinline__ Buf hrr_and_bra(const ClassDesc& d, double* sm, int T
 // kernel (store, per-integral DF-J digestion), 1 adds the several-density
 // digestion on FP64 tensor-core tiles (digest == 4), in a kernel of its own
 // so that the plain launches keep their register count.
-template <int kVar>
+template <int kVar, int NT>
 __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, double* sm) {
   const unsigned tid = threadIdx.x;
   const int T = d.T, G = d.G, mode = d.mode, lc = d.lc, Lab = d.Lab;
@@ -370,7 +423,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       // when the pair has no other sub-pair
       if (accum == 2 && d.digest == 0) {
         double* o = d.out + ((pair - d.out_pair0) * d.naux + aux0) * (long long)d.nblk;
-        for (int w = tid; w < tv * d.nblk; w += kThreads) o[w] = 0.0;
+        for (int w = tid; w < tv * d.nblk; w += NT) o[w] = 0.0;
       }
       return;
     }
@@ -379,7 +432,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
     __syncthreads();  // previous tile done with shared memory
     {
       // this sub-pair's primitive-pair records, in its orientation
-      for (int i = tid; i < kab * kPairRec; i += kThreads) {
+      for (int i = tid; i < kab * kPairRec; i += NT) {
         const int g = i / kPairRec, f = i - g * kPairRec;
         int fs = f;
         if (d.orient) {
@@ -405,17 +458,10 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
         else if (tid == 12) v = y * z;
         sm[d.ab_base + tid] = v;
       }
-      for (int i = tid; i < tv * auxsz; i += kThreads) {
+      for (int i = tid; i < tv * auxsz; i += NT) {
         int t = i / auxsz, r = i - t * auxsz;
         sm[d.aux_base + i] = r < 3 ? d.auxc[(long long)(aux0 + t) * 3 + r]
                                    : d.auxrec[(long long)(aux0 + t) * d.Kc * kAuxRec + (r - 3)];
-      }
-      FDiv fA;
-      fA.init(d.NACC);
-      for (unsigned w = tid; w < (unsigned)(T * d.NACC); w += kThreads) {
-        int t, a;
-        dec2(w, mode, fT, fA, t, a);
-        sm[BUF_T(d.P, a, t)] = 0.0;
       }
     }
     __syncthreads();
@@ -424,7 +470,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       const int p0 = chunk * G;
       const int gcnt = min(G, K - p0);
       // ---- stage A: geometry, Boys function, [00|0]^(m) and recurrence factors
-      for (unsigned w = tid; w < (unsigned)(T * G); w += kThreads) {
+      for (unsigned w = tid; w < (unsigned)(T * G); w += NT) {
         int t, g;
         if (mode == 0) {
           unsigned q = fT.div(w);
@@ -460,200 +506,224 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
         }
         sm[fb + 3 * fs] = rg;
         if (lc > 0) {
-          double X[3] = {gr * PCx, gr * PCy, gr * PCz};
-          for (int i = 0; i < 3; ++i) {
-            double v = X[i];
-            sm[fb + (4 + i * lc) * fs] = v;
-            for (int j = 2; j <= lc; ++j) {
-              v *= X[i];
-              sm[fb + (4 + i * lc + j - 1) * fs] = v;
-            }
-          }
-          double Y = 0.5 * r, v = Y;
-          sm[fb + (4 + 3 * lc) * fs] = v;
-          for (int k = 2; k <= lc; ++k) {
+          sm[fb + 4 * fs] = gr * PCx;
+          sm[fb + 5 * fs] = gr * PCy;
+          sm[fb + 6 * fs] = gr * PCz;
+          const double Y = 0.5 * r;
+          double v = Y;
+          for (int k = 1; k <= d.kmax; ++k) {
+            sm[fb + (6 + k) * fs] = v;
             v *= Y;
-            sm[fb + (4 + 3 * lc + k - 1) * fs] = v;
           }
         }
         boys_scaled(d.boys_tab, d.boys_mid, d.boys_cL, d.L, lc, Tb, pref, sm + BUF_TG(d.V, 0, g, t), d.V.si);
       }
       __syncthreads();
-      // ---- weights W_{k,n} = Y^k X^n (Eq. a0cv2)
+      // ---- weights W_{k,m} = Y^k s_{lc-k,m}(X), one item per (slot, |m|):
+      // (x + i y)^m, then Q_{l,m}(z, r^2) for l = m..lc by recursion; items of
+      // one m stand together (the loops' trip counts depend on it), and the
+      // last threads take them, as the first VRR1 level starts on the first
       {
-        FDiv fX;
-        fX.init(d.nW);
-        const unsigned n = (unsigned)(T * G * d.nW);
-        for (unsigned w = tid; w < n; w += kThreads) {
-          int t, g, x;
-          dec3(w, mode, fT, fG, fX, t, g, x);
+        FDiv fS;
+        const int ns = T * G, kmax = d.kmax;
+        fS.init(ns);
+        for (unsigned w = NT - 1 - tid; w < (unsigned)(ns * (lc + 1)); w += NT) {
+          const int m = (int)fS.div(w), slot = (int)w - m * ns;
+          int t, g;
+          if (mode == 0) {
+            g = (int)fT.div(slot);
+            t = slot - g * T;
+          } else {
+            t = (int)fG.div(slot);
+            g = slot - t * G;
+          }
           if (t >= tv || g >= gcnt) continue;
-          const int4 it = __ldg(d.wtab + x);
-          const int dst = it.x & 0xFFFF, cnt = it.z >> 16;
-          const int fb = BUF_TG(d.F, 0, g, t), fs = d.F.si;
-          double v = 1.0;
-          if (cnt > 0) v = sm[fb + (it.x >> 16) * fs];
-          if (cnt > 1) v *= sm[fb + (it.y & 0xFFFF) * fs];
-          if (cnt > 2) v *= sm[fb + (it.y >> 16) * fs];
-          if (cnt > 3) v *= sm[fb + (it.z & 0xFFFF) * fs];
-          sm[BUF_TG(d.W, dst, g, t)] = v;
+          const double* F = sm + BUF_TG(d.F, 0, g, t);
+          double* W = sm + BUF_TG(d.W, 0, g, t);
+          const int fs = d.F.si, ws = d.W.si;
+          if (lc == 0) {
+            W[0] = 1.0;
+            continue;
+          }
+          const double X = F[4 * fs], Yc = F[5 * fs], Z = F[6 * fs];
+          const double r2 = fma(Z, Z, fma(Yc, Yc, X * X));
+          double A = X, B = Yc;
+          for (int i = 1; i < m; ++i) {
+            const double An = fma(A, X, -B * Yc);
+            B = fma(A, Yc, B * X);
+            A = An;
+          }
+          double q0 = 0.0, q1 = 1.0;
+          for (int l = m; l <= lc; ++l) {
+            const int k = lc - l;
+            if (k <= kmax) {
+              const double v = k ? q1 * F[(6 + k) * fs] : q1;
+              const int o = k * (2 * lc + 2 - k) + l;  // m = 0 of degree l
+              if (m == 0) {
+                W[o * ws] = v;
+              } else {
+                W[(o + m) * ws] = v * A;
+                W[(o - m) * ws] = v * B;
+              }
+            }
+            if (l < lc) {
+              double n = Z * q1;
+              if (l > m) n = fma(-c_q[l * 6 + m] * r2, q0, n);
+              q0 = q1;
+              q1 = n;
+            }
+          }
         }
       }
-      // ---- VRR1, level by level (Eq. vrr1)
+      // ---- VRR1, level by level (Eq. vrr1).  A level is few targets and a
+      // barrier: with few triples every (target, primitive, triple) is an item
+      // of its own, with 16 or more an item is its target over the chunk's
+      // primitives ((dd|f) K = 3: 6.4 -> 6.1 ms; one triple: 93 -> 102 ms)
       for (int e = 1; e <= Lab; ++e) {
         const int j0 = d.vlev_start[e - 1];
-        const int nl = d.vlev_start[e] - j0;
-        FDiv fX;
-        fX.init(nl);
-        const unsigned n = (unsigned)(T * G * nl);
-        for (unsigned w = tid; w < n; w += kThreads) {
-          int t, g, x;
-          dec3(w, mode, fT, fG, fX, t, g, x);
-          if (t >= tv || g >= gcnt) continue;
-          const uint4 it = __ldg(d.vtab + j0 + x);
-          const int dst = it.x & 0xFFFF, a = it.x >> 16, an = it.y & 0xFFFF, b = it.y >> 16, bn = it.z & 0xFFFF;
-          const int axis = (it.z >> 16) & 0xF, nq = (it.z >> 20) & 0xF;
-          const int p = p0 + g;
-          const int ip = (int)fKc.div(p);
-          const double* pr = sm + d.pair_base + ip * kPairRec;
-          const int vb = BUF_TG(d.V, 0, g, t), vs = d.V.si;
-          const int fb = BUF_TG(d.F, 0, g, t), fs = d.F.si;
-          double val = pr[PR_PA + axis] * sm[vb + a * vs];
-          val = fma(-sm[fb + axis * fs], sm[vb + an * vs], val);
-          if (nq) {
-            double u = fma(-sm[fb + 3 * fs], sm[vb + bn * vs], sm[vb + b * vs]);
-            val = fma(pr[PR_NH + nq - 1], u, val);
+        const int nl = d.vlev_start[e] - j0, vs = d.V.si, fs = d.F.si;
+        const auto target = [&](const uint4& it, int axis, int nq, double pa, double nh, int g, int t) {
+          double* v = sm + BUF_TG(d.V, 0, g, t);
+          const double* f = sm + BUF_TG(d.F, 0, g, t);
+          double val = pa * v[(it.x >> 16) * vs];
+          val = fma(-f[axis * fs], v[(it.y & 0xFFFF) * vs], val);
+          if (nq) val = fma(nh, fma(-f[3 * fs], v[(it.z & 0xFFFF) * vs], v[(it.y >> 16) * vs]), val);
+          v[(it.x & 0xFFFF) * vs] = val;
+        };
+        if (T >= 16) {
+          stage<NT>(nl, T, tv, mode, [&](int x, int t0, int ts, auto tb) {
+            constexpr int TB = decltype(tb)::n;
+            const uint4 it = __ldg(d.vtab + j0 + x);
+            const int axis = (it.z >> 16) & 0xF, nq = (it.z >> 20) & 0xF;
+            for (int g = 0; g < gcnt; ++g) {
+              const double* pr = sm + d.pair_base + (int)fKc.div(p0 + g) * kPairRec;
+              const double pa = pr[PR_PA + axis], nh = nq ? pr[PR_NH + nq - 1] : 0.0;
+#pragma unroll
+              for (int k = 0; k < TB; ++k)
+                if (t0 + k * ts < tv) target(it, axis, nq, pa, nh, g, t0 + k * ts);
+            }
+          });
+        } else {
+          FDiv fX;
+          fX.init(nl);
+          for (unsigned w = tid; w < (unsigned)(T * G * nl); w += NT) {
+            int t, g, x;
+            dec3(w, mode, fT, fG, fX, t, g, x);
+            if (t >= tv || g >= gcnt) continue;
+            const uint4 it = __ldg(d.vtab + j0 + x);
+            const int axis = (it.z >> 16) & 0xF, nq = (it.z >> 20) & 0xF;
+            const double* pr = sm + d.pair_base + (int)fKc.div(p0 + g) * kPairRec;
+            target(it, axis, nq, pr[PR_PA + axis], nq ? pr[PR_NH + nq - 1] : 0.0, g, t);
           }
-          sm[vb + dst * vs] = val;
         }
         __syncthreads();
       }
       if (Lab == 0) __syncthreads();
-      // ---- accumulate CVRR2 prerequisites over the chunk's primitives; two
-      // independent accumulators per thread keep two FMA chains in flight
+      // ---- accumulate CVRR2 prerequisites over the chunk's primitives
       {
-        FDiv fX;
-        fX.init(d.NACC);
-        const unsigned n = (unsigned)(T * d.NACC);
-        for (unsigned w0 = tid; w0 < n; w0 += 2 * kThreads) {
-          const unsigned w1 = w0 + kThreads;
-          const bool has1 = w1 < n;
-          int t0, a0, t1, a1;
-          dec2(w0, mode, fT, fX, t0, a0);
-          dec2(has1 ? w1 : w0, mode, fT, fX, t1, a1);
-          const bool ok0 = t0 < tv, ok1 = has1 && t1 < tv;
-          const unsigned e0 = __ldg(d.atab + a0), e1 = __ldg(d.atab + a1);
-          const int pa0 = BUF_T(d.P, a0, t0), pa1 = BUF_T(d.P, a1, t1);
-          const int vb0 = BUF_TG(d.V, (int)(e0 & 0xFFFF), 0, t0), wb0 = BUF_TG(d.W, (int)(e0 >> 16), 0, t0);
-          const int vb1 = BUF_TG(d.V, (int)(e1 & 0xFFFF), 0, t1), wb1 = BUF_TG(d.W, (int)(e1 >> 16), 0, t1);
-          // FP64 instructions cost a whole warp slot, so only stored chains run
-          if (ok0 && ok1) {
-            double acc0 = sm[pa0], acc1 = sm[pa1];
-#pragma unroll 4
-            for (int g = 0; g < gcnt; ++g) {
-              acc0 = fma(sm[vb0 + g * d.V.sg], sm[wb0 + g * d.W.sg], acc0);
-              acc1 = fma(sm[vb1 + g * d.V.sg], sm[wb1 + g * d.W.sg], acc1);
-            }
-            sm[pa0] = acc0;
-            sm[pa1] = acc1;
-          } else if (ok0 || ok1) {
-            const int pa = ok0 ? pa0 : pa1, vb = ok0 ? vb0 : vb1, wb = ok0 ? wb0 : wb1;
-            double acc = sm[pa];
-#pragma unroll 4
-            for (int g = 0; g < gcnt; ++g) acc = fma(sm[vb + g * d.V.sg], sm[wb + g * d.W.sg], acc);
-            sm[pa] = acc;
+        const int vg = d.V.sg, wg = d.W.sg;
+        stage<NT>(d.NACC, T, tv, mode, [&](int x, int t0, int ts, auto tb) {
+          constexpr int TB = decltype(tb)::n;
+          const unsigned e = __ldg(d.atab + x);
+          const double* v = sm + BUF_TG(d.V, (int)(e & 0xFFFF), 0, t0);
+          const double* w = sm + BUF_TG(d.W, (int)(e >> 16), 0, t0);
+          double* p = sm + BUF_T(d.P, x, t0);
+          const int sv = d.V.st * ts, sw = d.W.st * ts, sp_ = d.P.st * ts;
+          double acc[TB];
+          const bool full = t0 + (TB - 1) * ts < tv;
+#pragma unroll
+          for (int k = 0; k < TB; ++k) acc[k] = (full || t0 + k * ts < tv) ? (chunk ? p[k * sp_] : 0.0) : 0.0;
+          if (full) {
+#pragma unroll 2
+            for (int g = 0; g < gcnt; ++g)
+#pragma unroll
+              for (int k = 0; k < TB; ++k) acc[k] = fma(v[k * sv + g * vg], w[k * sw + g * wg], acc[k]);
+#pragma unroll
+            for (int k = 0; k < TB; ++k) p[k * sp_] = acc[k];
+          } else {
+#pragma unroll
+            for (int k = 0; k < TB; ++k)
+              if (t0 + k * ts < tv) {
+                for (int g = 0; g < gcnt; ++g) acc[k] = fma(v[k * sv + g * vg], w[k * sw + g * wg], acc[k]);
+                p[k * sp_] = acc[k];
+              }
           }
-        }
+        });
       }
       __syncthreads();
     }
 
-    // ---- CVRR2 targets (a 0|c) by the n-quantum gather (Sec. 2.5.4)
-    {
+    // ---- CVRR2 targets (a 0|C) by the n-quantum gather (Sec. 2.5.4), the ket
+    // already solid harmonic
+    if (d.comp) {
       FDiv fX;
       fX.init(d.ngt);
-      const unsigned n = (unsigned)(T * d.ngt);
-      for (unsigned w = tid; w < n; w += kThreads) {
+      for (unsigned w = tid; w < (unsigned)(T * d.ngt); w += NT) {
         int t, r;
         dec2(w, mode, fT, fX, t, r);
         if (t >= tv) continue;
         const int id = __ldg(d.gdst + r);
-        double s = 0.0;
-        if (d.comp & 1) {
-          const int q0 = __ldg(d.gptr + id), q1 = __ldg(d.gptr + id + 1);
-          Dot2 acc;
-          for (int q = q0; q < q1; ++q) {
-            const unsigned e = __ldg(d.gterm + q);
-            acc.add(__ldg(d.pal + (e >> 20)), sm[BUF_T(d.P, e & 0xFFFFF, t)]);
-          }
-          s = acc.value();
-        } else if (mode == 0) {
-          // lanes share the target: CSR row, broadcast loads
-          const int q0 = __ldg(d.gptr + id), q1 = __ldg(d.gptr + id + 1);
-#pragma unroll 4
-          for (int q = q0; q < q1; ++q) {
-            const unsigned e = __ldg(d.gterm + q);
-            s = fma(__ldg(d.pal + (e >> 20)), sm[BUF_T(d.P, e & 0xFFFFF, t)], s);
-          }
-        } else {
-          // lanes take consecutive targets: sliced ELL, one coalesced line
-          // per term step and one trip count per slice
-          const int2 sl = __ldg(d.gslice + (r >> 5));
-          const unsigned* ge = d.gell + sl.x + (r & 31);
-#pragma unroll 4
-          for (int j = 0; j < sl.y; ++j) {
-            const unsigned e = __ldg(ge + 32 * j);
-            s = fma(__ldg(d.pal + (e >> 20)), sm[BUF_T(d.P, e & 0xFFFFF, t)], s);
-          }
+        Dot2 acc;
+        for (int q = __ldg(d.gptr + id); q < __ldg(d.gptr + id + 1); ++q) {
+          const unsigned e = __ldg(d.gterm + q);
+          acc.add(__ldg(d.pal + (e >> kGatherBits)), sm[BUF_T(d.P, e & kGatherMask, t)]);
         }
-        sm[BUF_T(d.Gb, id, t)] = s;
+        sm[BUF_T(d.H[0], id, t)] = acc.value();
       }
-    }
-    __syncthreads();
-    // ---- ket: Cartesian -> solid harmonic.  With targets across lanes
-    // (mode 1) the items run C-major, so a warp's lanes share one C and with
-    // it the loop trip count (a warp instruction costs the same whatever the
-    // number of active lanes).
-    {
-      FDiv fX, fC, fR;
-      const int nx = d.nkrow * d.nC;
-      fX.init(nx);
-      fC.init(d.nC);
-      fR.init(d.nkrow);
-      const unsigned n = (unsigned)(T * nx);
-      for (unsigned w = tid; w < n; w += kThreads) {
-        int t, x;
-        dec2(w, mode, fT, fX, t, x);
-        if (t >= tv) continue;
-        int row, C;
+    } else {
+      // lanes that share the target (mode 0) walk its CSR row by broadcast
+      // loads; lanes on consecutive targets (mode 1; the list padded to whole
+      // warps) a sliced-ELL copy, one coalesced line per term step and one trip
+      // count per slice
+      stage<NT>(mode == 0 ? d.ngt : (d.ngt + 31) & ~31, T, tv, mode, [&](int r, int t0, int ts, auto tb) {
+        constexpr int TB = decltype(tb)::n;
+        if (r >= d.ngt) return;
+        const int id = __ldg(d.gdst + r);
+        const unsigned* ge;
+        int n, step;
         if (mode == 0) {
-          row = (int)fC.div(x);
-          C = x - row * d.nC;
+          const int q0 = __ldg(d.gptr + id);
+          ge = d.gterm + q0;
+          n = __ldg(d.gptr + id + 1) - q0;
+          step = 1;
         } else {
-          C = (int)fR.div(x);
-          row = x - C * d.nkrow;
+          const int2 sl = __ldg(d.gslice + (r >> 5));
+          ge = d.gell + sl.x + (r & 31);
+          n = sl.y;
+          step = 32;
         }
-        x = row * d.nC + C;
-        const int q0 = __ldg(d.kptr + C), q1 = __ldg(d.kptr + C + 1);
-        double s = 0.0;
-        if (d.comp & 2) {
-          Dot2 acc;
-          for (int q = q0; q < q1; ++q) {
-            const int2 e = __ldg(d.kent + q);
-            acc.add(__ldg(d.pal + e.y), sm[BUF_T(d.Gb, row * d.ncc + e.x, t)]);
+        const double* P = sm + d.P.base + t0 * d.P.st;
+        const int st = d.P.st * ts, si = d.P.si;
+        double s[TB];
+#pragma unroll
+        for (int k = 0; k < TB; ++k) s[k] = 0.0;
+        const bool full = t0 + (TB - 1) * ts < tv;
+        if (full) {
+#pragma unroll 2
+          for (int j = 0; j < n; ++j) {
+            const unsigned e = __ldg(ge + j * step);
+            const double c = __ldg(d.pal + (e >> kGatherBits));
+            const double* p = P + (int)(e & kGatherMask) * si;
+#pragma unroll
+            for (int k = 0; k < TB; ++k) s[k] = fma(c, p[k * st], s[k]);
           }
-          s = acc.value();
         } else {
-          for (int q = q0; q < q1; ++q) {
-            const int2 e = __ldg(d.kent + q);
-            s = fma(__ldg(d.pal + e.y), sm[BUF_T(d.Gb, row * d.ncc + e.x, t)], s);
+          for (int j = 0; j < n; ++j) {
+            const unsigned e = __ldg(ge + j * step);
+            const double c = __ldg(d.pal + (e >> kGatherBits));
+            const double* p = P + (int)(e & kGatherMask) * si;
+#pragma unroll
+            for (int k = 0; k < TB; ++k)
+              if (t0 + k * ts < tv) s[k] = fma(c, p[k * st], s[k]);
           }
         }
-        sm[BUF_T(d.H[0], x, t)] = s;
-      }
+#pragma unroll
+        for (int k = 0; k < TB; ++k)
+          if (t0 + k * ts < tv) sm[BUF_T(d.H[0], id, t0 + k * ts)] = s[k];
+      });
     }
     __syncthreads();
-    Buf cur = hrr_and_bra(d, sm, T, tv, mode, fT);
+    Buf cur = hrr_and_bra<NT>(d, sm, T, tv, mode);
     if (d.digest == 3) {
       // ---- matrix store (2-centre metric (P|Q) = (P 1|Q), nB = 1): element
       // (t, A, C) of the tile goes to out[(ao_pair + A) * ldD + ao_ket + C]
@@ -663,7 +733,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       fAC.init(nAC);
       fC.init(nC);
       const unsigned n = (unsigned)(tv * nAC);
-      for (unsigned w = tid; w < n; w += kThreads) {
+      for (unsigned w = tid; w < n; w += NT) {
         const int t = (int)fAC.div(w), r = (int)(w - (unsigned)t * nAC);
         const int A = (int)fC.div(r), C = r - A * nC;
         d.out[(long long)(pao.x + A) * d.ldD + __ldg(d.aux_ao + aux0 + t) + C] = sm[BUF_T(cur, A * nC + C, t)];
@@ -681,14 +751,14 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       const int kAB = (nAB + 3) & ~3, kR = (R + 3) & ~3;
       double* Ds = sm + d.dscr;      // [kAB][8]
       double* Cs = Ds + kAB * 8;     // [kR][8]
-      for (int i = tid; i < kAB * 8; i += kThreads) {
+      for (int i = tid; i < kAB * 8; i += NT) {
         const int r = i >> 3, dd = i & 7;  // r: storage index of (A, B)
         const int A = d.orient ? r % nA : r / nB, B = d.orient ? r / nA : r % nB;
         Ds[i] = (d.gamma && r < nAB && dd < nd)
                     ? __ldg(d.D + dd * d.dstride + (long long)(pao.x + A) * d.ldD + pao.y + B)
                     : 0.0;
       }
-      for (int i = tid; i < kR * 8; i += kThreads) {
+      for (int i = tid; i < kR * 8; i += NT) {
         const int r = i >> 3, dd = i & 7;
         double v = 0.0;
         if (d.J && r < R && dd < nd) {
@@ -700,7 +770,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       __syncthreads();
       const Buf cb = cur;
       const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
-      constexpr int kWarps = kThreads / 32;
+      constexpr int kWarps = NT / 32;
       if (d.gamma) {
         for (int m0 = warp * 8; m0 < R; m0 += kWarps * 8) {
           const int m = m0 + g;
@@ -750,12 +820,12 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       double* Cs = Ds + nAB;
       const int sA = d.orient ? 1 : nB, sB = d.orient ? nA : 1;  // storage index of (A, B)
       if (d.gacc)
-        for (int s = tid; s < nAB; s += kThreads) {
+        for (int s = tid; s < nAB; s += NT) {
           const int A = s / nB, B = s - A * nB;
           Ds[A * sA + B * sB] = __ldg(d.D + (long long)(pao.x + A) * d.ldD + pao.y + B);
         }
       if (d.Jacc)
-        for (int i = tid; i < tv * nC; i += kThreads) {
+        for (int i = tid; i < tv * nC; i += NT) {
           const int t = i / nC, C = i - t * nC;
           Cs[i] = __ldg(d.cvec + __ldg(d.aux_ao + aux0 + t) + C);
         }
@@ -764,7 +834,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       FDiv fC;
       fC.init(nC);
       if (d.gacc)
-        seg_dot(tv * nC, nAB,
+        seg_dot<NT>(tv * nC, nAB,
                 [&](int o, int r, double acc) {
                   const int t = (int)fC.div(o), C = o - t * nC;
                   return fma(sm[BUF_T(cb, r * nC + C, t)], Ds[r], acc);
@@ -774,7 +844,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
                   fix_add(d.gacc + kFixWords * (__ldg(d.aux_ao + aux0 + t) + C), wg * v);
                 });
       if (d.Jacc)
-        seg_dot(nAB, tv * nC,
+        seg_dot<NT>(nAB, tv * nC,
                 [&](int o, int r, double acc) {
                   const int t = (int)fC.div(r), C = r - t * nC;
                   return fma(sm[BUF_T(cb, o * nC + C, t)], Cs[r], acc);
@@ -795,7 +865,7 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
       fC.init(d.nC);
       double* o = d.out + ((pair - d.out_pair0) * d.naux + aux0) * (long long)d.nblk;
       const unsigned n = (unsigned)(tv * d.nblk);
-      for (unsigned w = tid; w < n; w += kThreads) {
+      for (unsigned w = tid; w < n; w += NT) {
         const unsigned t = fB.div(w);
         const int idx = (int)(w - t * d.nblk);
         int sidx = idx;
@@ -812,16 +882,29 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
   }
 }
 
-// One class launch: CTAs stride over the class's tiles.
-__global__ void __launch_bounds__(kThreads) eri3c_kernel(const __grid_constant__ ClassDesc d) {
+// One class launch: CTAs stride over the class's tiles.  384 threads and 56
+// registers when three CTAs fit an SM's shared memory (their barriers overlap
+// better: (ff|g) K = 1 12.5 -> 10.8 ms), else 512 threads and two CTAs ((gg|i)
+// K = 6, one triple per tile, 99 -> 93 ms).  kVar 1: DF-J launches digesting
+// several densities.
+template <int kVar, int NT, int NB>
+__global__ void __launch_bounds__(NT, NB) eri3c_kernel(const __grid_constant__ ClassDesc d) {
   extern __shared__ double sm[];
-  for (long long tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) tile_body<0>(d, tile, sm);
+  for (long long tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) tile_body<kVar, NT>(d, tile, sm);
 }
 
-// The same for DF-J launches digesting several densities (digest == 4).
-__global__ void __launch_bounds__(kThreads) eri3c_multi_kernel(const __grid_constant__ ClassDesc d) {
+// Both orientations of a small plan (one tile per SM at most) side by side: the
+// first ga CTAs take a's tiles, the others b's.
+constexpr int kBothThreads = 512;
+__global__ void __launch_bounds__(kBothThreads, 1) eri3c_kernel_both(const __grid_constant__ ClassDesc a,
+                                                                     const __grid_constant__ ClassDesc b, int ga) {
   extern __shared__ double sm[];
-  for (long long tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) tile_body<1>(d, tile, sm);
+  if ((int)blockIdx.x < ga) {
+    for (long long tile = blockIdx.x; tile < a.ntiles; tile += ga) tile_body<0, kBothThreads>(a, tile, sm);
+  } else {
+    for (long long tile = blockIdx.x - ga; tile < b.ntiles; tile += gridDim.x - ga)
+      tile_body<0, kBothThreads>(b, tile, sm);
+  }
 }
 
 // (s s|C) classes (la = lb = 0) stored per integral, one thread per triple.
@@ -1242,12 +1325,13 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
 // ordered longest first on the host).  No CTA ever waits on another.  The
 // item's descriptor is staged in shared memory (re-copied only when the class
 // changes), so the tile body reads its fields from there, not from global
-// memory.  kMinBlocks = 3 caps the registers at 40 so that three 512-thread
-// CTAs fit an SM (with a few spills to L1: the descriptor fields the
-// parameter-space form keeps in constant banks now live in registers);
-// kMinBlocks = 1 leaves the compiler free (64 registers, two CTAs per SM).
+// memory.  kMinBlocks = 2 caps the registers at 64 so that two 512-thread
+// CTAs fit an SM, kMinBlocks = 1 (items whose shared memory lets only one fit)
+// leaves the compiler free.
+constexpr int kPersThreads = 512;
+
 template <int kMinBlocks>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) eri3c_persistent(const ClassDesc* __restrict__ descs,
+__global__ void __launch_bounds__(kPersThreads, kMinBlocks) eri3c_persistent(const ClassDesc* __restrict__ descs,
                                                                          const int2* __restrict__ work, long long nwork,
                                                                          unsigned long long* __restrict__ counter) {
   extern __shared__ double sm[];
@@ -1266,11 +1350,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) eri3c_persistent(const C
     if (wk.x != cur) {
       const unsigned long long* src = reinterpret_cast<const unsigned long long*>(descs + wk.x);
       unsigned long long* dst = reinterpret_cast<unsigned long long*>(&sd);
-      for (int i = threadIdx.x; i < kWords; i += kThreads) dst[i] = src[i];
+      for (int i = threadIdx.x; i < kWords; i += kPersThreads) dst[i] = src[i];
       cur = wk.x;
       __syncthreads();
     }
-    tile_body<0>(sd, wk.y, sm);
+    tile_body<0, kPersThreads>(sd, wk.y, sm);
   }
 }
 
@@ -1292,19 +1376,13 @@ cudaError_t init_constants() {
   return cudaMemcpyToSymbol(c_inv2m1, v, sizeof(v));
 }
 
-cudaError_t launch_pair_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb,
-                                   double* rec, double* ab, cudaStream_t st, int scale_a, int scale_b) {
-  long long n = npair * Ka * Kb;
+cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
+                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
+                              double* auxrec, double* auxc, cudaStream_t st) {
+  const long long n = npair * Ka * Kb + naux * Kc;
   if (n == 0) return cudaSuccess;
-  pair_precompute<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(orb, pairs, npair, Ka, Kb, rec, ab, scale_a, scale_b);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_aux_precompute(const DevBasis& aux, const int32_t* auxs, long long naux, int Kc, double* rec,
-                                  double* cxyz, cudaStream_t st) {
-  long long n = naux * Kc;
-  if (n == 0) return cudaSuccess;
-  aux_precompute<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(aux, auxs, naux, Kc, rec, cxyz);
+  precompute_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(orb, pairs, npair, Ka, Kb, rec, ab, aux, auxs, naux, Kc,
+                                                                auxrec, auxc);
   return cudaGetLastError();
 }
 
@@ -1321,15 +1399,48 @@ static int device_sms() {
   return n;
 }
 
+// Whether three CTAs of the 384-thread tile kernel fit an SM.
+static bool three_ctas(int smem_bytes) { return smem_bytes <= 233472 / 3 - 1024; }
+
+// Set once per process, from the first plan or occupancy query on.
+static cudaError_t tile_kernel_attributes() {
+  static const cudaError_t rc = [] {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void* f) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    };
+    set((const void*)eri3c_kernel<0, 512, 2>);
+    set((const void*)eri3c_kernel<0, 384, 3>);
+    set((const void*)eri3c_kernel<1, 512, 2>);
+    set((const void*)eri3c_kernel<1, 384, 3>);
+    set((const void*)eri3c_kernel_both);
+    return e;
+  }();
+  return rc;
+}
+
+// Whether a launch runs the tile kernel (not a register-resident one).
+static bool on_tile_kernel(const ClassDesc& d) {
+  if (d.digest == 4) return true;
+  if (d.la == 0 && d.lb == 0 && d.orient == 0 && (d.digest == 0 || (d.digest == 1 && d.tiles))) return false;
+  return !((d.digest == 0 || (d.digest == 1 && d.tiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 && (d.lc > 0 || d.K > 1));
+}
+
+bool can_launch_both(const ClassDesc& a, const ClassDesc& b) {
+  return a.digest == 0 && b.digest == 0 && on_tile_kernel(a) && on_tile_kernel(b);
+}
+
+cudaError_t launch_eri3c_both(const ClassDesc& a, int ga, const ClassDesc& b, int gb, cudaStream_t st) {
+  cudaError_t e = tile_kernel_attributes();
+  if (e != cudaSuccess) return e;
+  const int smem = std::max(a.smem_doubles, b.smem_doubles) * 8;
+  eri3c_kernel_both<<<ga + gb, kBothThreads, smem, st>>>(a, b, ga);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(eri3c_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(eri3c_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  cudaError_t e = tile_kernel_attributes();
+  if (e != cudaSuccess) return e;
   if (d.digest == 0 && d.la == 0 && d.lb == 0 && d.orient == 0) {
     // (s s|C): the register-resident form, one thread per triple
     const long long nb = (d.nsub * d.naux + kSsThreads - 1) / kSsThreads;
@@ -1382,10 +1493,16 @@ cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
       case 5: eri3c_ss_dfj_kernel<5><<<g, kSsThreads, 0, st>>>(d); break;
       default: eri3c_ss_dfj_kernel<6><<<g, kSsThreads, 0, st>>>(d); break;
     }
-  } else if (d.digest == 4)
-    eri3c_multi_kernel<<<grid, kThreads, (size_t)d.smem_doubles * 8, st>>>(d);
-  else
-    eri3c_kernel<<<grid, kThreads, (size_t)d.smem_doubles * 8, st>>>(d);
+  } else {
+    const int smem = d.smem_doubles * 8;
+    if (d.digest == 4) {
+      if (three_ctas(smem)) eri3c_kernel<1, 384, 3><<<grid, 384, smem, st>>>(d);
+      else eri3c_kernel<1, 512, 2><<<grid, 512, smem, st>>>(d);
+    } else {
+      if (three_ctas(smem)) eri3c_kernel<0, 384, 3><<<grid, 384, smem, st>>>(d);
+      else eri3c_kernel<0, 512, 2><<<grid, 512, smem, st>>>(d);
+    }
+  }
   return cudaGetLastError();
 }
 
@@ -1399,24 +1516,24 @@ cudaError_t launch_boys(const double* T, long long n, int mmax, const double* ta
 // The dynamic shared-memory attribute is set by persistent_occupancy(), which
 // callers run before any stream capture.
 cudaError_t launch_persistent(const ClassDesc* descs, const int2* work, long long nwork, unsigned long long* counter,
-                              int grid, int smem_bytes, int three, cudaStream_t st) {
-  if (three)
-    eri3c_persistent<3><<<grid, kThreads, smem_bytes, st>>>(descs, work, nwork, counter);
+                              int grid, int smem_bytes, int two, cudaStream_t st) {
+  if (two)
+    eri3c_persistent<2><<<grid, kPersThreads, smem_bytes, st>>>(descs, work, nwork, counter);
   else
-    eri3c_persistent<1><<<grid, kThreads, smem_bytes, st>>>(descs, work, nwork, counter);
+    eri3c_persistent<1><<<grid, kPersThreads, smem_bytes, st>>>(descs, work, nwork, counter);
   return cudaGetLastError();
 }
 
-int persistent_occupancy(int smem_bytes, int three) {
+int persistent_occupancy(int smem_bytes, int two) {
   int nb = 0;
   const int cap = 232448 - (int)sizeof(ClassDesc) - 64;
   cudaError_t e;
-  if (three) {
-    cudaFuncSetAttribute(eri3c_persistent<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_persistent<3>, kThreads, smem_bytes);
+  if (two) {
+    cudaFuncSetAttribute(eri3c_persistent<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_persistent<2>, kPersThreads, smem_bytes);
   } else {
     cudaFuncSetAttribute(eri3c_persistent<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_persistent<1>, kThreads, smem_bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_persistent<1>, kPersThreads, smem_bytes);
   }
   if (e != cudaSuccess) return 1;
   return nb < 1 ? 1 : nb;
@@ -1424,8 +1541,11 @@ int persistent_occupancy(int smem_bytes, int three) {
 
 int eri3c_occupancy(int smem_bytes) {
   int nb = 0;
-  cudaFuncSetAttribute(eri3c_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_kernel, kThreads, smem_bytes) != cudaSuccess) return 1;
+  if (tile_kernel_attributes() != cudaSuccess) return 1;
+  const cudaError_t e = three_ctas(smem_bytes)
+      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_kernel<0, 384, 3>, 384, smem_bytes)
+      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_kernel<0, 512, 2>, 512, smem_bytes);
+  if (e != cudaSuccess) return 1;
   return nb < 1 ? 1 : nb;
 }
 

@@ -1062,8 +1062,9 @@ struct HermPlan {
   double flops = 0, max_adds = 0;
 };
 
-cudaError_t launch_aux_precompute(const DevBasis& aux, const int32_t* auxs, long long naux, int Kc, double* rec,
-                                  double* cxyz, cudaStream_t st);
+cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
+                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
+                              double* auxrec, double* auxc, cudaStream_t st);
 
 void herm_destroy(HermPlan* p) {
   if (!p) return;
@@ -1441,7 +1442,8 @@ cudaError_t herm_begin(HermPlan* p, const double* D, bool dens, bool y, cudaStre
   cudaError_t e = cudaSuccess;
   if (y) e = cudaMemsetAsync(p->arena + p->zero_off, 0, p->zero_bytes, st);
   for (auto& k : p->kets)
-    if (e == cudaSuccess) e = launch_aux_precompute(p->aux->dev(), k.shells, k.n, k.Kc, k.rec, k.xyz, st);
+    if (e == cudaSuccess) e = launch_precompute(p->orb->dev(), nullptr, 0, 1, 1, nullptr, nullptr, p->aux->dev(), k.shells, k.n,
+                                                k.Kc, k.rec, k.xyz, st);
   if (e != cudaSuccess) return e;
   HermPairArgs a = p->pa;
   a.D = D;

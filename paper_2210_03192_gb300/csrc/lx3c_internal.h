@@ -9,7 +9,6 @@
 
 namespace lx3c {
 
-constexpr int kThreads = 512;            // threads per CTA of the integral kernels
 constexpr int kMaxLev = 16;              // VRR1 levels (la+lb) and HRR levels (lb)
 constexpr int kPairRec = 28;             // doubles per primitive-pair record
 constexpr int kPairNHalf = 13;           // offset of n/(2 gamma), n = 1..14
@@ -33,6 +32,10 @@ constexpr double kDefaultAmpMax = 300.0; // orientation: largest weighted HRR am
 // sub-pair whose recurrences run on centre B the PB and zb fields are copied
 // into the PA and za slots.
 enum PairField { PR_G = 0, PR_K = 1, PR_P = 2, PR_PA = 5, PR_PB = 8, PR_ZA = 11, PR_ZB = 12, PR_NH = kPairNHalf };
+
+// Gather term: accumulator index in the low kGatherBits, palette id above.
+constexpr int kGatherBits = 17;
+constexpr unsigned kGatherMask = (1u << kGatherBits) - 1;
 
 // A shared-memory buffer: element (idx, g, t) lives at base + idx*si + g*sg + t*st
 // (in doubles).  Per-triple buffers have sg = 0.
@@ -63,7 +66,7 @@ struct ClassDesc {
   int NV, NW, NF, NACC;
   // VRR1 levels e = 1..Lab: items [vlev_start[e-1], vlev_start[e])
   int vlev_start[kMaxLev + 1];
-  int nW;                  // weight items (= NW)
+  int kmax;                // weights Y^k s_{lc-k,m}(X), k = 0..kmax
   int ngt;                 // gather targets
   int nkrow;               // rows (bra Cartesian functions) entering the ket transform
   int nhrr;                // HRR rounds (lb for 1-q HRR; lb/2 + lb%2 for 2-q)
@@ -72,10 +75,9 @@ struct ClassDesc {
   int nbA, nbB;            // bra transform output rows (A,b) and (A,B), 0 if none
   // tables (device)
   const uint4* vtab;       // VRR1 items
-  const int4* wtab;        // weight items: F-buffer sources and count
   const unsigned* atab;    // accumulator -> vidx | widx<<16
   const int* gptr;         // gather CSR row pointers (by target id)
-  const unsigned* gterm;   // gather terms: pidx | coef_id<<20
+  const unsigned* gterm;   // gather terms: pidx | coef_id << kGatherBits
   // the same terms as sliced ELL for targets across lanes: slice s = targets
   // gdst[32s .. 32s+31], entry j of lane l at gell[gslice[s].x + 32 j + l]
   // (padded to the slice's longest row with zero-coefficient terms)
@@ -94,10 +96,10 @@ struct ClassDesc {
   const int2* bbent;
   // shared-memory layout (doubles)
   int pair_base, aux_base, ab_base;
-  Buf V, W, F, P, Gb, H[kMaxLev + 1], BA, BB, OUT;
+  Buf V, W, F, P, H[kMaxLev + 1], BA, BB, OUT;
   int smem_doubles;
-  // compensated (Dot2) summation in the contracted stages: bit 0 the CVRR2
-  // gather, bit 1 the ket transform
+  // compensated (Dot2) summation of the CVRR2 gather, which holds the ket
+  // transform (either bit)
   int comp;
   // data
   const double* pairrec;   // [npair][Kab][kPairRec]
@@ -155,7 +157,6 @@ struct ClassTables {
   int NV, NW, NF, NACC;
   std::vector<int> vlev_start;
   std::vector<uint4> vtab;
-  std::vector<int4> wtab;
   std::vector<unsigned> atab;
   std::vector<int> gptr, gdst;
   std::vector<unsigned> gterm;
@@ -176,15 +177,13 @@ struct ClassTables {
   // algorithmic FP64 flop counts (FMA = 2)
   double flops_prim;      // per primitive triple
   double flops_contr;     // per contracted triple (after the primitive loop)
-  // debug: (e comp, k, n comp) of each accumulator
-  std::vector<int4> acc_key;
+  int kmax = 0;
 };
 
 // Device-side constant tables (capi.cu)
 struct DevClass {
   void* blob = nullptr;
   const uint4* vtab;
-  const int4* wtab;
   const unsigned* atab;
   const int* gptr;
   const unsigned* gterm;
@@ -221,8 +220,8 @@ void fill_desc_common(ClassDesc& d, const ClassTables& ct, const DevClass& dc, c
                       const double* boys_mid, int orient, int kmax, int Kab_rec, int Kc, const LaunchShape& sh);
 // Device pointers of every class table inside one uploaded blob laid out by
 // class_blob (same offsets on host and device).
-std::vector<char> class_blob(const ClassTables& ct, size_t offs[16]);
-void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t offs[16]);
+std::vector<char> class_blob(const ClassTables& ct, size_t offs[15]);
+void class_blob_pointers(DevClass& dc, const void* dev_blob, const size_t offs[15]);
 
 // planner entry points (plan.cu)
 const ClassTables& class_tables(int la, int lb, int lc, int bra_pure);  // HRR variant from the hints

@@ -33,10 +33,9 @@
 #include "lx3c_internal.h"
 
 namespace lx3c {
-cudaError_t launch_pair_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb,
-                                   double* rec, double* ab, cudaStream_t st, int scale_a = 0, int scale_b = 0);
-cudaError_t launch_aux_precompute(const DevBasis& aux, const int32_t* auxs, long long naux, int Kc, double* rec,
-                                  double* cxyz, cudaStream_t st);
+cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
+                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
+                              double* auxrec, double* auxc, cudaStream_t st);
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st);
 int eri3c_occupancy(int smem_bytes);
 }  // namespace lx3c
@@ -588,8 +587,8 @@ lx3c_status lx3c_metric_execute(lx3c_metric* p, double* V, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   for (auto& g : p->groups) {
     const long long ns = (long long)g.shells.size();
-    MCUDA(launch_pair_precompute(p->bra->dev(), g.d_pairs, ns, g.K, 1, g.d_pairrec, g.d_pairab, st));
-    MCUDA(launch_aux_precompute(p->aux->dev(), g.d_kets, ns, g.K, g.d_auxrec, g.d_auxc, st));
+    MCUDA(launch_precompute(p->bra->dev(), g.d_pairs, ns, g.K, 1, g.d_pairrec, g.d_pairab, p->aux->dev(), g.d_kets, ns,
+                            g.K, g.d_auxrec, g.d_auxc, st));
   }
   for (auto& L : p->launches) {
     ClassDesc d = L.desc;
@@ -602,7 +601,7 @@ lx3c_status lx3c_metric_execute(lx3c_metric* p, double* V, void* stream) {
 lx3c_status lx3c_metric_info(const lx3c_metric* p, double* out, int n) {
   if (!p || (!out && n > 0)) return mfail(LX3C_EINVAL, "metric_info: null pointer");
   const double v[] = {(double)p->naux_ao, (double)p->groups.size(), (double)p->launches.size(),
-                      2.0 * p->groups.size() + p->launches.size(), p->flops,
+                      1.0 * p->groups.size() + p->launches.size(), p->flops,
                       (double)p->aux->nshell * (double)p->aux->nshell};
   for (int i = 0; i < n && i < 6; ++i) out[i] = v[i];
   return LX3C_OK;

@@ -21,10 +21,9 @@
 
 namespace lx3c {
 cudaError_t init_constants();
-cudaError_t launch_pair_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb,
-                                   double* rec, double* ab, cudaStream_t st, int scale_a = 0, int scale_b = 0);
-cudaError_t launch_aux_precompute(const DevBasis& aux, const int32_t* auxs, long long naux, int Kc, double* rec,
-                                  double* cxyz, cudaStream_t st);
+cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
+                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
+                              double* auxrec, double* auxc, cudaStream_t st);
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st);
 int eri3c_occupancy(int smem_bytes);
 void set_last_error(const std::string& msg);
@@ -122,7 +121,7 @@ __global__ void noalloc_orient(const int32_t* __restrict__ pairs, long long npai
 struct NaBlob {
   std::vector<char> bytes;
   size_t base[2] = {0, 0};
-  size_t offs[2][16] = {};
+  size_t offs[2][15] = {};
 };
 
 const NaBlob& na_blob(int la, int lb, int lc, int bra_pure, int split) {
@@ -218,8 +217,7 @@ extern "C" lx3c_status lx3c_eri3c_noalloc(int la, int lb, int lc, int ka, int kb
   if (e != cudaSuccess) return na_fail(LX3C_ECUDA, cudaGetErrorString(e));
   DevBasis orb{nullptr, nullptr, orb_off, orb_xyz, orb_exps, orb_coefs};
   DevBasis aux{nullptr, nullptr, aux_off, aux_xyz, aux_exps, aux_coefs};
-  e = launch_pair_precompute(orb, pairs, npair, ka, kb, pairrec, pairab, st);
-  if (e == cudaSuccess) e = launch_aux_precompute(aux, auxs, naux, kc, auxrec, auxc, st);
+  e = launch_precompute(orb, pairs, npair, ka, kb, pairrec, pairab, aux, auxs, naux, kc, auxrec, auxc, st);
   if (e == cudaSuccess) {
     noalloc_orient<<<(unsigned)((npair + 127) / 128), 128, 0, st>>>(pairs, npair, la, lb, ka, kb, orb_off, orb_xyz,
                                                                      orb_exps, orb_coefs, orientation_amp_max(), sub, prim);

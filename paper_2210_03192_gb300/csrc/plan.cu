@@ -5,12 +5,17 @@
 //   [00|0]^(m)       Sec. 2.5.2 (Boys function times the prefactor)
 //   VRR1             Eq. vrr1: [a+1_i 0|0]^(m) = PA_i [a]^(m) - rho/gamma PC_i [a]^(m+1)
 //                              + a_i/(2 gamma) ([a-1_i]^(m) - rho/gamma [a-1_i]^(m+1))
-//   CVRR2 prerequisites  Eq. a0cv2: (e 0)_{k,n} = sum_prim Y^k X^n [e 0|0]^(lc),
+//   CVRR2 prerequisites and targets  n-q form of Eq. cVRR2 (the printed closed
+//                    form is garbled; the reading used is (a 0|c) = sum over
+//                    u <= min(a,c) of prod_i C(a_i,u_i) C(c_i,u_i) u_i!
+//                    (a-u 0)_{|u|, c-u}) with the ket transform of Sec. 2.5.1
+//                    taken first: since sum_c T_Cc c!/(c-u)! X^{c-u} = d^u S_C(X)
+//                    is a solid harmonic of degree lc-|u|,
+//                      (a 0|C) = sum_u C(a,u) sum_m D^u_{Cm} (a-u 0)_{|u|,m},
+//                      (e 0)_{k,m} = sum_prim Y^k s_{lc-k,m}(X) [e 0|0]^(lc),
+//                    with 2(lc-k)+1 prerequisites per (e, k) where the monomials
+//                    X^n of Eq. a0cv2 give (lc-k+1)(lc-k+2)/2;
 //                    Y = rho/(2 gamma zeta_c) = 1/(2(gamma+zeta_c)), X = rho/zeta_c PC
-//   CVRR2 targets    n-q form of Eq. cVRR2 (the printed closed form is garbled; the
-//                    reading used is sum over u <= min(a,c) of
-//                    prod_i C(a_i,u_i) C(c_i,u_i) u_i! (a-u 0)_{|u|, c-u})
-//   ket transform    Sec. 2.5.1 (Cartesian ket to solid harmonic)
 //   HRR              Eq. hrr: (a b+1_i|C) = (a+1_i b|C) + AB_i (a b|C)
 //   bra transform    optional (solid-harmonic bra)
 #include <vector_types.h>
@@ -102,6 +107,100 @@ unsigned pal_id(std::vector<double>& pal, std::map<double, int>& ids, double v) 
   pal.push_back(v);
   ids[v] = id;
   return id;
+}
+
+// Homogeneous polynomials of degree l as coefficients over cart(l).
+typedef std::vector<long double> Poly;
+
+Poly times_coord(const Poly& p, int l, int axis) {
+  Poly r(ncart(l + 1), 0.0L);
+  for (auto& c : cart(l)) {
+    C3 d = c;
+    d.v[axis]++;
+    r[cart_index(d.v[0], d.v[1], d.v[2])] += p[cart_index(c.v[0], c.v[1], c.v[2])];
+  }
+  return r;
+}
+
+Poly derivative(const Poly& p, int l, int axis) {
+  Poly r(ncart(l - 1), 0.0L);
+  for (auto& c : cart(l))
+    if (c.v[axis] > 0) {
+      C3 d = c;
+      d.v[axis]--;
+      r[cart_index(d.v[0], d.v[1], d.v[2])] += c.v[axis] * p[cart_index(c.v[0], c.v[1], c.v[2])];
+    }
+  return r;
+}
+
+// The kernel's harmonic basis of degree l, m = -l..l: Q_{l,|m|}(z, r^2) times
+// the real (m >= 0) or imaginary part of (x + i y)^|m|, with
+// Q_{m,m} = 1, Q_{l+1,m} = z Q_{l,m} - (l^2-m^2)/(4l^2-1) r^2 Q_{l-1,m}.
+const std::vector<Poly>& harmonic_basis(int l) {
+  static std::map<int, std::vector<Poly>> cache;  // under class_tables_variant's lock
+  auto it = cache.find(l);
+  if (it != cache.end()) return it->second;
+  std::vector<Poly> out(2 * l + 1);
+  auto add = [](const Poly& a, const Poly& b, long double f) {
+    Poly r = a;
+    for (size_t i = 0; i < r.size(); ++i) r[i] += f * b[i];
+    return r;
+  };
+  Poly A{1.0L}, B{0.0L};
+  for (int m = 0; m <= l; ++m) {
+    if (m > 0) {
+      const Poly An = add(times_coord(A, m - 1, 0), times_coord(B, m - 1, 1), -1.0L);
+      B = add(times_coord(A, m - 1, 1), times_coord(B, m - 1, 0), 1.0L);
+      A = An;
+    }
+    for (int im = 0; im < (m > 0 ? 2 : 1); ++im) {
+      Poly q0(1, 0.0L), q1 = im ? B : A;  // Q_{k-1}, Q_k times the angular factor, degrees k-1 and k
+      for (int k = m; k < l; ++k) {
+        Poly n = times_coord(q1, k, 2);
+        if (k > m) {
+          Poly r2 = times_coord(times_coord(q0, k - 1, 0), k, 0);
+          for (int x = 1; x < 3; ++x) r2 = add(r2, times_coord(times_coord(q0, k - 1, x), k, x), 1.0L);
+          n = add(n, r2, -(long double)(k * k - m * m) / (4.0L * k * k - 1.0L));
+        }
+        q0 = q1;
+        q1 = n;
+      }
+      out[im ? l - m : l + m] = q1;
+    }
+  }
+  return cache.emplace(l, out).first->second;
+}
+
+// D^u: rows C of the solid harmonics S_C of degree lc, d^u S_C = sum_m D[C][m]
+// s_{lc-|u|,m}.  Harmonic polynomials of one degree and different m are
+// orthogonal under <x^a, x^b> = a! delta_ab (rotations preserve it).
+std::vector<double> harmonic_derivative(int lc, const C3& u) {
+  const int k = u.l(), l = lc - k;
+  const auto T = solid_matrix(lc);
+  const auto& s = harmonic_basis(l);
+  auto fac3 = [](const C3& c) { return (long double)(fact(c.v[0]) * fact(c.v[1]) * fact(c.v[2])); };
+  std::vector<double> D((2 * lc + 1) * (2 * l + 1), 0.0);
+  for (int C = 0; C < 2 * lc + 1; ++C) {
+    Poly p(T.begin() + C * ncart(lc), T.begin() + (C + 1) * ncart(lc));
+    int deg = lc;
+    for (int x = 0; x < 3; ++x)
+      for (int i = 0; i < u.v[x]; ++i) p = derivative(p, deg--, x);
+    long double big = 0.0L;
+    std::vector<long double> d(2 * l + 1);
+    for (int m = 0; m < 2 * l + 1; ++m) {
+      long double num = 0.0L, den = 0.0L;
+      for (auto& c : cart(l)) {
+        const int i = cart_index(c.v[0], c.v[1], c.v[2]);
+        num += fac3(c) * p[i] * s[m][i];
+        den += fac3(c) * s[m][i] * s[m][i];
+      }
+      d[m] = num / den;
+      big = std::max(big, std::fabs(d[m]));
+    }
+    for (int m = 0; m < 2 * l + 1; ++m)
+      D[C * (2 * l + 1) + m] = std::fabs(d[m]) > 1e-12L * big ? (double)d[m] : 0.0;
+  }
+  return D;
 }
 
 ClassTables build(int la, int lb, int lc, int bra_pure, int hrr2) {
@@ -282,112 +381,62 @@ ClassTables build(int la, int lb, int lc, int bra_pure, int hrr2) {
   }
   ct.vlev_start[Lab] = (int)ct.vtab.size();
 
-  // ---------------- weights W_{k,n} = Y^k X^n (Eq. a0cv2) ----------------
-  // F buffer: 0..2 (rho/gamma) PC, 3 rho/gamma, 4 + i*lc + (j-1) X_i^j, 4 + 3lc + (k-1) Y^k
-  ct.NF = 4 + 4 * lc;
-  std::vector<int> woff(lc + 2, 0);
-  for (int k = 0; k <= lc; ++k) woff[k + 1] = woff[k] + ncart(lc - k);
-  ct.NW = woff[lc + 1];
-  {
-    std::vector<std::pair<int, int4>> items;
-    for (int k = 0; k <= lc; ++k)
-      for (auto& n : cart(lc - k)) {
-        int w = woff[k] + cart_index(n.v[0], n.v[1], n.v[2]);
-        std::vector<int> src;
-        if (k > 0) src.push_back(4 + 3 * lc + (k - 1));
-        for (int i = 0; i < 3; ++i)
-          if (n.v[i] > 0) src.push_back(4 + i * lc + (n.v[i] - 1));
-        while (src.size() < 4) src.push_back(0xFFFF);
-        int cnt = 0;
-        for (int s : src) cnt += s != 0xFFFF;
-        int4 it{w | (src[0] << 16), src[1] | (src[2] << 16), src[3] | (cnt << 16), 0};
-        items.push_back({cnt, it});
-      }
-    std::stable_sort(items.begin(), items.end(), [](auto& x, auto& y) { return x.first < y.first; });
-    for (auto& it : items) ct.wtab.push_back(it.second);
-  }
+  // ---------------- weights W_{k,m} = Y^k s_{lc-k,m}(X) ----------------
+  // F buffer: 0..2 (rho/gamma) PC, 3 rho/gamma, 4..6 X, 7 + (k-1) Y^k
+  const int kmax = std::min(Lab, lc);
+  ct.kmax = kmax;
+  ct.NF = 4 + (lc > 0 ? 3 + kmax : 0);
+  ct.NW = (kmax + 1) * (2 * lc + 1 - kmax);
+  auto woff = [&](int k) { return k * (2 * lc + 2 - k); };
 
   // ---------------- CVRR2 targets and prerequisites (Sec. 2.5.4) ----------------
-  std::map<std::tuple<C3, int, C3>, int> accmap;
-  std::vector<std::tuple<C3, int, C3>> acckeys;
-  auto cl = cart(lc);
-  struct Tgt { int id; std::vector<unsigned> terms; };
-  std::vector<Tgt> tg;
-  std::vector<std::vector<std::pair<std::tuple<C3, int, C3>, double>>> rawterms;
-  for (int r = 0; r < ct.nkrow; ++r) {
-    const C3& a = erows[r];
-    for (size_t ic = 0; ic < cl.size(); ++ic) {
-      const C3& c = cl[ic];
-      std::vector<std::pair<std::tuple<C3, int, C3>, double>> terms;
-      for (int ux = 0; ux <= std::min(a.v[0], c.v[0]); ++ux)
-        for (int uy = 0; uy <= std::min(a.v[1], c.v[1]); ++uy)
-          for (int uz = 0; uz <= std::min(a.v[2], c.v[2]); ++uz) {
-            int u[3] = {ux, uy, uz};
-            double coef = 1.0;
-            C3 e, n;
-            for (int i = 0; i < 3; ++i) {
-              coef *= binom(a.v[i], u[i]) * binom(c.v[i], u[i]) * fact(u[i]);
-              e.v[i] = a.v[i] - u[i];
-              n.v[i] = c.v[i] - u[i];
-            }
-            terms.push_back({std::make_tuple(e, ux + uy + uz, n), coef});
-          }
-      rawterms.push_back(terms);
-      for (auto& t : terms)
-        if (!accmap.count(t.first)) { accmap[t.first] = 0; }
-    }
-  }
-  // accumulator order: by |e|, e, k, n
+  // prerequisites by (e, k), then m = -(lc-k)..lc-k, in the order |e|, e, k
+  std::map<std::pair<C3, int>, int> accmap;
+  for (int r = 0; r < ct.nkrow; ++r)
+    for (int ux = 0; ux <= erows[r].v[0]; ++ux)
+      for (int uy = 0; uy <= erows[r].v[1]; ++uy)
+        for (int uz = 0; uz <= erows[r].v[2] && ux + uy + uz <= lc; ++uz) {
+          const C3 e{{erows[r].v[0] - ux, erows[r].v[1] - uy, erows[r].v[2] - uz}};
+          accmap[{e, ux + uy + uz}] = 0;
+        }
+  std::vector<std::pair<C3, int>> acckeys;
   for (auto& kv : accmap) acckeys.push_back(kv.first);
   std::sort(acckeys.begin(), acckeys.end(), [](auto& x, auto& y) {
-    const C3 &ex = std::get<0>(x), &ey = std::get<0>(y);
-    if (ex.l() != ey.l()) return ex.l() < ey.l();
-    int ix = cart_index(ex.v[0], ex.v[1], ex.v[2]), iy = cart_index(ey.v[0], ey.v[1], ey.v[2]);
-    if (ix != iy) return ix < iy;
-    if (std::get<1>(x) != std::get<1>(y)) return std::get<1>(x) < std::get<1>(y);
-    const C3 &nx = std::get<2>(x), &ny = std::get<2>(y);
-    return cart_index(nx.v[0], nx.v[1], nx.v[2]) < cart_index(ny.v[0], ny.v[1], ny.v[2]);
+    if (x.first.l() != y.first.l()) return x.first.l() < y.first.l();
+    const int ix = cart_index(x.first.v[0], x.first.v[1], x.first.v[2]),
+              iy = cart_index(y.first.v[0], y.first.v[1], y.first.v[2]);
+    return ix != iy ? ix < iy : x.second < y.second;
   });
-  for (size_t i = 0; i < acckeys.size(); ++i) accmap[acckeys[i]] = (int)i;
-  ct.NACC = (int)acckeys.size();
+  ct.NACC = 0;
   for (auto& key : acckeys) {
-    const C3& e = std::get<0>(key);
-    int k = std::get<1>(key);
-    const C3& n = std::get<2>(key);
-    unsigned v = vidx(e.l(), lc, e);
-    unsigned w = woff[k] + cart_index(n.v[0], n.v[1], n.v[2]);
-    ct.atab.push_back(v | (w << 16));
-    ct.acc_key.push_back(int4{cart_index(e.v[0], e.v[1], e.v[2]) | (e.l() << 16), k,
-                              cart_index(n.v[0], n.v[1], n.v[2]) | ((lc - k) << 16), 0});
+    accmap[key] = ct.NACC;
+    const unsigned v = vidx(key.first.l(), lc, key.first);
+    for (int m = 0; m < 2 * (lc - key.second) + 1; ++m) ct.atab.push_back(v | ((unsigned)(woff(key.second) + m) << 16));
+    ct.NACC += 2 * (lc - key.second) + 1;
   }
-  {
-    // keep only the weights some accumulator reads (for la + lb < lc the
-    // targets reach k <= la + lb only) and renumber them densely
-    std::vector<int> remap(ct.NW, -1);
-    for (unsigned a : ct.atab) remap[a >> 16] = 0;
-    std::vector<int4> kept;
-    for (const int4& it : ct.wtab) {
-      const int dst = it.x & 0xFFFF;
-      if (remap[dst] < 0) continue;
-      remap[dst] = (int)kept.size();
-      int4 k2 = it;
-      k2.x = (it.x & ~0xFFFF) | remap[dst];
-      kept.push_back(k2);
-    }
-    for (unsigned& a : ct.atab) a = (a & 0xFFFF) | ((unsigned)remap[a >> 16] << 16);
-    ct.wtab = kept;
-    ct.NW = (int)kept.size();
-  }
-  // gather CSR by target id = row*ncc + c, items sorted by descending term count
-  int ngt = ct.nkrow * ct.ncc;
+  // gather CSR by target id = row*nC + C, items sorted by descending term count
+  int ngt = ct.nkrow * ct.nC;
   ct.gptr.assign(ngt + 1, 0);
-  for (int id = 0; id < ngt; ++id) {
-    for (auto& t : rawterms[id]) {
-      unsigned pid = (unsigned)accmap[t.first];
-      unsigned cid = pal_id(ct.pal, palids, t.second);
-      ct.gterm.push_back(pid | (cid << 20));
+  std::map<C3, std::vector<double>> dmap;
+  for (int r = 0; r < ct.nkrow; ++r) {
+    const C3& a = erows[r];
+    for (int C = 0; C < ct.nC; ++C) {
+      for (int ux = 0; ux <= a.v[0]; ++ux)
+        for (int uy = 0; uy <= a.v[1]; ++uy)
+          for (int uz = 0; uz <= a.v[2] && ux + uy + uz <= lc; ++uz) {
+            const C3 u{{ux, uy, uz}};
+            auto it = dmap.find(u);
+            if (it == dmap.end()) it = dmap.emplace(u, harmonic_derivative(lc, u)).first;
+            const int k = u.l(), nm = 2 * (lc - k) + 1;
+            const double bin = binom(a.v[0], ux) * binom(a.v[1], uy) * binom(a.v[2], uz);
+            const int p0 = accmap.at({C3{{a.v[0] - ux, a.v[1] - uy, a.v[2] - uz}}, k});
+            for (int m = 0; m < nm; ++m) {
+              const double d = it->second[C * nm + m];
+              if (d != 0.0) ct.gterm.push_back((unsigned)(p0 + m) | (pal_id(ct.pal, palids, bin * d) << kGatherBits));
+            }
+          }
+      ct.gptr[r * ct.nC + C + 1] = (int)ct.gterm.size();
     }
-    ct.gptr[id + 1] = (int)ct.gterm.size();
   }
   ct.gdst.resize(ngt);
   for (int i = 0; i < ngt; ++i) ct.gdst[i] = i;
@@ -396,7 +445,7 @@ ClassTables build(int la, int lb, int lc, int bra_pure, int hrr2) {
   });
   {
     // sliced ELL copy: padding terms read accumulator 0 with coefficient 0
-    const unsigned pad = 0u | (pal_id(ct.pal, palids, 0.0) << 20);
+    const unsigned pad = 0u | (pal_id(ct.pal, palids, 0.0) << kGatherBits);
     for (int s0 = 0; s0 < ngt; s0 += 32) {
       int mx = 0;
       for (int l = s0; l < std::min(ngt, s0 + 32); ++l) mx = std::max(mx, ct.gptr[ct.gdst[l] + 1] - ct.gptr[ct.gdst[l]]);
@@ -448,26 +497,28 @@ ClassTables build(int la, int lb, int lc, int bra_pure, int hrr2) {
     }
     ct.nbB = ct.nA * (2 * lb + 1);
   }
-  if (ct.pal.size() >= 4096) throw std::runtime_error("coefficient palette overflow");
-  if (ct.NACC >= (1 << 20) || ct.NV >= 65536 || ct.NW >= 65536) throw std::runtime_error("class too large");
+  if (ct.pal.size() >= (1u << (32 - kGatherBits))) throw std::runtime_error("coefficient palette overflow");
+  if (ct.NACC >= (1 << kGatherBits) || ct.NV >= 65536 || ct.NW >= 65536) throw std::runtime_error("class too large");
 
   // ---------------- algorithmic flop counts (FMA = 2) ----------------
   double fp = 0;
-  // geometry, rsqrt, prefactor, factor powers ((rho/gamma) PC only when VRR1 runs)
-  fp += 32 + (lc > 0 ? 4.0 * (lc - 1) : 0.0) - (Lab == 0 ? 3.0 : 0.0);
+  // geometry, rsqrt, prefactor, X and powers of Y ((rho/gamma) PC only when
+  // VRR1 runs)
+  fp += 32 + std::max(0, kmax - 1) - (Lab == 0 ? 3.0 : 0.0);
   // Boys and [00|0]^(m): one degree-7 polynomial for F_L; the exp(-T)
   // polynomial and the downward relation only when Lab > 0 (F_L..F_lc)
   fp += Lab == 0 ? 16.0 : 32.0 + 3.0 * Lab;
   for (int e = 1; e <= Lab; ++e)
     for (int i = ct.vlev_start[e - 1]; i < ct.vlev_start[e]; ++i) fp += ((ct.vtab[i].z >> 20) & 0xF) ? 7 : 3;
-  for (auto& w : ct.wtab) {
-    int cnt = (w.z >> 16) & 0xFFFF;
-    fp += cnt > 1 ? cnt - 1 : 0;
+  // weights, m by m: (x + i y)^m, the Q recursion, their products
+  if (lc > 0) fp += 5;
+  for (int m = 0; m <= lc; ++m) {
+    fp += 6.0 * std::max(0, m - 1) + 4.0 * std::max(0, lc - m - 1);
+    for (int k = 0; k <= kmax && k <= lc - m; ++k) fp += (k > 0) + (m > 0 ? 2 : 0);
   }
   fp += 2.0 * ct.NACC;
   ct.flops_prim = fp;
   double fc = 2.0 * ct.gterm.size();
-  fc += 2.0 * ct.kent.size() * ct.nkrow;
   for (const uint4& h : ct.htab) fc += 2.0 * ((h.x >> 16) - 1) * ct.nC;
   auto bra = [&](const std::vector<int>& ptr, const std::vector<int2>& ent, int nother) {
     double f = 0;
@@ -525,7 +576,7 @@ std::string check_class_tables(const ClassTables& ct) {
     return std::string(buf);
   };
   const int Lab = ct.la + ct.lb;
-  const unsigned NV = (unsigned)ct.NV, NW = (unsigned)ct.NW, NF = (unsigned)ct.NF, NACC = (unsigned)ct.NACC;
+  const unsigned NV = (unsigned)ct.NV, NW = (unsigned)ct.NW, NACC = (unsigned)ct.NACC;
   if ((int)ct.vlev_start.size() != Lab + 1) return "VRR1 level table size";
   // VRR1: indices in range; every entry above level 0 written once; level e
   // reads only entries written before it (levels are contiguous and ordered)
@@ -544,20 +595,12 @@ std::string check_class_tables(const ClassTables& ct) {
   }
   for (unsigned v = 0; v < NV; ++v)
     if (written[v] != (v <= (unsigned)Lab ? 0 : 1)) return bad("VRR1 entry not formed exactly once", v);
-  // weights and accumulators
-  for (size_t i = 0; i < ct.wtab.size(); ++i) {
-    const int4 w = ct.wtab[i];
-    const unsigned cnt = (unsigned)w.z >> 16;
-    const unsigned src[4] = {(unsigned)w.x >> 16, (unsigned)w.y & 0xFFFF, (unsigned)w.y >> 16, (unsigned)w.z & 0xFFFF};
-    if (((unsigned)w.x & 0xFFFF) >= NW || cnt > 4) return bad("weight item", (long long)i);
-    for (unsigned k = 0; k < cnt; ++k)
-      if (src[k] >= NF) return bad("weight factor index", (long long)i);
-  }
+  // accumulators
   if (ct.atab.size() != NACC) return "accumulator table size";
   for (size_t i = 0; i < ct.atab.size(); ++i)
     if ((ct.atab[i] & 0xFFFF) >= NV || (ct.atab[i] >> 16) >= NW) return bad("accumulator index", (long long)i);
   // gather: CSR and its sliced-ELL copy hold the same terms
-  const int ngt = ct.nkrow * ct.ncc;
+  const int ngt = ct.nkrow * ct.nC;
   if ((int)ct.gptr.size() != ngt + 1 || (int)ct.gdst.size() != ngt) return "gather table size";
   std::vector<int> seen(ngt, 0);
   for (int r = 0; r < ngt; ++r) {
@@ -568,7 +611,7 @@ std::string check_class_tables(const ClassTables& ct) {
   for (int id = 0; id < ngt; ++id)
     if (ct.gptr[id + 1] < ct.gptr[id]) return bad("gather row pointers", id);
   for (size_t q = 0; q < ct.gterm.size(); ++q)
-    if ((ct.gterm[q] & 0xFFFFF) >= NACC || (ct.gterm[q] >> 20) >= ct.pal.size()) return bad("gather term", (long long)q);
+    if ((ct.gterm[q] & kGatherMask) >= NACC || (ct.gterm[q] >> kGatherBits) >= ct.pal.size()) return bad("gather term", (long long)q);
   if ((int)ct.gslice.size() != (ngt + 31) / 32) return "sliced ELL slice count";
   for (int sl = 0; sl < (int)ct.gslice.size(); ++sl)
     for (int l = 0; l < 32; ++l) {
@@ -581,7 +624,7 @@ std::string check_class_tables(const ClassTables& ct) {
         if (q >= ct.gell.size()) return bad("sliced ELL entry out of range", r);
         const unsigned e = ct.gell[q];
         if (j < cnt ? e != ct.gterm[ct.gptr[id] + j]
-                    : ((e >> 20) >= ct.pal.size() || ct.pal[e >> 20] != 0.0 || (e & 0xFFFFF) >= NACC))
+                    : ((e >> kGatherBits) >= ct.pal.size() || ct.pal[e >> kGatherBits] != 0.0 || (e & kGatherMask) >= NACC))
           return bad("sliced ELL differs from the CSR terms", r);
       }
     }
@@ -670,22 +713,21 @@ void buffer_sizes(const ClassTables& ct, int Kab, int Kc, int T, int G, int mode
   if (mode == 0 && T > 1 && (T % 2 == 0)) Tp = T + 1;
   auto per_t = [&](int n) -> long long { return mode == 0 ? (long long)n * Tp : (long long)T * n; };
   auto per_tg = [&](int n) -> long long { return mode == 0 ? (long long)n * G * Tp : (long long)T * G * n; };
-  long long nK = (long long)ct.nkrow * ct.nC, nG = (long long)ct.nkrow * ct.ncc;
-  int lb = ct.lb;
+  const long long nK = (long long)ct.nkrow * ct.nC;
   s.pair = (long long)Kab * kPairRec + 16;  // + the tile's AB products
   s.aux = (long long)T * (3 + kAuxRec * Kc);
   s.loop = per_tg(ct.NV) + per_tg(ct.NW) + per_tg(ct.NF);
   s.P = per_t(ct.NACC);
-  // region assignment: Y holds P, level 0 (ket out) and even HRR levels;
-  // X holds the loop buffers, the gather output and odd HRR levels.
-  long long Y = std::max(s.P, per_t((int)nK));
-  long long X = std::max(s.loop, per_t((int)nG));
+  // region assignment: Y holds P and odd HRR levels; X holds the loop
+  // buffers, the gather output (level 0) and even HRR levels.
+  long long Y = s.P;
+  long long X = std::max(s.loop, per_t((int)nK));
   const int R = ct.nhrr;
   for (int j = 1; j <= R; ++j) {
     long long sz = per_t(ct.hrows[j] * ct.nC);
-    if (j & 1) X = std::max(X, sz); else Y = std::max(Y, sz);
+    if (j & 1) Y = std::max(Y, sz); else X = std::max(X, sz);
   }
-  int cur = (R & 1) ? 1 : 0;  // 0 = Y, 1 = X
+  int cur = (R & 1) ? 0 : 1;  // 0 = Y, 1 = X
   int baR = -1, bbR = -1;
   if (ct.nbA) { cur ^= 1; baR = cur; long long sz = per_t(ct.nbA * ct.nC); if (cur) X = std::max(X, sz); else Y = std::max(Y, sz); }
   if (ct.nbB) { cur ^= 1; bbR = cur; long long sz = per_t(ct.nbB * ct.nC); if (cur) X = std::max(X, sz); else Y = std::max(Y, sz); }
@@ -716,9 +758,8 @@ void buffer_sizes(const ClassTables& ct, int Kab, int Kc, int T, int G, int mode
   d->W = mk_tg(xbase + (int)per_tg(ct.NV), ct.NW);
   d->F = mk_tg(xbase + (int)(per_tg(ct.NV) + per_tg(ct.NW)), ct.NF);
   d->P = mk_t(ybase, ct.NACC);
-  d->Gb = mk_t(xbase, (int)nG);
-  d->H[0] = mk_t(ybase, (int)nK);
-  for (int j = 1; j <= R; ++j) d->H[j] = mk_t((j & 1) ? xbase : ybase, ct.hrows[j] * ct.nC);
+  d->H[0] = mk_t(xbase, (int)nK);
+  for (int j = 1; j <= R; ++j) d->H[j] = mk_t((j & 1) ? ybase : xbase, ct.hrows[j] * ct.nC);
   Buf last = d->H[R];
   if (ct.nbA) { d->BA = mk_t(baR ? xbase : ybase, ct.nbA * ct.nC); last = d->BA; }
   if (ct.nbB) { d->BB = mk_t(bbR ? xbase : ybase, ct.nbB * ct.nC); last = d->BB; }
