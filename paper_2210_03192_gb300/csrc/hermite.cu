@@ -18,13 +18,14 @@
 // GB300 layout.  FP64 issues one warp instruction per 16 SM clocks, so an FMA
 // may spend 16 clocks of shared-memory bandwidth and 64 issue slots on its
 // operands: every stage runs from per-lane shared-memory columns driven by
-// small index tables, with all 32 lanes on one table entry.  One warp is one
-// block and owns a tile (W kets x a range of primitive pairs, 32/W pairs at a
-// time); a lane reads and writes only its own columns, so there is no barrier
-// and no idle lane beyond the ragged end of a ket list.  Tables list the
-// terms of four outputs side by side: four independent FMA chains per warp
-// hide the latency at the two to four warps per SM that the largest classes'
-// columns leave room for.
+// small index tables, with all 32 lanes on one table entry.  A block owns a
+// tile (W kets x a range of primitive pairs, 32/W pairs at a time); a lane
+// reads and writes only its own columns, so a one-warp block needs no barrier
+// and no lane idles beyond the ragged end of a ket list.  An SM sub-partition
+// issues one FP64 warp instruction per 64 clocks, so it takes eight or more
+// warps to keep the four busy: where the columns of a class let fewer one-warp
+// blocks onto an SM, two or four warps share the columns and divide every
+// stage's outputs, with a barrier between stages.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -63,14 +64,18 @@ __host__ __device__ inline int hidx(int x, int y, int z) {
 // b closes its output, whose header word (destination byte offset | palette id
 // of its scale factor << 20; for y rows Hermite index | axes << 16) is the next
 // of h.  The queues' ragged ends multiply the zero column.
+// Each warp of the block has queues of its own: nb + 1 batches and hs headers
+// on from the one before.
 struct Stage {
   const uint4* a;
   const uint4* b;
   const unsigned* h;
-  long long nb;  // even
+  int nb;  // even
+  int hs;
 };
 
 struct HermCls {
+  int nw;  // warps per block
   int Lab, lc, Kc, L, nR, nY, ncc, nC, W, nket;
   int cX, cPW, cU, cB, cCP, cGA;  // column offsets (R at column 0)
   int cZero, cH;          // the zero column; the primitive pairs' densities
@@ -120,11 +125,12 @@ __device__ __forceinline__ void sts(char* base, unsigned off, double v) { *(doub
 // a warp alone reached 12 % of the FP64 pipe.  Queues closed one by one waste
 // no FMA on rows of unequal length (four rows in step wasted 10 to 40 %).
 template <class Flush>
-__device__ __forceinline__ void run_stage(const Stage& st, const char* A, const char* col, const Flush& flush) {
-  const uint4* pa = st.a;
-  const uint4* pb = st.b;
-  const unsigned* ph = st.h;
-  const int nb = (int)st.nb;
+__device__ __forceinline__ void run_stage(const Stage& st, int warp, const char* A, const char* col,
+                                          const Flush& flush) {
+  const int nb = st.nb;
+  const uint4* pa = st.a + warp * (nb + 1);
+  const uint4* pb = st.b + warp * (nb + 1);
+  const unsigned* ph = st.h + warp * st.hs;
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
   unsigned hd = __ldg(ph);
 #define HERM_LOAD(X, wa, wb)                                                                  \
@@ -179,12 +185,19 @@ struct StoreCols {
   }
 };
 
-// kMode: bit 0 gamma, bit 1 J, 4 gradient.
-template <int kMode>
-__global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ HermArgs g) {
+// y rows staged per warp before their kets are summed
+__host__ __device__ constexpr int stage_rows(int nw) { return nw == 1 ? 32 : 16; }
+
+// kMode: bit 0 gamma, bit 1 J, 4 gradient; kNW warps per block.
+template <int kMode, int kNW>
+__global__ void __launch_bounds__(32 * kNW, 16 / kNW) herm_kernel(const __grid_constant__ HermArgs g) {
   extern __shared__ double sm[];
+  constexpr int kRows = stage_rows(kNW);
   constexpr bool kG = (kMode & 1) != 0, kY = (kMode & 6) != 0, kF = (kMode & 4) != 0;
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = kNW > 1 ? threadIdx.x >> 5 : 0;
+  const auto sync = [] {
+    if (kNW > 1) __syncthreads();
+  };
   double* col = sm + lane;
   char* cb = (char*)col;
   const int4 tile = __ldg(g.tiles + blockIdx.x);
@@ -205,7 +218,7 @@ __global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ He
   PW[2 * (lc + 1) * 32] = 1.0;
   if (kY) {
     // the ket's q in Cartesian monomials, times their factorials
-    for (int n = 0; n < c.ncc; ++n) {
+    for (int n = warp; n < c.ncc; n += kNW) {
       double v = 0.0;
       for (int k = __ldg(c.cptr + n); k < __ldg(c.cptr + n + 1); ++k) {
         const int2 e = __ldg(c.cent + k);
@@ -215,7 +228,7 @@ __global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ He
     }
   }
   if (kG)
-    for (int n = 0; n < c.ncc; ++n) col[(c.cGA + n) * 32] = 0.0;
+    for (int n = warp; n < c.ncc; n += kNW) col[(c.cGA + n) * 32] = 0.0;
   for (int e0 = 0; e0 < tile.w; e0 += NP) {
     const int ie = e0 + sub;
     const int prim = tile.z + min(ie, tile.w - 1);
@@ -224,19 +237,21 @@ __global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ He
     const double gam = __ldg(pr);
     const double Rx = __ldg(pr + 1) - Cx, Ry = __ldg(pr + 2) - Cy, Rz = __ldg(pr + 3) - Cz;
     const double R2 = fma(Rz, Rz, fma(Ry, Ry, Rx * Rx));
+    if (kNW > 1) __syncthreads(); else __syncwarp();
     if (kG) {
       // the densities of the NP primitive pairs, side by side
-      __syncwarp();
       for (int s = 0; s < NP; ++s) {
         const double* H = c.H + (long long)(tile.z + min(e0 + s, tile.w - 1)) * c.nR;
-        for (int t = lane; t < c.nR; t += 32) sm[c.cH * 32 + s * c.nR + t] = __ldg(H + t);
+        for (int t = threadIdx.x; t < c.nR; t += 32 * kNW) sm[c.cH * 32 + s * c.nR + t] = __ldg(H + t);
       }
-      __syncwarp();
+      if (kNW == 1) __syncwarp();
     }
-    XC[0] = Rx;
-    XC[32] = Ry;
-    XC[64] = Rz;
-    if (lc > 0) {
+    if (warp == 0) {
+      XC[0] = Rx;
+      XC[32] = Ry;
+      XC[64] = Rz;
+    }
+    if (warp == 0 && lc > 0) {
       // R_i^j / j!
       double px = Rx, py = Ry, pz = Rz;
       double* P1 = PW + (lc + 1) * 32;
@@ -249,77 +264,90 @@ __global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ He
       }
     }
     for (int ic = 0; ic < c.Kc; ++ic) {
-      const double zc = __ldg(c.auxrec + ((long long)qc * c.Kc + ic) * kAuxRec);
-      const double ccp = __ldg(c.auxrec + ((long long)qc * c.Kc + ic) * kAuxRec + 1);
-      const double rs = rsqrt_fp64(gam + zc);
-      const double r = rs * rs;
-      const double gr = gam * r;
-      const double rho = gr * zc;
-      const double Tb = rho * R2, n2r = -2.0 * rho;
-      double pref = ccp * rs;
-      {
-        double b = gr;
-        for (int e = lc; e; e >>= 1) {
-          if (e & 1) pref *= b;
-          if (e > 1) b *= b;
-        }
-      }
-      if (!act) pref = 0.0;
-      double FL, ex;
-      boys_top(g.boys_tab, g.boys_mid, c.boys_cL, c.L, Lab > 0, Tb, FL, ex);
-      double fm = pref * FL;
-      if (Lab > 0) {
-        double b = n2r;
-        for (int e = Lab; e; e >>= 1) {
-          if (e & 1) fm *= b;
-          if (e > 1) b *= b;
-        }
-        double pe = pref * ex;
-        B[0] = pe;
-        for (int m = 1; m < Lab; ++m) {
-          pe *= n2r;
-          B[m * 32] = pe;
-        }
-      }
-      // R_e^(m), |e| <= Lab - m, in place from R^(m+1): degrees descend, so an
-      // entry is overwritten only after its last reader.  Operation words:
-      // destination, sources, then axis column | factor << 20 | scale << 24
-      col[0] = fm;
-      for (int m = Lab - 1; m >= 0; --m) {
-        const int b1 = c.rbeg[m + 1];
-        for (int b = c.rbeg[m]; b < b1; b += 4) {
-          double u[4];
-          unsigned dst[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint4 w = __ldg(c.rops + b + k);
-            const int kk = (int)((w.w >> 20) & 0xF), id = (int)(w.w >> 24);
-            double v = lds(cb, w.z);
-            if (kk > 1) v *= c_int[kk];
-            u[k] = kk ? fma(lds(cb, w.w & 0xFFFFFu), lds(cb, w.y), v) : lds(cb, w.w & 0xFFFFFu) * lds(cb, w.y);
-            if (id) u[k] *= __ldg(c.pal + id);  // 1/e! on the last level
-            dst[k] = w.x;
+      // geometry, Boys function and R recursion: the first warp (the others
+      // wait, and the SM's other blocks run)
+      if (ic > 0) sync();
+      if (warp == 0) {
+        const double zc = __ldg(c.auxrec + ((long long)qc * c.Kc + ic) * kAuxRec);
+        const double ccp = __ldg(c.auxrec + ((long long)qc * c.Kc + ic) * kAuxRec + 1);
+        const double rs = rsqrt_fp64(gam + zc);
+        const double r = rs * rs;
+        const double gr = gam * r;
+        const double rho = gr * zc;
+        const double Tb = rho * R2, n2r = -2.0 * rho;
+        double pref = ccp * rs;
+        {
+          double b = gr;
+          for (int e = lc; e; e >>= 1) {
+            if (e & 1) pref *= b;
+            if (e > 1) b *= b;
           }
-#pragma unroll
-          for (int k = 0; k < 4; ++k) sts(cb, dst[k], u[k]);
         }
-        fm = fma(-R2, fm, B[m * 32]) * c_inv[2 * (lc + m) + 1];
+        if (!act) pref = 0.0;
+        double FL, ex;
+        boys_top(g.boys_tab, g.boys_mid, c.boys_cL, c.L, Lab > 0, Tb, FL, ex);
+        double fm = pref * FL;
+        if (Lab > 0) {
+          double b = n2r;
+          for (int e = Lab; e; e >>= 1) {
+            if (e & 1) fm *= b;
+            if (e > 1) b *= b;
+          }
+          double pe = pref * ex;
+          B[0] = pe;
+          for (int m = 1; m < Lab; ++m) {
+            pe *= n2r;
+            B[m * 32] = pe;
+          }
+        }
+        // R_e^(m), |e| <= Lab - m, in place from R^(m+1): degrees descend, so an
+        // entry is overwritten only after its last reader.  Operation words:
+        // destination, sources, then axis column | factor << 20 | scale << 24
         col[0] = fm;
+        for (int m = Lab - 1; m >= 0; --m) {
+          const int b1 = c.rbeg[m + 1];
+          for (int b = c.rbeg[m]; b < b1; b += 4) {
+            double u[4];
+            unsigned dst[4];
+  #pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint4 w = __ldg(c.rops + b + k);
+              const int kk = (int)((w.w >> 20) & 0xF), id = (int)(w.w >> 24);
+              double v = lds(cb, w.z);
+              if (kk > 1) v *= c_int[kk];
+              u[k] = kk ? fma(lds(cb, w.w & 0xFFFFFu), lds(cb, w.y), v) : lds(cb, w.w & 0xFFFFFu) * lds(cb, w.y);
+              if (id) u[k] *= __ldg(c.pal + id);  // 1/e! on the last level
+              dst[k] = w.x;
+            }
+  #pragma unroll
+            for (int k = 0; k < 4; ++k) sts(cb, dst[k], u[k]);
+          }
+          fm = fma(-R2, fm, B[m * 32]) * c_inv[2 * (lc + m) + 1];
+          col[0] = fm;
+        }
       }
+      sync();
       if (kG) {
-        run_stage(c.Z, (const char*)(sm + c.cH * 32 + sub * c.nR), cb, StoreCols<true, false>{cb, c.pal});
-        run_stage(c.gz, cb, cb, StoreCols<false, false>{cb, c.pal});
-        run_stage(c.gy, cb, cb, StoreCols<false, false>{cb, c.pal});
-        run_stage(c.gx, cb, cb, StoreCols<false, true>{cb, c.pal});
+        run_stage(c.Z, warp, (const char*)(sm + c.cH * 32 + sub * c.nR), cb, StoreCols<true, false>{cb, c.pal});
+        sync();
+        run_stage(c.gz, warp, cb, cb, StoreCols<false, false>{cb, c.pal});
+        sync();
+        run_stage(c.gy, warp, cb, cb, StoreCols<false, false>{cb, c.pal});
+        sync();
+        run_stage(c.gx, warp, cb, cb, StoreCols<false, true>{cb, c.pal});
+        sync();
       }
       if (kY) {
-        run_stage(c.jx, cb, cb, StoreCols<false, false>{cb, c.pal});
-        run_stage(c.jy, cb, cb, StoreCols<false, false>{cb, c.pal});
-        run_stage(c.jw, cb, cb, StoreCols<true, false>{cb, c.pal});
+        run_stage(c.jx, warp, cb, cb, StoreCols<false, false>{cb, c.pal});
+        sync();
+        run_stage(c.jy, warp, cb, cb, StoreCols<false, false>{cb, c.pal});
+        sync();
+        run_stage(c.jw, warp, cb, cb, StoreCols<true, false>{cb, c.pal});
+        sync();
         // y_a rows of 32 lanes staged in the B columns (row stride 33); then
         // 32 / rows lanes per row, a power of two, sum the kets of each
         // primitive pair
-        double* stg = sm + c.cB * 32;
+        double* stg = sm + c.cB * 32 + warp * kRows * 33;
         const double* Hf = kF ? c.H + 3LL * prim * c.nY : nullptr;
         int row = 0, amine = 0;
         const auto drain = [&]() {
@@ -354,7 +382,7 @@ __global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ He
           __syncwarp();
           row = 0;
         };
-        run_stage(c.Y, cb, cb, [&](unsigned h, double v) {
+        run_stage(c.Y, warp, cb, cb, [&](unsigned h, double v) {
           stg[row * 33 + lane] = v;
           if (lane == row) amine = (int)(h & 0xFFFF);
           if (kF) {
@@ -363,14 +391,15 @@ __global__ void __launch_bounds__(32, 16) herm_kernel(const __grid_constant__ He
             if (h & 0x20000u) f1 = fma(__ldg(hf + c.nY), v, f1);
             if (h & 0x40000u) f2 = fma(__ldg(hf + 2 * c.nY), v, f2);
           }
-          if (++row == 32) drain();
+          if (++row == kRows) drain();
         });
         if (row) drain();
       }
     }
   }
-  if (kG && q < c.nket) {
-    for (int C = 0; C < c.nC; ++C) {
+  if (kG) {
+    sync();
+    for (int C = warp; C < c.nC && q < c.nket; C += kNW) {
       double v = 0.0;
       for (int k = __ldg(c.gptr + C); k < __ldg(c.gptr + C + 1); ++k) {
         const int2 e = __ldg(c.gent + k);
@@ -758,7 +787,7 @@ struct Row {
 struct HostStage {
   std::vector<uint4> a, b;
   std::vector<unsigned> h;
-  int nb = 0;
+  int nb = 0, hs = 0;
   long long terms = 0, rows = 0, scaled = 0;
 };
 
@@ -798,60 +827,66 @@ unsigned col_off(int c) { return (unsigned)(c * kColBytes); }
 // density, (Y): destinations are Hermite indices with their axes
 enum StageKind { kCols, kDensity, kRows };
 
-HostStage pack(std::vector<Row> rows, Pal pal, StageKind kind, int zero, const std::vector<std::array<int, 3>>& herm) {
+HostStage pack(std::vector<Row> rows, Pal pal, StageKind kind, int zero, const std::vector<std::array<int, 3>>& herm,
+               int nw) {
   HostStage s;
   std::stable_sort(rows.begin(), rows.end(), [](const Row& a, const Row& b) { return a.t.size() > b.t.size(); });
   const unsigned z = col_off(zero), za = kind == kDensity ? 0u : z;
-  // longest first onto the shortest of four queues
-  std::vector<const Row*> queue[4];
-  size_t len[4] = {0, 0, 0, 0};
+  // longest first onto the shortest of the warps' queues, four each
+  const int nq = 4 * nw;
+  std::vector<std::vector<const Row*>> queue(nq);
+  std::vector<size_t> len(nq, 0), at(nq, 0), term(nq, 0);
   for (const Row& r : rows) {
-    int k = 0;
-    for (int i = 1; i < 4; ++i)
-      if (len[i] < len[k]) k = i;
+    const int k = (int)(std::min_element(len.begin(), len.end()) - len.begin());
     queue[k].push_back(&r);
     len[k] += r.t.size();
     s.terms += (long long)r.t.size();
     ++s.rows;
+    s.scaled += pal.id(r.scale) != 0;
   }
-  size_t nb = *std::max_element(len, len + 4);
+  size_t nb = *std::max_element(len.begin(), len.end());
   nb += nb % 2;
-  size_t at[4] = {0, 0, 0, 0}, term[4] = {0, 0, 0, 0};
-  for (size_t j = 0; j < nb; ++j) {
-    unsigned x[4] = {za, za, za, za}, y[4] = {z, z, z, z};
-    for (int k = 0; k < 4; ++k) {
-      if (at[k] == queue[k].size()) continue;
-      const Row& r = *queue[k][at[k]];
-      const auto& t = r.t[term[k]];
-      x[k] = kind == kDensity ? (unsigned)(t.first * 8) : col_off(t.first);
-      y[k] = col_off(t.second);
-      if (++term[k] < r.t.size()) continue;
-      y[k] |= kLast;
-      ++at[k];
-      term[k] = 0;
-      if (kind == kRows) {
-        unsigned m = 0;
-        for (int i = 0; i < 3; ++i)
-          if (herm[r.dst][i] > 0) m |= 1u << i;
-        s.h.push_back((unsigned)r.dst | (m << 16));
-      } else {
-        const unsigned id = (unsigned)pal.id(r.scale);
-        s.scaled += id != 0;
-        s.h.push_back(col_off(r.dst) | (id << 20));
-      }
-    }
-    s.a.push_back(uint4{x[0], x[1], x[2], x[3]});
-    s.b.push_back(uint4{y[0], y[1], y[2], y[3]});
-  }
   s.nb = (int)nb;
-  // one batch and one header to fetch past the end
-  s.a.push_back(uint4{za, za, za, za});
-  s.b.push_back(uint4{z, z, z, z});
-  s.h.push_back(0u);
+  std::vector<std::vector<unsigned>> head(nw);
+  for (int w = 0; w < nw; ++w) {
+    for (size_t j = 0; j < nb; ++j) {
+      unsigned x[4] = {za, za, za, za}, y[4] = {z, z, z, z};
+      for (int i = 0; i < 4; ++i) {
+        const int k = 4 * w + i;
+        if (at[k] == queue[k].size()) continue;
+        const Row& r = *queue[k][at[k]];
+        const auto& t = r.t[term[k]];
+        x[i] = kind == kDensity ? (unsigned)(t.first * 8) : col_off(t.first);
+        y[i] = col_off(t.second);
+        if (++term[k] < r.t.size()) continue;
+        y[i] |= kLast;
+        ++at[k];
+        term[k] = 0;
+        if (kind == kRows) {
+          unsigned m = 0;
+          for (int ax = 0; ax < 3; ++ax)
+            if (herm[r.dst][ax] > 0) m |= 1u << ax;
+          head[w].push_back((unsigned)r.dst | (m << 16));
+        } else {
+          head[w].push_back(col_off(r.dst) | ((unsigned)pal.id(r.scale) << 20));
+        }
+      }
+      s.a.push_back(uint4{x[0], x[1], x[2], x[3]});
+      s.b.push_back(uint4{y[0], y[1], y[2], y[3]});
+    }
+    // one batch to fetch past the end
+    s.a.push_back(uint4{za, za, za, za});
+    s.b.push_back(uint4{z, z, z, z});
+    s.hs = std::max(s.hs, (int)head[w].size() + 1);  // and one header
+  }
+  for (int w = 0; w < nw; ++w) {
+    head[w].resize(s.hs, 0u);
+    s.h.insert(s.h.end(), head[w].begin(), head[w].end());
+  }
   return s;
 }
 
-Program build_program(int Lab, int lc) {
+Program build_program(int Lab, int lc, int nw) {
   Program p;
   p.Lab = Lab; p.lc = lc;
   p.K = std::min(Lab, lc);
@@ -876,7 +911,7 @@ Program build_program(int Lab, int lc) {
     for (int ny = 0; ux + ny <= lc; ++ny)
       for (int nz = 0; ux + ny + nz <= lc; ++nz) { int k = (int)iY.size(); iY[{ux, ny, nz}] = k; }
   const int nU = (int)iU.size();
-  const int sizeU = std::max(nU, (int)iY.size()), sizeB = std::max({(int)iZ.size(), 33, Lab + 1});
+  const int sizeU = std::max(nU, (int)iY.size()), sizeB = std::max({(int)iZ.size(), (nw * stage_rows(nw) * 33 + 31) / 32, Lab + 1});
   int c = p.nR;
   p.cZero = c; c += 1;
   p.cX = c; c += 3;
@@ -925,7 +960,7 @@ Program build_program(int Lab, int lc) {
     for (int i = 0; i < nherm(left); ++i) w.t.push_back({hidx(a[0] + herm[i][0], a[1] + herm[i][1], a[2] + herm[i][2]), i});
     r.push_back(w);
   }
-  p.Z = pack(r, pal, kDensity, p.cZero, herm);
+  p.Z = pack(r, pal, kDensity, p.cZero, herm, nw);
   r.clear();
   for (auto& z : iZ) {
     const int ux = z.first[0], uy = z.first[1], nz = z.first[2];
@@ -933,7 +968,7 @@ Program build_program(int Lab, int lc) {
     for (int uz = 0; uz <= std::min(nz, K - ux - uy); ++uz) w.t.push_back({p.cU + iU.at({ux, uy, uz}), PW(2, nz - uz)});
     r.push_back(w);
   }
-  p.gz = pack(r, pal, kCols, p.cZero, herm);
+  p.gz = pack(r, pal, kCols, p.cZero, herm, nw);
   r.clear();
   for (auto& y : iY) {
     const int ux = y.first[0], ny = y.first[1], nz = y.first[2];
@@ -941,7 +976,7 @@ Program build_program(int Lab, int lc) {
     for (int uy = 0; uy <= std::min(ny, K - ux); ++uy) w.t.push_back({p.cB + iZ.at({ux, uy, nz}), PW(1, ny - uy)});
     r.push_back(w);
   }
-  p.gy = pack(r, pal, kCols, p.cZero, herm);
+  p.gy = pack(r, pal, kCols, p.cZero, herm, nw);
   r.clear();
   for (int ny = 0; ny <= lc; ++ny)
     for (int nz = 0; ny + nz <= lc; ++nz) {
@@ -950,14 +985,14 @@ Program build_program(int Lab, int lc) {
       for (int ux = 0; ux <= std::min(nx, K); ++ux) w.t.push_back({p.cU + iY.at({ux, ny, nz}), PW(0, nx - ux)});
       r.push_back(w);
     }
-  p.gx = pack(r, pal, kCols, p.cZero, herm);
+  p.gx = pack(r, pal, kCols, p.cZero, herm, nw);
   // ---- J
   r.clear();
   for (auto& y : iY) {
     const int ux = y.first[0], ny = y.first[1], nz = y.first[2], nx = lc - ny - nz;
     r.push_back(Row{p.cU + y.second, 1.0, {{p.cCP + cart_index(nx, ny, nz), PW(0, nx - ux)}}});
   }
-  p.jx = pack(r, pal, kCols, p.cZero, herm);
+  p.jx = pack(r, pal, kCols, p.cZero, herm, nw);
   r.clear();
   for (auto& z : iZ) {
     const int ux = z.first[0], uy = z.first[1], nz = z.first[2];
@@ -965,7 +1000,7 @@ Program build_program(int Lab, int lc) {
     for (int ny = uy; ux + ny + nz <= lc; ++ny) w.t.push_back({p.cU + iY.at({ux, ny, nz}), PW(1, ny - uy)});
     r.push_back(w);
   }
-  p.jy = pack(r, pal, kCols, p.cZero, herm);
+  p.jy = pack(r, pal, kCols, p.cZero, herm, nw);
   r.clear();
   for (auto& u : iU) {
     const auto& a = u.first;
@@ -973,7 +1008,7 @@ Program build_program(int Lab, int lc) {
     for (int nz = a[2]; a[0] + a[1] + nz <= lc; ++nz) w.t.push_back({p.cB + iZ.at({a[0], a[1], nz}), PW(2, nz - a[2])});
     r.push_back(w);
   }
-  p.jw = pack(r, pal, kCols, p.cZero, herm);
+  p.jw = pack(r, pal, kCols, p.cZero, herm, nw);
   r.clear();
   for (int i = 0; i < p.nR; ++i) {
     const auto& a = herm[i];
@@ -984,7 +1019,7 @@ Program build_program(int Lab, int lc) {
           w.t.push_back({hidx(a[0] - ux, a[1] - uy, a[2] - uz), p.cU + iU.at({ux, uy, uz})});
     r.push_back(w);
   }
-  p.Y = pack(r, pal, kRows, p.cZero, herm);
+  p.Y = pack(r, pal, kRows, p.cZero, herm, nw);
   for (int i = 0; i < p.nR; ++i) p.ydeg.push_back(herm[i][0] + herm[i][1] + herm[i][2]);
   // ---- ket transforms with the monomials' factorials
   const auto T = solid_matrix(lc);
@@ -1011,12 +1046,13 @@ Program build_program(int Lab, int lc) {
   return p;
 }
 
-const Program& program(int Lab, int lc) {
+const Program& program(int Lab, int lc, int nw) {
   static std::mutex mu;
-  static std::map<std::pair<int, int>, Program> cache;
+  static std::map<std::tuple<int, int, int>, Program> cache;
   std::lock_guard<std::mutex> lk(mu);
-  auto it = cache.find({Lab, lc});
-  if (it == cache.end()) it = cache.emplace(std::make_pair(Lab, lc), build_program(Lab, lc)).first;
+  const auto key = std::make_tuple(Lab, lc, nw);
+  auto it = cache.find(key);
+  if (it == cache.end()) it = cache.emplace(key, build_program(Lab, lc, nw)).first;
   return it->second;
 }
 
@@ -1042,7 +1078,7 @@ struct HermPlan {
   bool grad = false;
   long long nao = 0, npair = 0, nprim = 0;
   struct Tier {
-    int smem;
+    int smem, nw;
     long long first, n;
   };
   std::vector<Tier> tiers;
@@ -1077,7 +1113,7 @@ double herm_flops(const HermPlan* p) { return p->flops; }
 double herm_max_adds(const HermPlan* p) { return p->max_adds; }
 
 double herm_class_flops(int Lab, int lc) {
-  const Program& p = program(Lab, lc);
+  const Program& p = program(Lab, lc, 1);
   return 2.0 * (p.instr_base + p.instr_gamma + p.instr_j);
 }
 
@@ -1208,9 +1244,16 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       }
       if (tri == 0) continue;
       const int Lp = L.Lab + (grad ? 1 : 0);
-      const Program& pg = program(Lp, k.lc);
+      // warps per block: as many as it takes to reach eight on an SM (asking
+      // for 12 or 16 leaves short stages with idle queues: DF-J of 32 atoms
+      // 105 -> 109 and 122 ms; one warp throughout: 110 ms)
+      const Program& p1 = program(Lp, k.lc, 1);
+      const int fit = kSmemSm / ((grad ? p1.ncol_grad : p1.ncol) * kColBytes + 2048);
+      const int nw = fit >= 8 ? 1 : (fit >= 4 ? 2 : 4);
+      const Program& pg = program(Lp, k.lc, nw);
       HermCls& c = x.c;
       std::memset(&c, 0, sizeof(c));
+      c.nw = nw;
       c.Lab = Lp; c.lc = k.lc; c.Kc = k.Kc; c.L = Lp + k.lc; c.nR = pg.nR; c.nY = pg.nR; c.ncc = pg.ncc; c.nC = pg.nC;
       c.nket = (int)k.shells.size();
       c.cX = pg.cX; c.cPW = pg.cPW; c.cU = pg.cU; c.cB = pg.cB; c.cCP = pg.cCP; c.cGA = pg.cGA;
@@ -1236,7 +1279,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       }
       p->flops += 2.0 * x.instr * tri;
       total += x.instr * best / 32.0;
-      auto key = std::make_pair(Lp, k.lc);
+      auto key = std::make_pair(Lp, k.lc);  // (nw follows from them)
       if (first_of.count(key)) {
         const ClsHost& f = cls[first_of[key]];
         x.rops = f.rops; x.cptr = f.cptr; x.cent = f.cent; x.gptr = f.gptr; x.gent = f.gent; x.pal = f.pal; x.ydeg = f.ydeg;
@@ -1255,7 +1298,10 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       {
         const HostStage* hs[8] = {&pg.Z, &pg.gz, &pg.gy, &pg.gx, &pg.jx, &pg.jy, &pg.jw, &pg.Y};
         Stage* ds_[8] = {&c.Z, &c.gz, &c.gy, &c.gx, &c.jx, &c.jy, &c.jw, &c.Y};
-        for (int s = 0; s < 8; ++s) ds_[s]->nb = hs[s]->nb;
+        for (int s = 0; s < 8; ++s) {
+          ds_[s]->nb = hs[s]->nb;
+          ds_[s]->hs = hs[s]->hs;
+        }
       }
       x.cnt = blob.add(x.counts);
       cls.push_back(std::move(x));
@@ -1267,8 +1313,10 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   std::vector<int> order(cls.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
   auto occ = [&](int smem) { return std::min(32, kSmemSm / (smem + 1024)); };
-  // classes of equal occupancy share a launch, the largest footprint first
+  // classes of equal block size and occupancy share a launch, the largest
+  // footprint first
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    if (cls[a].c.nw != cls[b].c.nw) return cls[a].c.nw > cls[b].c.nw;
     const int oa = occ(cls[a].smem), ob = occ(cls[b].smem);
     return oa != ob ? oa < ob : cls[a].instr > cls[b].instr;
   });
@@ -1281,8 +1329,8 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     const LabHost& L = labs[x.lab];
     int b = 0;
     while (b + 1 < 10 && bins[b + 1] <= occ(x.smem)) ++b;
-    if (b != bin) {
-      p->tiers.push_back(HermPlan::Tier{0, (long long)tiles.size(), 0});
+    if (b != bin || p->tiers.back().nw != x.c.nw) {
+      p->tiers.push_back(HermPlan::Tier{0, x.c.nw, (long long)tiles.size(), 0});
       bin = b;
     }
     HermPlan::Tier& t = p->tiers.back();
@@ -1304,7 +1352,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       set_last_error("dfj: too many tiles");
       return LX3C_ENOTSUP;
     }
-  p->max_adds = 32.0 * (double)tiles.size() + 2.0 * (double)p->npair;
+  p->max_adds = 4 * 32.0 * (double)tiles.size() + 2.0 * (double)p->npair;
   // ---- one allocation: tables and lists (uploaded), then the work buffers
   std::vector<double> sph;
   std::vector<int> sphoff;
@@ -1420,10 +1468,12 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   ma.boys_mid = dev_boys_mid(ds);
   cudaError_t e = cudaMemcpyAsync(A, blob.d.data(), blob.d.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
+  const void* kernels[] = {(const void*)herm_kernel<1, 1>, (const void*)herm_kernel<1, 2>, (const void*)herm_kernel<1, 4>,
+                           (const void*)herm_kernel<2, 1>, (const void*)herm_kernel<2, 2>, (const void*)herm_kernel<2, 4>,
+                           (const void*)herm_kernel<3, 1>, (const void*)herm_kernel<3, 2>, (const void*)herm_kernel<3, 4>,
+                           (const void*)herm_kernel<4, 1>, (const void*)herm_kernel<4, 2>, (const void*)herm_kernel<4, 4>};
+  for (const void* f : kernels)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_pre_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_pre_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(herm_post_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCta);
@@ -1458,7 +1508,9 @@ template <int kMode>
 cudaError_t herm_tiles(HermPlan* p, HermArgs a, cudaStream_t st) {
   for (auto& t : p->tiers) {
     a.tiles = p->ma.tiles + t.first;
-    herm_kernel<kMode><<<(unsigned)t.n, 32, t.smem, st>>>(a);
+    if (t.nw == 1) herm_kernel<kMode, 1><<<(unsigned)t.n, 32, t.smem, st>>>(a);
+    else if (t.nw == 2) herm_kernel<kMode, 2><<<(unsigned)t.n, 64, t.smem, st>>>(a);
+    else herm_kernel<kMode, 4><<<(unsigned)t.n, 128, t.smem, st>>>(a);
   }
   return cudaGetLastError();
 }
