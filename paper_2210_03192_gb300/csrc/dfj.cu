@@ -202,6 +202,37 @@ bool use_hermite(const HermBra& b, const HermKet& k) {
   return true;
 }
 
+// One device allocation for everything a plan keeps: arrays to upload
+// (copied at once) and work buffers.  Pointers are set by commit().  (A plan
+// has some 25 arrays per class group; one allocation and one copy for each was
+// 8 of the 18 ms that planning 12 atoms with g functions took.)
+struct PlanArena {
+  std::vector<char> up;
+  size_t work = 0;
+  std::vector<std::pair<void**, size_t>> fix_up, fix_work;
+  template <class T>
+  void add(T** ptr, const T* v, size_t n) {
+    const size_t off = (up.size() + 255) & ~size_t(255);
+    up.resize(off + std::max<size_t>(n, 1) * sizeof(T));
+    if (n) std::memcpy(up.data() + off, v, n * sizeof(T));
+    fix_up.push_back({(void**)ptr, off});
+  }
+  template <class T>
+  void take(T** ptr, size_t n) {
+    fix_work.push_back({(void**)ptr, work});
+    work += (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~size_t(255);
+  }
+  cudaError_t commit(char** base, cudaStream_t st) {
+    const size_t first = (up.size() + 255) & ~size_t(255);
+    cudaError_t e = cudaMalloc(base, std::max<size_t>(first + work, 256));
+    if (e == cudaSuccess && !up.empty()) e = cudaMemcpyAsync(*base, up.data(), up.size(), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    for (auto& f : fix_up) *f.first = *base + f.second;
+    for (auto& f : fix_work) *f.first = *base + first + f.second;
+    return cudaStreamSynchronize(st);
+  }
+};
+
 struct DfjLaunch {
   ClassDesc desc;
   int grid = 1;
@@ -209,6 +240,7 @@ struct DfjLaunch {
   int4* d_sub = nullptr;
   int* d_prim = nullptr;
   int4* d_tiles = nullptr;
+  bool own_tiles = false;  // re-tiled: d_tiles is its own allocation
   std::vector<int4> sub;   // host copy of the sub-pair list (re-tiling)
   int kmax = 0;
 };
@@ -243,6 +275,7 @@ struct lx3c_dfj {
   int natom = 0;
   bool gradient = false;
   std::vector<DfjGroup> groups;
+  char* arena = nullptr;            // every device array of the groups, and the accumulators
   HermPlan* hj = nullptr;           // gamma and J of the Hermite groups
   HermPlan* hg = nullptr;           // gradient of every group
   // exact fixed-point accumulators per element: gamma, J, gradient
@@ -259,18 +292,12 @@ extern "C" {
 
 void lx3c_dfj_destroy(lx3c_dfj* p) {
   if (!p) return;
-  for (auto& g : p->groups) {
-    cudaFree(g.d_pairs); cudaFree(g.d_auxs); cudaFree(g.d_pair_ao); cudaFree(g.d_aux_ao);
-    cudaFree(g.d_pairrec); cudaFree(g.d_pairab); cudaFree(g.d_auxrec); cudaFree(g.d_auxc);
-    for (auto& L : g.L) {
-      cudaFree(L.d_sub); cudaFree(L.d_prim); cudaFree(L.d_tiles);
-    }
-  }
+  for (auto& g : p->groups)
+    for (auto& L : g.L)
+      if (L.own_tiles) cudaFree(L.d_tiles);
+  cudaFree(p->arena);
   herm_destroy(p->hj);
   herm_destroy(p->hg);
-  cudaFree(p->d_gacc);
-  cudaFree(p->d_Jacc);
-  cudaFree(p->d_facc);
   delete p;
 }
 
@@ -295,7 +322,8 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   int rc = device_state_get(&ds);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  std::unique_ptr<lx3c_dfj> p(new lx3c_dfj);
+  std::unique_ptr<lx3c_dfj, void (*)(lx3c_dfj*)> p(new lx3c_dfj, lx3c_dfj_destroy);
+  PlanArena arena;
   p->orb = orb;
   p->aux = aux;
   p->tol = schwarz_tol;
@@ -412,18 +440,14 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       pao[i] = int4{ao[g.pairs[2 * i]], ao[g.pairs[2 * i + 1]], g.pairs[2 * i] == g.pairs[2 * i + 1] ? 1 : 0, 0};
     for (long long q = 0; q < na; ++q) aao[q] = aq[g.auxs[q]];
     const int Kab = g.Ka * g.Kb;
-    DCUDA(cudaMalloc(&g.d_pairs, np * 8));
-    DCUDA(cudaMalloc(&g.d_auxs, na * 4));
-    DCUDA(cudaMalloc(&g.d_pair_ao, np * sizeof(int4)));
-    DCUDA(cudaMalloc(&g.d_aux_ao, na * 4));
-    DCUDA(cudaMalloc(&g.d_pairrec, (size_t)np * Kab * kPairRec * 8));
-    DCUDA(cudaMalloc(&g.d_pairab, (size_t)np * 3 * 8));
-    DCUDA(cudaMalloc(&g.d_auxrec, (size_t)na * g.Kc * kAuxRec * 8));
-    DCUDA(cudaMalloc(&g.d_auxc, (size_t)na * 3 * 8));
-    DCUDA(cudaMemcpyAsync(g.d_pairs, g.pairs.data(), np * 8, cudaMemcpyHostToDevice, st));
-    DCUDA(cudaMemcpyAsync(g.d_auxs, g.auxs.data(), na * 4, cudaMemcpyHostToDevice, st));
-    DCUDA(cudaMemcpyAsync(g.d_pair_ao, pao.data(), np * sizeof(int4), cudaMemcpyHostToDevice, st));
-    DCUDA(cudaMemcpyAsync(g.d_aux_ao, aao.data(), na * 4, cudaMemcpyHostToDevice, st));
+    arena.add(&g.d_pairs, g.pairs.data(), g.pairs.size());
+    arena.add(&g.d_auxs, g.auxs.data(), g.auxs.size());
+    arena.add(&g.d_pair_ao, pao.data(), pao.size());
+    arena.add(&g.d_aux_ao, aao.data(), aao.size());
+    arena.take(&g.d_pairrec, (size_t)np * Kab * kPairRec);
+    arena.take(&g.d_pairab, (size_t)np * 3);
+    arena.take(&g.d_auxrec, (size_t)na * g.Kc * kAuxRec);
+    arena.take(&g.d_auxc, (size_t)na * 3);
     for (int o = 0; o < 2; ++o) {
       if (sub[o].empty()) continue;
       DfjLaunch& L = g.L[o];
@@ -460,35 +484,34 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       L.ntiles = (long long)tiles.size();
       L.sub = sub[o];
       L.kmax = kmax[o];
-      DCUDA(cudaMalloc(&L.d_sub, sub[o].size() * sizeof(int4)));
-      DCUDA(cudaMalloc(&L.d_prim, std::max<size_t>(prim[o].size(), 1) * sizeof(int)));
-      DCUDA(cudaMalloc(&L.d_tiles, tiles.size() * sizeof(int4)));
-      DCUDA(cudaMemcpyAsync(L.d_sub, sub[o].data(), sub[o].size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-      DCUDA(cudaMemcpyAsync(L.d_prim, prim[o].data(), prim[o].size() * sizeof(int), cudaMemcpyHostToDevice, st));
-      DCUDA(cudaMemcpyAsync(L.d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+      arena.add(&L.d_sub, sub[o].data(), sub[o].size());
+      arena.add(&L.d_prim, prim[o].data(), prim[o].size());
+      arena.add(&L.d_tiles, tiles.data(), tiles.size());
       d.npair = np;
       d.naux = na;
       d.nsub = (long long)sub[o].size();
       d.ntiles = L.ntiles;
       d.ntile_aux = 1;
-      d.tiles = L.d_tiles;
-      d.subpairs = L.d_sub;
-      d.primidx = L.d_prim;
-      d.pairrec = g.d_pairrec; d.pairab = g.d_pairab; d.auxrec = g.d_auxrec; d.auxc = g.d_auxc;
       d.digest = 1;
       set_digest_scratch(d);
       if ((long long)d.smem_doubles * 8 > 232448) return dfail(LX3C_ENOTSUP, "digestion scratch does not fit");
       d.ldD = p->nao;
-      d.pair_ao = g.d_pair_ao;
-      d.aux_ao = g.d_aux_ao;
       const int occ = eri3c_occupancy(d.smem_doubles * 8);
       L.grid = (int)std::min<long long>(L.ntiles, (long long)dev_nsm(ds) * occ * 8);
     }
   }
-  DCUDA(cudaMalloc(&p->d_gacc, (size_t)p->naux_ao * kFixBytes));
-  DCUDA(cudaMalloc(&p->d_Jacc, (size_t)p->nao * p->nao * kFixBytes));
-  if (want_grad) DCUDA(cudaMalloc(&p->d_facc, (size_t)p->natom * 3 * kFixBytes));
-  DCUDA(cudaStreamSynchronize(st));
+  arena.take(&p->d_gacc, (size_t)p->naux_ao * kFixWords);
+  arena.take(&p->d_Jacc, (size_t)p->nao * p->nao * kFixWords);
+  if (want_grad) arena.take(&p->d_facc, (size_t)p->natom * 3 * kFixWords);
+  DCUDA(arena.commit(&p->arena, st));
+  for (auto& g : p->groups)
+    for (auto& L : g.L) {
+      if (!L.ntiles) continue;
+      ClassDesc& d = L.desc;
+      d.tiles = L.d_tiles; d.subpairs = L.d_sub; d.primidx = L.d_prim;
+      d.pairrec = g.d_pairrec; d.pairab = g.d_pairab; d.auxrec = g.d_auxrec; d.auxc = g.d_auxc;
+      d.pair_ao = g.d_pair_ao; d.aux_ao = g.d_aux_ao;
+    }
   *out = p.release();
   return LX3C_OK;
 }
@@ -677,8 +700,9 @@ bool retile(DfjLaunch& L, const DfjGroup& g, const DevState* ds, int T) {
   int4* dt = nullptr;
   if (cudaMalloc(&dt, tiles.size() * sizeof(int4)) != cudaSuccess) return false;
   cudaMemcpy(dt, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice);
-  cudaFree(L.d_tiles);
+  if (L.own_tiles) cudaFree(L.d_tiles);
   L.d_tiles = dt;
+  L.own_tiles = true;
   L.ntiles = (long long)tiles.size();
   nd.tiles = dt;
   nd.ntiles = L.ntiles;

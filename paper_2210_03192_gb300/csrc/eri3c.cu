@@ -1539,14 +1539,10 @@ int persistent_occupancy(int smem_bytes, int two) {
   return nb < 1 ? 1 : nb;
 }
 
+// CTAs of the tile kernel per SM: its launch bounds, or what the shared memory
+// of an SM holds (233,472 bytes, 1 KB of it per CTA reserved).
 int eri3c_occupancy(int smem_bytes) {
-  int nb = 0;
-  if (tile_kernel_attributes() != cudaSuccess) return 1;
-  const cudaError_t e = three_ctas(smem_bytes)
-      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_kernel<0, 384, 3>, 384, smem_bytes)
-      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eri3c_kernel<0, 512, 2>, 512, smem_bytes);
-  if (e != cudaSuccess) return 1;
-  return nb < 1 ? 1 : nb;
+  return std::max(1, std::min(three_ctas(smem_bytes) ? 3 : 2, 233472 / (smem_bytes + 1024)));
 }
 
 }  // namespace lx3c
