@@ -225,10 +225,10 @@ __device__ __forceinline__ void stage_items(int nx, int T, int tv, int mode, con
 }
 
 // Blocks of four, two or one triples, as T divides, as long as the items still
-// fill the block's threads and (mode 0) a warp keeps to one target.
+// fill the block's threads and (mode 0) a warp holds two targets at most.
 template <int NT, class F>
 __device__ __forceinline__ void stage(int nx, int T, int tv, int mode, const F& f) {
-  const int most = mode == 0 ? T >> 5 : 4;
+  const int most = mode == 0 ? T >> 4 : 4;
   if ((T & 3) == 0 && most >= 4 && nx * T >= 4 * NT)
     stage_items<NT, 4>(nx, T, tv, mode, [&](int x, int t0, int ts) { f(x, t0, ts, Int<4>()); });
   else if ((T & 1) == 0 && most >= 2 && nx * T >= 2 * NT)
