@@ -240,6 +240,7 @@ struct DfjLaunch {
   int4* d_sub = nullptr;
   int* d_prim = nullptr;
   int4* d_tiles = nullptr;
+  int4* d_wtiles = nullptr;  // register-resident kernels (ClassDesc::wtiles)
   bool own_tiles = false;  // re-tiled: d_tiles is its own allocation
   std::vector<int4> sub;   // host copy of the sub-pair list (re-tiling)
   int kmax = 0;
@@ -487,6 +488,30 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       arena.add(&L.d_sub, sub[o].data(), sub[o].size());
       arena.add(&L.d_prim, prim[o].data(), prim[o].size());
       arena.add(&L.d_tiles, tiles.data(), tiles.size());
+      if (!g.herm) {
+        // tiles of the register-resident kernel: the width that leaves fewest
+        // lanes idle at the ends of the ket lists (a small charge for the
+        // sub-pairs of unequal contraction that then share a warp), the most
+        // contracted sub-pairs first.  (One tile of the tile kernel's T per
+        // warp left half the lanes idle from f on: (s s|h) of 16 atoms 256
+        // instructions per primitive triple where (s s|g) took 108.)
+        double best = 1e300;
+        for (int W = 32; W >= 1; W /= 2) {
+          double slots = 0;
+          for (auto& sp : sub[o]) slots += (double)((g.counts[sp.x] + W - 1) / W * W) * sp.z;
+          slots *= 1.0 + 0.03 * (32 / W - 1);
+          if (slots < 0.999 * best) { best = slots; d.warpW = W; }
+        }
+        std::vector<int4> wt;
+        for (size_t s = 0; s < sub[o].size(); ++s) {
+          const int cnt = g.counts[sub[o][s].x];
+          for (int a0 = 0; a0 < cnt; a0 += d.warpW)
+            wt.push_back(int4{(int)s, a0, std::min(d.warpW, cnt - a0), sub[o][s].z});
+        }
+        std::stable_sort(wt.begin(), wt.end(), [](const int4& x, const int4& y) { return x.w > y.w; });
+        d.nwtiles = (long long)wt.size();
+        arena.add(&L.d_wtiles, wt.data(), wt.size());
+      }
       d.npair = np;
       d.naux = na;
       d.nsub = (long long)sub[o].size();
@@ -508,7 +533,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       ClassDesc& d = L.desc;
-      d.tiles = L.d_tiles; d.subpairs = L.d_sub; d.primidx = L.d_prim;
+      d.tiles = L.d_tiles; d.wtiles = L.d_wtiles; d.subpairs = L.d_sub; d.primidx = L.d_prim;
       d.pairrec = g.d_pairrec; d.pairab = g.d_pairab; d.auxrec = g.d_auxrec; d.auxc = g.d_auxc;
       d.pair_ao = g.d_pair_ao; d.aux_ao = g.d_aux_ao;
     }
@@ -925,6 +950,7 @@ lx3c_status lx3c_batch_plan(lx3c_batch** out, int nmol, const lx3c_basis* const*
     for (int T : cands) {
       if (!retile(L, g, b->ds, T)) continue;
       ClassDesc d = L.desc;
+      d.wtiles = nullptr;  // the tile kernel, whose T this is
       d.D = tD; d.cvec = tc;
       d.gacc = (unsigned long long*)tg; d.Jacc = (unsigned long long*)tJ;
       long long nt = 0;

@@ -1017,55 +1017,51 @@ __global__ void __launch_bounds__(kSsThreads) eri3c_ss_kernel(const __grid_const
   }
 }
 
-// (s s|C) DF-J launches digesting per integral (digest == 1), one warp per
-// tile, lanes over the tile's kets: gamma_P[C] += w D_ab (ss|P)_C per lane,
+// (s s|C) DF-J launches digesting per integral (digest == 1), lanes over the
+// kets of 32 / warpW tiles: gamma_P[C] += w D_ab (ss|P)_C per lane,
 // and J_ab += w_J sum over the tile's kets and C of (ss|P)_C c_PC, reduced
-// across the warp into one add.  The same sums as the tile kernel's digest.
+// across the tile's lanes into one add.  The same sums as the tile kernel's
+// digest.
 template <int LC>
 __global__ void __launch_bounds__(kSsThreads) eri3c_ss_dfj_kernel(const __grid_constant__ ClassDesc d) {
   constexpr int NC = (LC + 1) * (LC + 2) / 2, NS = 2 * LC + 1;
   __shared__ double sP[kSsThreads * (NC + 1)];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double* row = sP + threadIdx.x * (NC + 1);
+  const int W = d.warpW, NP = 32 / W, g = lane / W, t = lane - g * W;
   const long long nwarps = (long long)gridDim.x * (kSsThreads / 32);
-  for (long long tile = blockIdx.x * (long long)(kSsThreads / 32) + warp; tile < d.ntiles; tile += nwarps) {
-    const int4 tt = __ldg(d.tiles + tile);
+  for (long long w0 = (blockIdx.x * (long long)(kSsThreads / 32) + warp) * NP; w0 < d.nwtiles; w0 += nwarps * NP) {
+    const int4 tt = w0 + g < d.nwtiles ? __ldg(d.wtiles + w0 + g) : int4{0, 0, 0, 0};
     const int4 sp = __ldg(d.subpairs + tt.x);
     const long long pair = sp.x;
     const int4 pao = __ldg(d.pair_ao + pair);
     const double wg = pao.z ? 1.0 : 2.0, wj = pao.z ? 0.5 : 1.0;
     const double Dab = d.gacc ? __ldg(d.D + (long long)pao.x * d.ldD + pao.y) : 0.0;
     double jsum = 0.0;
-    for (int t0 = 0; t0 < tt.z; t0 += 32) {
-      const int t = t0 + lane;
-      const bool live = t < tt.z;
-      double acc[NC];
+    const bool live = t < tt.z;
+    double acc[NC];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] = 0.0;
-      const long long q = tt.y + t;
-      if (live) ss_prims<LC>(d, pair, sp, q, acc);
+    for (int c = 0; c < NC; ++c) acc[c] = 0.0;
+    const long long q = tt.y + t;
+    if (live) {
+      ss_prims<LC>(d, pair, sp, q, acc);
 #pragma unroll
       for (int c = 0; c < NC; ++c) row[c] = acc[c];
-      __syncwarp();
-      if (live) {
-        const int ao = __ldg(d.aux_ao + q);
+      const int ao = __ldg(d.aux_ao + q);
 #pragma unroll
-        for (int C = 0; C < NS; ++C) {
-          double v = 0.0;
-          for (int k = __ldg(d.kptr + C); k < __ldg(d.kptr + C + 1); ++k) {
-            const int2 e = __ldg(d.kent + k);
-            v = fma(__ldg(d.pal + e.y), row[e.x], v);
-          }
-          if (d.gacc) fix_add(d.gacc + kFixWords * (ao + C), wg * Dab * v);
-          if (d.Jacc) jsum = fma(v, __ldg(d.cvec + ao + C), jsum);
+      for (int C = 0; C < NS; ++C) {
+        double v = 0.0;
+        for (int k = __ldg(d.kptr + C); k < __ldg(d.kptr + C + 1); ++k) {
+          const int2 e = __ldg(d.kent + k);
+          v = fma(__ldg(d.pal + e.y), row[e.x], v);
         }
+        if (d.gacc) fix_add(d.gacc + kFixWords * (ao + C), wg * Dab * v);
+        if (d.Jacc) jsum = fma(v, __ldg(d.cvec + ao + C), jsum);
       }
-      __syncwarp();
     }
     if (d.Jacc) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) jsum += __shfl_xor_sync(0xffffffffu, jsum, o);
-      if (lane == 0) fix_add(d.Jacc + kFixWords * ((long long)pao.x * d.ldD + pao.y), wj * jsum);
+      for (int o = W >> 1; o > 0; o >>= 1) jsum += __shfl_xor_sync(0xffffffffu, jsum, o);
+      if (t == 0 && tt.z) fix_add(d.Jacc + kFixWords * ((long long)pao.x * d.ldD + pao.y), wj * jsum);
     }
   }
 }
@@ -1265,9 +1261,10 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double* row = sG + threadIdx.x * 3 * (NC + 1);
   double* out = sO + threadIdx.x * NB;
+  const int W = d.warpW, NP = 32 / W, g = lane / W, t = lane - g * W;
   const long long nwarps = (long long)gridDim.x * (kPsThreads / 32);
-  for (long long tile = blockIdx.x * (long long)(kPsThreads / 32) + warp; tile < d.ntiles; tile += nwarps) {
-    const int4 tt = __ldg(d.tiles + tile);
+  for (long long w0 = (blockIdx.x * (long long)(kPsThreads / 32) + warp) * NP; w0 < d.nwtiles; w0 += nwarps * NP) {
+    const int4 tt = w0 + g < d.nwtiles ? __ldg(d.wtiles + w0 + g) : int4{0, 0, 0, 0};
     const int4 sp = __ldg(d.subpairs + tt.x);
     const long long pair = sp.x;
     const int4 pao = __ldg(d.pair_ao + pair);
@@ -1279,29 +1276,26 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
         Ds[s] = d.orient ? __ldg(d.D + (long long)pao.x * d.ldD + pao.y + s)
                          : __ldg(d.D + (long long)(pao.x + s) * d.ldD + pao.y);
     double js[3] = {0.0, 0.0, 0.0};
-    for (int t0 = 0; t0 < tt.z; t0 += 32) {
-      const int t = t0 + lane;
-      if (t < tt.z) {
-        const long long q = tt.y + t;
-        double A[3][NC], Bm[NCM];
+    if (t < tt.z) {
+      const long long q = tt.y + t;
+      double A[3][NC], Bm[NCM];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) A[0][c] = A[1][c] = A[2][c] = 0.0;
+      for (int c = 0; c < NC; ++c) A[0][c] = A[1][c] = A[2][c] = 0.0;
 #pragma unroll
-        for (int n = 0; n < NCM; ++n) Bm[n] = 0.0;
-        ps_prims<LC>(d, pair, sp, q, A, Bm);
-        ps_targets<LC>(A, Bm, row);
-        ps_transform<LC>(d, row, out);
-        const int ao = __ldg(d.aux_ao + q);
+      for (int n = 0; n < NCM; ++n) Bm[n] = 0.0;
+      ps_prims<LC>(d, pair, sp, q, A, Bm);
+      ps_targets<LC>(A, Bm, row);
+      ps_transform<LC>(d, row, out);
+      const int ao = __ldg(d.aux_ao + q);
 #pragma unroll
-        for (int C = 0; C < NS; ++C) {
-          const double i0 = out[C], i1 = out[NS + C], i2 = out[2 * NS + C];
-          if (d.gacc) fix_add(d.gacc + kFixWords * (ao + C), wg * fma(Ds[0], i0, fma(Ds[1], i1, Ds[2] * i2)));
-          if (d.Jacc) {
-            const double cv = __ldg(d.cvec + ao + C);
-            js[0] = fma(i0, cv, js[0]);
-            js[1] = fma(i1, cv, js[1]);
-            js[2] = fma(i2, cv, js[2]);
-          }
+      for (int C = 0; C < NS; ++C) {
+        const double i0 = out[C], i1 = out[NS + C], i2 = out[2 * NS + C];
+        if (d.gacc) fix_add(d.gacc + kFixWords * (ao + C), wg * fma(Ds[0], i0, fma(Ds[1], i1, Ds[2] * i2)));
+        if (d.Jacc) {
+          const double cv = __ldg(d.cvec + ao + C);
+          js[0] = fma(i0, cv, js[0]);
+          js[1] = fma(i1, cv, js[1]);
+          js[2] = fma(i2, cv, js[2]);
         }
       }
     }
@@ -1309,9 +1303,8 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
         double v = js[s];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) {
+        for (int o = W >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (t == 0 && tt.z) {
           const long long e = d.orient ? (long long)pao.x * d.ldD + pao.y + s : (long long)(pao.x + s) * d.ldD + pao.y;
           fix_add(d.Jacc + kFixWords * e, wj * v);
         }
@@ -1422,8 +1415,8 @@ static cudaError_t tile_kernel_attributes() {
 // Whether a launch runs the tile kernel (not a register-resident one).
 static bool on_tile_kernel(const ClassDesc& d) {
   if (d.digest == 4) return true;
-  if (d.la == 0 && d.lb == 0 && d.orient == 0 && (d.digest == 0 || (d.digest == 1 && d.tiles))) return false;
-  return !((d.digest == 0 || (d.digest == 1 && d.tiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 && (d.lc > 0 || d.K > 1));
+  if (d.la == 0 && d.lb == 0 && d.orient == 0 && (d.digest == 0 || (d.digest == 1 && d.wtiles))) return false;
+  return !((d.digest == 0 || (d.digest == 1 && d.wtiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 && (d.lc > 0 || d.K > 1));
 }
 
 bool can_launch_both(const ClassDesc& a, const ClassDesc& b) {
@@ -1454,14 +1447,14 @@ cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
       case 5: eri3c_ss_kernel<5><<<g, kSsThreads, 0, st>>>(d); break;
       default: eri3c_ss_kernel<6><<<g, kSsThreads, 0, st>>>(d); break;
     }
-  } else if ((d.digest == 0 || (d.digest == 1 && d.tiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 &&
+  } else if ((d.digest == 0 || (d.digest == 1 && d.wtiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 &&
              (d.lc > 0 || d.K > 1)) {
     // (p s|C) and B-oriented (s p|C) (whose descriptor holds the (p s|C)
     // tables with orient = 1), 1 <= lc <= 4 or contracted: register-resident.
     // (p s|s) with one primitive per triple stays on the tile kernel, which
     // measured faster there.
-    const long long items = d.digest ? d.ntiles : d.nsub * d.naux;
-    const long long per = d.digest ? kPsThreads / 32 : kPsThreads;
+    const long long items = d.digest ? d.nwtiles : d.nsub * d.naux;
+    const long long per = d.digest ? kPsThreads / d.warpW : kPsThreads;
     const unsigned g = (unsigned)std::min<long long>(std::max<long long>((items + per - 1) / per, 1), (long long)device_sms() * 64);
     if (d.digest) {
       switch (d.lc) {
@@ -1480,9 +1473,9 @@ cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
         default: eri3c_ps_kernel<4><<<g, kPsThreads, 0, st>>>(d); break;
       }
     }
-  } else if (d.digest == 1 && d.la == 0 && d.lb == 0 && d.orient == 0 && d.tiles) {
-    // (s s|C) DF-J: one warp per tile
-    const long long nb = (d.ntiles + kSsThreads / 32 - 1) / (kSsThreads / 32);
+  } else if (d.digest == 1 && d.la == 0 && d.lb == 0 && d.orient == 0 && d.wtiles) {
+    // (s s|C) DF-J
+    const long long per = kSsThreads / d.warpW, nb = (d.nwtiles + per - 1) / per;
     const unsigned g = (unsigned)std::min<long long>(std::max<long long>(nb, 1), (long long)device_sms() * 32);
     switch (d.lc) {
       case 0: eri3c_ss_dfj_kernel<0><<<g, kSsThreads, 0, st>>>(d); break;

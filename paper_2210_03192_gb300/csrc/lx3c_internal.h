@@ -114,6 +114,11 @@ struct ClassDesc {
   // optional explicit tile table {sub-pair, first ket-list entry, ket count, 0};
   // when null, tiles are (sub-pair, T consecutive ket shells) over all naux
   const int4* tiles;
+  // the register-resident DF-J kernels' tiles: as above but at most warpW (a
+  // power of two up to 32) kets each, 32 / warpW of them side by side in a warp
+  const int4* wtiles;
+  long long nwtiles;
+  int warpW;
   // DF-J digestion instead of the store (Sec. 3: integral digestion callable):
   //   gamma[aux_ao[q] + C] += w * sum_AB I[A][B][C] D[ao_a + A][ao_b + B]
   //   J[ao_a + A][ao_b + B] += wj * sum_{q,C} I[A][B][C] c[aux_ao[q] + C]

@@ -75,3 +75,20 @@ def test_gradient(lx, name):
     G = plan.gradient(torch.tensor(D, device="cuda"), torch.tensor(c, device="cuda")).cpu().numpy()
     Go = oracle.dfj_grad(orb, aux, D, c, plan.natom, tasks=plan.tasks(), mode="quad")
     assert np.abs(G - Go).max() <= 1e-11 * np.abs(Go).max()
+
+
+@pytest.mark.parametrize("count", [1, 2, 3, 5, 17, 31, 32, 33, 65])
+def test_register_kernels_ket_widths(lx, count):
+    """(s s|C) and (p s|C) ket lists of every width that shares a warp, the
+    last group of a launch partly empty, primitives of unequal number."""
+    rng = np.random.default_rng(100 + count)
+    coords = np.array([[0.0, 0.0, 0.0], [1.7, 0.4, -0.6], [-0.9, 1.5, 3.0]])
+    orb = shells(rng, [(0, 3, 1), (0, 2, 3), (1, 2, 2), (1, 1, 1)], coords, 0.1, 300.0)
+    aux = shells(rng, [(0, count, 1), (2, count, 1), (3, 1, 2), (6, 2, 1)], coords, 0.1, 300.0)
+    n, na = int(oracle.ao_offsets(orb)[-1]), int(oracle.ao_offsets(aux)[-1])
+    D, c = W.density(rng, n), rng.standard_normal(na)
+    plan = lx.DFJPlan(orb, aux, 1e-10)
+    g, J = (x.cpu().numpy() for x in plan.execute(torch.tensor(D, device="cuda"), torch.tensor(c, device="cuda")))
+    go, Jo = oracle.dfj(orb, aux, D, c, tasks=plan.tasks(), mode="quad")
+    assert np.abs(g - go).max() <= 1e-12 * np.abs(go).max()
+    assert np.abs(J - Jo).max() <= 1e-12 * np.abs(Jo).max()
