@@ -39,6 +39,7 @@
 #include "boys_device.cuh"
 #include "fixed128.cuh"
 #include "hermite.h"
+#include "hermite_device.cuh"
 #include "primitives.h"
 
 namespace lx3c {
@@ -46,72 +47,6 @@ namespace lx3c {
 namespace {
 
 __constant__ double c_int[16] = {0., 1., 2., 3., 4., 5., 6., 7., 8., 9., 10., 11., 12., 13., 14., 15.};
-
-constexpr int kMaxDeg = 13;  // Hermite degrees 0..13 (la + lb <= 12, one more for the gradient)
-constexpr unsigned kLast = 0x80000000u;
-constexpr int kColBytes = 32 * 8;  // one column: a double per lane
-
-__host__ __device__ constexpr int nherm(int L) { return (L + 1) * (L + 2) * (L + 3) / 6; }
-// position of (x, y, z) in the graded Hermite order
-__host__ __device__ inline int hidx(int x, int y, int z) {
-  const int n = x + y + z, m = y + z;
-  return n * (n + 1) * (n + 2) / 6 + m * (m + 1) / 2 + z;
-}
-
-// A list of outputs, each a sum of products of two columns.  Four queues of
-// outputs run side by side, balanced in length: a batch is one term of each
-// queue, the two factors as byte offsets in a and b; the sign bit of a queue's
-// b closes its output, whose header word (destination byte offset | palette id
-// of its scale factor << 20; for y rows Hermite index | axes << 16) is the next
-// of h.  The queues' ragged ends multiply the zero column.
-// Each warp of the block has queues of its own: nb + 1 batches and hs headers
-// on from the one before.
-struct Stage {
-  const uint4* a;
-  const uint4* b;
-  const unsigned* h;
-  int nb;  // even
-  int hs;
-};
-
-struct HermCls {
-  int nw;  // warps per block
-  int Lab, lc, Kc, L, nR, nY, ncc, nC, W, nket;
-  int cX, cPW, cU, cB, cCP, cGA;  // column offsets (R at column 0)
-  int cZero, cH;          // the zero column; the primitive pairs' densities
-  int rbeg[kMaxDeg + 2];  // R recursion: operations of level m at rops[rbeg[m]] ...
-  const uint4* rops;
-  Stage Z, gz, gy, gx;    // gamma: Z_u, then the shift's transpose along z, y, x
-  Stage jx, jy, jw;       // J: the shift of q along x, y, z
-  Stage Y;                // y_a
-  const int* cptr;        // Cartesian c -> (C, T_Cc c!) and its transpose
-  const int2* cent;
-  const int* gptr;
-  const int2* gent;
-  const double* pal;
-  const int* ydeg;        // degree of Hermite index a
-  double boys_cL;
-  // data
-  const double* prim;     // [nprim][8]: gamma, P, 1/(2 gamma), K_ab
-  const int* primpair;    // primitive -> pair position
-  const int* cnt;         // kets kept by each pair
-  const double* H;        // [nprim][nR], gradient: [nprim][3][nY]
-  unsigned long long* Yacc;
-  const double* auxrec;   // [nket][Kc][2]
-  const double* auxc;     // [nket][3]
-  const int* aux_ao;
-  const int* aux_atom;
-};
-
-struct HermArgs {
-  const HermCls* cls;
-  const int4* tiles;  // {class, first ket, first primitive, primitives}
-  const double* boys_tab;
-  const double* boys_mid;
-  const double* cvec;
-  unsigned long long* gacc;
-  unsigned long long* facc;
-};
 
 __device__ __forceinline__ double lds(const char* base, unsigned off) { return *(const double*)(base + off); }
 __device__ __forceinline__ void sts(char* base, unsigned off, double v) { *(double*)(base + off) = v; }
@@ -351,35 +286,7 @@ __global__ void __launch_bounds__(32 * kNW, 16 / kNW) herm_kernel(const __grid_c
         const double* Hf = kF ? c.H + 3LL * prim * c.nY : nullptr;
         int row = 0, amine = 0;
         const auto drain = [&]() {
-          __syncwarp();
-          const int lg = row > 16 ? 0 : (row > 8 ? 1 : (row > 4 ? 2 : (row > 2 ? 3 : (row > 1 ? 4 : 5))));
-          const int w = 32 >> lg, r = lane >> lg, part = lane & ((1 << lg) - 1);
-          const int a = __shfl_sync(0xffffffffu, amine, r);
-          const int seg = min(w, W);  // kets summed by this lane for one primitive pair
-          const double* x = stg + r * 33 + part * w;
-          for (int s0 = 0; s0 < w; s0 += seg) {
-            double v0 = 0.0, v1 = 0.0;
-            if (r < row) {
-              int i = 0;
-              for (; i + 1 < seg; i += 2) {
-                v0 += x[s0 + i];
-                v1 += x[s0 + i + 1];
-              }
-              if (i < seg) v0 += x[s0 + i];
-            }
-            double v = seg > 1 ? v0 + v1 : v0;
-            for (int o = 1; o * w < W; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            const int at = part * w + s0, s = at / W;
-            if (r < row && at == s * W && e0 + s < tile.w) {
-              const int ps = tile.z + e0 + s;
-              const double* prs = c.prim + 8LL * ps;
-              v *= __ldg(prs + 5);
-              const double h = __ldg(prs + 4);
-              for (int k = __ldg(c.ydeg + a); k > 0; --k) v *= h;
-              fix_add(c.Yacc + kFixWords * ((long long)ps * c.nY + a), v);
-            }
-          }
-          __syncwarp();
+          sum_rows(c, stg, row, tile, e0, lane, [&](int r) { return __shfl_sync(0xffffffffu, amine, r); });
           row = 0;
         };
         run_stage(c.Y, warp, cb, cb, [&](unsigned h, double v) {
@@ -1078,7 +985,7 @@ struct HermPlan {
   bool grad = false;
   long long nao = 0, npair = 0, nprim = 0;
   struct Tier {
-    int smem, nw;
+    int smem, nw, Lab;  // nw = 0: the unrolled kernel of this Lab
     long long first, n;
   };
   std::vector<Tier> tiers;
@@ -1113,6 +1020,10 @@ double herm_flops(const HermPlan* p) { return p->flops; }
 double herm_max_adds(const HermPlan* p) { return p->max_adds; }
 
 double herm_class_flops(int Lab, int lc) {
+  if (herm_unrolled(Lab, lc)) {
+    const UnrolledCost u = herm_unrolled_cost(Lab, lc);
+    return 2.0 * (u.base + u.gamma + u.j);
+  }
   const Program& p = program(Lab, lc, 1);
   return 2.0 * (p.instr_base + p.instr_gamma + p.instr_j);
 }
@@ -1249,8 +1160,9 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       // 105 -> 109 and 122 ms; one warp throughout: 110 ms)
       const Program& p1 = program(Lp, k.lc, 1);
       const int fit = kSmemSm / ((grad ? p1.ncol_grad : p1.ncol) * kColBytes + 2048);
-      const int nw = fit >= 8 ? 1 : (fit >= 4 ? 2 : 4);
-      const Program& pg = program(Lp, k.lc, nw);
+      const bool unr = herm_unrolled(Lp, k.lc);
+      const int nw = unr ? 0 : (fit >= 8 ? 1 : (fit >= 4 ? 2 : 4));  // 0: the unrolled kernel
+      const Program& pg = program(Lp, k.lc, std::max(nw, 1));
       HermCls& c = x.c;
       std::memset(&c, 0, sizeof(c));
       c.nw = nw;
@@ -1261,7 +1173,9 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       c.cH = grad ? pg.ncol_grad : pg.ncol;
       for (int m = 0; m < kMaxDeg + 2; ++m) c.rbeg[m] = pg.rbeg[m];
       c.boys_cL = boys_large_const(c.L);
-      x.instr = (pg.instr_base + pg.instr_j + (grad ? 3.0 * pg.nR : pg.instr_gamma)) * k.Kc;
+      const UnrolledCost uc = unr ? herm_unrolled_cost(Lp, k.lc)
+                                  : UnrolledCost{pg.instr_base, pg.instr_gamma, pg.instr_j};
+      x.instr = (uc.base + uc.j + (grad ? 3.0 * pg.nR : uc.gamma)) * k.Kc;
       // W kets side by side: the widest power of two whose ragged end wastes
       // least (narrower tiles pay one more y row sum per primitive pair)
       double best = 1e300;
@@ -1272,7 +1186,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
         const double cost = slots * (1.0 + 0.02 * (32 / W - 1));
         if (cost < best * 0.999) { best = cost; c.W = W; }
       }
-      x.smem = c.cH * kColBytes + (grad ? 0 : 32 / c.W * pg.nR * 8);
+      x.smem = unr ? herm_unrolled_smem(Lp, k.lc, c.W) : c.cH * kColBytes + (grad ? 0 : 32 / c.W * pg.nR * 8);
       if (x.smem > kSmemCta) {
         set_last_error("dfj: Hermite class does not fit in shared memory");
         return LX3C_ENOTSUP;
@@ -1286,10 +1200,11 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
         std::memcpy(x.st, f.st, sizeof(x.st));
       } else {
         first_of[key] = (int)cls.size();
-        x.rops = blob.add(pg.rops); x.cptr = blob.add(pg.cptr); x.cent = blob.add(pg.cent); x.gptr = blob.add(pg.gptr);
+        x.rops = unr ? 0 : blob.add(pg.rops); x.cptr = blob.add(pg.cptr); x.cent = blob.add(pg.cent); x.gptr = blob.add(pg.gptr);
         x.gent = blob.add(pg.gent); x.pal = blob.add(pg.pal); x.ydeg = blob.add(pg.ydeg);
         const HostStage* hs[8] = {&pg.Z, &pg.gz, &pg.gy, &pg.gx, &pg.jx, &pg.jy, &pg.jw, &pg.Y};
-        for (int s = 0; s < 8; ++s) {
+        std::memset(x.st, 0, sizeof(x.st));
+        for (int s = 0; s < 8 && !unr; ++s) {
           x.st[s][0] = blob.add(hs[s]->a);
           x.st[s][1] = blob.add(hs[s]->b);
           x.st[s][2] = blob.add(hs[s]->h);
@@ -1317,6 +1232,8 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   // footprint first
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
     if (cls[a].c.nw != cls[b].c.nw) return cls[a].c.nw > cls[b].c.nw;
+    if (!cls[a].c.nw)
+      return cls[a].c.Lab != cls[b].c.Lab ? cls[a].c.Lab > cls[b].c.Lab : cls[a].instr > cls[b].instr;
     const int oa = occ(cls[a].smem), ob = occ(cls[b].smem);
     return oa != ob ? oa < ob : cls[a].instr > cls[b].instr;
   });
@@ -1328,9 +1245,10 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     ClsHost& x = cls[ci];
     const LabHost& L = labs[x.lab];
     int b = 0;
-    while (b + 1 < 10 && bins[b + 1] <= occ(x.smem)) ++b;
+    while (x.c.nw && b + 1 < 10 && bins[b + 1] <= occ(x.smem)) ++b;
+    if (!x.c.nw) b = 100 + x.c.Lab;  // one launch per Lab
     if (b != bin || p->tiers.back().nw != x.c.nw) {
-      p->tiers.push_back(HermPlan::Tier{0, x.c.nw, (long long)tiles.size(), 0});
+      p->tiers.push_back(HermPlan::Tier{0, x.c.nw, x.c.Lab, (long long)tiles.size(), 0});
       bin = b;
     }
     HermPlan::Tier& t = p->tiers.back();
@@ -1468,6 +1386,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   ma.boys_mid = dev_boys_mid(ds);
   cudaError_t e = cudaMemcpyAsync(A, blob.d.data(), blob.d.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = herm_unrolled_setup();
   const void* kernels[] = {(const void*)herm_kernel<1, 1>, (const void*)herm_kernel<1, 2>, (const void*)herm_kernel<1, 4>,
                            (const void*)herm_kernel<2, 1>, (const void*)herm_kernel<2, 2>, (const void*)herm_kernel<2, 4>,
                            (const void*)herm_kernel<3, 1>, (const void*)herm_kernel<3, 2>, (const void*)herm_kernel<3, 4>,
@@ -1508,7 +1427,10 @@ template <int kMode>
 cudaError_t herm_tiles(HermPlan* p, HermArgs a, cudaStream_t st) {
   for (auto& t : p->tiers) {
     a.tiles = p->ma.tiles + t.first;
-    if (t.nw == 1) herm_kernel<kMode, 1><<<(unsigned)t.n, 32, t.smem, st>>>(a);
+    if (t.nw == 0) {
+      const cudaError_t e = launch_herm_unrolled(t.Lab, a, kMode, t.smem, t.n, st);
+      if (e != cudaSuccess) return e;
+    } else if (t.nw == 1) herm_kernel<kMode, 1><<<(unsigned)t.n, 32, t.smem, st>>>(a);
     else if (t.nw == 2) herm_kernel<kMode, 2><<<(unsigned)t.n, 64, t.smem, st>>>(a);
     else herm_kernel<kMode, 4><<<(unsigned)t.n, 128, t.smem, st>>>(a);
   }

@@ -92,3 +92,28 @@ def test_register_kernels_ket_widths(lx, count):
     go, Jo = oracle.dfj(orb, aux, D, c, tasks=plan.tasks(), mode="quad")
     assert np.abs(g - go).max() <= 1e-12 * np.abs(go).max()
     assert np.abs(J - Jo).max() <= 1e-12 * np.abs(Jo).max()
+
+
+@pytest.mark.parametrize("lc", range(6))
+@pytest.mark.parametrize("la,lb", [(1, 1), (2, 1), (2, 2), (3, 2), (3, 3)])
+def test_unrolled_classes(lx, la, lb, lc):
+    """Every class of the unrolled kernel, and its neighbours on the table
+    kernel: one shell more than half a tile, contracted and plain kets, values
+    and gradient."""
+    rng = np.random.default_rng(1000 + 100 * la + 10 * lb + lc)
+    coords = np.array([[0.0, 0.0, 0.0], [1.7, 0.4, -0.6], [-0.9, 1.5, 3.0]])
+    orb = shells(rng, [(la, 1, 2), (lb, 2, 1)], coords, 0.1, 100.0)
+    aux = shells(rng, [(lc, 17, 1), (lc, 2, 2)], coords, 0.1, 100.0)
+    n, na = int(oracle.ao_offsets(orb)[-1]), int(oracle.ao_offsets(aux)[-1])
+    D, c = W.density(rng, n), rng.standard_normal(na)
+    Dt, ct = torch.tensor(D, device="cuda"), torch.tensor(c, device="cuda")
+    plan = lx.DFJPlan(orb, aux, 1e-10, gradient=True)
+    g, J = plan.execute(Dt, ct)
+    go, Jo = oracle.dfj(orb, aux, D, c, tasks=plan.tasks(), mode="quad")
+    assert np.abs(g.cpu().numpy() - go).max() <= 1e-12 * np.abs(go).max()
+    assert np.abs(J.cpu().numpy() - Jo).max() <= 1e-12 * np.abs(Jo).max()
+    assert torch.equal(plan.execute(Dt, ct, outputs="gamma")[0], g)
+    assert torch.equal(plan.execute(Dt, ct, outputs="J")[1], J)
+    G = plan.gradient(Dt, ct).cpu().numpy()
+    Go = oracle.dfj_grad(orb, aux, D, c, plan.natom, tasks=plan.tasks(), mode="quad")
+    assert np.abs(G - Go).max() <= 1e-11 * np.abs(Go).max()
