@@ -112,11 +112,17 @@ __device__ __forceinline__ void sum_rows(const HermCls& c, const double* stg, in
   __syncwarp();
 }
 
-// Classes (Lab, lc) of the unrolled kernel.
-constexpr int kUnrollLab0 = 2, kUnrollLab1 = 4;
-inline bool herm_unrolled(int Lab, int lc) {
-  return Lab >= kUnrollLab0 && Lab <= kUnrollLab1 && lc <= (Lab == 4 ? 4 : 5);
+// Classes (Lab, lc) of the unrolled kernel: up to degree 6, as far as the
+// shared-memory columns let five or more one-warp blocks onto an SM.  (l s|C)
+// classes below lc = 5 belong to the register kernels of eri3c.cu.
+__host__ __device__ constexpr bool herm_unrolled(int Lab, int lc) {
+  return lc <= 6 && (Lab == 1 ? lc >= 5 : Lab >= 2 && Lab <= 6 && lc <= (Lab < 5 ? 6 : 5));
 }
+__host__ __device__ constexpr bool unrolled_m_shared(int Lab, int lc) { return Lab >= 5 || lc == 6 || Lab + lc >= 9; }
+template <int Lab>
+cudaError_t herm_unrolled_setup();
+template <int Lab>
+cudaError_t herm_unrolled_launch(const HermArgs& a, int mode, int smem, long long n, cudaStream_t st);
 struct UnrolledCost {
   double base, gamma, j;  // FP64 instructions per primitive triple
 };

@@ -94,8 +94,8 @@ def test_register_kernels_ket_widths(lx, count):
     assert np.abs(J - Jo).max() <= 1e-12 * np.abs(Jo).max()
 
 
-@pytest.mark.parametrize("lc", range(6))
-@pytest.mark.parametrize("la,lb", [(1, 1), (2, 1), (2, 2), (3, 2), (3, 3)])
+@pytest.mark.parametrize("lc", range(7))
+@pytest.mark.parametrize("la,lb", [(1, 0), (1, 1), (2, 1), (2, 2), (3, 2), (3, 3)])
 def test_unrolled_classes(lx, la, lb, lc):
     """Every class of the unrolled kernel, and its neighbours on the table
     kernel: one shell more than half a tile, contracted and plain kets, values
