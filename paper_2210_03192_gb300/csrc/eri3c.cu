@@ -1017,12 +1017,43 @@ __global__ void __launch_bounds__(kSsThreads) eri3c_ss_kernel(const __grid_const
   }
 }
 
+// Sums js[k] over the W lanes of a tile for eight densities: while there are
+// values left to share, each step hands half of them to the other half of the
+// lanes (nine additions instead of 40 for W = 32); then adds w times each sum to
+// its density's J element.
+__device__ __forceinline__ void multi_j(const ClassDesc& d, double (&js)[8], int W, int t, bool store, double w,
+                                        long long elem) {
+  int first = 0, left = 8, o = W >> 1;
+#pragma unroll
+  for (int n = 4; n > 0; n >>= 1) {
+    if (o > 0) {
+      const bool up = (t & o) != 0;
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        const double other = __shfl_xor_sync(0xffffffffu, up ? js[k] : js[k + n], o);
+        js[k] = (up ? js[k + n] : js[k]) + other;
+      }
+      first += up ? n : 0;
+      left = n;
+      o >>= 1;
+    }
+  }
+  const int rest = (o << 1) - 1;  // lanes below this mask hold partial sums of one density
+  for (; o > 0; o >>= 1) js[0] += __shfl_xor_sync(0xffffffffu, js[0], o);
+  if (store && (rest <= 0 || (t & rest) == 0)) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < left && first + k < d.nd) atomicAdd(d.J + (first + k) * d.dstride + elem, w * js[k]);
+  }
+}
+
 // (s s|C) DF-J launches digesting per integral (digest == 1), lanes over the
 // kets of 32 / warpW tiles: gamma_P[C] += w D_ab (ss|P)_C per lane,
 // and J_ab += w_J sum over the tile's kets and C of (ss|P)_C c_PC, reduced
 // across the tile's lanes into one add.  The same sums as the tile kernel's
-// digest.
-template <int LC>
+// digest.  kMulti: up to eight densities (digest == 4), the integrals formed
+// once; gamma and J by FP64 atomics as in the tile kernel.
+template <int LC, bool kMulti>
 __global__ void __launch_bounds__(kSsThreads) eri3c_ss_dfj_kernel(const __grid_constant__ ClassDesc d) {
   constexpr int NC = (LC + 1) * (LC + 2) / 2, NS = 2 * LC + 1;
   __shared__ double sP[kSsThreads * (NC + 1)];
@@ -1036,8 +1067,13 @@ __global__ void __launch_bounds__(kSsThreads) eri3c_ss_dfj_kernel(const __grid_c
     const long long pair = sp.x;
     const int4 pao = __ldg(d.pair_ao + pair);
     const double wg = pao.z ? 1.0 : 2.0, wj = pao.z ? 0.5 : 1.0;
-    const double Dab = d.gacc ? __ldg(d.D + (long long)pao.x * d.ldD + pao.y) : 0.0;
+    const long long elem = (long long)pao.x * d.ldD + pao.y;
+    const double Dab = !kMulti && d.gacc ? __ldg(d.D + elem) : 0.0;
     double jsum = 0.0;
+    double js[8];
+    if (kMulti)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) js[k] = 0.0;
     const bool live = t < tt.z;
     double acc[NC];
 #pragma unroll
@@ -1055,13 +1091,24 @@ __global__ void __launch_bounds__(kSsThreads) eri3c_ss_dfj_kernel(const __grid_c
           const int2 e = __ldg(d.kent + k);
           v = fma(__ldg(d.pal + e.y), row[e.x], v);
         }
+        if (kMulti) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            if (k >= d.nd) break;
+            if (d.gamma) atomicAdd(d.gamma + k * d.cstride + ao + C, wg * v * __ldg(d.D + k * d.dstride + elem));
+            if (d.J) js[k] = fma(v, __ldg(d.cvec + k * d.cstride + ao + C), js[k]);
+          }
+          continue;
+        }
         if (d.gacc) fix_add(d.gacc + kFixWords * (ao + C), wg * Dab * v);
         if (d.Jacc) jsum = fma(v, __ldg(d.cvec + ao + C), jsum);
       }
     }
-    if (d.Jacc) {
+    if (kMulti) {
+      if (d.J) multi_j(d, js, W, t, tt.z > 0, wj, elem);
+    } else if (d.Jacc) {
       for (int o = W >> 1; o > 0; o >>= 1) jsum += __shfl_xor_sync(0xffffffffu, jsum, o);
-      if (t == 0 && tt.z) fix_add(d.Jacc + kFixWords * ((long long)pao.x * d.ldD + pao.y), wj * jsum);
+      if (t == 0 && tt.z) fix_add(d.Jacc + kFixWords * elem, wj * jsum);
     }
   }
 }
@@ -1252,7 +1299,7 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_kernel(const __grid_const
 // its kets; gamma_P[C] += w sum_s D_s (ps|P)_{sC} per lane and
 // J_s += w_J sum over the tile's kets and C of (ps|P)_{sC} c_PC, reduced
 // across the warp.
-template <int LC>
+template <int LC, bool kMulti>
 __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_constant__ ClassDesc d) {
   constexpr int NC = (LC + 1) * (LC + 2) / 2, NS = 2 * LC + 1, NB = 3 * NS;
   constexpr int NCM = LC > 0 ? LC * (LC + 1) / 2 : 1;
@@ -1269,12 +1316,15 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
     const long long pair = sp.x;
     const int4 pao = __ldg(d.pair_ao + pair);
     const double wg = pao.z ? 1.0 : 2.0, wj = pao.z ? 0.5 : 1.0;
+    const long long elem = (long long)pao.x * d.ldD + pao.y, step = d.orient ? 1 : d.ldD;
     double Ds[3] = {0.0, 0.0, 0.0};
-    if (d.gacc)
+    if (!kMulti && d.gacc)
 #pragma unroll
-      for (int s = 0; s < 3; ++s)
-        Ds[s] = d.orient ? __ldg(d.D + (long long)pao.x * d.ldD + pao.y + s)
-                         : __ldg(d.D + (long long)(pao.x + s) * d.ldD + pao.y);
+      for (int s = 0; s < 3; ++s) Ds[s] = __ldg(d.D + elem + s * step);
+    double jm[3][8];
+    if (kMulti)
+#pragma unroll
+      for (int k = 0; k < 24; ++k) jm[k >> 3][k & 7] = 0.0;
     double js[3] = {0.0, 0.0, 0.0};
     if (t < tt.z) {
       const long long q = tt.y + t;
@@ -1287,6 +1337,26 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
       ps_targets<LC>(A, Bm, row);
       ps_transform<LC>(d, row, out);
       const int ao = __ldg(d.aux_ao + q);
+      if (kMulti) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (k >= d.nd) break;
+          const double* D = d.D + k * d.dstride + elem;
+          double D0 = 0.0, D1 = 0.0, D2 = 0.0;
+          if (d.gamma) { D0 = __ldg(D); D1 = __ldg(D + step); D2 = __ldg(D + 2 * step); }
+#pragma unroll
+          for (int C = 0; C < NS; ++C) {
+            const double i0 = out[C], i1 = out[NS + C], i2 = out[2 * NS + C];
+            if (d.gamma) atomicAdd(d.gamma + k * d.cstride + ao + C, wg * fma(D0, i0, fma(D1, i1, D2 * i2)));
+            if (d.J) {
+              const double cv = __ldg(d.cvec + k * d.cstride + ao + C);
+              jm[0][k] = fma(i0, cv, jm[0][k]);
+              jm[1][k] = fma(i1, cv, jm[1][k]);
+              jm[2][k] = fma(i2, cv, jm[2][k]);
+            }
+          }
+        }
+      } else
 #pragma unroll
       for (int C = 0; C < NS; ++C) {
         const double i0 = out[C], i1 = out[NS + C], i2 = out[2 * NS + C];
@@ -1299,14 +1369,17 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_c
         }
       }
     }
-    if (d.Jacc) {
+    if (kMulti) {
+      if (d.J)
+#pragma unroll
+        for (int s = 0; s < 3; ++s) multi_j(d, jm[s], W, t, tt.z > 0, wj, elem + s * step);
+    } else if (d.Jacc) {
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
         double v = js[s];
         for (int o = W >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (t == 0 && tt.z) {
-          const long long e = d.orient ? (long long)pao.x * d.ldD + pao.y + s : (long long)(pao.x + s) * d.ldD + pao.y;
-          fix_add(d.Jacc + kFixWords * e, wj * v);
+          fix_add(d.Jacc + kFixWords * (elem + s * step), wj * v);
         }
       }
     }
@@ -1412,11 +1485,30 @@ static cudaError_t tile_kernel_attributes() {
   return rc;
 }
 
-// Whether a launch runs the tile kernel (not a register-resident one).
-static bool on_tile_kernel(const ClassDesc& d) {
-  if (d.digest == 4) return true;
-  if (d.la == 0 && d.lb == 0 && d.orient == 0 && (d.digest == 0 || (d.digest == 1 && d.wtiles))) return false;
-  return !((d.digest == 0 || (d.digest == 1 && d.wtiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 && (d.lc > 0 || d.K > 1));
+// Whether a launch runs on a register-resident kernel: (s s|C), or (p s|C) and
+// B-oriented (s p|C) (whose descriptor holds the (p s|C) tables with orient =
+// 1) with 1 <= lc <= 4 or contracted; (p s|s) with one primitive per triple
+// measured faster on the tile kernel.  Stores and per-integral DF-J, for one
+// density or several, the latter with the kernels' own tiles (several densities
+// on 16 atoms: these classes 9.3 of 26.3 ms on the tile kernel).
+static bool on_register_kernel(const ClassDesc& d) {
+  if (d.digest != 0 && !((d.digest == 1 || d.digest == 4) && d.wtiles)) return false;
+  if (d.la == 0 && d.lb == 0) return d.orient == 0;
+  return d.la == 1 && d.lb == 0 && d.lc <= 4 && (d.lc > 0 || d.K > 1);
+}
+static bool on_tile_kernel(const ClassDesc& d) { return !on_register_kernel(d); }
+
+template <int LC>
+static void launch_ss(const ClassDesc& d, unsigned g, cudaStream_t st) {
+  if (d.digest == 0) eri3c_ss_kernel<LC><<<g, kSsThreads, 0, st>>>(d);
+  else if (d.digest == 1) eri3c_ss_dfj_kernel<LC, false><<<g, kSsThreads, 0, st>>>(d);
+  else eri3c_ss_dfj_kernel<LC, true><<<g, kSsThreads, 0, st>>>(d);
+}
+template <int LC>
+static void launch_ps(const ClassDesc& d, unsigned g, cudaStream_t st) {
+  if (d.digest == 0) eri3c_ps_kernel<LC><<<g, kPsThreads, 0, st>>>(d);
+  else if (d.digest == 1) eri3c_ps_dfj_kernel<LC, false><<<g, kPsThreads, 0, st>>>(d);
+  else eri3c_ps_dfj_kernel<LC, true><<<g, kPsThreads, 0, st>>>(d);
 }
 
 bool can_launch_both(const ClassDesc& a, const ClassDesc& b) {
@@ -1434,57 +1526,30 @@ cudaError_t launch_eri3c_both(const ClassDesc& a, int ga, const ClassDesc& b, in
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
   cudaError_t e = tile_kernel_attributes();
   if (e != cudaSuccess) return e;
-  if (d.digest == 0 && d.la == 0 && d.lb == 0 && d.orient == 0) {
-    // (s s|C): the register-resident form, one thread per triple
-    const long long nb = (d.nsub * d.naux + kSsThreads - 1) / kSsThreads;
-    const unsigned g = (unsigned)std::min<long long>(std::max<long long>(nb, 1), (long long)device_sms() * 32);
-    switch (d.lc) {
-      case 0: eri3c_ss_kernel<0><<<g, kSsThreads, 0, st>>>(d); break;
-      case 1: eri3c_ss_kernel<1><<<g, kSsThreads, 0, st>>>(d); break;
-      case 2: eri3c_ss_kernel<2><<<g, kSsThreads, 0, st>>>(d); break;
-      case 3: eri3c_ss_kernel<3><<<g, kSsThreads, 0, st>>>(d); break;
-      case 4: eri3c_ss_kernel<4><<<g, kSsThreads, 0, st>>>(d); break;
-      case 5: eri3c_ss_kernel<5><<<g, kSsThreads, 0, st>>>(d); break;
-      default: eri3c_ss_kernel<6><<<g, kSsThreads, 0, st>>>(d); break;
-    }
-  } else if ((d.digest == 0 || (d.digest == 1 && d.wtiles)) && d.la == 1 && d.lb == 0 && d.lc <= 4 &&
-             (d.lc > 0 || d.K > 1)) {
-    // (p s|C) and B-oriented (s p|C) (whose descriptor holds the (p s|C)
-    // tables with orient = 1), 1 <= lc <= 4 or contracted: register-resident.
-    // (p s|s) with one primitive per triple stays on the tile kernel, which
-    // measured faster there.
+  if (on_register_kernel(d)) {
+    const int threads = d.la ? kPsThreads : kSsThreads;
     const long long items = d.digest ? d.nwtiles : d.nsub * d.naux;
-    const long long per = d.digest ? kPsThreads / d.warpW : kPsThreads;
-    const unsigned g = (unsigned)std::min<long long>(std::max<long long>((items + per - 1) / per, 1), (long long)device_sms() * 64);
-    if (d.digest) {
+    const long long per = d.digest ? threads / d.warpW : threads;
+    const unsigned g = (unsigned)std::min<long long>(std::max<long long>((items + per - 1) / per, 1),
+                                                     (long long)device_sms() * (d.la ? 64 : 32));
+    if (d.la == 0) {
       switch (d.lc) {
-        case 0: eri3c_ps_dfj_kernel<0><<<g, kPsThreads, 0, st>>>(d); break;
-        case 1: eri3c_ps_dfj_kernel<1><<<g, kPsThreads, 0, st>>>(d); break;
-        case 2: eri3c_ps_dfj_kernel<2><<<g, kPsThreads, 0, st>>>(d); break;
-        case 3: eri3c_ps_dfj_kernel<3><<<g, kPsThreads, 0, st>>>(d); break;
-        default: eri3c_ps_dfj_kernel<4><<<g, kPsThreads, 0, st>>>(d); break;
+        case 0: launch_ss<0>(d, g, st); break;
+        case 1: launch_ss<1>(d, g, st); break;
+        case 2: launch_ss<2>(d, g, st); break;
+        case 3: launch_ss<3>(d, g, st); break;
+        case 4: launch_ss<4>(d, g, st); break;
+        case 5: launch_ss<5>(d, g, st); break;
+        default: launch_ss<6>(d, g, st); break;
       }
     } else {
       switch (d.lc) {
-        case 0: eri3c_ps_kernel<0><<<g, kPsThreads, 0, st>>>(d); break;
-        case 1: eri3c_ps_kernel<1><<<g, kPsThreads, 0, st>>>(d); break;
-        case 2: eri3c_ps_kernel<2><<<g, kPsThreads, 0, st>>>(d); break;
-        case 3: eri3c_ps_kernel<3><<<g, kPsThreads, 0, st>>>(d); break;
-        default: eri3c_ps_kernel<4><<<g, kPsThreads, 0, st>>>(d); break;
+        case 0: launch_ps<0>(d, g, st); break;
+        case 1: launch_ps<1>(d, g, st); break;
+        case 2: launch_ps<2>(d, g, st); break;
+        case 3: launch_ps<3>(d, g, st); break;
+        default: launch_ps<4>(d, g, st); break;
       }
-    }
-  } else if (d.digest == 1 && d.la == 0 && d.lb == 0 && d.orient == 0 && d.wtiles) {
-    // (s s|C) DF-J
-    const long long per = kSsThreads / d.warpW, nb = (d.nwtiles + per - 1) / per;
-    const unsigned g = (unsigned)std::min<long long>(std::max<long long>(nb, 1), (long long)device_sms() * 32);
-    switch (d.lc) {
-      case 0: eri3c_ss_dfj_kernel<0><<<g, kSsThreads, 0, st>>>(d); break;
-      case 1: eri3c_ss_dfj_kernel<1><<<g, kSsThreads, 0, st>>>(d); break;
-      case 2: eri3c_ss_dfj_kernel<2><<<g, kSsThreads, 0, st>>>(d); break;
-      case 3: eri3c_ss_dfj_kernel<3><<<g, kSsThreads, 0, st>>>(d); break;
-      case 4: eri3c_ss_dfj_kernel<4><<<g, kSsThreads, 0, st>>>(d); break;
-      case 5: eri3c_ss_dfj_kernel<5><<<g, kSsThreads, 0, st>>>(d); break;
-      default: eri3c_ss_dfj_kernel<6><<<g, kSsThreads, 0, st>>>(d); break;
     }
   } else {
     const int smem = d.smem_doubles * 8;

@@ -117,3 +117,25 @@ def test_unrolled_classes(lx, la, lb, lc):
     G = plan.gradient(Dt, ct).cpu().numpy()
     Go = oracle.dfj_grad(orb, aux, D, c, plan.natom, tasks=plan.tasks(), mode="quad")
     assert np.abs(G - Go).max() <= 1e-11 * np.abs(Go).max()
+
+
+@pytest.mark.parametrize("nd", [1, 2, 3, 5, 8])
+@pytest.mark.parametrize("count", [1, 2, 3, 7, 16, 33])
+def test_register_kernels_several_densities(lx, count, nd):
+    """(s s|C) and (p s|C) for several densities at every width of a tile:
+    each density as by itself (1e-13, only the order of sums differs)."""
+    rng = np.random.default_rng(500 + 10 * count + nd)
+    coords = np.array([[0.0, 0.0, 0.0], [1.7, 0.4, -0.6], [-0.9, 1.5, 3.0]])
+    orb = shells(rng, [(0, 3, 1), (0, 2, 3), (1, 2, 2), (1, 1, 1)], coords, 0.1, 300.0)
+    aux = shells(rng, [(0, count, 1), (2, count, 1), (4, 1, 2), (6, 2, 1)], coords, 0.1, 300.0)
+    n, na = int(oracle.ao_offsets(orb)[-1]), int(oracle.ao_offsets(aux)[-1])
+    plan = lx.DFJPlan(orb, aux, 1e-10)
+    D = torch.tensor(np.stack([W.density(rng, n) for _ in range(nd)]), device="cuda")
+    c = torch.tensor(rng.standard_normal((nd, na)), device="cuda")
+    g, J = plan.execute_multi(D, c)
+    for k in range(nd):
+        g1, J1 = plan.execute(D[k].contiguous(), c[k].contiguous())
+        assert (g[k] - g1).abs().max() <= 1e-13 * g1.abs().max()
+        assert (J[k] - J1).abs().max() <= 1e-13 * J1.abs().max()
+    assert (plan.execute_multi(D, None, outputs="gamma")[0] - g).abs().max() <= 1e-13 * g.abs().max()
+    assert (plan.execute_multi(None, c, outputs="J")[1] - J).abs().max() <= 1e-13 * J.abs().max()
