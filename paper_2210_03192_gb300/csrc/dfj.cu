@@ -51,9 +51,8 @@ using namespace lx3c;
 namespace {
 
 // Ket-count bound for the shape chooser from the tile fill: the largest T
-// (a power of two up to 512) at which this launch's tiles hold at least 80%
-// screened triples, returned as T/2 (the chooser allows T up to twice the
-// count it is given), and never above the longest ket list.
+// (a power of two up to 512, at least 2) at which this launch's tiles hold at
+// least 80% screened triples, and never above the longest ket list.
 long long fill_bound(const std::vector<int4>& sub, const std::vector<int>& counts, int cmax) {
   long long tot = 0;
   for (auto& s : sub) tot += counts[s.x];

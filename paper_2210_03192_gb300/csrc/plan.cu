@@ -831,7 +831,9 @@ LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long n
   bool found = false;
   for (long long budget : budgets) {
     for (int T : Ts) {
-      if (T > 1 && T > 2 * naux && T != 1) continue;
+      // never a tile that half its size would hold ((pp|d) with 32 kets: T = 64
+      // 28.7 us a call, T = 32 26.7)
+      if (T > 1 && T >= 2 * naux) continue;
       int mode = T >= 32 ? 0 : 1;
       buffer_sizes(ct, Kab, Kc, T, 1, mode, s, nullptr);
       if (s.total > budget) continue;
