@@ -62,7 +62,7 @@ long long fill_bound(const std::vector<int4>& sub, const std::vector<int>& count
     for (auto& s : sub) slots += (long long)((counts[s.x] + T - 1) / T) * T;
     if (tot * 5 >= slots * 4) { pick = T; break; }
   }
-  return std::min<long long>(cmax, std::max(1, pick / 2));
+  return std::min<long long>(cmax, std::max(2, pick));
 }
 
 
@@ -275,6 +275,10 @@ struct lx3c_dfj {
   int natom = 0;
   bool gradient = false;
   std::vector<DfjGroup> groups;
+  // records of every group: the groups outside the Hermite basis first
+  PrecomputeJob* d_jobs = nullptr;
+  int njobs = 0, njobs_plain = 0;
+  long long job_blocks = 0, job_blocks_plain = 0;
   char* arena = nullptr;            // every device array of the groups, and the accumulators
   HermPlan* hj = nullptr;           // gamma and J of the Hermite groups
   HermPlan* hg = nullptr;           // gradient of every group
@@ -527,6 +531,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   arena.take(&p->d_gacc, (size_t)p->naux_ao * kFixWords);
   arena.take(&p->d_Jacc, (size_t)p->nao * p->nao * kFixWords);
   if (want_grad) arena.take(&p->d_facc, (size_t)p->natom * 3 * kFixWords);
+  arena.take(&p->d_jobs, p->groups.size());
   DCUDA(arena.commit(&p->arena, st));
   for (auto& g : p->groups)
     for (auto& L : g.L) {
@@ -536,8 +541,32 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       d.pairrec = g.d_pairrec; d.pairab = g.d_pairab; d.auxrec = g.d_auxrec; d.auxc = g.d_auxc;
       d.pair_ao = g.d_pair_ao; d.aux_ao = g.d_aux_ao;
     }
+  std::vector<PrecomputeJob> jobs;
+  for (int herm = 0; herm < 2; ++herm) {
+    for (auto& g : p->groups)
+      if ((int)g.herm == herm) {
+        jobs.push_back(PrecomputeJob{g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
+                                     g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, p->job_blocks});
+        p->job_blocks += jobs.back().blocks();
+      }
+    if (!herm) {
+      p->njobs_plain = (int)jobs.size();
+      p->job_blocks_plain = p->job_blocks;
+    }
+  }
+  p->njobs = (int)jobs.size();
+  if (!jobs.empty())
+    DCUDA(cudaMemcpyAsync(p->d_jobs, jobs.data(), jobs.size() * sizeof(PrecomputeJob), cudaMemcpyHostToDevice, st));
+  DCUDA(cudaStreamSynchronize(st));
   *out = p.release();
   return LX3C_OK;
+}
+
+// The pair and ket records of a plan's groups (all, or those that do not run in
+// the Hermite basis).
+static cudaError_t group_records(const lx3c_dfj* p, bool all, cudaStream_t st) {
+  return launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->d_jobs, all ? p->njobs : p->njobs_plain,
+                                all ? p->job_blocks : p->job_blocks_plain, st);
 }
 
 lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, double* gamma, double* J, void* stream) {
@@ -547,11 +576,9 @@ lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, doub
   if (gamma) DCUDA(cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, st));
   if (J) DCUDA(cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, st));
   if (p->hj) DCUDA(herm_execute(p->hj, D, c, gamma ? p->d_gacc : nullptr, J ? p->d_Jacc : nullptr, st));
+  DCUDA(group_records(p, false, st));
   for (auto& g : p->groups) {
     if (g.herm) continue;
-    const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
-    DCUDA(launch_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, p->aux->dev(), g.d_auxs,
-                            na, g.Kc, g.d_auxrec, g.d_auxc, st));
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       ClassDesc d = L.desc;
@@ -598,10 +625,8 @@ lx3c_status lx3c_dfj_execute_multi(lx3c_dfj* p, int nd, const double* D, const d
   if (gamma) DCUDA(cudaMemsetAsync(gamma, 0, (size_t)nd * cstride * 8, st));
   if (J) DCUDA(cudaMemsetAsync(J, 0, (size_t)nd * dstride * 8, st));
   size_t li = 0;
+  DCUDA(group_records(p, true, st));
   for (auto& g : p->groups) {
-    const long long np = (long long)g.counts.size(), na = (long long)g.auxs.size();
-    DCUDA(launch_precompute(p->orb->dev(), g.d_pairs, np, g.Ka, g.Kb, g.d_pairrec, g.d_pairab, p->aux->dev(), g.d_auxs,
-                            na, g.Kc, g.d_auxrec, g.d_auxc, st));
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       DCUDA(launch_eri3c(descs[li], grids[li], st));
@@ -661,8 +686,9 @@ lx3c_status lx3c_dfj_info(const lx3c_dfj* p, double* out, int n) {
     tasks += (double)g.ntasks;
     nint += g.nint;
     flops += g.flops;
-    if (!g.herm) launches += 1 + (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
+    if (!g.herm) launches += (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
   }
+  launches += p->njobs_plain > 0;
   const double v[] = {(double)p->groups.size(), tasks, nint, flops, launches, (double)p->nao, (double)p->naux_ao,
                       (double)p->natom, gflops, glaunches, slots};
   for (int i = 0; i < n && i < 11; ++i) out[i] = v[i];
@@ -796,12 +822,8 @@ cudaError_t capture_branches(lx3c_batch* b, const std::vector<ClassDesc>& descs,
       lx3c_dfj* p = b->mols[m];
       cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
       cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
-      for (auto& g : p->groups) {
-        if (g.herm) continue;
-        launch_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
-                          p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
-        ++kernels;
-      }
+      group_records(p, false, cap);
+      kernels += p->njobs_plain > 0;
     }
     cudaEventRecord(fork, cap);
     double load[kBranches] = {};
@@ -1005,10 +1027,9 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
   b->plain_launches = 0;
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];
-    b->plain_launches += 2 + (p->hj ? herm_launches(p->hj) : 0);
+    b->plain_launches += 2 + (p->njobs_plain > 0) + (p->hj ? herm_launches(p->hj) : 0);
     for (auto& g : p->groups) {
       if (g.herm) continue;
-      b->plain_launches += 1;
       for (auto& L : g.L) {
         if (!L.ntiles) continue;
         ++b->plain_launches;
@@ -1066,12 +1087,8 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     lx3c_dfj* p = b->mols[m];
     cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
     cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
-    for (auto& g : p->groups) {
-      if (g.herm) continue;
-      launch_precompute(p->orb->dev(), g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
-                        p->aux->dev(), g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, cap);
-      b->graph_kernels += 1;
-    }
+    group_records(p, false, cap);
+    b->graph_kernels += p->njobs_plain > 0;
   }
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];

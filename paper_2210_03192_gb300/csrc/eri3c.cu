@@ -167,6 +167,22 @@ __global__ void precompute_kernel(DevBasis orb, const int32_t* __restrict__ pair
     aux_record(aux, auxs, Kc, auxrec, auxc, i - n);
 }
 
+// The same for many lists in one launch (a DF-J build has dozens of groups, and
+// a launch each of a few microseconds came to 0.6 of 22.3 ms for eight densities
+// on 16 atoms).  Each warp finds its block's job among the first blocks.
+__global__ void precompute_jobs_kernel(DevBasis orb, DevBasis aux, const PrecomputeJob* __restrict__ jobs, int n) {
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+  for (int b = 0; b < n; b += 32)
+    at += __popc(__ballot_sync(0xffffffffu, b + lane < n && jobs[b + lane].first <= (long long)blockIdx.x));
+  const PrecomputeJob& j = jobs[at - 1];
+  const long long i = (blockIdx.x - j.first) * blockDim.x + threadIdx.x, np = j.npair * j.Ka * j.Kb;
+  if (i < np)
+    pair_record(orb, j.pairs, j.Ka, j.Kb, j.rec, j.ab, i);
+  else if (i - np < j.naux * j.Kc)
+    aux_record(aux, j.auxs, j.Kc, j.auxrec, j.auxc, i - np);
+}
+
 // ---------------------------------------------------------------------------
 // integral kernel
 // ---------------------------------------------------------------------------
@@ -1449,6 +1465,13 @@ cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long lo
   if (n == 0) return cudaSuccess;
   precompute_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(orb, pairs, npair, Ka, Kb, rec, ab, aux, auxs, naux, Kc,
                                                                 auxrec, auxc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_precompute_jobs(const DevBasis& orb, const DevBasis& aux, const PrecomputeJob* jobs, int n,
+                                   long long blocks, cudaStream_t st) {
+  if (n == 0 || blocks == 0) return cudaSuccess;
+  precompute_jobs_kernel<<<(unsigned)blocks, 128, 0, st>>>(orb, aux, jobs, n);
   return cudaGetLastError();
 }
 

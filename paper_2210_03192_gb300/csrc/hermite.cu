@@ -989,14 +989,9 @@ struct HermPlan {
     long long first, n;
   };
   std::vector<Tier> tiers;
-  struct Ket {
-    int32_t* shells;
-    long long n;
-    int Kc;
-    double* rec;
-    double* xyz;
-  };
-  std::vector<Ket> kets;
+  const PrecomputeJob* jobs = nullptr;  // the ket lists' records
+  int njobs = 0;
+  long long job_blocks = 0;
   char* arena = nullptr;
   size_t zero_off = 0, zero_bytes = 0;  // the fixed-point y of all primitives
   HermPairArgs pa;
@@ -1005,17 +1000,13 @@ struct HermPlan {
   double flops = 0, max_adds = 0;
 };
 
-cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
-                              double* ab, const DevBasis& aux, const int32_t* auxs, long long naux, int Kc,
-                              double* auxrec, double* auxc, cudaStream_t st);
-
 void herm_destroy(HermPlan* p) {
   if (!p) return;
   cudaFree(p->arena);
   delete p;
 }
 
-int herm_launches(const HermPlan* p) { return 2 + (int)p->kets.size() + (int)p->tiers.size(); }
+int herm_launches(const HermPlan* p) { return 3 + (int)p->tiers.size(); }
 double herm_flops(const HermPlan* p) { return p->flops; }
 double herm_max_adds(const HermPlan* p) { return p->max_adds; }
 
@@ -1304,6 +1295,8 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   const size_t o_lab = blob.add(ld);
   std::vector<HermCls> hc(cls.size());
   const size_t o_cls = blob.add(hc);
+  std::vector<PrecomputeJob> jobs(kets.size());
+  const size_t o_jobs = blob.add(jobs);
   size_t top = blob.d.size();
   auto take = [&](size_t bytes) {
     top = (top + 255) & ~size_t(255);
@@ -1366,9 +1359,15 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     hc[i] = c;
   }
   std::memcpy(blob.d.data() + o_cls, hc.data(), hc.size() * sizeof(HermCls));
-  for (size_t k = 0; k < kets.size(); ++k)
-    p->kets.push_back(HermPlan::Ket{(int32_t*)(A + ko[k].shells), (long long)kets[k].shells.size(), kets[k].Kc,
-                                    (double*)(A + ko[k].rec), (double*)(A + ko[k].xyz)});
+  for (size_t k = 0; k < kets.size(); ++k) {
+    jobs[k] = PrecomputeJob{nullptr, 0, 1, 1, nullptr, nullptr, (const int32_t*)(A + ko[k].shells),
+                            (long long)kets[k].shells.size(), kets[k].Kc, (double*)(A + ko[k].rec),
+                            (double*)(A + ko[k].xyz), p->job_blocks};
+    p->job_blocks += jobs[k].blocks();
+  }
+  std::memcpy(blob.d.data() + o_jobs, jobs.data(), jobs.size() * sizeof(PrecomputeJob));
+  p->jobs = (const PrecomputeJob*)(A + o_jobs);
+  p->njobs = (int)jobs.size();
   HermPairArgs& pa = p->pa;
   pa.orb = orb->dev();
   pa.pairs = (const int4*)(A + o_pairs);
@@ -1410,9 +1409,7 @@ namespace {
 cudaError_t herm_begin(HermPlan* p, const double* D, bool dens, bool y, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (y) e = cudaMemsetAsync(p->arena + p->zero_off, 0, p->zero_bytes, st);
-  for (auto& k : p->kets)
-    if (e == cudaSuccess) e = launch_precompute(p->orb->dev(), nullptr, 0, 1, 1, nullptr, nullptr, p->aux->dev(), k.shells, k.n,
-                                                k.Kc, k.rec, k.xyz, st);
+  if (e == cudaSuccess) e = launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->jobs, p->njobs, p->job_blocks, st);
   if (e != cudaSuccess) return e;
   HermPairArgs a = p->pa;
   a.D = D;

@@ -295,4 +295,23 @@ int basis_upload(lx3c_basis* b, cudaStream_t st);
 // at most the orientation threshold, else each to its more compact centre.
 void split_orientation(const lx3c_basis* orb, int a, int b, int la, int lb, std::vector<int>& primA,
                        std::vector<int>& primB);
+// One pair list and ket list whose records a launch over many computes, from
+// block `first` on (blocks of 128 records).
+struct PrecomputeJob {
+  const int32_t* pairs;
+  long long npair;
+  int Ka, Kb;
+  double* rec;
+  double* ab;
+  const int32_t* auxs;
+  long long naux;
+  int Kc;
+  double* auxrec;
+  double* auxc;
+  long long first;
+  long long blocks() const { return (npair * Ka * Kb + naux * Kc + 127) / 128; }
+};
+cudaError_t launch_precompute_jobs(const DevBasis& orb, const DevBasis& aux, const PrecomputeJob* jobs, int n,
+                                   long long blocks, cudaStream_t st);
+
 }  // namespace lx3c
