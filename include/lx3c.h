@@ -180,7 +180,8 @@ lx3c_status lx3c_class_flops(int la, int lb, int lc, int Kab, int Kc, int bra_pu
 
 /*
  * Launch-shape tuning (not in the paper).  The planner sizes a tile (triples
- * per tile T, primitive chunk G) for two CTAs per SM by default.
+ * per tile T, primitive chunk G) for two CTAs per SM by default, or three where
+ * they take no fewer triples a tile (or still 32).
  * lx3c_shape_hint makes every later plan of class (la, lb | lc) -- as the
  * planner orients it, so (lb, la | lc) for the B-oriented launch -- with kab
  * primitive pairs in its largest sub-pair and kc ket primitives size its tile

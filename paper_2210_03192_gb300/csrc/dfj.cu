@@ -734,7 +734,7 @@ bool retile(DfjLaunch& L, const DfjGroup& g, const DevState* ds, int T) {
   ClassDesc d = L.desc;
   const int mode = T >= 32 ? 0 : 1;
   // keep G from the planner's choice for this T
-  LaunchShape sh = choose_shape(ct, L.kmax, d.Kc, T, dev_smem(ds));
+  LaunchShape sh = largest_tile(ct, L.kmax, d.Kc, T, dev_smem(ds), 2);
   sh.T = T;
   sh.mode = mode;
   ClassDesc nd = d;

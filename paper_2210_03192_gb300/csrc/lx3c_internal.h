@@ -259,6 +259,7 @@ std::string check_class_tables(const ClassTables& ct);  // "" when every table i
 // integrals (exact for any weight), see lx3c_hrr_tables_check.
 double hrr_moment_error(const ClassTables& ct, const double AB[3]);
 LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit);
+LaunchShape largest_tile(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas);
 LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas);
 void set_shape_hint(int la, int lb, int lc, int bra_pure, int Kab, int Kc, int ctas);
 void set_tile_hint(int la, int lb, int lc, int bra_pure, int Kab, int Kc, int T, int G);

@@ -819,49 +819,69 @@ LaunchShape tile_hint_shape(const ClassTables& ct, int Kab, int Kc, int smem_lim
   return LaunchShape{T, G, mode, (int)(s.total * 8)};
 }
 
-// Largest T (then largest balanced G) whose tile fits `ctas` CTAs per SM,
-// falling back to fewer CTAs per SM when nothing fits.
-LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas) {
-  const int K = Kab * Kc;
-  std::vector<long long> budgets;
-  for (int c = std::max(1, ctas); c >= 1; --c) budgets.push_back((smem_limit / c - 1024) / 8);
-  LaunchShape best{1, 1, 1, 0};
+namespace {
+
+// Largest T, then largest balanced G, whose tile fits `budget` doubles with at
+// least gmin(T) primitives side by side (or all of them); smem_bytes = -1 when
+// none does.
+template <class GMin>
+LaunchShape fit_shape(const ClassTables& ct, int Kab, int Kc, long long naux, long long budget, const GMin& gmin) {
+  const int K = Kab * Kc, Gmax = std::min(K, 8);
   Sizes s;
-  int Ts[] = {512, 256, 128, 64, 32, 16, 8, 4, 2, 1};
-  bool found = false;
-  for (long long budget : budgets) {
-    for (int T : Ts) {
-      // never a tile that half its size would hold ((pp|d) with 32 kets: T = 64
-      // 28.7 us a call, T = 32 26.7)
-      if (T > 1 && T >= 2 * naux) continue;
-      int mode = T >= 32 ? 0 : 1;
-      buffer_sizes(ct, Kab, Kc, T, 1, mode, s, nullptr);
-      if (s.total > budget) continue;
-      // enough independent work per stage?  prefer the largest T that fits
-      int G = 1;
-      int Gmax = std::min(K, 8);
-      while (G < Gmax) {
-        buffer_sizes(ct, Kab, Kc, T, G + 1, mode, s, nullptr);
-        if (s.total > budget) break;
-        ++G;
-      }
-      // balance the primitive chunks: same number of chunks, equal sizes
-      const int nch = (K + G - 1) / G;
-      G = (K + nch - 1) / nch;
-      buffer_sizes(ct, Kab, Kc, T, G, mode, s, nullptr);
-      best = LaunchShape{T, G, mode, (int)(s.total * 8)};
-      found = true;
-      break;
+  for (int T : {512, 256, 128, 64, 32, 16, 8, 4, 2, 1}) {
+    // never a tile that half its size would hold ((pp|d) with 32 kets: T = 64
+    // 28.7 us a call, T = 32 26.7)
+    if (T > 1 && T >= 2 * naux) continue;
+    const int mode = T >= 32 ? 0 : 1;
+    int G = 0;
+    while (G < Gmax) {
+      buffer_sizes(ct, Kab, Kc, T, G + 1, mode, s, nullptr);
+      if (s.total > budget) break;
+      ++G;
     }
-    if (found) break;
+    if (G < std::min(K, std::max(1, gmin(T)))) continue;
+    // balance the primitive chunks: same number of chunks, equal sizes
+    const int nch = (K + G - 1) / G;
+    G = (K + nch - 1) / nch;
+    buffer_sizes(ct, Kab, Kc, T, G, mode, s, nullptr);
+    return LaunchShape{T, G, mode, (int)(s.total * 8)};
   }
-  if (!found) best.smem_bytes = -1;
-  return best;
+  return LaunchShape{1, 1, 1, -1};
+}
+
+}  // namespace
+
+// The largest tile for `ctas` CTAs per SM.
+LaunchShape largest_tile(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas) {
+  return fit_shape(ct, Kab, Kc, naux, (smem_limit / ctas - 1024) / 8, [](int) { return 1; });
+}
+
+// Shape for one or three CTAs per SM: the largest tile, or that of fewer CTAs
+// when nothing fits.  For two, the default: wide tiles (T >= 64) only with three
+// primitives side by side, as each chunk of primitives costs the barriers of
+// its stages ((pp|p) K = 36: T, G = 128, 2 1.53 ms, 64, 6 1.35; (pp|d) K = 9:
+// 128, 1 0.90, 64, 3 0.77); and a third CTA (of 384 threads) where it takes no
+// fewer triples a tile, or still a full warp of them, and two primitives: the
+// barriers of three overlap better ((fd|f) K = 9 8, 5 7.64 ms, 8, 3 6.76; (ff|d)
+// K = 4 8, 4 6.25, 8, 2 5.43; (gg|i) K = 36 92.4 -> 86.0), while fewer triples lose
+// more than that ((dd|f) K = 9 16, 5 4.15, 8, 5 4.53), and so does one primitive at
+// a time ((gs|d) K = 9 32, 3 1.56, 32, 1 1.73).
+LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas) {
+  if (ctas != 2) {
+    const LaunchShape sh = largest_tile(ct, Kab, Kc, naux, smem_limit, std::max(1, ctas));
+    return sh.smem_bytes < 0 && ctas > 1 ? choose_shape_for(ct, Kab, Kc, naux, smem_limit, ctas - 1) : sh;
+  }
+  const LaunchShape two =
+      fit_shape(ct, Kab, Kc, naux, (smem_limit / 2 - 1024) / 8, [](int T) { return T >= 64 ? 3 : 1; });
+  if (two.smem_bytes < 0) return choose_shape_for(ct, Kab, Kc, naux, smem_limit, 1);
+  const LaunchShape three =
+      fit_shape(ct, Kab, Kc, naux, (smem_limit / 3 - 1024) / 8, [](int T) { return T >= 128 ? 3 : 2; });
+  return three.smem_bytes >= 0 && three.T >= std::min(two.T, 32) ? three : two;
 }
 
 // The planner's shape: a tuned tile hint (T, G) for this class, contraction
-// and ket contraction when one is set and fits; else two CTAs per SM unless
-// a tuned CTAs-per-SM hint says otherwise.
+// and ket contraction when one is set and fits, or a tuned number of CTAs per
+// SM, or the default.
 LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit) {
   const LaunchShape th = tile_hint_shape(ct, Kab, Kc, smem_limit);
   if (th.smem_bytes >= 0) return th;

@@ -328,3 +328,19 @@ def test_hrr_tables_exact_on_moment_integrals(variant):
                 assert L.lx3c_hrr_tables_check(la, lb, lc, 1, variant, AB.ctypes.data, ctypes.byref(e)) == 0, \
                     L.lx3c_last_error()
                 assert e.value < 1e-14, (la, lb, lc, e.value)
+
+
+@pytest.mark.parametrize("naux", [1, 2, 3, 31, 32, 33, 64, 65, 512])
+@pytest.mark.parametrize("la,lb,lc,kab", [(1, 1, 2, 1), (1, 1, 1, 36), (2, 1, 2, 6), (3, 2, 3, 9), (4, 4, 6, 36), (4, 0, 2, 9)])
+def test_default_shape_rule(la, lb, lc, kab, naux):
+    """The planner's tile is never one that half its size would hold, fits two
+    CTAs per SM (or the largest that one takes), and wide tiles keep three
+    primitives side by side."""
+    import paper_2210_03192_gb300 as lx
+    smem = 233472
+    T, G, mode, sb = lx.shape_query(la, lb, lc, kab, 1, naux, 0)
+    assert T == 1 or T < 2 * naux
+    assert mode == (0 if T >= 32 else 1)
+    assert sb <= smem // 2 - 1024 or (T, G, mode, sb) == lx.shape_query(la, lb, lc, kab, 1, naux, 1)
+    chunks = -(-kab // G)
+    assert T < 64 or chunks <= -(-kab // min(kab, 2))
