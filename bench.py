@@ -415,7 +415,7 @@ def extra_dfj(dev):
     cp = lx.DFJPlan(cl.orb, cl.aux, 1e-12, contract=True)
     csetup = time.time() - t0
     _, cfused, cgonly, cjonly = times(cp)
-    # the contracted build does fewer flops; its fraction is of its own flops
+    # with the contraction flag; its fraction is of its own flops
     out["contracted"] = dict(setup_s=round(csetup, 2), fused_s=round(cfused / 1e3, 3),
                              gamma_only_s=round(cgonly / 1e3, 3), J_only_s=round(cjonly / 1e3, 3),
                              flops_ratio=round(cp.flops / pflops, 4),
@@ -487,8 +487,8 @@ def extra_grad(dev):
 
 def extra_dfj_multi(dev):
     """Per-density DF-J time with one density and with eight at once
-    (lx3c_dfj_execute_multi), and the single-density build contracted at the
-    (e0|c) level, 32-atom cluster of the 256-atom recipe."""
+    (lx3c_dfj_execute_multi), and the single-density build with the contraction
+    flag, 32-atom cluster of the 256-atom recipe."""
     import torch
     import paper_2210_03192_gb300 as lx
     from paper_2210_03192_gb300 import workloads as W

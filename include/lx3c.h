@@ -451,9 +451,8 @@ lx3c_status lx3c_dfj_coulomb(lx3c_dfj* plan, const double* L, int64_t lda, const
  *   alive while the batch is executed), orders the class launches longest
  *   first and captures two CUDA graphs of the whole build (zeroing,
  *   precompute, integrals, J finish): graph 1 runs every (class launch,
- *   tile) work item in persistent kernels, one per occupancy tier (the
- *   items that fit three CTAs per SM of the 40-register persistent kernel,
- *   then two CTAs of the unrestricted one, then the rest), each sized for its
+ *   tile) work item outside the Hermite basis in persistent kernels, one per
+ *   occupancy tier (the items that fit two CTAs per SM, then the rest), each sized for its
  *   tier's largest item and pulling items longest first from its own atomic
  *   counter (no CTA waits on another); graph 2 runs the class launches
  *   themselves on four parallel graph branches.  Setup; may
