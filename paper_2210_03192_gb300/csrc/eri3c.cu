@@ -1320,10 +1320,10 @@ __global__ void __launch_bounds__(kPsThreads) eri3c_ps_kernel(const __grid_const
   }
 }
 
-// (p s|C) DF-J launches digesting per integral: one warp per tile, lanes over
-// its kets; gamma_P[C] += w sum_s D_s (ps|P)_{sC} per lane and
-// J_s += w_J sum over the tile's kets and C of (ps|P)_{sC} c_PC, reduced
-// across the warp.
+// (p s|C) DF-J launches digesting per integral, lanes over the kets of 32 /
+// warpW tiles as in eri3c_ss_dfj_kernel: gamma_P[C] += w sum_s D_s (ps|P)_{sC}
+// per lane and J_s += w_J sum over the tile's kets and C of (ps|P)_{sC} c_PC,
+// reduced across the tile's lanes.  kMulti: up to eight densities.
 template <int LC, bool kMulti>
 __global__ void __launch_bounds__(kPsThreads) eri3c_ps_dfj_kernel(const __grid_constant__ ClassDesc d) {
   constexpr int NC = (LC + 1) * (LC + 2) / 2, NS = 2 * LC + 1, NB = 3 * NS;

@@ -15,6 +15,10 @@
 // is formed: (ff|h) costs about 2.8e3 FP64 instructions per triple where
 // forming and digesting its integrals took 3.4e4 flops.
 //
+// The classes of degree up to 6 run on the unrolled kernel of
+// hermite_unrolled.cuh; this file has the tables and the kernel for the others,
+// the kernels per pair, and the plans of both.
+//
 // GB300 layout.  FP64 issues one warp instruction per 16 SM clocks, so an FMA
 // may spend 16 clocks of shared-memory bandwidth and 64 issue slots on its
 // operands: every stage runs from per-lane shared-memory columns driven by
