@@ -303,7 +303,10 @@ lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap
  *   (each contribution rounded to a multiple of 2^-72, every partial sum
  *   below 2^55 in magnitude) and rounded once to FP64, so the
  *   result does not depend on the order in which tiles finish: repeated
- *   executes of a plan are bitwise equal.
+ *   executes of a plan are bitwise equal.  The Hermite potentials behind J
+ *   and the gradient are summed in the same way, each scaled to the size of
+ *   its terms in J or in the force, with 16 bits more at either end (2^-88,
+ *   2^71).
  * lx3c_dfj_execute_multi: the same build for nd (1..8) densities and
  *   coefficient vectors at once, sharing every integral: D (device, nd x nao
  *   x nao), c (device, nd x naux_ao) in; gamma (nd x naux_ao) and J (nd x nao

@@ -16,6 +16,8 @@
 //   contributions per accumulator (the planners check the gradient's
 //   per-atom counts; gamma and J elements get at most two per shell pair or
 //   ket shell).
+// The Hermite potentials y behind J and the forces have a wider form of their
+// own (wide_add, below).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -71,6 +73,65 @@ __device__ __forceinline__ double fix_decode(const unsigned long long* acc) {
   }
   const double mag = fma((double)hi, 18446744073709551616.0, (double)lo);
   const double v = ldexp(mag, -kFixShift);
+  return neg ? -v : v;
+}
+
+// Accumulator of one Hermite potential: N = round(v 2^kWideShift) of 160 bits in
+// four words, N = A3 2^96 + A2 2^64 + A1 2^32 + A0.  A contribution adds its
+// magnitude's 32-bit digits with its own sign (the words are signed sums), so
+// that two or three of the four words are touched whatever the sign; up to
+// 2^31 contributions.  y enters scaled to the size of its terms in J or in the
+// force (hermite.cu, potential_scale); a J element is a sum over up to 455
+// terms that partly cancel, so the words have 16 bits more than J's at either
+// end: resolution 2^-88, range 2^71.  Unscaled and in J's 128 bits, y_0 of a
+// unit-normalised (g g| pair with exponents 1e4 passed 2^55 (6e16, read back
+// as -1e16), and one rounding cost 2e-11 of an (i i| pair's J at 0.02.
+constexpr int kWideShift = 88;
+constexpr int kWideWords = 4;
+constexpr int kWideBytes = 8 * kWideWords;
+
+__device__ __forceinline__ void wide_add(unsigned long long* acc, double v) {
+  const long long bits = __double_as_longlong(v);
+  const int e = (int)((bits >> 52) & 0x7FF);
+  if (e == 0) return;
+  unsigned long long m = (bits & ((1ULL << 52) - 1)) | (1ULL << 52);
+  int sh = e - 1075 + kWideShift;  // |N| = m 2^sh
+  if (sh < 0) {
+    if (sh < -53) return;
+    m = (m + (1ULL << (-sh - 1))) >> -sh;
+    sh = 0;
+  }
+  const int off = sh & 31, w = sh >> 5;  // m 2^off fills digits w, w + 1, w + 2
+  const unsigned long long lo = m << off, hi = off ? m >> (64 - off) : 0ULL;
+  const unsigned long long d[3] = {lo & 0xFFFFFFFFULL, lo >> 32, hi};
+  unsigned long long top = 0ULL;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (w + k < 3) {
+      if (d[k]) atomicAdd(acc + w + k, bits < 0 ? 0ULL - d[k] : d[k]);
+    } else if (w + k < 5) {
+      top += d[k] << (32 * (w + k - 3));
+    }
+  }
+  if (top) atomicAdd(acc + 3, bits < 0 ? 0ULL - top : top);
+}
+
+// {A0, .., A3} -> the nearest FP64 value of N 2^-kWideShift (to within an ulp).
+__device__ __forceinline__ double wide_decode(const unsigned long long* acc) {
+  const long long a0 = (long long)acc[0];
+  const long long a1 = (long long)acc[1] + (a0 >> 32);
+  const long long a2 = (long long)acc[2] + (a1 >> 32);
+  unsigned long long hi = acc[3] + (unsigned long long)(a2 >> 32);
+  unsigned long long mid = ((unsigned long long)a2 << 32) | (a1 & 0xFFFFFFFFULL);
+  unsigned long long lo = a0 & 0xFFFFFFFFULL;
+  const bool neg = (long long)hi < 0;
+  if (neg) {
+    lo = (0ULL - lo) & 0xFFFFFFFFULL;
+    mid = ~mid + (lo == 0ULL ? 1ULL : 0ULL);
+    hi = ~hi + (lo == 0ULL && mid == 0ULL ? 1ULL : 0ULL);
+  }
+  const double mag = fma(fma((double)hi, 18446744073709551616.0, (double)mid), 4294967296.0, (double)lo);
+  const double v = ldexp(mag, -kWideShift);
   return neg ? -v : v;
 }
 

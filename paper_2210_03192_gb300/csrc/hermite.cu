@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(32 * kNW, 16 / kNW) herm_kernel(const __grid_c
     const int ie = e0 + sub;
     const int prim = tile.z + min(ie, tile.w - 1);
     const bool act = ie < tile.w && q < __ldg(c.cnt + __ldg(c.primpair + prim));
-    const double* pr = c.prim + 8LL * prim;
+    const double* pr = c.prim + 4LL * prim;
     const double gam = __ldg(pr);
     const double Rx = __ldg(pr + 1) - Cx, Ry = __ldg(pr + 2) - Cy, Rz = __ldg(pr + 3) - Cz;
     const double R2 = fma(Rz, Rz, fma(Ry, Ry, Rx * Rx));
@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(32 * kNW, 16 / kNW) herm_kernel(const __grid_c
 
 struct HermLabDev {
   double* prim;
+  double* scale;
   const int* primab;  // ia Kb + ib of each primitive pair
   double* H;
   unsigned long long* Y;
@@ -407,6 +408,29 @@ __device__ __forceinline__ PairGeom pair_geom(const DevBasis& o, int sa, int sb,
   return r;
 }
 
+// The power of two 2^e by which y_a of degree t is held: about the largest
+// |E~^ab_a| it is multiplied by (with 2 gamma, for the forces), so that the
+// fixed-point words see the size of its term in J (in the force).  E~_t is the
+// mean of the t-th derivative of (x + PA)^i (x + PB)^j over a normal
+// distribution of variance h = 1/(2 gamma), i + j = n: about n!/(n - t)! times
+// the largest n - t of the factors, each sqrt(|PA|^2 + h (n - t)/e).  (Between
+// the tightest and the most diffuse shells it spans h^6.)
+__device__ __forceinline__ int potential_scale(int la, int lb, double pa2, double pb2, double h, int t, bool grad) {
+  if (grad) ++la;
+  const int n = la + lb, m = n - t;
+  const float hm = (float)(h * m) * 0.36787944f;
+  float ra = (float)pa2 + hm, rb = (float)pb2 + hm;
+  const int small = ra < rb ? la : lb;           // factors of the smaller kind
+  const int k = max(small - t, 0);               // of them, those left
+  float f = 1.0f;
+  for (int i = 0; i < t; ++i) f *= (float)(n - i);
+  float l = log2f(f) + 0.5f * (k * log2f(fminf(ra, rb)) + (m - k) * log2f(fmaxf(ra, rb)));
+  if (m == 0) l = log2f(f);                      // (no factor: the logarithm may be infinite)
+  else if (k == 0) l = log2f(f) + 0.5f * m * log2f(fmaxf(ra, rb));
+  if (grad) l -= log2f((float)h);
+  return (int)rintf(fminf(fmaxf(l, -500.0f), 500.0f));
+}
+
 // (y, z) of index w in the graded order of two exponents
 __device__ __forceinline__ void yz_of(int w, int& y, int& z) {
   int n = 0;
@@ -478,12 +502,23 @@ __global__ void __launch_bounds__(32) herm_pre_kernel(const __grid_constant__ He
     const int prim = p1.w + k, ab = __ldg(L.primab + prim);
     const PairGeom pg = pair_geom(g.orb, p1.x, p1.y, ab / Kb, ab % Kb);
     if (lane == 0) {
-      double* o = L.prim + 8LL * prim;
+      double* o = L.prim + 4LL * prim;
       o[0] = pg.g;
       o[1] = pg.P[0]; o[2] = pg.P[1]; o[3] = pg.P[2];
-      o[4] = pg.h;
-      o[5] = pg.K;
-      o[6] = pg.za; o[7] = pg.zb;
+    }
+    const int nT = kGrad ? Lab + 2 : Lab + 1;
+    if (lane < nT) {
+      const double pa2 = pg.PA[0] * pg.PA[0] + pg.PA[1] * pg.PA[1] + pg.PA[2] * pg.PA[2];
+      const double pb2 = pg.PB[0] * pg.PB[0] + pg.PB[1] * pg.PB[1] + pg.PB[2] * pg.PB[2];
+      const int e = potential_scale(la, lb, pa2, pb2, pg.h, lane, kGrad);
+      double s = pg.K, b = pg.h;
+      for (int k = lane; k; k >>= 1) {
+        if (k & 1) s *= b;
+        b *= b;
+      }
+      double* o = L.scale + 2LL * prim * nT + lane;
+      o[0] = ldexp(s, e);
+      o[nT] = ldexp(1.0, -e);
     }
     if (!dens) continue;
     __syncwarp();
@@ -531,6 +566,16 @@ __global__ void __launch_bounds__(32) herm_pre_kernel(const __grid_constant__ He
   }
 }
 
+// y of one primitive pair, degrees 0..deg, from its fixed-point words.
+__device__ __forceinline__ void potentials(const HermLabDev& L, int prim, int deg, double* Ys) {
+  const double* inv = L.scale + (2LL * prim + 1) * (deg + 1);
+  for (int n = 0; n <= deg; ++n) {
+    const double f = __ldg(inv + n);
+    for (int t = nherm(n - 1) + threadIdx.x; t < nherm(n); t += 32)
+      Ys[t] = f * wide_decode(L.Y + kWideWords * ((long long)prim * L.nY + t));
+  }
+}
+
 // J block of each pair: J_ab = wj sum over primitives of E~ y, through the
 // Cartesian block, one warp per shell pair.
 __global__ void __launch_bounds__(32) herm_post_kernel(const __grid_constant__ HermPairArgs g) {
@@ -550,7 +595,7 @@ __global__ void __launch_bounds__(32) herm_post_kernel(const __grid_constant__ H
     const int prim = p1.w + k, ab = __ldg(L.primab + prim);
     const PairGeom pg = pair_geom(g.orb, p1.x, p1.y, ab / Kb, ab % Kb);
     __syncwarp();
-    for (int t = lane; t < nherm(Lab); t += 32) Ys[t] = fix_decode(L.Y + kFixWords * ((long long)prim * L.nY + t));
+    potentials(L, prim, Lab, Ys);
     etables(E, la, lb, nt, pg.PA, pg.PB, pg.h);
     for (int ax = 0; ax <= la; ++ax)
       for (int bx = 0; bx <= lb; ++bx) {
@@ -621,7 +666,7 @@ __global__ void __launch_bounds__(32) herm_force_kernel(const __grid_constant__ 
     const int prim = p1.w + k, ab = __ldg(L.primab + prim);
     const PairGeom pg = pair_geom(g.orb, p1.x, p1.y, ab / Kb, ab % Kb);
     __syncwarp();
-    for (int t = lane; t < nherm(Lab + 1); t += 32) Ys[t] = fix_decode(L.Y + kFixWords * ((long long)prim * L.nY + t));
+    potentials(L, prim, Lab + 1, Ys);
     etables(E, la + 1, lb, nt, pg.PA, pg.PB, pg.h);
     for (int w = lane; w < 3 * sf; w += 32) {
       const int ax = w / sf, rem = w - ax * sf, i = rem / si, r = rem - i * si;
@@ -1059,7 +1104,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     std::vector<PairRef> pr;
     std::vector<long long> prim0;  // first primitive of each pair, and the end
     std::vector<int> primab, primpair;
-    size_t H, Y, prim, o_ab, o_pair;  // arena offsets
+    size_t H, Y, prim, scale, o_ab, o_pair;  // arena offsets
   };
   std::vector<LabHost> labs;
   std::vector<int> laboff(kMaxDeg + 2, -1);
@@ -1314,11 +1359,12 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   }
   for (auto& L : labs) {
     const long long nY = nherm(L.Lab + (grad ? 1 : 0));
-    L.prim = take((size_t)L.nprim * 64);
+    L.prim = take((size_t)L.nprim * 32);
+    L.scale = take((size_t)L.nprim * 2 * (L.Lab + (grad ? 2 : 1)) * 8);
     L.H = take((size_t)L.nprim * (grad ? 3 * nY : nY) * 8);
   }
   p->zero_off = take(0);
-  for (auto& L : labs) L.Y = take((size_t)L.nprim * nherm(L.Lab + (grad ? 1 : 0)) * kFixBytes);
+  for (auto& L : labs) L.Y = take((size_t)L.nprim * nherm(L.Lab + (grad ? 1 : 0)) * kWideBytes);
   p->zero_bytes = top - p->zero_off;
   if (cudaMalloc(&p->arena, top) != cudaSuccess) {
     cudaGetLastError();
@@ -1329,6 +1375,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   for (size_t i = 0; i < labs.size(); ++i) {
     const LabHost& L = labs[i];
     ld[i].prim = (double*)(A + L.prim);
+    ld[i].scale = (double*)(A + L.scale);
     ld[i].primab = (const int*)(A + L.o_ab);
     ld[i].H = (double*)(A + L.H);
     ld[i].Y = (unsigned long long*)(A + L.Y);
@@ -1353,6 +1400,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     c.cnt = (const int*)(A + x.cnt);
     const LabHost& L = labs[x.lab];
     c.prim = (const double*)(A + L.prim);
+    c.scale = (const double*)(A + L.scale);
     c.primpair = (const int*)(A + L.o_pair);
     c.H = (const double*)(A + L.H);
     c.Yacc = (unsigned long long*)(A + L.Y);

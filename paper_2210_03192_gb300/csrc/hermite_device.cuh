@@ -53,7 +53,8 @@ struct HermCls {
   const int* ydeg;        // degree of Hermite index a
   double boys_cL;
   // data
-  const double* prim;     // [nprim][8]: gamma, P, 1/(2 gamma), K_ab
+  const double* prim;     // [nprim][4]: gamma, P
+  const double* scale;    // [nprim][2][Lab + 1]: factor of y_a by degree, power of two it holds (inverse)
   const int* primpair;    // primitive -> pair position
   const int* cnt;         // kets kept by each pair
   const double* H;        // [nprim][nR], gradient: [nprim][3][nY]
@@ -102,11 +103,8 @@ __device__ __forceinline__ void sum_rows(const HermCls& c, const double* stg, in
     const int at = part * w + s0, s = at / W;
     if (r < row && at == s * W && e0 + s < tile.w) {
       const int ps = tile.z + e0 + s;
-      const double* prs = c.prim + 8LL * ps;
-      v *= __ldg(prs + 5);
-      const double h = __ldg(prs + 4);
-      for (int k = __ldg(c.ydeg + a); k > 0; --k) v *= h;
-      fix_add(c.Yacc + kFixWords * ((long long)ps * c.nY + a), v);
+      v *= __ldg(c.scale + 2LL * ps * (c.Lab + 1) + __ldg(c.ydeg + a));
+      wide_add(c.Yacc + kWideWords * ((long long)ps * c.nY + a), v);
     }
   }
   __syncwarp();

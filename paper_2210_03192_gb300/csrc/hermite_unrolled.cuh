@@ -135,7 +135,7 @@ __device__ __forceinline__ void herm_tile(const HermArgs& g, const HermCls& c, c
     const int ie = e0 + grp;
     const int prim = tile.z + min(ie, tile.w - 1);
     const bool act = ie < tile.w && q < __ldg(c.cnt + __ldg(c.primpair + prim));
-    const double* pr = c.prim + 8LL * prim;
+    const double* pr = c.prim + 4LL * prim;
     const double gam = __ldg(pr);
     const double R3[3] = {__ldg(pr + 1) - Cx, __ldg(pr + 2) - Cy, __ldg(pr + 3) - Cz};
     const double R2 = fma(R3[2], R3[2], fma(R3[1], R3[1], R3[0] * R3[0]));
