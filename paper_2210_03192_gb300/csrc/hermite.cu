@@ -1217,20 +1217,25 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
                                   : UnrolledCost{pg.instr_base, pg.instr_gamma, pg.instr_j};
       x.instr = (uc.base + uc.j + (grad ? 3.0 * pg.nR : uc.gamma)) * k.Kc;
       // W kets side by side: the widest power of two whose ragged end wastes
-      // least (narrower tiles pay one more y row sum per primitive pair)
+      // least (narrower tiles pay one more y row sum per primitive pair), of
+      // those whose 32 / W densities fit beside the columns (one ket at a time
+      // takes 116 KB of them at degree 12)
+      const auto smem_of = [&](int W) {
+        return unr ? herm_unrolled_smem(Lp, k.lc, W) : c.cH * kColBytes + (grad ? 0 : 32 / W * pg.nR * 8);
+      };
       double best = 1e300;
-      for (int W = 32; W >= 1; W /= 2) {
+      for (int W = 32; W >= 1 && smem_of(W) <= kSmemCta; W /= 2) {
         double slots = 0;
         for (size_t i = 0; i < L.pr.size(); ++i)
           slots += (double)((x.counts[i] + W - 1) / W * W) * (double)(L.prim0[i + 1] - L.prim0[i]);
         const double cost = slots * (1.0 + 0.02 * (32 / W - 1));
         if (cost < best * 0.999) { best = cost; c.W = W; }
       }
-      x.smem = unr ? herm_unrolled_smem(Lp, k.lc, c.W) : c.cH * kColBytes + (grad ? 0 : 32 / c.W * pg.nR * 8);
-      if (x.smem > kSmemCta) {
+      if (!c.W) {
         set_last_error("dfj: Hermite class does not fit in shared memory");
         return LX3C_ENOTSUP;
       }
+      x.smem = smem_of(c.W);
       p->flops += 2.0 * x.instr * tri;
       total += x.instr * best / 32.0;
       auto key = std::make_pair(Lp, k.lc);  // (nw follows from them)

@@ -1,4 +1,4 @@
-"""J and forces from unit-normalised shells, l = 4 and 5, exponents from 0.01 to
+"""J and forces from unit-normalised shells, l = 4 to 6, exponents from 0.01 to
 1e4 on one centre and one beside it: the Hermite potentials behind them span
 h^-6 (h = 1/(2 gamma)) where J itself is of the size of c, for coefficients c
 of 1e-8, 1 and 1e8.  Tolerances as for the other DF-J and gradient tests, with
@@ -53,7 +53,7 @@ def density_and_c(orb, aux, l, scale):
 
 
 @pytest.mark.parametrize("scale", [1e-8, 1.0, 1e8])
-@pytest.mark.parametrize("l", [4, 5])
+@pytest.mark.parametrize("l", [4, 5, 6])
 def test_J_of_normalised_shells(lx, l, scale):
     orb, aux = problem(l)
     D, c = density_and_c(orb, aux, l, scale)
