@@ -64,6 +64,7 @@ struct lx3c::DevState {
   double* boys_mid = nullptr;
   int nsm = 0;
   int smem_per_sm = 0;
+  bool ready = false;  // every step of the set-up done
   std::map<std::tuple<int, int, int, int>, DevClass> classes;
   // host-buffer path (lx3c_eri3c_host): the two output chunk buffers (grown,
   // never shrunk), the copy stream and its events, made on first use and kept;
@@ -85,16 +86,17 @@ lx3c_status device_state(DevState** out) {
   CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_mu);
   DevState& s = g_dev[dev];
-  if (!s.boys_tab) {
+  if (!s.ready) {
     std::vector<double> tab, mid;
     boys_tables(tab, mid);
-    CUDA_TRY(cudaMalloc(&s.boys_tab, tab.size() * 8));
-    CUDA_TRY(cudaMalloc(&s.boys_mid, mid.size() * 8));
+    if (!s.boys_tab) CUDA_TRY(cudaMalloc(&s.boys_tab, tab.size() * 8));
+    if (!s.boys_mid) CUDA_TRY(cudaMalloc(&s.boys_mid, mid.size() * 8));
     CUDA_TRY(cudaMemcpy(s.boys_tab, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(s.boys_mid, mid.data(), mid.size() * 8, cudaMemcpyHostToDevice));
     CUDA_TRY(init_constants());
     CUDA_TRY(cudaDeviceGetAttribute(&s.nsm, cudaDevAttrMultiProcessorCount, dev));
     CUDA_TRY(cudaDeviceGetAttribute(&s.smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    s.ready = true;
   }
   *out = &s;
   return LX3C_OK;

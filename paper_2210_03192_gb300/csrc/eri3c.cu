@@ -1461,10 +1461,18 @@ __global__ void boys_kernel(const double* __restrict__ Tv, long long n, int mmax
 // host-side launch helpers (called from capi.cu)
 // ---------------------------------------------------------------------------
 
+// The current device's constants and the tile kernels' shared-memory limit (an
+// attribute of the kernel on that device), with each device's first plan or
+// allocation-free call.
 cudaError_t init_constants() {
   double v[32];
   for (int m = 0; m < 32; ++m) v[m] = 1.0 / (2 * m + 1);
-  return cudaMemcpyToSymbol(c_inv2m1, v, sizeof(v));
+  cudaError_t e = cudaMemcpyToSymbol(c_inv2m1, v, sizeof(v));
+  for (const void* f : {(const void*)eri3c_kernel<0, 512, 2>, (const void*)eri3c_kernel<0, 384, 3>,
+                        (const void*)eri3c_kernel<1, 512, 2>, (const void*)eri3c_kernel<1, 384, 3>,
+                        (const void*)eri3c_kernel_both})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  return e;
 }
 
 cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
@@ -1500,23 +1508,6 @@ static int device_sms() {
 // Whether three CTAs of the 384-thread tile kernel fit an SM.
 static bool three_ctas(int smem_bytes) { return smem_bytes <= 233472 / 3 - 1024; }
 
-// Set once per process, from the first plan or occupancy query on.
-static cudaError_t tile_kernel_attributes() {
-  static const cudaError_t rc = [] {
-    cudaError_t e = cudaSuccess;
-    auto set = [&](const void* f) {
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    };
-    set((const void*)eri3c_kernel<0, 512, 2>);
-    set((const void*)eri3c_kernel<0, 384, 3>);
-    set((const void*)eri3c_kernel<1, 512, 2>);
-    set((const void*)eri3c_kernel<1, 384, 3>);
-    set((const void*)eri3c_kernel_both);
-    return e;
-  }();
-  return rc;
-}
-
 // Whether a launch runs on a register-resident kernel: (s s|C), or (p s|C) and
 // B-oriented (s p|C) (whose descriptor holds the (p s|C) tables with orient =
 // 1) with 1 <= lc <= 4 or contracted; (p s|s) with one primitive per triple
@@ -1548,16 +1539,12 @@ bool can_launch_both(const ClassDesc& a, const ClassDesc& b) {
 }
 
 cudaError_t launch_eri3c_both(const ClassDesc& a, int ga, const ClassDesc& b, int gb, cudaStream_t st) {
-  cudaError_t e = tile_kernel_attributes();
-  if (e != cudaSuccess) return e;
   const int smem = std::max(a.smem_doubles, b.smem_doubles) * 8;
   eri3c_kernel_both<<<ga + gb, kBothThreads, smem, st>>>(a, b, ga);
   return cudaGetLastError();
 }
 
 cudaError_t launch_eri3c(const ClassDesc& d, int grid, cudaStream_t st) {
-  cudaError_t e = tile_kernel_attributes();
-  if (e != cudaSuccess) return e;
   if (on_register_kernel(d)) {
     const int threads = d.la ? kPsThreads : kSsThreads;
     const long long items = d.digest ? d.nwtiles : d.nsub * d.naux;
