@@ -17,20 +17,22 @@ static __constant__ double c_inv[48] = {
 
 // FP64 <-> FP32 by shifting bits: the conversion instructions run at the FP64
 // rate (17 SM clocks per warp, measured), these in the integer pipe.  Values
-// outside the float range saturate to infinity and to zero.
+// from 2^128 on give infinity, those below 2^-127 zero (high word clamped, low
+// word cleared).
 __device__ __forceinline__ float to_float_bits(double x) {  // x >= 0, truncated
-  const int hi = min(max(__double2hiint(x), 0x38000000), 0x47F00000);
-  return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)(hi - 0x38000000), 3));
+  const int h = __double2hiint(x), hi = min(max(h, 0x38000000), 0x47F00000);
+  const unsigned lo = h == hi ? (unsigned)__double2loint(x) : 0u;
+  return __int_as_float((int)__funnelshift_l(lo, (unsigned)(hi - 0x38000000), 3));
 }
-__device__ __forceinline__ double to_double_bits(float y) {  // y > 0, or 0
+__device__ __forceinline__ double to_double_bits(float y) {  // finite y > 0, or 0
   const int b = __float_as_int(y);
   return __hiloint2double(b ? (b >> 3) + 0x38000000 : 0, b << 29);
 }
 
-// 1/sqrt(x) for x > 0 in FP64: single-precision seed, then one Newton-Raphson
-// step carrying the second-order term (y1 = y0 (1 + e/2 + 3e^2/8),
-// e = 1 - x y0^2), which takes the ~1e-7 seed error to FP64 rounding level
-// with five FP64 operations.
+// 1/sqrt(x) in FP64 for x in the range of a normal float: single-precision
+// seed, then one Newton-Raphson step carrying the second-order term
+// (y1 = y0 (1 + e/2 + 3e^2/8), e = 1 - x y0^2), which takes the ~1e-7 seed
+// error to FP64 rounding level with five FP64 operations.  0 from 2^128 on.
 __device__ __forceinline__ double rsqrt_fp64(double x) {
   double y0 = to_double_bits(rsqrtf(to_float_bits(x)));
   double t = x * y0;
@@ -61,7 +63,10 @@ __device__ __forceinline__ void boys_top(const double* __restrict__ tab, const d
       ex = fma(fma(fma(fma(fma(fma(fma(e3.y, dx, e3.x), dx, e2.y), dx, e2.x), dx, e1.y), dx, e1.x), dx, e0.y), dx, e0.x);
     }
   } else {
-    const double rs = rsqrt_fp64(T);
+    // the root of T 4^-k in [1, 4), for any finite T (NaN and infinity give NaN)
+    const int k = h < 0x7FF00000 ? ((h >> 20) - 1023) >> 1 : 0;
+    const double rs = rsqrt_fp64(__hiloint2double(h - (k << 21), __double2loint(T))) *
+                      __hiloint2double((1023 - k) << 20, 0);
     double b = rs * rs;  // 1/T, one Newton step from the root
     b = fma(b, fma(-T, b, 1.0), b);
     double p = rs;
