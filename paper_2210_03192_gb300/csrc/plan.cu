@@ -510,15 +510,30 @@ ClassTables build(int la, int lb, int lc, int bra_pure, int hrr2) {
   fp += Lab == 0 ? 16.0 : 32.0 + 3.0 * Lab;
   for (int e = 1; e <= Lab; ++e)
     for (int i = ct.vlev_start[e - 1]; i < ct.vlev_start[e]; ++i) fp += ((ct.vtab[i].z >> 20) & 0xF) ? 7 : 3;
-  // weights, m by m: (x + i y)^m, the Q recursion, their products
-  if (lc > 0) fp += 5;
-  for (int m = 0; m <= lc; ++m) {
-    fp += 6.0 * std::max(0, m - 1) + 4.0 * std::max(0, lc - m - 1);
-    for (int k = 0; k <= kmax && k <= lc - m; ++k) fp += (k > 0) + (m > 0 ? 2 : 0);
+  double fc;
+  if (Lab == 0 || (la == 1 && lb == 0 && lc <= 4)) {
+    // (s s|C) and (p s|C) run on the register-resident kernels: powers of X,
+    // the monomials Y^k X^n the accumulators read, 3 ncart(lc) + ncart(lc - 1)
+    // accumulators for (p s|C) or ncart(lc), a target's one or two terms, the
+    // ket transform
+    const int rows = Lab ? 3 : 1;
+    fp += lc > 0 ? 4.0 * (lc - 1) - std::max(0, kmax - 1) : 0.0;
+    for (int k = 0; k <= kmax; ++k)
+      for (auto& n : cart(lc - k)) fp += std::max(0, (n.v[0] > 0) + (n.v[1] > 0) + (n.v[2] > 0) + k - 1);
+    const int nmono = ct.ncc, nless = kmax ? ncart(lc - 1) : 0;
+    fp += 2.0 * (rows * nmono + nless);
+    fc = 2.0 * rows * (nmono + nless) + 2.0 * ct.kent.size() * rows;
+  } else {
+    // weights: (x + i y)^m, the Q recursion for each m, their products
+    if (lc > 0) fp += 5 + 6.0 * (lc - 1);
+    for (int m = 0; m <= lc; ++m) {
+      fp += 4.0 * std::max(0, lc - m - 1);
+      for (int k = 0; k <= kmax && k <= lc - m; ++k) fp += (k > 0) + (m > 0 ? 2 : 0);
+    }
+    fp += 2.0 * ct.NACC;
+    fc = 2.0 * ct.gterm.size();
   }
-  fp += 2.0 * ct.NACC;
   ct.flops_prim = fp;
-  double fc = 2.0 * ct.gterm.size();
   for (const uint4& h : ct.htab) fc += 2.0 * ((h.x >> 16) - 1) * ct.nC;
   auto bra = [&](const std::vector<int>& ptr, const std::vector<int2>& ent, int nother) {
     double f = 0;
