@@ -634,7 +634,7 @@ def make_line(args, res, classes, world, cpu, extras):
         higher_is_better=True, scaling="weak", vs_baseline=None, dtype="f64",
         data="synthetic (per-class sweep recipe, seeded)",
         config=dict(sweep_config(args, classes, world),
-                    tile_shapes=("planner default + %d tuned hints (shape_hints_gb300.txt)" % getattr(args, "hints", 0)
+                    tile_shapes=("planner default + %d tuned hints" % getattr(args, "hints", 0)
                                  if getattr(args, "hints", 0) else "planner default"),
                     hrr=("1-q rounds + %d tuned 2-q classes (hrr_hints_gb300.txt)" % getattr(args, "hrr_hints", 0)
                          if getattr(args, "hrr_hints", 0) else "1-q rounds")),
@@ -647,7 +647,8 @@ def make_line(args, res, classes, world, cpu, extras):
     )
     if "e2e" in res:
         line["e2e"] = res["e2e"]
-    line.update(extras)
+    # an extra of a contract key's name (the fitting metric) stands beside it
+    line.update({("extra_" + k if k in line else k): v for k, v in extras.items()})
     return line
 
 
