@@ -256,14 +256,29 @@ lx3c_status lx3c_class_tables_check(int la, int lb, int lc, int bra_pure);
 lx3c_status lx3c_shape_query(int la, int lb, int lc, int bra_pure, int kab, int kc, int64_t naux, int ctas_per_sm,
                              int32_t* out);
 
+/*
+ * Host evaluation of the tables the kernels form (a 0|C) by, |a| = la..la+lb,
+ * for one primitive triple (for checks of their values; no device needed):
+ * VRR1 items (Eq. vrr1), the ket's harmonic weights, accumulators and the
+ * n-quantum gather (Sec. 2.5.4) on the solid-harmonic ket.
+ *   geom[12]  PA[3], (rho/gamma) PC[3], rho/gamma, 1/(2 gamma), X[3] =
+ *             (rho/zeta_c) PC, Y = 1/(2(gamma+zeta_c)); need not belong together
+ *   base      [00|0]^(m), m = lc..lc+la+lb
+ * *nrow rows, of which up to cap are written: rows[3*i..] the exponents of a,
+ * out[i*(2 lc+1) + C] its targets.
+ */
+lx3c_status lx3c_cvrr2_tables_eval(int la, int lb, int lc, const double* geom, const double* base, int32_t cap,
+                                   double* out, int32_t* rows, int32_t* nrow);
+
 /* Library's solid-harmonic matrix for shell l: out[(m+l)*ncart(l) + c]. */
 lx3c_status lx3c_solid_harmonics(int l, double* out);
 
 /*
- * n-quantum CVRR2 expansion (Sec. 2.5.4) of the contracted target (a 0|c)
- * as the library tabulates it: for bra exponents a[3], ket exponents c[3]
- * writes up to cap terms (e[3], k, n[3], coef) into terms[8*i..8*i+7] as
- * doubles and their count into *nterms.
+ * n-quantum CVRR2 expansion (Sec. 2.5.4) of the contracted target (a 0|c),
+ * the closed form on a Cartesian ket: for bra exponents a[3], ket exponents
+ * c[3] writes up to cap terms (e[3], k, n[3], coef) into terms[8*i..8*i+7] as
+ * doubles and their count into *nterms.  (The kernels' tables hold the same
+ * targets with the ket transform taken first: lx3c_cvrr2_tables_eval.)
  */
 lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap, double* terms,
                                  int32_t* nterms);

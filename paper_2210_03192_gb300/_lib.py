@@ -80,6 +80,8 @@ EXPORTS = {
     "lx3c_shape_hint": (ctypes.c_int, [ctypes.c_int] * 7),
     "lx3c_tile_hint": (ctypes.c_int, [ctypes.c_int] * 8),
     "lx3c_hrr_hint": (ctypes.c_int, [ctypes.c_int] * 5),
+    "lx3c_cvrr2_tables_eval": (ctypes.c_int, [ctypes.c_int] * 3 + [ctypes.c_void_p] * 2 + [ctypes.c_int32] +
+                               [ctypes.c_void_p] * 3),
     "lx3c_hrr_tables_check": (ctypes.c_int, [ctypes.c_int] * 5 + [ctypes.c_void_p, c_f64p]),
     "lx3c_set_orientation_threshold": (ctypes.c_int, [ctypes.c_double]),
     "lx3c_set_compensation": (ctypes.c_int, [ctypes.c_int]),

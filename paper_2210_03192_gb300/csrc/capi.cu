@@ -742,6 +742,28 @@ lx3c_status lx3c_hrr_tables_check(int la, int lb, int lc, int bra_pure, int vari
   return LX3C_OK;
 }
 
+lx3c_status lx3c_cvrr2_tables_eval(int la, int lb, int lc, const double* geom, const double* base, int32_t cap,
+                                   double* out, int32_t* rows, int32_t* nrow) {
+  if (!geom || !base || !nrow || (cap > 0 && (!out || !rows)) || cap < 0 || la < 0 || lb < 0 || lc < 0 ||
+      la > LX3C_LMAX_ORB || lb > LX3C_LMAX_ORB || lc > LX3C_LMAX_AUX)
+    return fail(LX3C_EINVAL, "cvrr2_tables_eval: bad argument");
+  try {
+    const ClassTables& ct = class_tables_variant(la, lb, lc, 0, 0);
+    const std::vector<double> v =
+        eval_targets(ct, geom, geom + 3, geom[6], geom[7], geom + 8, geom[11], base);
+    *nrow = ct.nkrow;
+    for (int r = 0; r < std::min<int>(cap, ct.nkrow); ++r) {
+      rows[3 * r] = ct.erow_xyz[r].x;
+      rows[3 * r + 1] = ct.erow_xyz[r].y;
+      rows[3 * r + 2] = ct.erow_xyz[r].z;
+      std::copy(v.begin() + (size_t)r * ct.nC, v.begin() + (size_t)(r + 1) * ct.nC, out + (size_t)r * ct.nC);
+    }
+  } catch (std::exception& e) {
+    return fail(LX3C_ENOTSUP, e.what());
+  }
+  return LX3C_OK;
+}
+
 lx3c_status lx3c_hrr_hint(int la, int lb, int lc, int bra_pure, int variant) {
   if (la < 0 || lb < 0 || lc < 0 || la > LX3C_LMAX_ORB + 1 || lb > LX3C_LMAX_ORB + 1 || lc > LX3C_LMAX_AUX ||
       variant < -1 || variant > 1)

@@ -29,17 +29,14 @@
 
 #include "boys_device.cuh"
 #include "fixed128.cuh"
+#include "harmonic_weights.h"
 #include "lx3c_internal.h"
 
 namespace lx3c {
 
 __constant__ double c_inv2m1[32];  // 1/(2m+1)
 
-// (l^2 - m^2) / (4 l^2 - 1): the solid-harmonic recursion
-// Q_{l+1,m} = z Q_{l,m} - c r^2 Q_{l-1,m}, l, m <= 5
-#define QC(l, m) ((double)((l) * (l) - (m) * (m)) / (4.0 * (l) * (l) - 1.0))
-#define QROW(l) QC(l, 0), QC(l, 1), QC(l, 2), QC(l, 3), QC(l, 4), QC(l, 5)
-__constant__ double c_q[36] = {0, 0, 0, 0, 0, 0, QROW(1), QROW(2), QROW(3), QROW(4), QROW(5)};
+__constant__ double c_q[36] = LX3C_QTABLE;
 
 template <int N>
 struct Int {
@@ -535,10 +532,10 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
         boys_scaled(d.boys_tab, d.boys_mid, d.boys_cL, d.L, lc, Tb, pref, sm + BUF_TG(d.V, 0, g, t), d.V.si);
       }
       __syncthreads();
-      // ---- weights W_{k,m} = Y^k s_{lc-k,m}(X), one item per (slot, |m|):
-      // (x + i y)^m, then Q_{l,m}(z, r^2) for l = m..lc by recursion; items of
-      // one m stand together (the loops' trip counts depend on it), and the
-      // last threads take them, as the first VRR1 level starts on the first
+      // ---- weights W_{k,m} = Y^k s_{lc-k,m}(X), one item per (slot, |m|);
+      // items of one m stand together (the loops' trip counts depend on it),
+      // and the last threads take them, as the first VRR1 level starts on the
+      // first
       {
         FDiv fS;
         const int ns = T * G, kmax = d.kmax;
@@ -561,34 +558,9 @@ __device__ __forceinline__ void tile_body(const ClassDesc& d, long long tile, do
             W[0] = 1.0;
             continue;
           }
-          const double X = F[4 * fs], Yc = F[5 * fs], Z = F[6 * fs];
-          const double r2 = fma(Z, Z, fma(Yc, Yc, X * X));
-          double A = X, B = Yc;
-          for (int i = 1; i < m; ++i) {
-            const double An = fma(A, X, -B * Yc);
-            B = fma(A, Yc, B * X);
-            A = An;
-          }
-          double q0 = 0.0, q1 = 1.0;
-          for (int l = m; l <= lc; ++l) {
-            const int k = lc - l;
-            if (k <= kmax) {
-              const double v = k ? q1 * F[(6 + k) * fs] : q1;
-              const int o = k * (2 * lc + 2 - k) + l;  // m = 0 of degree l
-              if (m == 0) {
-                W[o * ws] = v;
-              } else {
-                W[(o + m) * ws] = v * A;
-                W[(o - m) * ws] = v * B;
-              }
-            }
-            if (l < lc) {
-              double n = Z * q1;
-              if (l > m) n = fma(-c_q[l * 6 + m] * r2, q0, n);
-              q0 = q1;
-              q1 = n;
-            }
-          }
+          harmonic_weights(
+              lc, kmax, m, F[4 * fs], F[5 * fs], F[6 * fs], c_q, [&](int k) { return F[(6 + k) * fs]; },
+              [&](int i, double v) { W[i * ws] = v; });
         }
       }
       // ---- VRR1, level by level (Eq. vrr1).  A level is few targets and a

@@ -258,6 +258,9 @@ std::string check_class_tables(const ClassTables& ct);  // "" when every table i
 // Largest relative error of the class's HRR tables applied to moment
 // integrals (exact for any weight), see lx3c_hrr_tables_check.
 double hrr_moment_error(const ClassTables& ct, const double AB[3]);
+// Host evaluation of the class's (a 0|C) tables, see lx3c_cvrr2_tables_eval.
+std::vector<double> eval_targets(const ClassTables& ct, const double PA[3], const double f[3], double rg, double h,
+                                 const double X[3], double Y, const double* base);
 LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit);
 LaunchShape largest_tile(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas);
 LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas);

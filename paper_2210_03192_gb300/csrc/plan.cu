@@ -30,6 +30,7 @@
 #include <string>
 #include <tuple>
 
+#include "harmonic_weights.h"
 #include "lx3c_internal.h"
 
 namespace lx3c {
@@ -666,6 +667,30 @@ std::string check_class_tables(const ClassTables& ct) {
     for (size_t q = 0; q < ct.bbent.size(); ++q)
       if (ct.bbent[q].x < 0 || ct.bbent[q].x >= ct.ncB) return bad("bra B entry", (long long)q);
   return "";
+}
+
+// The tables behind (a 0|C) on one primitive, as the kernel walks them: VRR1
+// items from base[i] = [00|0]^(lc+i), weights, accumulators, gather.
+std::vector<double> eval_targets(const ClassTables& ct, const double PA[3], const double f[3], double rg, double h,
+                                 const double X[3], double Y, const double* base) {
+  static const double q[36] = LX3C_QTABLE;
+  const int Lab = ct.la + ct.lb, lc = ct.lc;
+  std::vector<double> v(ct.NV), W(ct.NW, 1.0), P(ct.NACC), out((size_t)ct.nkrow * ct.nC);
+  for (int i = 0; i <= Lab; ++i) v[i] = base[i];
+  for (const uint4& it : ct.vtab) {
+    const int axis = (it.z >> 16) & 0xF, nq = (it.z >> 20) & 0xF;
+    double x = PA[axis] * v[it.x >> 16] - f[axis] * v[it.y & 0xFFFF];
+    if (nq) x += nq * h * (v[it.y >> 16] - rg * v[it.z & 0xFFFF]);
+    v[it.x & 0xFFFF] = x;
+  }
+  for (int m = 0; m <= lc && lc > 0; ++m)
+    harmonic_weights(
+        lc, ct.kmax, m, X[0], X[1], X[2], q, [&](int k) { return std::pow(Y, k); }, [&](int i, double w) { W[i] = w; });
+  for (int i = 0; i < ct.NACC; ++i) P[i] = v[ct.atab[i] & 0xFFFF] * W[ct.atab[i] >> 16];
+  for (size_t id = 0; id < out.size(); ++id)
+    for (int t = ct.gptr[id]; t < ct.gptr[id + 1]; ++t)
+      out[id] += ct.pal[ct.gterm[t] >> kGatherBits] * P[ct.gterm[t] & kGatherMask];
+  return out;
 }
 
 // HRR holds exactly for moment integrals M(a, b) = int (x-A)^a (x-B)^b w(x) dx
