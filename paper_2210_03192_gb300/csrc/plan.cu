@@ -900,7 +900,8 @@ LaunchShape largest_tile(const ClassTables& ct, int Kab, int Kc, long long naux,
 // when nothing fits.  For two, the default: wide tiles (T >= 64) only with three
 // primitives side by side, as each chunk of primitives costs the barriers of
 // its stages ((pp|p) K = 36: T, G = 128, 2 1.53 ms, 64, 6 1.35; (pp|d) K = 9:
-// 128, 1 0.90, 64, 3 0.77); and a third CTA (of 384 threads) where it takes no
+// 128, 1 0.90, 64, 3 0.77; asking for two gives the same shapes, as a tile of
+// two leaves room for the three CTAs below); and a third CTA (of 384 threads) where it takes no
 // fewer triples a tile, or still a full warp of them, and two primitives: the
 // barriers of three overlap better ((fd|f) K = 9 8, 5 7.64 ms, 8, 3 6.76; (ff|d)
 // K = 4 8, 4 6.25, 8, 2 5.43; (gg|i) K = 36 92.4 -> 86.0), while fewer triples lose
