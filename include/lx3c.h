@@ -232,12 +232,14 @@ lx3c_status lx3c_hrr_tables_check(int la, int lb, int lc, int bra_pure, int vari
  *   more compact centre (a second, transposed launch).  Smaller values split
  *   more pairs (more accurate, more post-contraction work).  amp_max >= 1,
  *   or 0 for the default 300; else LX3C_EINVAL.
- * lx3c_set_compensation: bits selecting compensated (Dot2: TwoProduct by FMA
- *   and TwoSum) summation in the contracted stages -- bit 0 the n-quantum
- *   CVRR2 gather (Sec. 2.5.4), bit 1 the ket Cartesian-to-solid-harmonic
- *   transform; 0 (the default) for plain FMA chains.  bits outside 0..3 give
- *   LX3C_EINVAL.  (Both settings act on launches that form integrals; the
- *   Hermite-basis DF-J and gradient have neither an HRR nor these stages.)
+ * lx3c_set_compensation: compensated (Dot2: TwoProduct by FMA and TwoSum)
+ *   summation of the n-quantum CVRR2 gather (Sec. 2.5.4), which delivers
+ *   solid-harmonic ket components: bit 0 for the gather, bit 1 for the ket
+ *   transform it contains; either selects the one sum.  0 (the default) for
+ *   plain FMA chains.  bits outside 0..3 give LX3C_EINVAL.  (Both settings
+ *   act on the tile kernel's launches that form integrals; the register-
+ *   resident (s s|C) and (p s|C) kernels have no gather, the Hermite-basis
+ *   DF-J and gradient neither an HRR nor this stage.)
  */
 lx3c_status lx3c_set_orientation_threshold(double amp_max);
 lx3c_status lx3c_set_compensation(int bits);

@@ -510,8 +510,8 @@ def set_orientation_threshold(amp_max=0.0):
 
 
 def set_compensation(bits=0):
-    """Compensated summation in later plans' contracted stages: bit 0 gather,
-    bit 1 ket transform (lx3c_set_compensation)."""
+    """Compensated summation of later plans' gather, which holds the ket
+    transform: bit 0 or bit 1 (lx3c_set_compensation)."""
     check(_lib.load().lx3c_set_compensation(int(bits)), "lx3c_set_compensation")
 
 
