@@ -273,6 +273,7 @@ struct lx3c_dfj {
   long long nao = 0, naux_ao = 0;
   double tol = 0;
   int natom = 0;
+  int nsm = 0;
   bool gradient = false;
   std::vector<DfjGroup> groups;
   // records of every group: the groups outside the Hermite basis first
@@ -331,6 +332,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   p->orb = orb;
   p->aux = aux;
   p->tol = schwarz_tol;
+  p->nsm = dev_nsm(ds);
   std::vector<int> ao(orb->nshell + 1, 0), aq(aux->nshell + 1, 0);
   for (int64_t s = 0; s < orb->nshell; ++s) ao[s + 1] = ao[s] + 2 * orb->l[s] + 1;
   for (int64_t s = 0; s < aux->nshell; ++s) aq[s + 1] = aq[s] + 2 * aux->l[s] + 1;
@@ -618,6 +620,13 @@ lx3c_status lx3c_dfj_execute_multi(lx3c_dfj* p, int nd, const double* D, const d
       d.J = J;
       const long long kAB = ((long long)d.onA * d.onB + 3) & ~3LL, kR = ((long long)d.T * d.nC + 3) & ~3LL;
       d.dscr = place_epilogue_scratch(d, 8 * (kAB + kR));
+      // the register-resident kernels from two warps per SM on: a warp runs its
+      // tiles' primitives, components and densities one after another, 170 us
+      // for (s s|h) whatever the number of warps, where the tile kernel spreads
+      // a tile over its threads (2 atoms, eight densities: 3.45 ms a build with
+      // the register kernels, 2.73 without; 4 atoms 3.13 and 2.52, 16 atoms
+      // 21.7 and 25.2)
+      if (d.wtiles && (d.nwtiles * d.warpW + 31) / 32 < 2LL * p->nsm) d.wtiles = nullptr;
       if ((long long)d.smem_doubles * 8 > 232448) return dfail(LX3C_ENOTSUP, "execute_multi: scratch does not fit");
       descs.push_back(d);
       grids.push_back(L.grid);

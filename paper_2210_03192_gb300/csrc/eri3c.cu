@@ -1485,7 +1485,8 @@ static bool three_ctas(int smem_bytes) { return smem_bytes <= 233472 / 3 - 1024;
 // 1) with 1 <= lc <= 4 or contracted; (p s|s) with one primitive per triple
 // measured faster on the tile kernel.  Stores and per-integral DF-J, for one
 // density or several, the latter with the kernels' own tiles (several densities
-// on 16 atoms: these classes 9.3 of 26.3 ms on the tile kernel).
+// on 16 atoms: these classes 9.3 of 26.3 ms on the tile kernel; the caller
+// leaves out the tiles of launches too small for it).
 static bool on_register_kernel(const ClassDesc& d) {
   if (d.digest != 0 && !((d.digest == 1 || d.digest == 4) && d.wtiles)) return false;
   if (d.la == 0 && d.lb == 0) return d.orient == 0;
