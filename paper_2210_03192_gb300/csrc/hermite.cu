@@ -348,7 +348,8 @@ struct HermPairArgs {
   const double* sph;   // solid-harmonic matrices
   const int* sphoff;
   const double* D;
-  long long ldD, npair;
+  long long ldD;
+  int chunk;           // primitives of a pair per warp
   unsigned long long* Jacc;
   unsigned long long* facc;
   const int* atom;     // atom of each orbital shell
@@ -482,9 +483,18 @@ __device__ __forceinline__ double dens_yz(const double* Dc, int nb, int da, int 
   return v;
 }
 
+// The per-pair kernels run one warp per shell pair and range of `chunk` of its
+// primitives (blockIdx.y).  A warp takes some 10 us a primitive, so pairs of
+// many primitives are cut where there are few pairs (one (p p| pair of 256
+// primitives: 3.2 ms a build uncut, 0.12 cut); the more ranges, the more
+// often the pair's density is transformed and its J block added.
+__device__ __forceinline__ int2 prim_range(const HermPairArgs& g, const int4& p2) {
+  const int k0 = (int)blockIdx.y * g.chunk;
+  return int2{k0, min(p2.w, k0 + g.chunk)};
+}
+
 // Primitive records, and with dens the Hermite densities H~_a = K h^|a| sum
-// Dc E~_a (gradient: the three arrays of (a_i + 1) H~_a at a + 1_i).  One warp
-// per shell pair.
+// Dc E~_a (gradient: the three arrays of (a_i + 1) H~_a at a + 1_i).
 template <bool kGrad>
 __global__ void __launch_bounds__(32) herm_pre_kernel(const __grid_constant__ HermPairArgs g, int dens) {
   extern __shared__ double sm[];
@@ -497,8 +507,10 @@ __global__ void __launch_bounds__(32) herm_pre_kernel(const __grid_constant__ He
   double* E = Dc + na * nb;
   double* Hs = E + 3 * (la + 1) * (lb + 1) * nt;  // also dens_cart's scratch
   const int sj = nt, si = (lb + 1) * nt, sa = (la + 1) * si;
+  const int2 kr = prim_range(g, p2);
+  if (kr.x >= kr.y) return;
   if (dens) dens_cart(g, la, lb, p2, Hs, Dc);
-  for (int k = 0; k < p2.w; ++k) {
+  for (int k = kr.x; k < kr.y; ++k) {
     const int prim = p1.w + k, ab = __ldg(L.primab + prim);
     const PairGeom pg = pair_geom(g.orb, p1.x, p1.y, ab / Kb, ab % Kb);
     if (lane == 0) {
@@ -577,7 +589,7 @@ __device__ __forceinline__ void potentials(const HermLabDev& L, int prim, int de
 }
 
 // J block of each pair: J_ab = wj sum over primitives of E~ y, through the
-// Cartesian block, one warp per shell pair.
+// Cartesian block.
 __global__ void __launch_bounds__(32) herm_post_kernel(const __grid_constant__ HermPairArgs g) {
   extern __shared__ double sm[];
   const int lane = threadIdx.x;
@@ -590,8 +602,10 @@ __global__ void __launch_bounds__(32) herm_post_kernel(const __grid_constant__ H
   double* Ys = E + 3 * (la + 1) * (lb + 1) * nt;
   double* Ns = Ys + nherm(Lab);  // [(Lab + 1)(Lab + 2) / 2], also the transform's scratch
   const int sj = nt, si = (lb + 1) * nt, sa = (la + 1) * si;
+  const int2 kr = prim_range(g, p2);
+  if (kr.x >= kr.y) return;
   for (int w = lane; w < na * nb; w += 32) Jc[w] = 0.0;
-  for (int k = 0; k < p2.w; ++k) {
+  for (int k = kr.x; k < kr.y; ++k) {
     const int prim = p1.w + k, ab = __ldg(L.primab + prim);
     const PairGeom pg = pair_geom(g.orb, p1.x, p1.y, ab / Kb, ab % Kb);
     __syncwarp();
@@ -660,9 +674,11 @@ __global__ void __launch_bounds__(32) herm_force_kernel(const __grid_constant__ 
   double* F = E + 3 * (la + 2) * (lb + 1) * nt;        // derivative tables, (la, lb)
   double* Ys = F + 3 * (la + 1) * (lb + 1) * nt;       // also dens_cart's scratch
   const int sj = nt, si = (lb + 1) * nt, sa = (la + 2) * si, sf = (la + 1) * si;
+  const int2 kr = prim_range(g, p2);
+  if (kr.x >= kr.y) return;
   dens_cart(g, la, lb, p2, Ys, Dc);
   double dA[3] = {0.0, 0.0, 0.0}, dP[3] = {0.0, 0.0, 0.0};
-  for (int k = 0; k < p2.w; ++k) {
+  for (int k = kr.x; k < kr.y; ++k) {
     const int prim = p1.w + k, ab = __ldg(L.primab + prim);
     const PairGeom pg = pair_geom(g.orb, p1.x, p1.y, ab / Kb, ab % Kb);
     __syncwarp();
@@ -1046,6 +1062,7 @@ struct HermPlan {
   HermPairArgs pa;
   HermArgs ma;
   int smem_pre = 0, smem_post = 0;
+  int nchunk = 1;              // ranges of a pair's primitives (HermPairArgs::chunk)
   double flops = 0, max_adds = 0;
 };
 
@@ -1165,6 +1182,12 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     labs.push_back(std::move(L));
   }
   p->npair = (long long)pairs.size();
+  // ranges of primitives: 16 warps an SM's worth of them, four or more each
+  const int per = (int)std::max<long long>(4, p->nprim / (dev_nsm(ds) * 16));
+  int most = 1;
+  for (const int4& q : pairs2) most = std::max(most, q.w);
+  p->nchunk = (most + per - 1) / per;
+  p->pa.chunk = per;
   p->smem_pre = smem_pre * 8;
   p->smem_post = smem_post * 8;
   // classes and their tables
@@ -1315,7 +1338,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       set_last_error("dfj: too many tiles");
       return LX3C_ENOTSUP;
     }
-  p->max_adds = 4 * 32.0 * (double)tiles.size() + 2.0 * (double)p->npair;
+  p->max_adds = 4 * 32.0 * (double)tiles.size() + 2.0 * (double)p->npair * p->nchunk;
   // ---- one allocation: tables and lists (uploaded), then the work buffers
   std::vector<double> sph;
   std::vector<int> sphoff;
@@ -1433,7 +1456,6 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   pa.sph = (const double*)(A + o_sph);
   pa.sphoff = (const int*)(A + o_sphoff);
   pa.ldD = nao;
-  pa.npair = p->npair;
   pa.atom = (const int*)(A + o_atom);
   HermArgs& ma = p->ma;
   ma.cls = (const HermCls*)(A + o_cls);
@@ -1463,6 +1485,8 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
 
 namespace {
 
+dim3 pair_grid(const HermPlan* p) { return dim3((unsigned)p->npair, (unsigned)p->nchunk); }
+
 cudaError_t herm_begin(HermPlan* p, const double* D, bool dens, bool y, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (y) e = cudaMemsetAsync(p->arena + p->zero_off, 0, p->zero_bytes, st);
@@ -1471,9 +1495,9 @@ cudaError_t herm_begin(HermPlan* p, const double* D, bool dens, bool y, cudaStre
   HermPairArgs a = p->pa;
   a.D = D;
   if (p->grad)
-    herm_pre_kernel<true><<<(unsigned)p->npair, 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
+    herm_pre_kernel<true><<<pair_grid(p), 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
   else
-    herm_pre_kernel<false><<<(unsigned)p->npair, 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
+    herm_pre_kernel<false><<<pair_grid(p), 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1507,7 +1531,7 @@ cudaError_t herm_execute(HermPlan* p, const double* D, const double* c, unsigned
   if (e != cudaSuccess || !Jacc) return e;
   HermPairArgs b = p->pa;
   b.Jacc = Jacc;
-  herm_post_kernel<<<(unsigned)p->npair, 32, p->smem_post, st>>>(b);
+  herm_post_kernel<<<pair_grid(p), 32, p->smem_post, st>>>(b);
   return cudaGetLastError();
 }
 
@@ -1523,7 +1547,7 @@ cudaError_t herm_gradient(HermPlan* p, const double* D, const double* c, unsigne
   HermPairArgs b = p->pa;
   b.D = D;
   b.facc = facc;
-  herm_force_kernel<<<(unsigned)p->npair, 32, p->smem_post, st>>>(b);
+  herm_force_kernel<<<pair_grid(p), 32, p->smem_post, st>>>(b);
   return cudaGetLastError();
 }
 
