@@ -8,10 +8,10 @@
 // Setup (lx3c_dfj_plan): Schwarz-type screening estimates Q_ab, Q_P; every
 // (la lb | lc) class group keeps its ket shells sorted by Q_P so that the
 // ket shells surviving Q_ab Q_P >= tol for a pair form a prefix of the list.
-// Execution: the (s s|C) and (p s|C) groups run the register-resident class
-// kernels in digest mode on tabulated tiles (sub-pair, ket range); all others,
-// and the gradient of every group, run in the Hermite basis (hermite.cu),
-// which forms no integral.  gamma, J and the gradient are accumulated into
+// Execution: the (s s|C) and (p s|C) groups, and strongly contracted ones of low
+// angular momentum, run the class kernels in digest mode on tabulated tiles
+// (sub-pair, ket range); all others, and the gradient of every group, run in
+// the Hermite basis (hermite.cu), which forms no integral.  gamma, J and the gradient are accumulated into
 // exact fixed-point accumulators (fixed128.cuh), so the result does not
 // depend on the order of the contributions; final kernels convert them to
 // FP64 and symmetrise J.
@@ -34,6 +34,7 @@
 #include "fixed128.cuh"
 #include "hermite.h"
 #include "lx3c_internal.h"
+#include "primitives.h"
 
 namespace lx3c {
 cudaError_t launch_precompute(const DevBasis& orb, const int32_t* pairs, long long npair, int Ka, int Kb, double* rec,
@@ -191,14 +192,68 @@ int kets_kept(double qpair, const std::vector<double>& qket, double tol) {
   return lo;
 }
 
-// Every group runs in the Hermite basis except those with a register-resident
-// class kernel, (s s|C) and (p s|C) with lc <= 4 (contracted when lc = 0):
-// there the digestion is a few FMAs per contracted triple, where the Hermite
-// form pays its two contractions per primitive triple.
-bool use_hermite(const HermBra& b, const HermKet& k) {
-  if (b.la + b.lb == 0) return false;
-  if (b.la + b.lb == 1) return k.lc > 4 || (k.lc == 0 && b.Ka * b.Kb * k.Kc == 1);
-  return true;
+// The modes (hermite.h) in which a group runs in the Hermite basis: all, except
+// where its integrals cost less.  The Hermite form pays its contractions per
+// primitive triple, where the digestion of integrals is a few FMAs per
+// contracted one: the groups with a register-resident class kernel, (s s|C) and
+// (p s|C) with lc <= 4 (contracted when lc = 0), never do, and strongly
+// contracted ones of low angular momentum not in every mode.  For these the
+// line is drawn on operation counts.  Over 197 classes (la, lb <= 4, lc <= 4, 4
+// to 100 primitive triples a triple) the time of the Hermite form over the tile
+// kernel's is, to 13 %, the ratio of their counts (the contracted stages taken
+// 1.5 times), times 0.8 beyond lc = 0; the tile kernel is taken where that makes
+// it a tenth faster, or faster at all for 18 primitive triples and more up to
+// la + lb = 4, where it comes out low.  Both outputs together, ms before and
+// after: (d s|s) K = 36 5.5 and 3.0, (f s|d) 16.1 and 10.6, (p p|s) 4.3 and 2.6,
+// (p p|d) 6.7 and 5.2; left in the Hermite basis: (p p|s) K = 4 0.54 (tile kernel
+// 0.66), (f f|s) K = 36 4.2 (5.3).  gamma alone is the cheaper half of the
+// Hermite form and always its.
+int hermite_modes(const HermBra& b, const HermKet& k) {
+  if (b.la + b.lb == 0) return 0;
+  if (b.la + b.lb == 1 && k.lc <= 4) return k.lc == 0 && b.Ka * b.Kb * k.Kc == 1 ? kHermBuild : 0;
+  // (the tile kernel runs a tile's primitives in chunks one after another, a
+  // Hermite launch spreads them: fewer tiles than SMs go there.  Under 32 tiles
+  // an SM the weakly contracted gain less than their launches cost: a batch of
+  // three molecules 8.37 -> 8.6 ms with (d s|s), (f s|s), (g s|s) on the tile
+  // kernel.)
+  const double n = b.nprim * k.Kc;
+  if (n < 4 || (double)b.q.size() * ((k.shells.size() + 31) / 32) < (n >= 18 ? 152 : 32 * 152)) return kHermBuild;
+  try {
+    const ClassTables& ct = class_tables(b.la, b.lb, k.lc, 1);
+    const double nint = (2.0 * b.la + 1) * (2 * b.lb + 1) * (2 * k.lc + 1);
+    const double tile = ct.flops_prim * n + 1.5 * (ct.flops_contr + 4.0 * nint);
+    const double least = n >= 18 && b.la + b.lb <= 4 ? 1.0 : 1.1;
+    int modes = 1 << 1;
+    for (int mode = 2; mode <= 3; ++mode)
+      if ((k.lc == 0 ? 1.0 : 0.8) * n * herm_class_flops(b.la + b.lb, k.lc, mode) < least * tile) modes |= 1 << mode;
+    return modes;
+  } catch (std::exception&) {
+    return kHermBuild;  // no tile kernel for the class
+  }
+}
+
+// Contributing primitive pairs of a bra class's shell pairs, averaged over up
+// to 64 of them.
+double mean_prims(const lx3c_basis* orb, const HermBra& b) {
+  if (b.Ka * b.Kb < 4) return b.Ka * b.Kb;
+  const size_t np = b.q.size(), step = std::max<size_t>(1, np / 64);
+  long long kept = 0, seen = 0;
+  std::vector<double> q(b.Ka * b.Kb), K(b.Ka * b.Kb);
+  for (size_t i = 0; i < np; i += step, ++seen) {
+    const int sa = b.pairs[2 * i], sb = b.pairs[2 * i + 1];
+    double ab2 = 0, qmax = 0;
+    for (int x = 0; x < 3; ++x) {
+      const double d = orb->xyz[3 * sa + x] - orb->xyz[3 * sb + x];
+      ab2 += d * d;
+    }
+    for (int r = 0; r < b.Ka * b.Kb; ++r) {
+      const long long ia = orb->off[sa] + r / b.Kb, ib = orb->off[sb] + r % b.Kb;
+      q[r] = prim_bound(orb->exps[ia], orb->coefs[ia], orb->exps[ib], orb->coefs[ib], ab2, b.la, b.lb, &K[r]);
+      qmax = std::max(qmax, q[r]);
+    }
+    for (int r = 0; r < b.Ka * b.Kb; ++r) kept += prim_kept(K[r], q[r], qmax);
+  }
+  return (double)kept / (double)std::max(1LL, seen);
 }
 
 // One device allocation for everything a plan keeps: arrays to upload
@@ -260,9 +315,10 @@ struct DfjGroup {
   double* d_auxrec = nullptr;
   double* d_auxc = nullptr;
   DfjLaunch L[2];
-  // the group runs in the Hermite basis; its class launches L serve the
-  // several-density build alone
-  bool herm = false;
+  // the modes in which the group runs in the Hermite basis; its class launches
+  // L serve the others and the several-density build
+  int herm = 0;
+  bool hermite(int mode) const { return herm >> mode & 1; }
 };
 
 }  // namespace
@@ -276,10 +332,11 @@ struct lx3c_dfj {
   int nsm = 0;
   bool gradient = false;
   std::vector<DfjGroup> groups;
-  // records of every group: the groups outside the Hermite basis first
+  // records of every group: those never in the Hermite basis first, then those
+  // sometimes; a mode takes as many as it runs class launches of
   PrecomputeJob* d_jobs = nullptr;
-  int njobs = 0, njobs_plain = 0;
-  long long job_blocks = 0, job_blocks_plain = 0;
+  int njobs = 0, njobs_mode[4] = {0, 0, 0, 0};
+  long long job_blocks = 0, job_blocks_mode[4] = {0, 0, 0, 0};
   char* arena = nullptr;            // every device array of the groups, and the accumulators
   HermPlan* hj = nullptr;           // gamma and J of the Hermite groups
   HermPlan* hg = nullptr;           // gradient of every group
@@ -360,12 +417,13 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   std::vector<HermBra> hbra;
   std::vector<HermKet> hket;
   for (auto& bk : bra) {
-    HermBra h{std::get<0>(bk.first), std::get<2>(bk.first), std::get<1>(bk.first), std::get<3>(bk.first), {}, {}};
+    HermBra h{std::get<0>(bk.first), std::get<2>(bk.first), std::get<1>(bk.first), std::get<3>(bk.first), {}, {}, 0.0};
     for (auto& e : bk.second) {
       h.pairs.push_back(e.first);
       h.pairs.push_back(e.second);
     }
     h.q = braq[bk.first];
+    h.nprim = mean_prims(orb, h);
     hbra.push_back(std::move(h));
   }
   for (auto& kk : kets) {
@@ -382,7 +440,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       g.la = hb.la; g.Ka = hb.Ka;
       g.lb = hb.lb; g.Kb = hb.Kb;
       g.lc = hk.lc; g.Kc = hk.Kc;
-      g.herm = use_hermite(hb, hk);
+      g.herm = hermite_modes(hb, hk);
       g.auxs = hk.shells;
       for (size_t i = 0; i < hb.q.size(); ++i) {
         const int lo = kets_kept(hb.q[i], hk.q, schwarz_tol);
@@ -397,9 +455,9 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       p->groups.push_back(std::move(g));
     }
   }
-  rc = herm_build(&p->hj, orb, aux, hbra, hket, use_hermite, kets_kept, schwarz_tol, false, p->nao, st);
+  rc = herm_build(&p->hj, orb, aux, hbra, hket, hermite_modes, kets_kept, schwarz_tol, false, p->nao, st);
   if (!rc && want_grad)
-    rc = herm_build(&p->hg, orb, aux, hbra, hket, [](const HermBra&, const HermKet&) { return true; }, kets_kept,
+    rc = herm_build(&p->hg, orb, aux, hbra, hket, [](const HermBra&, const HermKet&) { return kHermGrad; }, kets_kept,
                     schwarz_tol, true, p->nao, st);
   if (rc) return rc;
   // contributions to one element of the gradient's fixed-point accumulators
@@ -479,8 +537,8 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
           tris += g.counts[sp.x];
           primtris += (double)g.counts[sp.x] * sp.z * g.Kc;
         }
-        g.flops += g.herm ? primtris * herm_class_flops(g.la + g.lb, g.lc)
-                          : primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nbra * nket);
+        g.flops += g.hermite(3) ? primtris * herm_class_flops(g.la + g.lb, g.lc, 3)
+                                : primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nbra * nket);
       }
       std::vector<int4> tiles;
       for (size_t s = 0; s < sub[o].size(); ++s) {
@@ -493,7 +551,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       arena.add(&L.d_sub, sub[o].data(), sub[o].size());
       arena.add(&L.d_prim, prim[o].data(), prim[o].size());
       arena.add(&L.d_tiles, tiles.data(), tiles.size());
-      if (!g.herm) {
+      if (!g.herm && g.la + g.lb <= 1) {
         // tiles of the register-resident kernel: the width that leaves fewest
         // lanes idle at the ends of the ket lists (a small charge for the
         // sub-pairs of unequal contraction that then share a warp), the most
@@ -544,18 +602,18 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       d.pair_ao = g.d_pair_ao; d.aux_ao = g.d_aux_ao;
     }
   std::vector<PrecomputeJob> jobs;
-  for (int herm = 0; herm < 2; ++herm) {
-    for (auto& g : p->groups)
-      if ((int)g.herm == herm) {
-        jobs.push_back(PrecomputeJob{g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
-                                     g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, p->job_blocks});
-        p->job_blocks += jobs.back().blocks();
-      }
-    if (!herm) {
-      p->njobs_plain = (int)jobs.size();
-      p->job_blocks_plain = p->job_blocks;
+  for (int part = 0; part < 3; ++part)
+    for (auto& g : p->groups) {
+      if (part != (g.herm == 0 ? 0 : (g.herm == kHermBuild ? 2 : 1))) continue;
+      jobs.push_back(PrecomputeJob{g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
+                                   g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, p->job_blocks});
+      p->job_blocks += jobs.back().blocks();
+      for (int mode = 1; mode <= 3; ++mode)
+        if (!g.hermite(mode)) {
+          p->njobs_mode[mode] = (int)jobs.size();
+          p->job_blocks_mode[mode] = p->job_blocks;
+        }
     }
-  }
   p->njobs = (int)jobs.size();
   if (!jobs.empty())
     DCUDA(cudaMemcpyAsync(p->d_jobs, jobs.data(), jobs.size() * sizeof(PrecomputeJob), cudaMemcpyHostToDevice, st));
@@ -564,11 +622,11 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   return LX3C_OK;
 }
 
-// The pair and ket records of a plan's groups (all, or those that do not run in
-// the Hermite basis).
-static cudaError_t group_records(const lx3c_dfj* p, bool all, cudaStream_t st) {
-  return launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->d_jobs, all ? p->njobs : p->njobs_plain,
-                                all ? p->job_blocks : p->job_blocks_plain, st);
+// The pair and ket records of a plan's groups: those of the mode's class
+// launches, or of all (mode 0).
+static cudaError_t group_records(const lx3c_dfj* p, int mode, cudaStream_t st) {
+  return launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->d_jobs, mode ? p->njobs_mode[mode] : p->njobs,
+                                mode ? p->job_blocks_mode[mode] : p->job_blocks, st);
 }
 
 lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, double* gamma, double* J, void* stream) {
@@ -578,9 +636,10 @@ lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, doub
   if (gamma) DCUDA(cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, st));
   if (J) DCUDA(cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, st));
   if (p->hj) DCUDA(herm_execute(p->hj, D, c, gamma ? p->d_gacc : nullptr, J ? p->d_Jacc : nullptr, st));
-  DCUDA(group_records(p, false, st));
+  const int mode = (gamma ? 1 : 0) | (J ? 2 : 0);
+  DCUDA(group_records(p, mode, st));
   for (auto& g : p->groups) {
-    if (g.herm) continue;
+    if (g.hermite(mode)) continue;
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       ClassDesc d = L.desc;
@@ -634,7 +693,7 @@ lx3c_status lx3c_dfj_execute_multi(lx3c_dfj* p, int nd, const double* D, const d
   if (gamma) DCUDA(cudaMemsetAsync(gamma, 0, (size_t)nd * cstride * 8, st));
   if (J) DCUDA(cudaMemsetAsync(J, 0, (size_t)nd * dstride * 8, st));
   size_t li = 0;
-  DCUDA(group_records(p, true, st));
+  DCUDA(group_records(p, 0, st));
   for (auto& g : p->groups) {
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
@@ -695,9 +754,9 @@ lx3c_status lx3c_dfj_info(const lx3c_dfj* p, double* out, int n) {
     tasks += (double)g.ntasks;
     nint += g.nint;
     flops += g.flops;
-    if (!g.herm) launches += (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
+    if (!g.hermite(3)) launches += (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
   }
-  launches += p->njobs_plain > 0;
+  launches += p->njobs_mode[3] > 0;
   const double v[] = {(double)p->groups.size(), tasks, nint, flops, launches, (double)p->nao, (double)p->naux_ao,
                       (double)p->natom, gflops, glaunches, slots};
   for (int i = 0; i < n && i < 11; ++i) out[i] = v[i];
@@ -831,8 +890,8 @@ cudaError_t capture_branches(lx3c_batch* b, const std::vector<ClassDesc>& descs,
       lx3c_dfj* p = b->mols[m];
       cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
       cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
-      group_records(p, false, cap);
-      kernels += p->njobs_plain > 0;
+      group_records(p, 3, cap);
+      kernels += p->njobs_mode[3] > 0;
     }
     cudaEventRecord(fork, cap);
     double load[kBranches] = {};
@@ -1036,9 +1095,9 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
   b->plain_launches = 0;
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];
-    b->plain_launches += 2 + (p->njobs_plain > 0) + (p->hj ? herm_launches(p->hj) : 0);
+    b->plain_launches += 2 + (p->njobs_mode[3] > 0) + (p->hj ? herm_launches(p->hj) : 0);
     for (auto& g : p->groups) {
-      if (g.herm) continue;
+      if (g.hermite(3)) continue;
       for (auto& L : g.L) {
         if (!L.ntiles) continue;
         ++b->plain_launches;
@@ -1096,8 +1155,8 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     lx3c_dfj* p = b->mols[m];
     cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
     cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
-    group_records(p, false, cap);
-    b->graph_kernels += p->njobs_plain > 0;
+    group_records(p, 3, cap);
+    b->graph_kernels += p->njobs_mode[3] > 0;
   }
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];
