@@ -1343,7 +1343,15 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     HermPlan::Tier& t = p->tiers.back();
     t.smem = std::max(t.smem, x.smem);
     const int W = x.c.W, NP = 32 / W;
-    const long long step = NP * std::max<long long>(1, std::min<long long>(64, (long long)(target / x.instr)));
+    // a tile ends with three atomics for each of a lane's sums (a ket's gamma, or
+    // its force), which cost the chip about as much as 30 FP64 instructions
+    // each: tiles of a few primitives on light classes are mostly flushes (20
+    // contracted p shells over 160 kets, gamma alone 1.18 ms), so a tile has
+    // three times their cost of work, if that leaves a warp for each slot (0.44;
+    // the batch of three molecules 8.34 -> 8.08)
+    const double flush = 100.0 * 3.0 * (grad ? 3 : x.c.nC);
+    const double work = std::max(target, std::min(flush, 16.0 * target));
+    const long long step = NP * std::max<long long>(1, std::min<long long>(64, (long long)(work / x.instr + 0.5)));
     for (int k0 = 0; k0 < x.c.nket; k0 += W) {
       // pairs keeping ket k0: a prefix, save for pairs this class does not use
       size_t np = x.counts.size();

@@ -1,0 +1,36 @@
+"""Small Hermite-basis builds of light classes are not mostly the atomics their
+tiles end with: gamma of 20 contracted p shells over 160 kets took 1.18 ms in
+tiles of one or two primitives (0.91 when the integrals were formed), 0.44 in
+tiles with work enough to carry them.  Values against the several-density
+build, to rounding."""
+import numpy as np
+import pytest
+
+from paper_2210_03192_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def test_gamma_of_contracted_p_shells():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2210_03192_gb300 as lx
+    rng = np.random.default_rng(3)
+    orb = W.random_shells(rng, 20, 1, 6, 3.0, 0.1, 30.0)
+    aux = W.concat(*[W.random_shells(rng, n, l, 1, 3.0, 0.2, 3.0) for l, n in ((0, 60), (2, 60), (4, 40))])
+    plan = lx.DFJPlan(orb, aux, 0.0)
+    D = torch.tensor(W.density(rng, plan.nao), device="cuda")
+    c = torch.tensor(rng.standard_normal(plan.naux_ao), device="cuda")
+    g = plan.execute(D, c, outputs="gamma")[0]
+    g1 = plan.execute_multi(D[None].contiguous(), None, outputs="gamma")[0][0]
+    assert (g - g1).abs().max() <= 1e-13 * g.abs().max()
+    best = 1e30
+    for _ in range(6):
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        e[0].record()
+        plan.execute(D, c, outputs="gamma")
+        e[1].record()
+        torch.cuda.synchronize()
+        best = min(best, e[0].elapsed_time(e[1]))
+    assert best < 0.75, best
