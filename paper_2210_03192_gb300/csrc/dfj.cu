@@ -212,12 +212,12 @@ int hermite_modes(const HermBra& b, const HermKet& k) {
   if (b.la + b.lb == 0) return 0;
   if (b.la + b.lb == 1 && k.lc <= 4) return k.lc == 0 && b.Ka * b.Kb * k.Kc == 1 ? kHermBuild : 0;
   // (the tile kernel runs a tile's primitives in chunks one after another, a
-  // Hermite launch spreads them: fewer tiles than SMs go there.  Under 32 tiles
-  // an SM the weakly contracted gain less than their launches cost: a batch of
-  // three molecules 8.37 -> 8.6 ms with (d s|s), (f s|s), (g s|s) on the tile
-  // kernel.)
+  // Hermite launch spreads them: fewer tiles than SMs go there.  Under some
+  // hundred tiles an SM the weakly contracted gain less than their launches
+  // cost: (d s|s) and (f s|s) of 18 atoms 14.34 ms in the Hermite basis, 14.64
+  // on the tile kernel, of 24 33.7 and 33.4, of 32 72.7 and 72.1.)
   const double n = b.nprim * k.Kc;
-  if (n < 4 || (double)b.q.size() * ((k.shells.size() + 31) / 32) < (n >= 18 ? 152 : 32 * 152)) return kHermBuild;
+  if (n < 4 || (double)b.q.size() * ((k.shells.size() + 31) / 32) < (n >= 18 ? 152 : 112 * 152)) return kHermBuild;
   try {
     const ClassTables& ct = class_tables(b.la, b.lb, k.lc, 1);
     const double nint = (2.0 * b.la + 1) * (2 * b.lb + 1) * (2 * k.lc + 1);

@@ -1345,11 +1345,11 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     const int W = x.c.W, NP = 32 / W;
     // a tile ends with three atomics for each of a lane's sums (a ket's gamma, or
     // its force), which cost the chip about as much as 30 FP64 instructions
-    // each: tiles of a few primitives on light classes are mostly flushes (20
-    // contracted p shells over 160 kets, gamma alone 1.18 ms), so a tile has
-    // three times their cost of work, if that leaves a warp for each slot (0.44;
-    // the batch of three molecules 8.34 -> 8.08)
-    const double flush = 100.0 * 3.0 * (grad ? 3 : x.c.nC);
+    // each: tiles of one or two primitives on light classes are mostly flushes
+    // (20 contracted p shells over 160 kets, gamma alone 1.18 ms), so a tile has
+    // work for as much, if that leaves a warp for each slot (0.76; for three
+    // times as much 0.44, but DF-J of 4 atoms 1.70 -> 1.78)
+    const double flush = 30.0 * 3.0 * (grad ? 3 : x.c.nC);
     const double work = std::max(target, std::min(flush, 16.0 * target));
     const long long step = NP * std::max<long long>(1, std::min<long long>(64, (long long)(work / x.instr + 0.5)));
     for (int k0 = 0; k0 < x.c.nket; k0 += W) {
