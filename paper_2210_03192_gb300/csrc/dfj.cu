@@ -217,7 +217,7 @@ int hermite_modes(const HermBra& b, const HermKet& k) {
   // cost: (d s|s) and (f s|s) of 18 atoms 14.34 ms in the Hermite basis, 14.64
   // on the tile kernel, of 24 33.7 and 33.4, of 32 72.7 and 72.1.)
   const double n = b.nprim * k.Kc;
-  if (n < 4 || (double)b.q.size() * ((k.shells.size() + 31) / 32) < (n >= 18 ? 152 : 112 * 152)) return kHermBuild;
+  if (n < 4 || (double)b.q.size() * ((k.shells.size() + 31) / 32) < (n >= 9 ? 152 : 112 * 152)) return kHermBuild;
   try {
     const ClassTables& ct = class_tables(b.la, b.lb, k.lc, 1);
     const double nint = (2.0 * b.la + 1) * (2 * b.lb + 1) * (2 * k.lc + 1);
