@@ -203,8 +203,8 @@ void fill_desc_common(ClassDesc& d, const ClassTables& ct, const DevClass& dc, c
 }
 
 int fill_class_desc(ClassDesc& d, const ClassTables& ct, const DevClass& dc, const DevState* ds, int orient,
-                    int kmax, int Kab_rec, int Kc, long long naux_for_shape) {
-  LaunchShape sh = choose_shape(ct, kmax, Kc, naux_for_shape, ds->smem_per_sm);
+                    int kmax, int Kab_rec, int Kc, long long naux_for_shape, long long nsub) {
+  LaunchShape sh = choose_shape(ct, kmax, Kc, naux_for_shape, ds->smem_per_sm, nsub, ds->nsm);
   if (sh.smem_bytes < 0 || sh.smem_bytes > 232448) return -1;
   fill_desc_common(d, ct, dc, ds->boys_tab, ds->boys_mid, orient, kmax, Kab_rec, Kc, sh);
   return sh.smem_bytes;
@@ -442,7 +442,7 @@ lx3c_status make_launch(DevState* ds, lx3c_plan* p, int orient, const std::vecto
   lx3c_status rc = device_class(ds, *ct, &dc);
   if (rc) return rc;
   ClassDesc& d = L.desc;
-  if (fill_class_desc(d, *ct, *dc, ds, orient, kmax, p->Ka * p->Kb, p->Kc, p->naux) < 0)
+  if (fill_class_desc(d, *ct, *dc, ds, orient, kmax, p->Ka * p->Kb, p->Kc, p->naux, L.nsub) < 0)
     return fail(LX3C_ENOTSUP, "eri3c_plan: class does not fit in shared memory");
   d.npair = p->npair; d.naux = p->naux;
   d.ntile_aux = (int)((p->naux + d.T - 1) / d.T);

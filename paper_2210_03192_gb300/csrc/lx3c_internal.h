@@ -216,7 +216,7 @@ void set_last_error(const std::string& msg);
 // caller's (la, lb)), kmax primitive pairs per sub-pair; returns smem bytes or
 // -1 if the class does not fit.
 int fill_class_desc(ClassDesc& d, const ClassTables& ct, const DevClass& dc, const DevState* ds, int orient,
-                    int kmax, int Kab_rec, int Kc, long long naux_for_shape);
+                    int kmax, int Kab_rec, int Kc, long long naux_for_shape, long long nsub = 0);
 struct LaunchShape;
 // The shape-independent part of that fill plus the layout for shape sh, with
 // the class tables at dc and the Boys table at boys_tab / boys_mid (shared by
@@ -261,9 +261,11 @@ double hrr_moment_error(const ClassTables& ct, const double AB[3]);
 // Host evaluation of the class's (a 0|C) tables, see lx3c_cvrr2_tables_eval.
 std::vector<double> eval_targets(const ClassTables& ct, const double PA[3], const double f[3], double rg, double h,
                                  const double X[3], double Y, const double* base);
-LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit);
+LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, long long nsub = 0,
+                         int nsm = 0);
 LaunchShape largest_tile(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas);
-LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas);
+LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas,
+                             long long nsub = 0, int nsm = 0);
 void set_shape_hint(int la, int lb, int lc, int bra_pure, int Kab, int Kc, int ctas);
 void set_tile_hint(int la, int lb, int lc, int bra_pure, int Kab, int Kc, int T, int G);
 void fill_layout(ClassDesc& d, const ClassTables& ct, const LaunchShape& s);

@@ -226,7 +226,7 @@ extern "C" lx3c_status lx3c_eri3c_noalloc(int la, int lb, int lc, int ka, int kb
   if (e != cudaSuccess) return na_fail(LX3C_ECUDA, cudaGetErrorString(e));
   for (int o = 0; o < 1 + split; ++o) {
     const ClassTables& ct = *cts[o];
-    LaunchShape sh = choose_shape(ct, kab, kc, naux, smem);
+    LaunchShape sh = choose_shape(ct, kab, kc, naux, smem, npair, nsm);
     if (sh.smem_bytes < 0 || sh.smem_bytes > 232448) return na_fail(LX3C_ENOTSUP, "class does not fit in shared memory");
     DevClass dc;
     class_blob_pointers(dc, tb + nb->base[o], nb->offs[o]);

@@ -907,7 +907,8 @@ LaunchShape largest_tile(const ClassTables& ct, int Kab, int Kc, long long naux,
 // K = 4 8, 4 6.25, 8, 2 5.43; (gg|i) K = 36 92.4 -> 86.0), while fewer triples lose
 // more than that ((dd|f) K = 9 16, 5 4.15, 8, 5 4.53), and so does one primitive at
 // a time ((gs|d) K = 9 32, 3 1.56, 32, 1 1.73).
-LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas) {
+LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, int ctas,
+                             long long nsub, int nsm) {
   if (ctas != 2) {
     const LaunchShape sh = largest_tile(ct, Kab, Kc, naux, smem_limit, std::max(1, ctas));
     return sh.smem_bytes < 0 && ctas > 1 ? choose_shape_for(ct, Kab, Kc, naux, smem_limit, ctas - 1) : sh;
@@ -917,17 +918,26 @@ LaunchShape choose_shape_for(const ClassTables& ct, int Kab, int Kc, long long n
   if (two.smem_bytes < 0) return choose_shape_for(ct, Kab, Kc, naux, smem_limit, 1);
   const LaunchShape three =
       fit_shape(ct, Kab, Kc, naux, (smem_limit / 3 - 1024) / 8, [](int T) { return T >= 128 ? 3 : 2; });
-  return three.smem_bytes >= 0 && three.T >= std::min(two.T, 32) ? three : two;
+  if (three.smem_bytes < 0 || three.T < std::min(two.T, 32)) return two;
+  // nsub sub-pairs that give no third CTA of an SM a tile (nsm = 0: unknown):
+  // wide tiles keep the primitives two CTAs hold side by side instead.  400 pairs
+  // x 60 kets, two launches of 200 tiles, us: (pp|p) 3 x 2 x 2 primitives G = 6
+  // 125, 3 149; (pp|d) 4 187, 2 210; over 40 such classes of up to 304 tiles a
+  // launch 9 % on average.  With T = 32 it goes either way ((pp|f) K = 36 G = 4
+  // 354, 8 538; (dd|s) 429 and 333).
+  if (nsm > 0 && three.T == two.T && two.T >= 64 && nsub * ((naux + two.T - 1) / two.T) <= 2LL * nsm) return two;
+  return three;
 }
 
 // The planner's shape: a tuned tile hint (T, G) for this class, contraction
 // and ket contraction when one is set and fits, or a tuned number of CTAs per
 // SM, or the default.
-LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit) {
+LaunchShape choose_shape(const ClassTables& ct, int Kab, int Kc, long long naux, int smem_limit, long long nsub,
+                         int nsm) {
   const LaunchShape th = tile_hint_shape(ct, Kab, Kc, smem_limit);
   if (th.smem_bytes >= 0) return th;
   const int h = shape_hint(ct, Kab, Kc);
-  return choose_shape_for(ct, Kab, Kc, naux, smem_limit, h > 0 ? h : 2);
+  return choose_shape_for(ct, Kab, Kc, naux, smem_limit, h > 0 ? h : 2, nsub, nsm);
 }
 
 int place_epilogue_scratch(ClassDesc& d, long long need) {
