@@ -336,11 +336,12 @@ lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap
  *   class's scratch does not fit.  Asynchronous.
  * lx3c_dfj_energy: gamma as above (J skipped) and *energy = c^T gamma
  *   (device scalar), the DF-J energy whose gradient lx3c_dfj_grad returns.
- * lx3c_dfj_info: out[0..10] = groups, screened (pair, ket shell) triples,
+ * lx3c_dfj_info: out[0..11] = groups, screened (pair, ket shell) triples,
  *   integrals digested, algorithmic FP64 flops per execute, kernel launches
  *   per execute, nao, naux_ao, natom, gradient FP64 flops, gradient launches,
  *   tile slots of the integral launches (screened triples / slots is the
- *   tile fill).
+ *   tile fill), an upper bound of the contributions to one atom's force
+ *   accumulators (below 2^32, or lx3c_dfj_plan refuses; 0 without gradient).
  * lx3c_dfj_grad: dE/dR for E = c^T gamma with D and c held fixed (not in the
  *   paper), in the Hermite Gaussian basis: per screened triple the potential
  *   y_a = sum_P (Lambda_a|P) c_P up to |a| = la + lb + 1 and the force on the

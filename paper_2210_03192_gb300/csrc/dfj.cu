@@ -758,8 +758,8 @@ lx3c_status lx3c_dfj_info(const lx3c_dfj* p, double* out, int n) {
   }
   launches += p->njobs_mode[3] > 0;
   const double v[] = {(double)p->groups.size(), tasks, nint, flops, launches, (double)p->nao, (double)p->naux_ao,
-                      (double)p->natom, gflops, glaunches, slots};
-  for (int i = 0; i < n && i < 11; ++i) out[i] = v[i];
+                      (double)p->natom, gflops, glaunches, slots, p->hg ? herm_max_adds(p->hg) : 0.0};
+  for (int i = 0; i < n && i < 12; ++i) out[i] = v[i];
   return LX3C_OK;
 }
 

@@ -1327,6 +1327,10 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     return oa != ob ? oa < ob : cls[a].instr > cls[b].instr;
   });
   std::vector<int4> tiles;
+  int natom = 1;
+  for (int a : orb->atom) natom = std::max(natom, a + 1);
+  for (int a : aux->atom) natom = std::max(natom, a + 1);
+  std::vector<double> adds(natom, 0.0);  // contributions to each atom's force accumulators
   const double target = total / (dev_nsm(ds) * 8 * 16.0);
   int bin = -1;
   const int bins[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32};
@@ -1359,6 +1363,9 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       const long long ne = L.prim0[np];
       for (long long e = 0; e < ne; e += step)
         tiles.push_back(int4{ci, k0, (int)e, (int)std::min<long long>(step, ne - e)});
+      if (grad)  // one contribution per axis from each lane with the ket, of each warp
+        for (int q = k0; q < std::min(k0 + W, x.c.nket); ++q)
+          adds[aux->atom[kets[x.ket].shells[q]]] += (double)((ne + step - 1) / step) * NP * std::max(x.c.nw, 1);
     }
     t.n = (long long)tiles.size() - t.first;
   }
@@ -1367,7 +1374,11 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       set_last_error("dfj: too many tiles");
       return LX3C_ENOTSUP;
     }
-  p->max_adds = 4 * 32.0 * (double)tiles.size() + 2.0 * (double)p->npair * p->nchunk;
+  if (grad) {
+    for (const int4& q : pairs)
+      for (int s : {q.x, q.y}) adds[orb->atom[s]] += p->nchunk;
+    p->max_adds = *std::max_element(adds.begin(), adds.end());
+  }
   // ---- one allocation: tables and lists (uploaded), then the work buffers
   std::vector<double> sph;
   std::vector<int> sphoff;
