@@ -136,8 +136,8 @@ void lx3c_plan_destroy(lx3c_plan* plan);
  * tables, lists and the output are host memory; device memory is allocated
  * and freed inside the call, which synchronises `stream` before returning.
  * out_host receives npair*naux*nA*nB*nC doubles (same layout as execute).
- * The output is produced in pair-range chunks of about 512 MB that alternate
- * between two device buffers; each chunk is copied to out_host on a second
+ * The output is produced in pair-range chunks, a quarter of it each within 64
+ * to 512 MB, that alternate between two device buffers; each chunk is copied to out_host on a second
  * stream while the next is computed, so the device holds two chunks, not the
  * whole output.  The two buffers (at most ~1 GB, or two pairs' blocks if
  * larger), the copy stream and its events are made on the first call and
@@ -301,8 +301,9 @@ lx3c_status lx3c_cvrr2_expansion(const int32_t* a, const int32_t* c, int32_t cap
  *   (Sec. 4).  Every plan does so where it is the faster form: in a Hermite
  *   Gaussian basis, gamma_P = sum_a H_a (Lambda_a|P) with H the pair's
  *   density in Hermite Gaussians and J_ab = sum_a E^ab_a sum_P (Lambda_a|P) c_P,
- *   for all classes but (s s|C) and (p s|C), lc <= 4, whose integrals are
- *   digested one by one.  The flag is accepted and changes nothing.
+ *   for all classes but (s s|C) and (p s|C), lc <= 4, and strongly contracted
+ *   ones of low angular momentum, whose integrals are digested one by one.
+ *   The flag is accepted and changes nothing.
  *   Screening: a (pair, ket) triple is kept when Q_ab Q_P >= schwarz_tol, with
  *   Q_ab = 20 sum over primitive pairs of |c_a c_b| exp(-za zb/g AB^2)
  *   sqrt(2 pi^{5/2}/(g^2 sqrt(2g))) (|PA|^2+1/(2g))^{la/2} (|PB|^2+1/(2g))^{lb/2}
@@ -424,7 +425,7 @@ void lx3c_dfj_destroy(lx3c_dfj* plan);
  * lx3c_cholesky: in-place Cholesky V = L L^T of the symmetric positive
  *   definite A (device, n x n row-major, leading dimension lda >= n), reading
  *   and writing only the lower triangle (the strictly upper triangle is left
- *   as it was).  Blocked right-looking, 64-wide panels, FP64 throughout.
+ *   as it was).  Blocked right-looking, 32-wide panels, FP64 throughout.
  *   info (device int32, may be NULL) is set to 0, or to the 1-based index of
  *   the first non-positive pivot (the factor then holds NaN from there on).
  *   drop_tol = 0: info gets the first non-positive pivot as above.

@@ -192,43 +192,38 @@ int kets_kept(double qpair, const std::vector<double>& qket, double tol) {
   return lo;
 }
 
-// The modes (hermite.h) in which a group runs in the Hermite basis: all, except
-// where its integrals cost less.  The Hermite form pays its contractions per
-// primitive triple, where the digestion of integrals is a few FMAs per
-// contracted one: the groups with a register-resident class kernel, (s s|C) and
-// (p s|C) with lc <= 4 (contracted when lc = 0), never do, and strongly
-// contracted ones of low angular momentum not in every mode.  For these the
-// line is drawn on operation counts.  Over 197 classes (la, lb <= 4, lc <= 4, 4
-// to 100 primitive triples a triple) the time of the Hermite form over the tile
-// kernel's is, to 13 %, the ratio of their counts (the contracted stages taken
-// 1.5 times), times 0.8 beyond lc = 0; the tile kernel is taken where that makes
-// it a tenth faster, or faster at all for 18 primitive triples and more up to
-// la + lb = 4, where it comes out low.  Both outputs together, ms before and
-// after: (d s|s) K = 36 5.5 and 3.0, (f s|d) 16.1 and 10.6, (p p|s) 4.3 and 2.6,
-// (p p|d) 6.7 and 5.2; left in the Hermite basis: (p p|s) K = 4 0.54 (tile kernel
-// 0.66), (f f|s) K = 36 4.2 (5.3).  gamma alone is the cheaper half of the
-// Hermite form and always its.
-int hermite_modes(const HermBra& b, const HermKet& k) {
-  if (b.la + b.lb == 0) return 0;
-  if (b.la + b.lb == 1 && k.lc <= 4) return k.lc == 0 && b.Ka * b.Kb * k.Kc == 1 ? kHermBuild : 0;
-  // (the tile kernel runs a tile's primitives in chunks one after another, a
-  // Hermite launch spreads them: fewer tiles than SMs go there.  Under some
-  // hundred tiles an SM the weakly contracted gain less than their launches
-  // cost: (d s|s) and (f s|s) of 18 atoms 14.34 ms in the Hermite basis, 14.64
-  // on the tile kernel, of 24 33.7 and 33.4, of 32 72.7 and 72.1.)
+// Every group runs in the Hermite basis except those whose integrals cost less.
+// The Hermite form pays its two contractions per primitive triple, where the
+// digestion of integrals is a few FMAs per contracted one: the groups with a
+// register-resident class kernel, (s s|C) and (p s|C) with lc <= 4 (contracted
+// when lc = 0), and strongly contracted ones of low angular momentum.  For these
+// the line is drawn on operation counts.  Over 197 classes (la, lb <= 4, lc <= 4,
+// 4 to 100 primitive triples a triple) the time of the Hermite form over the
+// tile kernel's, gamma and J together, is, to 13 %, the ratio of their counts
+// (the contracted stages taken 1.5 times), times 0.8 beyond lc = 0; the tile
+// kernel is taken where that makes it a fifth faster (three tenths with two
+// shells above s, where it scatters more).  ms before and after:
+// (d s|s) K = 36 5.5 and 3.0, (f s|d) 16.1 and 10.6, (p p|s) 4.3 and 2.6; left in
+// the Hermite basis: (p p|s) K = 4 0.54 (tile kernel 0.66), (f f|s) K = 36 4.2
+// (5.3).  One route for every output: gamma or J alone are bit for bit those of
+// both, which costs gamma alone, 0.6 of the Hermite form, up to a quarter at the
+// line and little for lc = 0 ((p p|s) K = 36 2.51 and 2.57).
+// Fewer than 12 primitive triples gain little and fewer tiles than SMs lose: the
+// tile kernel runs a tile's primitives in chunks one after another, a Hermite
+// launch spreads them ((d s|s) and (f s|s), K = 6, of 18 atoms 14.34 ms in the
+// Hermite basis, 14.64 on the tile kernel).
+bool use_hermite(const HermBra& b, const HermKet& k) {
+  if (b.la + b.lb == 0) return false;
+  if (b.la + b.lb == 1) return k.lc > 4 || (k.lc == 0 && b.Ka * b.Kb * k.Kc == 1);
   const double n = b.nprim * k.Kc;
-  if (n < 4 || (double)b.q.size() * ((k.shells.size() + 31) / 32) < (n >= 9 ? 152 : 112 * 152)) return kHermBuild;
+  if (n < 12 || b.q.size() * ((k.shells.size() + 31) / 32) < 152) return true;
   try {
     const ClassTables& ct = class_tables(b.la, b.lb, k.lc, 1);
     const double nint = (2.0 * b.la + 1) * (2 * b.lb + 1) * (2 * k.lc + 1);
     const double tile = ct.flops_prim * n + 1.5 * (ct.flops_contr + 4.0 * nint);
-    const double least = n >= 18 && b.la + b.lb <= 4 ? 1.0 : 1.1;
-    int modes = 1 << 1;
-    for (int mode = 2; mode <= 3; ++mode)
-      if ((k.lc == 0 ? 1.0 : 0.8) * n * herm_class_flops(b.la + b.lb, k.lc, mode) < least * tile) modes |= 1 << mode;
-    return modes;
+    return (k.lc == 0 ? 1.0 : 0.8) * n * herm_class_flops(b.la + b.lb, k.lc) < (b.lb ? 1.3 : 1.2) * tile;
   } catch (std::exception&) {
-    return kHermBuild;  // no tile kernel for the class
+    return true;  // no tile kernel for the class
   }
 }
 
@@ -315,10 +310,9 @@ struct DfjGroup {
   double* d_auxrec = nullptr;
   double* d_auxc = nullptr;
   DfjLaunch L[2];
-  // the modes in which the group runs in the Hermite basis; its class launches
-  // L serve the others and the several-density build
-  int herm = 0;
-  bool hermite(int mode) const { return herm >> mode & 1; }
+  // the group runs in the Hermite basis; its class launches L serve the
+  // several-density build alone
+  bool herm = false;
 };
 
 }  // namespace
@@ -332,11 +326,10 @@ struct lx3c_dfj {
   int nsm = 0;
   bool gradient = false;
   std::vector<DfjGroup> groups;
-  // records of every group: those never in the Hermite basis first, then those
-  // sometimes; a mode takes as many as it runs class launches of
+  // records of every group: the groups outside the Hermite basis first
   PrecomputeJob* d_jobs = nullptr;
-  int njobs = 0, njobs_mode[4] = {0, 0, 0, 0};
-  long long job_blocks = 0, job_blocks_mode[4] = {0, 0, 0, 0};
+  int njobs = 0, njobs_plain = 0;
+  long long job_blocks = 0, job_blocks_plain = 0;
   char* arena = nullptr;            // every device array of the groups, and the accumulators
   HermPlan* hj = nullptr;           // gamma and J of the Hermite groups
   HermPlan* hg = nullptr;           // gradient of every group
@@ -440,7 +433,7 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       g.la = hb.la; g.Ka = hb.Ka;
       g.lb = hb.lb; g.Kb = hb.Kb;
       g.lc = hk.lc; g.Kc = hk.Kc;
-      g.herm = hermite_modes(hb, hk);
+      g.herm = use_hermite(hb, hk);
       g.auxs = hk.shells;
       for (size_t i = 0; i < hb.q.size(); ++i) {
         const int lo = kets_kept(hb.q[i], hk.q, schwarz_tol);
@@ -455,9 +448,9 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       p->groups.push_back(std::move(g));
     }
   }
-  rc = herm_build(&p->hj, orb, aux, hbra, hket, hermite_modes, kets_kept, schwarz_tol, false, p->nao, st);
+  rc = herm_build(&p->hj, orb, aux, hbra, hket, use_hermite, kets_kept, schwarz_tol, false, p->nao, st);
   if (!rc && want_grad)
-    rc = herm_build(&p->hg, orb, aux, hbra, hket, [](const HermBra&, const HermKet&) { return kHermGrad; }, kets_kept,
+    rc = herm_build(&p->hg, orb, aux, hbra, hket, [](const HermBra&, const HermKet&) { return true; }, kets_kept,
                     schwarz_tol, true, p->nao, st);
   if (rc) return rc;
   // contributions to one element of the gradient's fixed-point accumulators
@@ -537,8 +530,8 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
           tris += g.counts[sp.x];
           primtris += (double)g.counts[sp.x] * sp.z * g.Kc;
         }
-        g.flops += g.hermite(3) ? primtris * herm_class_flops(g.la + g.lb, g.lc, 3)
-                                : primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nbra * nket);
+        g.flops += g.herm ? primtris * herm_class_flops(g.la + g.lb, g.lc)
+                          : primtris * ct->flops_prim + tris * (ct->flops_contr + 4.0 * nbra * nket);
       }
       std::vector<int4> tiles;
       for (size_t s = 0; s < sub[o].size(); ++s) {
@@ -602,18 +595,18 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
       d.pair_ao = g.d_pair_ao; d.aux_ao = g.d_aux_ao;
     }
   std::vector<PrecomputeJob> jobs;
-  for (int part = 0; part < 3; ++part)
-    for (auto& g : p->groups) {
-      if (part != (g.herm == 0 ? 0 : (g.herm == kHermBuild ? 2 : 1))) continue;
-      jobs.push_back(PrecomputeJob{g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
-                                   g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, p->job_blocks});
-      p->job_blocks += jobs.back().blocks();
-      for (int mode = 1; mode <= 3; ++mode)
-        if (!g.hermite(mode)) {
-          p->njobs_mode[mode] = (int)jobs.size();
-          p->job_blocks_mode[mode] = p->job_blocks;
-        }
+  for (int herm = 0; herm < 2; ++herm) {
+    for (auto& g : p->groups)
+      if ((int)g.herm == herm) {
+        jobs.push_back(PrecomputeJob{g.d_pairs, (long long)g.counts.size(), g.Ka, g.Kb, g.d_pairrec, g.d_pairab,
+                                     g.d_auxs, (long long)g.auxs.size(), g.Kc, g.d_auxrec, g.d_auxc, p->job_blocks});
+        p->job_blocks += jobs.back().blocks();
+      }
+    if (!herm) {
+      p->njobs_plain = (int)jobs.size();
+      p->job_blocks_plain = p->job_blocks;
     }
+  }
   p->njobs = (int)jobs.size();
   if (!jobs.empty())
     DCUDA(cudaMemcpyAsync(p->d_jobs, jobs.data(), jobs.size() * sizeof(PrecomputeJob), cudaMemcpyHostToDevice, st));
@@ -622,11 +615,11 @@ lx3c_status lx3c_dfj_plan(lx3c_dfj** out, const lx3c_basis* orb, const lx3c_basi
   return LX3C_OK;
 }
 
-// The pair and ket records of a plan's groups: those of the mode's class
-// launches, or of all (mode 0).
-static cudaError_t group_records(const lx3c_dfj* p, int mode, cudaStream_t st) {
-  return launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->d_jobs, mode ? p->njobs_mode[mode] : p->njobs,
-                                mode ? p->job_blocks_mode[mode] : p->job_blocks, st);
+// The pair and ket records of a plan's groups (all, or those that do not run in
+// the Hermite basis).
+static cudaError_t group_records(const lx3c_dfj* p, bool all, cudaStream_t st) {
+  return launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->d_jobs, all ? p->njobs : p->njobs_plain,
+                                all ? p->job_blocks : p->job_blocks_plain, st);
 }
 
 lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, double* gamma, double* J, void* stream) {
@@ -636,10 +629,9 @@ lx3c_status lx3c_dfj_execute(lx3c_dfj* p, const double* D, const double* c, doub
   if (gamma) DCUDA(cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, st));
   if (J) DCUDA(cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, st));
   if (p->hj) DCUDA(herm_execute(p->hj, D, c, gamma ? p->d_gacc : nullptr, J ? p->d_Jacc : nullptr, st));
-  const int mode = (gamma ? 1 : 0) | (J ? 2 : 0);
-  DCUDA(group_records(p, mode, st));
+  DCUDA(group_records(p, false, st));
   for (auto& g : p->groups) {
-    if (g.hermite(mode)) continue;
+    if (g.herm) continue;
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
       ClassDesc d = L.desc;
@@ -693,7 +685,7 @@ lx3c_status lx3c_dfj_execute_multi(lx3c_dfj* p, int nd, const double* D, const d
   if (gamma) DCUDA(cudaMemsetAsync(gamma, 0, (size_t)nd * cstride * 8, st));
   if (J) DCUDA(cudaMemsetAsync(J, 0, (size_t)nd * dstride * 8, st));
   size_t li = 0;
-  DCUDA(group_records(p, 0, st));
+  DCUDA(group_records(p, true, st));
   for (auto& g : p->groups) {
     for (auto& L : g.L) {
       if (!L.ntiles) continue;
@@ -754,9 +746,9 @@ lx3c_status lx3c_dfj_info(const lx3c_dfj* p, double* out, int n) {
     tasks += (double)g.ntasks;
     nint += g.nint;
     flops += g.flops;
-    if (!g.hermite(3)) launches += (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
+    if (!g.herm) launches += (g.L[0].ntiles > 0) + (g.L[1].ntiles > 0);
   }
-  launches += p->njobs_mode[3] > 0;
+  launches += p->njobs_plain > 0;
   const double v[] = {(double)p->groups.size(), tasks, nint, flops, launches, (double)p->nao, (double)p->naux_ao,
                       (double)p->natom, gflops, glaunches, slots, p->hg ? herm_max_adds(p->hg) : 0.0};
   for (int i = 0; i < n && i < 12; ++i) out[i] = v[i];
@@ -890,8 +882,8 @@ cudaError_t capture_branches(lx3c_batch* b, const std::vector<ClassDesc>& descs,
       lx3c_dfj* p = b->mols[m];
       cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
       cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
-      group_records(p, 3, cap);
-      kernels += p->njobs_mode[3] > 0;
+      group_records(p, false, cap);
+      kernels += p->njobs_plain > 0;
     }
     cudaEventRecord(fork, cap);
     double load[kBranches] = {};
@@ -1095,9 +1087,9 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
   b->plain_launches = 0;
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];
-    b->plain_launches += 2 + (p->njobs_mode[3] > 0) + (p->hj ? herm_launches(p->hj) : 0);
+    b->plain_launches += 2 + (p->njobs_plain > 0) + (p->hj ? herm_launches(p->hj) : 0);
     for (auto& g : p->groups) {
-      if (g.hermite(3)) continue;
+      if (g.herm) continue;
       for (auto& L : g.L) {
         if (!L.ntiles) continue;
         ++b->plain_launches;
@@ -1155,8 +1147,8 @@ lx3c_status lx3c_batch_bind(lx3c_batch* b, const double* const* D, const double*
     lx3c_dfj* p = b->mols[m];
     cudaMemsetAsync(p->d_gacc, 0, p->naux_ao * kFixBytes, cap);
     cudaMemsetAsync(p->d_Jacc, 0, p->nao * p->nao * kFixBytes, cap);
-    group_records(p, 3, cap);
-    b->graph_kernels += p->njobs_mode[3] > 0;
+    group_records(p, false, cap);
+    b->graph_kernels += p->njobs_plain > 0;
   }
   for (int m = 0; m < nmol; ++m) {
     lx3c_dfj* p = b->mols[m];

@@ -1,7 +1,7 @@
 // Device kernels for contracted 3-center Coulomb integrals (ab|C)
 // (arXiv:2210.03192, HGPA scheme of Sec. 2.5.1):
-//   pair_precompute  primitive-pair quantities gamma, P, PA, K_ab (Appendix A)
-//   aux_precompute   ket primitive records
+//   precompute_kernel  primitive-pair records gamma, P, PA, K_ab (Appendix A) and
+//                    ket primitive records; precompute_jobs_kernel many lists
 //   eri3c_kernel     per tile of (one pair, T ket shells):
 //                      [00|0]^(m) from the Boys function       Sec. 2.5.2
 //                      VRR1                                      Eq. vrr1
@@ -83,8 +83,8 @@ __device__ __forceinline__ void dmma_8x8x4(double a, double b, double& c0, doubl
 }
 
 // pref * F_m(T) for m = hi down to lo, written to v[(m - lo) * stride].
-// F_hi and exp(-T) come from the interpolation table (T < 117) or the
-// asymptotic form (T >= 117, exp(-T) = 0); lower orders by the downward
+// F_hi and exp(-T) come from the interpolation table (T < 2^24; exp(-T) = 0
+// from 117 on) or the asymptotic form beyond; lower orders by the downward
 // relation (2m+1) F_m = 2T F_{m+1} + exp(-T).
 __device__ __forceinline__ void boys_scaled(const double* __restrict__ tab, const double* __restrict__ mid,
                                             double cL, int hi, int lo, double T, double pref, double* v,

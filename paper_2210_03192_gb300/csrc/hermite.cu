@@ -1049,10 +1049,8 @@ struct HermPlan {
   const lx3c_basis* aux = nullptr;
   bool grad = false;
   long long nao = 0, npair = 0, nprim = 0;
-  long long npair_mode[5] = {0, 0, 0, 0, 0};  // leading pairs with a class in each mode
   struct Tier {
     int smem, nw, Lab;  // nw = 0: the unrolled kernel of this Lab
-    int modes;          // in which it runs (mask)
     long long first, n;
   };
   std::vector<Tier> tiers;
@@ -1074,26 +1072,21 @@ void herm_destroy(HermPlan* p) {
   delete p;
 }
 
-int herm_launches(const HermPlan* p) {
-  int n = 3;
-  for (auto& t : p->tiers) n += t.modes >> (p->grad ? 4 : 3) & 1;
-  return n;
-}
+int herm_launches(const HermPlan* p) { return 3 + (int)p->tiers.size(); }
 double herm_flops(const HermPlan* p) { return p->flops; }
 double herm_max_adds(const HermPlan* p) { return p->max_adds; }
 
-double herm_class_flops(int Lab, int lc, int mode) {
-  const double g = mode & 1, j = mode >> 1 & 1;
+double herm_class_flops(int Lab, int lc) {
   if (herm_unrolled(Lab, lc)) {
     const UnrolledCost u = herm_unrolled_cost(Lab, lc);
-    return 2.0 * (u.base + g * u.gamma + j * u.j);
+    return 2.0 * (u.base + u.gamma + u.j);
   }
   const Program& p = program(Lab, lc, 1);
-  return 2.0 * (p.instr_base + g * p.instr_gamma + j * p.instr_j);
+  return 2.0 * (p.instr_base + p.instr_gamma + p.instr_j);
 }
 
 int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, const std::vector<HermBra>& bras,
-               const std::vector<HermKet>& kets, int (*use)(const HermBra&, const HermKet&), HermKeep keep, double tol,
+               const std::vector<HermKet>& kets, bool (*use)(const HermBra&, const HermKet&), HermKeep keep, double tol,
                bool grad, long long nao, cudaStream_t st) {
   *out = nullptr;
   DevState* ds;
@@ -1101,28 +1094,18 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   if (rc) return rc;
   std::unique_ptr<HermPlan, void (*)(HermPlan*)> p(new HermPlan, herm_destroy);
   p->orb = orb; p->aux = aux; p->grad = grad; p->nao = nao;
-  // lists of pairs of one Lab, most strongly coupled first, so that the pairs
-  // keeping a given ket are a prefix.  A bra class that some ket lists use in
-  // some modes only has a list of its own, and those that both outputs together
-  // use, then J alone, come first: a call's per-pair kernels run the leading
-  // lists it has a class for.
+  // pairs by Lab, most strongly coupled first, so that the pairs keeping a
+  // given ket are a prefix
   struct PairRef { double q; int bra, i; };
-  std::map<std::array<int, 3>, std::vector<PairRef>> byL;  // {modes left out, Lab, bra class + 1 of a list of its own}
-  std::vector<std::vector<int>> uses(bras.size(), std::vector<int>(kets.size()));
+  std::map<int, std::vector<PairRef>> byL;
   for (size_t b = 0; b < bras.size(); ++b) {
-    int any = 0;
-    bool part = false;
-    for (size_t k = 0; k < kets.size(); ++k) {
-      const int m = uses[b][k] = use(bras[b], kets[k]);
-      any |= m;
-      part = part || (m && m != (grad ? kHermGrad : kHermBuild));
-    }
+    bool any = false;
+    for (auto& k : kets) any = any || use(bras[b], k);
     if (!any) continue;
-    const std::array<int, 3> key{grad || (any >> 3 & 1) ? 0 : (any >> 2 & 1 ? 1 : 2), bras[b].la + bras[b].lb, part ? (int)b + 1 : 0};
     for (size_t i = 0; i < bras[b].q.size(); ++i)
-      for (size_t k = 0; k < kets.size(); ++k)
-        if (uses[b][k] && keep(bras[b].q[i], kets[k].q, tol) > 0) {
-          byL[key].push_back(PairRef{bras[b].q[i], (int)b, (int)i});
+      for (auto& k : kets)
+        if (use(bras[b], k) && keep(bras[b].q[i], k.q, tol) > 0) {
+          byL[bras[b].la + bras[b].lb].push_back(PairRef{bras[b].q[i], (int)b, (int)i});
           break;
         }
   }
@@ -1141,13 +1124,14 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     size_t H, Y, prim, scale, o_ab, o_pair;  // arena offsets
   };
   std::vector<LabHost> labs;
-  std::vector<long long> lab_pairs;  // pairs up to the end of each list
+  std::vector<int> laboff(kMaxDeg + 2, -1);
   int smem_pre = 0, smem_post = 0;
   for (auto& kv : byL) {
     LabHost L;
-    L.Lab = kv.first[1];
+    L.Lab = kv.first;
     L.pr = std::move(kv.second);
     std::stable_sort(L.pr.begin(), L.pr.end(), [](const PairRef& a, const PairRef& b) { return a.q > b.q; });
+    laboff[L.Lab] = (int)labs.size();
     for (size_t i = 0; i < L.pr.size(); ++i) {
       const HermBra& b = bras[L.pr[i].bra];
       const int sa = b.pairs[2 * L.pr[i].i], sb = b.pairs[2 * L.pr[i].i + 1];
@@ -1156,7 +1140,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
         return LX3C_ENOTSUP;
       }
       L.prim0.push_back(L.nprim);
-      pairs.push_back(int4{sa, sb, (int)labs.size(), (int)L.nprim});
+      pairs.push_back(int4{sa, sb, laboff[L.Lab], (int)L.nprim});
       {
         // the contributing primitive pairs
         double ab2 = 0, q[LX3C_KMAX * LX3C_KMAX], K[LX3C_KMAX * LX3C_KMAX], qmax = 0;
@@ -1196,7 +1180,6 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     L.prim0.push_back(L.nprim);
     p->nprim += L.nprim;
     labs.push_back(std::move(L));
-    lab_pairs.push_back((long long)pairs.size());
   }
   p->npair = (long long)pairs.size();
   // ranges of primitives: 16 warps an SM's worth of them, four or more each
@@ -1210,7 +1193,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   // classes and their tables
   struct ClsHost {
     HermCls c;
-    int lab, ket, modes;
+    int lab, ket;
     size_t rops, cptr, cent, gptr, gent, pal, ydeg, cnt, st[8][3];
     std::vector<int> counts;
     double instr;
@@ -1226,17 +1209,14 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
       ClsHost x;
       x.lab = (int)li; x.ket = (int)ki;
       x.counts.resize(L.pr.size());
-      x.modes = 0;
       double tri = 0;
+      std::vector<char> used(bras.size());
+      for (size_t b = 0; b < bras.size(); ++b) used[b] = use(bras[b], k);
       for (size_t i = 0; i < L.pr.size(); ++i) {
-        const int m = uses[L.pr[i].bra][ki];
-        x.modes |= m;
-        x.counts[i] = m ? keep(L.pr[i].q, k.q, tol) : 0;
+        x.counts[i] = used[L.pr[i].bra] ? keep(L.pr[i].q, k.q, tol) : 0;
         tri += (double)x.counts[i] * (double)(L.prim0[i + 1] - L.prim0[i]);
       }
       if (tri == 0) continue;
-      for (int m = 1; m <= 4; ++m)
-        if (x.modes >> m & 1) p->npair_mode[m] = std::max(p->npair_mode[m], lab_pairs[li]);
       const int Lp = L.Lab + (grad ? 1 : 0);
       // warps per block: as many as it takes to reach eight on an SM (asking
       // for 12 or 16 leaves short stages with idle queues: DF-J of 32 atoms
@@ -1279,7 +1259,7 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
         return LX3C_ENOTSUP;
       }
       x.smem = smem_of(c.W);
-      if (x.modes >> (grad ? 4 : 3) & 1) p->flops += 2.0 * x.instr * tri;
+      p->flops += 2.0 * x.instr * tri;
       total += x.instr * best / 32.0;
       auto key = std::make_pair(Lp, k.lc);  // (nw follows from them)
       if (first_of.count(key)) {
@@ -1316,10 +1296,9 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
   std::vector<int> order(cls.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
   auto occ = [&](int smem) { return std::min(32, kSmemSm / (smem + 1024)); };
-  // classes of equal modes, block size and occupancy share a launch, the
-  // largest footprint first
+  // classes of equal block size and occupancy share a launch, the largest
+  // footprint first
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-    if (cls[a].modes != cls[b].modes) return cls[a].modes > cls[b].modes;
     if (cls[a].c.nw != cls[b].c.nw) return cls[a].c.nw > cls[b].c.nw;
     if (!cls[a].c.nw)
       return cls[a].c.Lab != cls[b].c.Lab ? cls[a].c.Lab > cls[b].c.Lab : cls[a].instr > cls[b].instr;
@@ -1340,8 +1319,8 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
     int b = 0;
     while (x.c.nw && b + 1 < 10 && bins[b + 1] <= occ(x.smem)) ++b;
     if (!x.c.nw) b = 100 + x.c.Lab;  // one launch per Lab
-    if (b != bin || p->tiers.back().nw != x.c.nw || p->tiers.back().modes != x.modes) {
-      p->tiers.push_back(HermPlan::Tier{0, x.c.nw, x.c.Lab, x.modes, (long long)tiles.size(), 0});
+    if (b != bin || p->tiers.back().nw != x.c.nw) {
+      p->tiers.push_back(HermPlan::Tier{0, x.c.nw, x.c.Lab, (long long)tiles.size(), 0});
       bin = b;
     }
     HermPlan::Tier& t = p->tiers.back();
@@ -1525,10 +1504,9 @@ int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, con
 
 namespace {
 
-dim3 pair_grid(const HermPlan* p, int mode) { return dim3((unsigned)p->npair_mode[mode], (unsigned)p->nchunk); }
+dim3 pair_grid(const HermPlan* p) { return dim3((unsigned)p->npair, (unsigned)p->nchunk); }
 
-cudaError_t herm_begin(HermPlan* p, const double* D, int mode, cudaStream_t st) {
-  const bool dens = mode != 2, y = mode != 1;
+cudaError_t herm_begin(HermPlan* p, const double* D, bool dens, bool y, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (y) e = cudaMemsetAsync(p->arena + p->zero_off, 0, p->zero_bytes, st);
   if (e == cudaSuccess) e = launch_precompute_jobs(p->orb->dev(), p->aux->dev(), p->jobs, p->njobs, p->job_blocks, st);
@@ -1536,16 +1514,15 @@ cudaError_t herm_begin(HermPlan* p, const double* D, int mode, cudaStream_t st) 
   HermPairArgs a = p->pa;
   a.D = D;
   if (p->grad)
-    herm_pre_kernel<true><<<pair_grid(p, mode), 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
+    herm_pre_kernel<true><<<pair_grid(p), 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
   else
-    herm_pre_kernel<false><<<pair_grid(p, mode), 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
+    herm_pre_kernel<false><<<pair_grid(p), 32, p->smem_pre, st>>>(a, dens ? 1 : 0);
   return cudaGetLastError();
 }
 
 template <int kMode>
 cudaError_t herm_tiles(HermPlan* p, HermArgs a, cudaStream_t st) {
   for (auto& t : p->tiers) {
-    if (!(t.modes >> kMode & 1)) continue;
     a.tiles = p->ma.tiles + t.first;
     if (t.nw == 0) {
       const cudaError_t e = launch_herm_unrolled(t.Lab, a, kMode, t.smem, t.n, st);
@@ -1561,9 +1538,7 @@ cudaError_t herm_tiles(HermPlan* p, HermArgs a, cudaStream_t st) {
 
 cudaError_t herm_execute(HermPlan* p, const double* D, const double* c, unsigned long long* gacc,
                          unsigned long long* Jacc, cudaStream_t st) {
-  const int mode = (gacc ? 1 : 0) | (Jacc ? 2 : 0);
-  if (!p->npair_mode[mode]) return cudaSuccess;
-  cudaError_t e = herm_begin(p, D, mode, st);
+  cudaError_t e = herm_begin(p, D, gacc != nullptr, Jacc != nullptr, st);
   if (e != cudaSuccess) return e;
   HermArgs a = p->ma;
   a.cvec = c;
@@ -1575,12 +1550,12 @@ cudaError_t herm_execute(HermPlan* p, const double* D, const double* c, unsigned
   if (e != cudaSuccess || !Jacc) return e;
   HermPairArgs b = p->pa;
   b.Jacc = Jacc;
-  herm_post_kernel<<<pair_grid(p, mode), 32, p->smem_post, st>>>(b);
+  herm_post_kernel<<<pair_grid(p), 32, p->smem_post, st>>>(b);
   return cudaGetLastError();
 }
 
 cudaError_t herm_gradient(HermPlan* p, const double* D, const double* c, unsigned long long* facc, cudaStream_t st) {
-  cudaError_t e = herm_begin(p, D, 4, st);
+  cudaError_t e = herm_begin(p, D, true, true, st);
   if (e != cudaSuccess) return e;
   HermArgs a = p->ma;
   a.cvec = c;
@@ -1591,7 +1566,7 @@ cudaError_t herm_gradient(HermPlan* p, const double* D, const double* c, unsigne
   HermPairArgs b = p->pa;
   b.D = D;
   b.facc = facc;
-  herm_force_kernel<<<pair_grid(p, 4), 32, p->smem_post, st>>>(b);
+  herm_force_kernel<<<pair_grid(p), 32, p->smem_post, st>>>(b);
   return cudaGetLastError();
 }
 

@@ -30,15 +30,10 @@ struct HermPlan;
 // Number of kets of the sorted list that a pair of factor q keeps.
 typedef int (*HermKeep)(double qpair, const std::vector<double>& qket, double tol);
 
-// The outputs of a call: gamma (1), J (2), both (3), the gradient (4).  A set of
-// them is a mask with bit `mode`.
-constexpr int kHermBuild = 1 << 1 | 1 << 2 | 1 << 3, kHermGrad = 1 << 4;
-
-// Build the plan for the (bra, ket) classes, in the modes that use(bra, ket)
-// gives as a mask.  grad: energy gradient (programs one Hermite degree higher).
-// Returns an lx3c_status.
+// Build the plan for the (bra, ket) classes where use(bra, ket) holds.  grad:
+// energy gradient (programs one Hermite degree higher).  Returns an lx3c_status.
 int herm_build(HermPlan** out, const lx3c_basis* orb, const lx3c_basis* aux, const std::vector<HermBra>& bras,
-               const std::vector<HermKet>& kets, int (*use)(const HermBra&, const HermKet&), HermKeep keep, double tol,
+               const std::vector<HermKet>& kets, bool (*use)(const HermBra&, const HermKet&), HermKeep keep, double tol,
                bool grad, long long nao, cudaStream_t st);
 void herm_destroy(HermPlan* p);
 // gamma (gacc) and J (Jacc) into the fixed-point accumulators; either may be null.
@@ -48,7 +43,7 @@ cudaError_t herm_execute(HermPlan* p, const double* D, const double* c, unsigned
 cudaError_t herm_gradient(HermPlan* p, const double* D, const double* c, unsigned long long* facc, cudaStream_t st);
 int herm_launches(const HermPlan* p);       // kernels of one execute (or gradient)
 double herm_flops(const HermPlan* p);       // FP64 flops of one fused execute (or gradient)
-double herm_class_flops(int Lab, int lc, int mode);  // per primitive triple: gamma, J or both fused
+double herm_class_flops(int Lab, int lc);   // per primitive triple, gamma and J fused
 double herm_max_adds(const HermPlan* p);    // upper bound of the additions into one gradient accumulator
 
 }  // namespace lx3c
